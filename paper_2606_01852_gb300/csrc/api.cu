@@ -247,7 +247,7 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
       } else if (sr.cls == TN_CLASS_SPLITK) {
         launch_contract_splitk(a, nbs, cplx, reinterpret_cast<double*>(P.dev + P.off_scratch), st);
       } else {
-        launch_contract_simt(a, nbs, cplx, st);
+        launch_contract_simt(a, nbs, cplx, P.num_sms, st);
       }
       if (P.prof_on) {
         TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(pr.e1), st));

@@ -2,8 +2,7 @@
 //   stage_leaves      : leaf staging and slicing (declared order -> planned order,
 //                       sliced labels fixed per batch entry, complex64 -> planar fp32
 //                       or, for operands of BF16x3 steps, split BF16)
-//   contract_simt     : any pairwise step C[b] = A[b](m x k) . B[b](n x k)^T, FP32 FMA,
-//                       written through the separable row/column offset maps
+//   contract_chain    : a run of tiny pairwise steps in one launch
 //   contract_stream   : big x small steps (n*k tiny), one pass over the big operand
 //   accumulate_root   : compensated FP64 sum of the root over the slice batch; the last
 //                       pass writes the FP64 result and its log scale
@@ -371,144 +370,6 @@ void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, int3
 }
 
 // ---------------------------------------------------------------------------------
-// generic step kernel: 64 x 64 output tile, 16-deep k slices, 256 threads, 4 x 4
-// outputs per thread (rows ty*4.., columns tx + 16j so a half-warp stores 16
-// consecutive columns). MAXPLUS (real only): C = max_k (A + B), -inf padding.
-
-template <bool CPLX, bool MAXPLUS = false>
-__global__ void __launch_bounds__(256) contract_simt_kernel(StepArgs a) {
-  static_assert(!(CPLX && MAXPLUS), "the max-plus semiring is real");
-  const float kZero = MAXPLUS ? __int_as_float(0xff800000) : 0.f;  // the semiring's zero (-inf)
-  constexpr int BM = 64, BN = 64, BK = 16, NP = CPLX ? 2 : 1;
-  __shared__ float As[NP][BK][BM + 4];
-  __shared__ float Bs[NP][BK][BN + 4];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int64_t tiles_n = (a.n + BN - 1) / BN;
-  const int64_t tile = blockIdx.x;
-  const int64_t m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN;
-  const int b = blockIdx.y;
-  const float* A = a.A + b * a.a_bstride;
-  const float* B = a.B + b * a.b_bstride;
-  float* C = a.C + b * a.c_bstride;
-  // this CTA's part of k (all of it unless the step is split, blockIdx.z = part)
-  const int64_t kc = a.ksplit > 1 ? ((a.k + a.ksplit - 1) / a.ksplit + BK - 1) / BK * BK : a.k;
-  const int64_t kbeg = blockIdx.z * kc, kend = kbeg + kc < a.k ? kbeg + kc : a.k;
-  float sa = 1.f, sb = 1.f;
-  if (a.recs) {
-    const ScaleRec* ra = a.recs + a.rec_a + (a.a_bstride ? b : 0);
-    const ScaleRec* rb = a.recs + a.rec_b + (a.b_bstride ? b : 0);
-    sa = pow2_neg(scale_exp(ra));
-    sb = pow2_neg(scale_exp(rb));
-  }
-  float accr[4][4], acci[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) accr[i][j] = acci[i][j] = kZero;
-
-  const int lr = tid >> 2, lk = (tid & 3) * 4;  // loader: row lr, k lk..lk+3
-  for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int64_t kk = k0 + lk + q;
-        const int64_t ra = m0 + lr, rb = n0 + lr;
-        float va = kZero, vb = kZero;
-        if (ra < a.m && kk < kend) va = A[p * a.a_plane + ra * a.k + kk] * sa;
-        if (rb < a.n && kk < kend) vb = B[p * a.b_plane + rb * a.k + kk] * sb;
-        As[p][lk + q][lr] = va;
-        Bs[p][lk + q][lr] = vb;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float ar[4], br[4], ai[4], bi[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        ar[i] = As[0][kk][ty * 4 + i];
-        br[i] = Bs[0][kk][tx + 16 * i];
-        if (CPLX) {
-          ai[i] = As[1][kk][ty * 4 + i];
-          bi[i] = Bs[1][kk][tx + 16 * i];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (CPLX) {
-            accr[i][j] = fmaf(ar[i], br[j], accr[i][j]);
-            accr[i][j] = fmaf(-ai[i], bi[j], accr[i][j]);
-            acci[i][j] = fmaf(ar[i], bi[j], acci[i][j]);
-            acci[i][j] = fmaf(ai[i], br[j], acci[i][j]);
-          } else if (MAXPLUS) {
-            accr[i][j] = fmaxf(accr[i][j], ar[i] + br[j]);
-          } else {
-            accr[i][j] = fmaf(ar[i], br[j], accr[i][j]);
-          }
-        }
-    }
-    __syncthreads();
-  }
-  if (a.ksplit > 1) {
-    // partial tile of this part of k, dense [part][b][plane][m][n]; combined and written
-    // through the offset maps by simt_combine_kernel
-    float* P0 = a.part + ((int64_t(blockIdx.z) * gridDim.y + b) * NP) * a.m * a.n;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int64_t m = m0 + ty * 4 + i;
-      if (m >= a.m) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int64_t n = n0 + tx + 16 * j;
-        if (n >= a.n) continue;
-        P0[m * a.n + n] = accr[i][j];
-        if (CPLX) P0[a.m * a.n + m * a.n + n] = acci[i][j];
-      }
-    }
-    return;
-  }
-  // epilogue through the offset maps
-  int64_t coff[4];
-  bool cok[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int64_t n = n0 + tx + 16 * j;
-    cok[j] = n < a.n;
-    coff[j] = cok[j] ? map_offset(a.cols, n) : 0;
-  }
-  int lmax = -127;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t m = m0 + ty * 4 + i;
-    if (m >= a.m) continue;
-    const int64_t ro = map_offset(a.rows, m);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (!cok[j]) continue;
-      if (CPLX) store_cplx(C, a.c_plane, ro + coff[j], accr[i][j], acci[i][j], a.c_split);
-      else C[ro + coff[j]] = accr[i][j];
-      if (a.recs) lmax = max(lmax, exp_of(CPLX ? fmaxf(fabsf(accr[i][j]), fabsf(acci[i][j]))
-                                               : fabsf(accr[i][j])));
-    }
-  }
-  if (a.recs) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-    ScaleRec* rc = a.recs + a.rec_c + (a.c_bstride ? b : 0);
-    if ((tid & 31) == 0) atomicMax(&rc->emax, lmax);
-    if (tile == 0 && tid == 0) {
-      const ScaleRec* ra = a.recs + a.rec_a + (a.a_bstride ? b : 0);
-      const ScaleRec* rb = a.recs + a.rec_b + (a.b_bstride ? b : 0);
-      rc->log2 = ra->log2 + rb->log2 + scale_exp(ra) + scale_exp(rb);
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------
 // step chains: a run of tiny steps in one CTA. Each step's outputs are spread over the
 // threads (thread = output element, batch entry by batch entry), each summed over k in
 // order with the FMAs of contract_simt_kernel (the same bits); the CTA barrier between
@@ -864,57 +725,6 @@ void launch_stream_tma(const StepArgs& a, int32_t nb, int num_sms, int* err, cud
   int64_t gx = (int64_t(num_sms) * per_sm + nb - 1) / nb;
   gx = std::max<int64_t>(1, std::min<int64_t>(gx, tiles));
   contract_stream_tma_kernel<CPLX, NMAX, K><<<dim3((unsigned)gx, (unsigned)nb), 256, smem, st>>>(a, err);
-}
-
-// Combine the k parts of a split SIMT step in part order (sum, or max for max-plus) and
-// write C through the offset maps. One thread per output element of every batch entry.
-__global__ void simt_combine_kernel(StepArgs a, int32_t nb, int32_t cplx) {
-  const int64_t mn = a.m * a.n, np = cplx ? 2 : 1;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nb * mn;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / mn, o = e - b * mn;
-    const float* P0 = a.part + b * np * mn + o;
-    const int64_t pstride = (int64_t)nb * np * mn;  // one part to the next
-    float vr = P0[0], vi = cplx ? P0[mn] : 0.f;
-    for (int s = 1; s < a.ksplit; ++s) {
-      const float xr = P0[s * pstride];
-      if (a.maxplus) {
-        vr = fmaxf(vr, xr);
-      } else {
-        vr += xr;
-        if (cplx) vi += P0[s * pstride + mn];
-      }
-    }
-    const int64_t i = o / a.n, j = o - i * a.n;
-    const int64_t off = map_offset(a.rows, i) + map_offset(a.cols, j);
-    float* C = a.C + b * a.c_bstride;
-    if (cplx) store_cplx(C, a.c_plane, off, vr, vi, a.c_split);
-    else C[off] = vr;
-  }
-}
-
-int32_t simt_ksplit(int64_t m, int64_t n, int64_t k, int64_t copies, int num_sms, bool scaled) {
-  if (scaled || k < 2048) return 1;
-  // aim at four 256-thread CTAs per SM (the kernel's blocks are short-lived)
-  const int64_t tiles = ((m + 63) / 64) * ((n + 63) / 64) * copies;
-  if (tiles >= 2 * int64_t(num_sms)) return 1;
-  int64_t s = (4 * int64_t(num_sms) + tiles - 1) / tiles;
-  s = std::min<int64_t>(s, k / 1024);
-  s = std::min<int64_t>(s, 32);
-  return s > 1 ? int32_t(s) : 1;
-}
-
-void launch_contract_simt(const StepArgs& a, int32_t nb, bool cplx, cudaStream_t st) {
-  const int64_t tiles = ((a.m + 63) / 64) * ((a.n + 63) / 64);
-  dim3 grid((unsigned)tiles, (unsigned)nb, (unsigned)(a.ksplit > 1 ? a.ksplit : 1));
-  if (cplx) contract_simt_kernel<true><<<grid, 256, 0, st>>>(a);
-  else if (a.maxplus) contract_simt_kernel<false, true><<<grid, 256, 0, st>>>(a);
-  else contract_simt_kernel<false><<<grid, 256, 0, st>>>(a);
-  if (a.ksplit > 1) {
-    const int64_t total = int64_t(nb) * a.m * a.n;
-    const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 4096);
-    simt_combine_kernel<<<blocks, 256, 0, st>>>(a, nb, cplx ? 1 : 0);
-  }
 }
 
 // The bulk-copy form takes k = 4, 8, 16 with the big operand's planes and batch entries

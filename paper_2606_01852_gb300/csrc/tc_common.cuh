@@ -208,10 +208,12 @@ __device__ __forceinline__ void store_run_real(float* C, int64_t off, const floa
 // The address-ordered stores of one block, lanes taking V = 2^VB consecutive addresses.
 // e[k], src[k]: the k-th smallest bit weight (log2) and which bit of r (0-4) or c (5-9)
 // carries it; the VB smallest weights are 1, 2, ..., 2^(VB-1).
-// REAL: a real result, t holds the one plane and C is FP32.
+// REAL: a real result, t holds the one plane and C is FP32. part of parts: the stores this
+// warp makes when several share the block.
 template <int VB, bool REAL = false>
 __device__ __forceinline__ void store_sorted(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
-                                             int64_t base, const int* e, const int* src, int lane) {
+                                             int64_t base, const int* e, const int* src, int lane, int part = 0,
+                                             int parts = 1) {
   constexpr int V = 1 << VB;
   // r and c take disjoint bits, so t's index r * pitch + c is a sum of one increment per
   // set bit: the lane's part, the store's part and, per element of the run, du[u]
@@ -232,7 +234,7 @@ __device__ __forceinline__ void store_sorted(float* C, int64_t plane, int split,
       il += step(VB + k);
       al += int64_t(1) << e[VB + k];
     }
-  for (int s = 0; s < (32 >> VB); ++s) {
+  for (int s = part; s < (32 >> VB); s += parts) {
     int is = il;
     int64_t ah = 0;
 #pragma unroll
@@ -320,19 +322,20 @@ __device__ __forceinline__ BlockOrder block_order(int64_t ro_rel, int64_t co_rel
 // V-aligned; 16 bytes at most).
 template <bool REAL = false>
 __device__ __forceinline__ void store_ordered(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
-                                              int64_t base, const BlockOrder& o, int lane) {
+                                              int64_t base, const BlockOrder& o, int lane, int part = 0,
+                                              int parts = 1) {
   int vb = 0;
   while (vb < (!REAL && split ? 3 : 2) && o.e[vb] == vb) ++vb;
   while (vb > 0 && ((base | plane) & ((int64_t(1) << vb) - 1)) != 0) --vb;
   if constexpr (!REAL) {
     if (vb == 3) {
-      store_sorted<3>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane);
+      store_sorted<3>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
       return;
     }
   }
-  if (vb == 2) store_sorted<2, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane);
-  else if (vb == 1) store_sorted<1, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane);
-  else store_sorted<0, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane);
+  if (vb == 2) store_sorted<2, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
+  else if (vb == 1) store_sorted<1, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
+  else store_sorted<0, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
 }
 
 // Store one 32 x 32 block of a result tile from shared memory (t[r * pitch + c] = Re,
@@ -345,17 +348,19 @@ __device__ __forceinline__ void store_ordered(float* C, int64_t plane, int split
 // following weights continue the sequence (interleaved row/column layouts included).
 // Otherwise (ragged block, other extents) it falls back to one row per store. ro / co:
 // this lane's row / column offset; row_ok / col_ok: in range. REAL: a real FP32 result
-// (one plane in t; plane, split and cs unused).
+// (one plane in t; plane, split and cs unused). part of parts: the share of the stores this
+// warp makes when several warps store one block.
 template <bool REAL = false>
 __device__ __forceinline__ void store_block(float* C, int64_t plane, int split, const float* t, int pitch,
-                                            int cs, int64_t ro, int64_t co, bool row_ok, bool col_ok, int lane) {
+                                            int cs, int64_t ro, int64_t co, bool row_ok, bool col_ok, int lane,
+                                            int part = 0, int parts = 1) {
   const int64_t ro0 = __shfl_sync(0xffffffffu, ro, 0), co0 = __shfl_sync(0xffffffffu, co, 0);
   const BlockOrder o = block_order(ro - ro0, co - co0, row_ok && col_ok, lane);
   if (o.ok) {
-    store_ordered<REAL>(C, plane, split, t, pitch, cs, ro0 + co0, o, lane);
+    store_ordered<REAL>(C, plane, split, t, pitch, cs, ro0 + co0, o, lane, part, parts);
     return;
   }
-  for (int r = 0; r < 32; ++r) {
+  for (int r = part; r < 32; r += parts) {
     const int64_t ro_r = __shfl_sync(0xffffffffu, ro, r);
     const bool ok_r = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, r) != 0;
     if (ok_r && col_ok) {
