@@ -25,8 +25,18 @@ thread_local std::string g_last_error;
     }                                                                             \
   } while (0)
 
-int64_t batch_footprint(Plan& P, int64_t b) {
-  assign_workspace(P, b);
+// Level-ordered chains keep their (small) tensors alive together: they may hold this much, else
+// the chains run in path order.
+constexpr int64_t kLevelOrderBytes = int64_t(64) << 20;
+
+// Assign the workspace for b slices a pass, chains in level order if that fits `budget` and
+// costs little; its size.
+int64_t batch_footprint(Plan& P, int64_t b, int64_t budget) {
+  assign_workspace(P, b, true);
+  int64_t held = 0;
+  for (const StepRec& st : P.steps)
+    if (st.chain >= 0) held += P.tensors[st.out].bytes;
+  if (held > kLevelOrderBytes || P.total_bytes > budget || !P.workspace_ok) assign_workspace(P, b, false);
   return P.total_bytes;
 }
 
@@ -94,16 +104,52 @@ tn_status check_device_error(Plan& P) {
 
 tn_status upload_chain_table(Plan& P) {
   if (P.chains.empty() || !P.dev) return TN_OK;
+  auto packed = [](uint32_t e) {
+    const uint32_t sh = (e & (e - 1u)) == 0u ? static_cast<uint32_t>(__builtin_ctz(e)) : 0xffu;
+    return e | (sh << 24);
+  };
   std::vector<ChainStep> table;
   for (const ChainRec& c : P.chains)
     for (int32_t q = c.first; q < c.first + c.n; ++q) {
+      const StepArgs a = step_args(P, P.steps[q]);
       ChainStep cs{};
-      cs.a = step_args(P, P.steps[q]);
+      cs.A = a.A;
+      cs.B = a.B;
+      cs.C = a.C;
+      cs.recs = a.recs;
+      cs.n = (int32_t)a.n;
+      cs.n_shift = (a.n & (a.n - 1)) == 0 ? __builtin_ctzll((unsigned long long)a.n) : -1;
+      cs.k = (int32_t)a.k;
+      cs.a_plane = (int32_t)a.a_plane;
+      cs.b_plane = (int32_t)a.b_plane;
+      cs.c_plane = (int32_t)a.c_plane;
+      cs.a_bstride = (int32_t)a.a_bstride;
+      cs.b_bstride = (int32_t)a.b_bstride;
+      cs.c_bstride = (int32_t)a.c_bstride;
+      cs.rec_a = a.rec_a;
+      cs.rec_b = a.rec_b;
+      cs.rec_c = a.rec_c;
+      cs.c_split = a.c_split;
       cs.batched = P.steps[q].batched ? 1 : 0;
+      cs.nr = a.rows.n;
+      cs.nc = a.cols.n;
+      for (int d = 0; d < a.rows.n; ++d) {
+        cs.ext[d] = packed(a.rows.ext[d]);
+        cs.stride[d] = (int32_t)a.rows.stride[d];
+      }
+      for (int d = 0; d < a.cols.n; ++d) {
+        cs.ext[kMaxDims + d] = packed(a.cols.ext[d]);
+        cs.stride[kMaxDims + d] = (int32_t)a.cols.stride[d];
+      }
       table.push_back(cs);
     }
   cudaError_t e = cudaMemcpy(P.dev + P.off_chain, table.data(), sizeof(ChainStep) * table.size(),
                              cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(P.dev + P.off_chain_tasks, P.chain_tasks.data(), 4 * P.chain_tasks.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(P.dev + P.off_chain_levels, P.chain_levels.data(), 4 * P.chain_levels.size(),
+                   cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     set_error(std::string("writing the step-chain table: ") + cudaGetErrorString(e));
     return TN_ERR_CUDA;
@@ -214,8 +260,11 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
           }
           TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(pr.e0), st));
         }
-        launch_contract_chain(reinterpret_cast<const ChainStep*>(P.dev + P.off_chain) + c.table, c.n, nb, p > 0,
-                              cplx, P.policy.semiring == TN_SEMIRING_MAXPLUS, st);
+        TN_CUDA_TRY(launch_contract_chain(reinterpret_cast<const ChainStep*>(P.dev + P.off_chain),
+                                          reinterpret_cast<const ChainTask*>(P.dev + P.off_chain_tasks),
+                                          reinterpret_cast<const int32_t*>(P.dev + P.off_chain_levels) + c.level0,
+                                          c.n_levels, c.ctas, nb, p > 0, cplx,
+                                          P.policy.semiring == TN_SEMIRING_MAXPLUS, st));
         if (P.prof_on) {
           TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(pr.e1), st));
           P.prof_pending.push_back(pr);
@@ -339,7 +388,7 @@ tn_status tn_plan(const tn_network* net, const tn_path* path, const int32_t* sli
   want = std::min<int64_t>(want, 65535);  // the batch is a grid dimension
   if (host_only) {
     if (policy.max_slice_batch <= 0) want = 1;
-    assign_workspace(P, want);
+    batch_footprint(P, want, INT64_MAX);
     if (!P.workspace_ok) {
       set_error("internal error: workspace assignment failed its self-check");
       delete h;
@@ -360,8 +409,8 @@ tn_status tn_plan(const tn_network* net, const tn_path* path, const int32_t* sli
   }
   const int64_t budget = int64_t(double(free_b) * 0.9);
   int64_t b = want;
-  while (b > 1 && batch_footprint(P, b) > budget) b = (b + 1) / 2;
-  if (batch_footprint(P, b) > budget || !P.workspace_ok) {
+  while (b > 1 && batch_footprint(P, b, budget) > budget) b = (b + 1) / 2;
+  if (batch_footprint(P, b, budget) > budget || !P.workspace_ok) {
     if (!P.workspace_ok) {
       set_error("internal error: workspace assignment failed its self-check");
       delete h;

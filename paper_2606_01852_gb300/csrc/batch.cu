@@ -530,7 +530,7 @@ tn_status tn_batch_plan(int32_t n_nets, const tn_network* nets, const tn_path* p
       set_error("tn_batch_plan: network " + std::to_string(w) + " has open labels (closed networks only)");
       return TN_ERR_UNSUPPORTED;
     }
-    assign_workspace(P, 1);
+    assign_workspace(P, 1, false);
     if (!P.workspace_ok) {
       set_error("tn_batch_plan: workspace self-check failed");
       return TN_ERR_INVALID;

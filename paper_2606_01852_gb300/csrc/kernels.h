@@ -77,21 +77,40 @@ struct StepArgs {
   float* part;                              // ksplit * nb * planes * m * n floats, or null
 };
 
-// A run of consecutive tiny CUDA-core steps executed by one CTA in one launch (the step
-// chain): each step's StepArgs as for launch_contract_simt, and whether it is batched.
+// A step of a step chain (a run of consecutive tiny CUDA-core steps in one launch): what
+// StepArgs says, in 32 bits where a tiny step fits (kChainMaxWork).
 struct ChainStep {
-  StepArgs a;
-  int32_t batched;
-  int32_t pad;
+  const float* A;
+  const float* B;
+  float* C;
+  ScaleRec* recs;
+  int32_t n, n_shift, k;                    // n_shift: log2 n, -1 when n is not a power of two
+  int32_t a_plane, b_plane, c_plane;
+  int32_t a_bstride, b_bstride, c_bstride;
+  int32_t rec_a, rec_b, rec_c;
+  int32_t c_split, batched, nr, nc;
+  // merged dims: rows at 0 .. nr - 1, columns at kMaxDims .. kMaxDims + nc - 1; the extent in the
+  // low 24 bits, its log2 (0xff: not a power of two) above
+  uint32_t ext[2 * kMaxDims];
+  int32_t stride[2 * kMaxDims];
 };
+// A warp's share of a chain level: outputs first .. first + count - 1 (row-major m x n) of batch
+// entry b of table entry `step`.
+struct ChainTask {
+  int32_t step, first, count, b;
+};
+constexpr int32_t kChainMaxCtas = 16;  // CTAs of a chain's cluster at most (two levels or more)
+constexpr int32_t kChainCtaWarps = 16;
 // A chain step's work bound: m n k (x the slice batch when batched) at most this many
 // multiply-adds (complex ones count four).
 constexpr int64_t kChainMaxWork = int64_t(1) << 16;
-// steps[0 .. n): the run, in path order; nb: slices of this pass; skip_unbatched: a pass
-// after the first (the slice-invariant steps were computed by the first and are kept).
-// Every step's outputs are the same bits as launch_contract_simt's (k summed in order by FMA).
-void launch_contract_chain(const ChainStep* steps, int32_t n, int32_t nb, bool skip_unbatched, bool cplx,
-                           bool maxplus, cudaStream_t st);
+// The chain's table, its tasks sorted by level, level l's being levels[l] .. levels[l + 1] - 1;
+// ctas: the cluster's size (the grid's, for one level); nb: slices of this pass; skip_unbatched: a pass after the first (the
+// slice-invariant steps were computed by the first and are kept). Every step's outputs are the
+// same bits as launch_contract_simt's (k summed in order by FMA).
+cudaError_t launch_contract_chain(const ChainStep* steps, const ChainTask* tasks, const int32_t* levels,
+                                  int32_t n_levels, int32_t ctas, int32_t nb, bool skip_unbatched, bool cplx,
+                                  bool maxplus, cudaStream_t st);
 
 // Small leaves: one CTA per leaf. Large leaves (LeafDesc::tiled): the tiled permutation
 // kernel, one launch per leaf; host_descs is the host copy of the table (grid sizes).

@@ -543,6 +543,82 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
   return TN_OK;
 }
 
+// Step chains: maximal runs (two or more) of consecutive tiny CUDA-core steps, each run one
+// launch instead of a launch per step (launch-bound paths). Its steps are sorted by level --
+// one more than the deepest of their operands made in the run; by position in path order without
+// level_order -- and each level's outputs cut into tasks, about one for each warp of the cluster.
+static void find_chains(Plan& P, int64_t batch, bool level_order) {
+  const int32_t S = (int32_t)P.steps.size(), T = P.n_leaves;
+  for (StepRec& st : P.steps) {
+    st.ksplit = st.cls == TN_CLASS_SIMT ? simt_ksplit(st.m, st.n, st.k, st.batched ? batch : 1, P.num_sms,
+                                                      P.policy.exp_scaling != 0)
+                                        : 1;
+    st.chain = -1;
+  }
+  P.chains.clear();
+  P.chain_tasks.clear();
+  P.chain_levels.clear();
+  const int64_t cw = P.is_complex ? 4 : 1;
+  auto tiny = [&](const StepRec& st) {
+    return st.cls == TN_CLASS_SIMT && st.ksplit == 1 &&
+           double(st.m) * double(st.n) * double(st.k) * double(cw * (st.batched ? batch : 1)) <=
+               double(kChainMaxWork);
+  };
+  int32_t n_table = 0;
+  std::vector<int32_t> level(S, 0);
+  for (int32_t s = 0; s < S;) {
+    int32_t e = s;
+    while (e < S && tiny(P.steps[e])) ++e;
+    if (e - s >= 2) {
+      ChainRec c;
+      c.first = s;
+      c.n = e - s;
+      c.table = n_table;
+      c.level0 = (int32_t)P.chain_levels.size();
+      int32_t deepest = 0;
+      for (int32_t q = s; q < e; ++q) {
+        StepRec& st = P.steps[q];
+        st.chain = (int32_t)P.chains.size();
+        c.any_batched = c.any_batched || st.batched;
+        level[q] = level_order ? 0 : q - s;
+        for (int32_t x : {st.a, st.b})
+          if (level_order && x - T >= s) level[q] = std::max(level[q], level[x - T] + 1);
+        deepest = std::max(deepest, level[q]);
+      }
+      c.n_levels = deepest + 1;
+      std::vector<std::vector<int32_t>> at(c.n_levels);
+      std::vector<int64_t> outs(c.n_levels, 0);
+      for (int32_t q = s; q < e; ++q) {
+        at[level[q]].push_back(q);
+        outs[level[q]] += P.steps[q].m * P.steps[q].n * (P.steps[q].batched ? batch : 1);
+      }
+      // CTAs until the widest level has a lane per output: one cluster's, or (one level, no barrier)
+      // any number
+      const int64_t widest = *std::max_element(outs.begin(), outs.end());
+      const int64_t most = c.n_levels == 1 ? 4096 : kChainMaxCtas;
+      while (c.ctas < most && int64_t(c.ctas) * kChainCtaWarps * 32 < widest) c.ctas *= 2;
+      const int64_t lanes = int64_t(c.ctas) * kChainCtaWarps * 32;
+      for (int32_t l = 0; l < c.n_levels; ++l) {
+        P.chain_levels.push_back((int32_t)(P.chain_tasks.size() / 4));
+        const int64_t per = 32 * ((outs[l] + lanes - 1) / lanes);
+        for (int32_t q : at[l]) {
+          const StepRec& st = P.steps[q];
+          for (int64_t b = 0; b < (st.batched ? batch : 1); ++b)
+            for (int64_t o = 0; o < st.m * st.n; o += per) {
+              const int64_t cnt = std::min(per, st.m * st.n - o);
+              P.chain_tasks.insert(P.chain_tasks.end(),
+                                   {c.table + q - s, (int32_t)o, (int32_t)cnt, (int32_t)b});
+            }
+        }
+      }
+      P.chain_levels.push_back((int32_t)(P.chain_tasks.size() / 4));
+      n_table += c.n;
+      P.chains.push_back(c);
+    }
+    s = e > s ? e : s + 1;
+  }
+}
+
 // Liveness: a leaf is born when the pass stages it (event -1) and a step output at its
 // step; each dies at its consuming step (the root after the final accumulation). Two
 // tensors share memory only if their lifetimes are disjoint. Offsets are static, so
@@ -550,17 +626,28 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
 // first pass, read by every pass) is reserved over the whole timeline [-1, inf]: a
 // tensor that dies before the pinned one is made in the first pass is made again in
 // later passes, and must not land on it.
-void assign_workspace(Plan& P, int64_t batch) {
+void assign_workspace(Plan& P, int64_t batch, bool level_order) {
   P.batch = batch;
   const int32_t T = P.n_leaves, S = (int32_t)P.steps.size();
   const int64_t eb = elem_bytes(P);
   const int32_t N = T + S;
   const int32_t kInf = S + 1;
+  find_chains(P, batch, level_order);
+  // the time a step's output is written from, and its operands are read until: with level order
+  // a chain is one event that lasts from its first step to its last
+  auto writes = [&](int32_t s) {
+    return level_order && P.steps[s].chain >= 0 ? P.chains[P.steps[s].chain].first : s;
+  };
+  auto reads = [&](int32_t s) {
+    if (!level_order || P.steps[s].chain < 0) return s;
+    const ChainRec& c = P.chains[P.steps[s].chain];
+    return c.first + c.n - 1;
+  };
   std::vector<int32_t> birth(N), death(N);
   for (int32_t t = 0; t < N; ++t) {
     TensorRec& R = P.tensors[t];
-    birth[t] = t < T ? -1 : R.producer;
-    death[t] = R.consumer < 0 ? S : R.consumer;
+    birth[t] = t < T ? -1 : writes(R.producer);
+    death[t] = R.consumer < 0 ? S : reads(R.consumer);
     if (R.pinned) {
       birth[t] = -1;
       death[t] = kInf;
@@ -665,14 +752,10 @@ void assign_workspace(Plan& P, int64_t batch) {
   cur += kAlign;
   // split-K partials: the largest need of any split-K step (one pass)
   int64_t scratch = 0;
-  for (StepRec& st : P.steps) {
-    st.ksplit = st.cls == TN_CLASS_SIMT ? simt_ksplit(st.m, st.n, st.k, st.batched ? batch : 1, P.num_sms,
-                                                      P.policy.exp_scaling != 0)
-                                        : 1;
+  for (const StepRec& st : P.steps)
     if (st.ksplit > 1)
       scratch = std::max(scratch, int64_t(st.ksplit) * (st.batched ? batch : 1) * st.m * st.n *
                                       (P.is_complex ? 2 : 1) * 4);
-  }
   for (const StepRec& st : P.steps)
     if (st.cls == TN_CLASS_SPLITK)
       scratch = std::max(scratch, (st.batched ? batch : 1) * ((st.k + kSplitChunk - 1) / kSplitChunk) *
@@ -680,36 +763,13 @@ void assign_workspace(Plan& P, int64_t batch) {
   P.off_scratch = cur;
   P.scratch_bytes = scratch;
   cur += align_up(scratch, kAlign);
-  // step chains: maximal runs (two or more) of consecutive tiny CUDA-core steps, each run
-  // one launch of a single CTA instead of a launch per step (launch-bound paths)
-  P.chains.clear();
-  int32_t n_table = 0;
-  const int64_t cw = P.is_complex ? 4 : 1;
-  auto tiny = [&](const StepRec& st) {
-    return st.cls == TN_CLASS_SIMT && st.ksplit == 1 &&
-           double(st.m) * double(st.n) * double(st.k) * double(cw * (st.batched ? batch : 1)) <=
-               double(kChainMaxWork);
-  };
-  for (StepRec& st : P.steps) st.chain = -1;
-  for (int32_t s = 0; s < (int32_t)P.steps.size();) {
-    int32_t e = s;
-    while (e < (int32_t)P.steps.size() && tiny(P.steps[e])) ++e;
-    if (e - s >= 2) {
-      ChainRec c;
-      c.first = s;
-      c.n = e - s;
-      c.table = n_table;
-      for (int32_t q = s; q < e; ++q) {
-        P.steps[q].chain = (int32_t)P.chains.size();
-        c.any_batched = c.any_batched || P.steps[q].batched;
-      }
-      n_table += c.n;
-      P.chains.push_back(c);
-    }
-    s = e > s ? e : s + 1;
-  }
   P.off_chain = cur;
-  cur += align_up(int64_t(n_table) * (int64_t)sizeof(ChainStep), kAlign);
+  if (!P.chains.empty())
+    cur += align_up(int64_t(P.chains.back().table + P.chains.back().n) * (int64_t)sizeof(ChainStep), kAlign);
+  P.off_chain_tasks = cur;
+  cur += align_up(int64_t(P.chain_tasks.size()) * 4, kAlign);
+  P.off_chain_levels = cur;
+  cur += align_up(int64_t(P.chain_levels.size()) * 4, kAlign);
   P.off_leafdesc = cur;
   cur += align_up(int64_t(T) * (int64_t)sizeof(LeafDesc), kAlign);
   P.off_stage_in = cur;

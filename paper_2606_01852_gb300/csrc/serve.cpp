@@ -188,7 +188,12 @@ struct tn_server_s {
     const bool simt_only = std::all_of(P.steps.begin(), P.steps.end(),
                                        [](const StepRec& st) { return st.cls != TN_CLASS_TC; });
     std::string why;
-    if (simt_only && P.batch == 1 && batch_template(P, pt.T, why)) {
+    Plan path_order;  // the batched kernel runs the steps one after another: the smaller arena
+    if (simt_only && P.batch == 1) {
+      path_order = P;
+      assign_workspace(path_order, 1, false);
+    }
+    if (simt_only && P.batch == 1 && path_order.workspace_ok && batch_template(path_order, pt.T, why)) {
       pt.ok = true;
       const bool maxplus = P.policy.semiring == TN_SEMIRING_MAXPLUS;
       pt.kind = P.is_complex ? 1 : (maxplus ? 4 : (P.policy.exp_scaling ? 3 : 2));

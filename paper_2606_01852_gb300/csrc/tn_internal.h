@@ -89,9 +89,11 @@ struct StepRec {
 };
 
 // A step chain: steps first .. first + n - 1 run in one launch (entries table .. table + n - 1
-// of the device table at off_chain)
+// of the device table at off_chain), level by level: the tasks of its level l are
+// chain_levels[level0 + l] .. chain_levels[level0 + l + 1] - 1
 struct ChainRec {
   int32_t first = 0, n = 0, table = 0;
+  int32_t level0 = 0, n_levels = 0, ctas = 1;
   bool any_batched = false;
 };
 
@@ -124,6 +126,9 @@ struct Plan {
   int64_t off_leafdesc = 0;         // LeafDesc table
   int64_t off_chain = 0;            // ChainStep table of the step chains
   std::vector<ChainRec> chains;
+  std::vector<int32_t> chain_tasks;   // ChainTask, four ints each
+  std::vector<int32_t> chain_levels;
+  int64_t off_chain_tasks = 0, off_chain_levels = 0;
   int64_t off_stage_in = 0;         // device copies of host inputs (tn_contract_host)
   std::vector<int64_t> stage_in_off;
   int64_t total_bytes = 0;
@@ -167,8 +172,10 @@ extern tn_cost_model g_cost;
 // planner (host only)
 tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* sliced,
                      int32_t n_sliced, const tn_dtype_policy& pol, Plan& P, std::string& err);
-// liveness assignment of workspace offsets for a given slice batch
-void assign_workspace(Plan& P, int64_t batch);
+// Liveness assignment of workspace offsets for a given slice batch. level_order: a step chain
+// runs its steps by tree level, so every tensor it touches is alive for the whole chain; else
+// (no chain is launched, or memory is short) tensors live in path order, and chains run in it.
+void assign_workspace(Plan& P, int64_t batch, bool level_order = true);
 
 // executor
 // pinned: null (descriptors copied from pageable host memory, staged before the call
