@@ -817,186 +817,160 @@ void launch_accumulate_root(const float* root, int64_t size, int32_t nb, int64_t
 
 // ---------------------------------------------------------------------------------
 // split-K steps (m*n <= kSplitMaxOut outputs, very long k; e.g. the final scalar of a
-// closed network, a dot product of two large tensors). Pass 1: CTA (chunk, b) sums
-// its k-range for every output -- FP32 over the few terms each thread owns, FP64
-// across threads -- and writes one FP64 partial per output to scratch[b][chunk].
-// Pass 2: per (b, output), the partials are added in chunk order in FP64 and the
-// result stored through the offset maps. Deterministic: no atomics.
+// closed network, a dot product of two large tensors). Pass 1: CTA (chunk, b, output) sums its
+// k-range -- FP32 over the few terms each thread owns, FP64 across threads -- and writes one FP64
+// partial to scratch[b][chunk][output]. Pass 2: per (b, output), the partials are added in chunk
+// order in FP64 and the result stored through the offset maps. Deterministic: no atomics.
+//
+// What bounds it: HBM for one output of a long k, latency for several outputs of a short one.
+// An output has CTAs of its own: one CTA summing all sixteen over 16384 terms left 148 SMs idle
+// (197 us, now 10; the operands come from L2 after their first read). All of a thread's loads of
+// the chunk are issued before its first FMA. The FP64 pipe is narrow (1.7 adds a clock and SM):
+// the two halves of a warp reduce the real and the imaginary part side by side, five adds a lane
+// instead of ten, in the same tree (8 x 2^23 terms 376 -> 170 us, 6.3 TB/s).
 
 template <bool CPLX, bool MAXPLUS = false>
 __global__ void __launch_bounds__(256) splitk_partial_kernel(StepArgs a, double* scratch, int64_t kc,
                                                              int32_t chunks) {
   static_assert(!(CPLX && MAXPLUS), "the max-plus semiring is real");
-  const int chunk = blockIdx.x, b = blockIdx.y;
-  const int m = (int)a.m, n = (int)a.n, mn = m * n;
-  const float* A = a.A + b * a.a_bstride;
-  const float* B = a.B + b * a.b_bstride;
+  const int chunk = blockIdx.x, b = blockIdx.y, o = blockIdx.z;
+  const int n = (int)a.n, mn = (int)a.m * n;
+  const float* A = a.A + b * a.a_bstride + (o / n) * a.k;
+  const float* B = a.B + b * a.b_bstride + (o - (o / n) * n) * a.k;
   float sa = 1.f, sb = 1.f;
   if (a.recs) {
     sa = pow2_neg(scale_exp(a.recs + a.rec_a + (a.a_bstride ? b : 0)));
     sb = pow2_neg(scale_exp(a.recs + a.rec_b + (a.b_bstride ? b : 0)));
   }
-  float accr[kSplitMaxOut], acci[kSplitMaxOut];
   const float zero = MAXPLUS ? __int_as_float(0xff800000) : 0.f;  // the semiring's zero
-#pragma unroll
-  for (int o = 0; o < kSplitMaxOut; ++o) accr[o] = acci[o] = zero;
+  float accr = zero, acci = 0.f;
   const int64_t k0 = (int64_t)chunk * kc;
   const int64_t k1 = min(a.k, k0 + kc);
-  if (MAXPLUS) {
-    for (int64_t kk = k0 + threadIdx.x; kk < k1; kk += blockDim.x) {
-#pragma unroll
-      for (int o = 0; o < kSplitMaxOut; ++o) {
-        if (o < mn) {
-          const int i = o / n, j = o - (o / n) * n;
-          accr[o] = fmaxf(accr[o], A[i * a.k + kk] + B[j * a.k + kk]);
-        }
-      }
-    }
-  }
-  // the output index o is a compile-time constant in every unrolled iteration, so the
-  // accumulators stay in registers
   const bool vec = !MAXPLUS && (a.k & 3) == 0 && (a.a_plane & 3) == 0 && (a.b_plane & 3) == 0 &&
                    ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
   if (vec) {
-    // 16-byte loads, four k-steps of the block unrolled: every thread has all of its
-    // loads of the chunk in flight before its first FMA (the step is HBM-bound)
-#pragma unroll 4
-    for (int64_t kk = k0 + 4 * threadIdx.x; kk < k1; kk += 4 * blockDim.x) {
+    // 16-byte loads; the chunk is at most U rounds of the block
+    constexpr int U = (int)(kSplitChunk / 1024);
+    float4 xr[U], yr[U], xi[CPLX ? U : 1], yi[CPLX ? U : 1];
+    const int64_t kt = k0 + 4 * threadIdx.x;
 #pragma unroll
-      for (int o = 0; o < kSplitMaxOut; ++o) {
-        if (o < mn) {
-          const int i = o / n, j = o - (o / n) * n;
-          const float4 xr = *reinterpret_cast<const float4*>(A + i * a.k + kk);
-          const float4 yr = *reinterpret_cast<const float4*>(B + j * a.k + kk);
-          if (CPLX) {
-            const float4 xi = *reinterpret_cast<const float4*>(A + a.a_plane + i * a.k + kk);
-            const float4 yi = *reinterpret_cast<const float4*>(B + a.b_plane + j * a.k + kk);
-            const float ar[4] = {xr.x * sa, xr.y * sa, xr.z * sa, xr.w * sa};
-            const float ai[4] = {xi.x * sa, xi.y * sa, xi.z * sa, xi.w * sa};
-            const float br[4] = {yr.x * sb, yr.y * sb, yr.z * sb, yr.w * sb};
-            const float bi[4] = {yi.x * sb, yi.y * sb, yi.z * sb, yi.w * sb};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              accr[o] = fmaf(ar[e], br[e], fmaf(-ai[e], bi[e], accr[o]));
-              acci[o] = fmaf(ar[e], bi[e], fmaf(ai[e], br[e], acci[o]));
-            }
-          } else {
-            accr[o] = fmaf(xr.x * sa, yr.x * sb, accr[o]);
-            accr[o] = fmaf(xr.y * sa, yr.y * sb, accr[o]);
-            accr[o] = fmaf(xr.z * sa, yr.z * sb, accr[o]);
-            accr[o] = fmaf(xr.w * sa, yr.w * sb, accr[o]);
-          }
-        }
+    for (int u = 0; u < U; ++u) {
+      const int64_t kk = kt + 1024 * u;
+      if (kk >= k1) break;
+      xr[u] = *reinterpret_cast<const float4*>(A + kk);
+      yr[u] = *reinterpret_cast<const float4*>(B + kk);
+      if (CPLX) {
+        xi[u] = *reinterpret_cast<const float4*>(A + a.a_plane + kk);
+        yi[u] = *reinterpret_cast<const float4*>(B + a.b_plane + kk);
       }
     }
-  }
-  for (int64_t kk = k0 + threadIdx.x; !MAXPLUS && !vec && kk < k1; kk += blockDim.x) {
 #pragma unroll
-    for (int o = 0; o < kSplitMaxOut; ++o) {
-      if (o < mn) {
-        const int i = o / n, j = o - (o / n) * n;
-        const float xr = A[i * a.k + kk] * sa;
-        const float yr = B[j * a.k + kk] * sb;
-        if (CPLX) {
-          const float xi = A[a.a_plane + i * a.k + kk] * sa;
-          const float yi = B[a.b_plane + j * a.k + kk] * sb;
-          accr[o] = fmaf(xr, yr, fmaf(-xi, yi, accr[o]));
-          acci[o] = fmaf(xr, yi, fmaf(xi, yr, acci[o]));
-        } else {
-          accr[o] = fmaf(xr, yr, accr[o]);
+    for (int u = 0; u < U; ++u) {
+      if (kt + 1024 * u >= k1) break;
+      const float ar[4] = {xr[u].x * sa, xr[u].y * sa, xr[u].z * sa, xr[u].w * sa};
+      const float br[4] = {yr[u].x * sb, yr[u].y * sb, yr[u].z * sb, yr[u].w * sb};
+      if (CPLX) {
+        const float ai[4] = {xi[u].x * sa, xi[u].y * sa, xi[u].z * sa, xi[u].w * sa};
+        const float bi[4] = {yi[u].x * sb, yi[u].y * sb, yi[u].z * sb, yi[u].w * sb};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          accr = fmaf(ar[e], br[e], fmaf(-ai[e], bi[e], accr));
+          acci = fmaf(ar[e], bi[e], fmaf(ai[e], br[e], acci));
         }
-      }
-    }
-  }
-  __shared__ double red[2][kSplitMaxOut][8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 0; o < kSplitMaxOut; ++o) {
-    if (o >= mn) break;
-    double vr = accr[o], vi = acci[o];
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-      if (MAXPLUS) {
-        vr = fmax(vr, __shfl_xor_sync(0xffffffffu, vr, s));
       } else {
-        vr += __shfl_xor_sync(0xffffffffu, vr, s);
-        vi += __shfl_xor_sync(0xffffffffu, vi, s);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) accr = fmaf(ar[e], br[e], accr);
       }
     }
-    if (lane == 0) {
-      red[0][o][warp] = vr;
-      red[1][o][warp] = vi;
+  } else {
+#pragma unroll 4
+    for (int64_t kk = k0 + threadIdx.x; kk < k1; kk += blockDim.x) {
+      const float xr = A[kk] * sa, yr = B[kk] * sb;
+      if (MAXPLUS) {
+        accr = fmaxf(accr, xr + yr);
+      } else if (CPLX) {
+        const float xi = A[a.a_plane + kk] * sa, yi = B[a.b_plane + kk] * sb;
+        accr = fmaf(xr, yr, fmaf(-xi, yi, accr));
+        acci = fmaf(xr, yi, fmaf(xi, yr, acci));
+      } else {
+        accr = fmaf(xr, yr, accr);
+      }
     }
+  }
+  // the warp's sums in lane 0 (and the imaginary part's in lane 16), the warps' in order
+  __shared__ double red[2][8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (MAXPLUS) {
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) accr = fmaxf(accr, __shfl_xor_sync(0xffffffffu, accr, s));
+    if (lane == 0) red[0][warp] = accr;
+  } else {
+    double v = accr;
+    if (CPLX) {
+      const float mine = lane < 16 ? accr : acci, other = lane < 16 ? acci : accr;
+      v = (double)mine + (double)__shfl_xor_sync(0xffffffffu, other, 16);
+    } else {
+      v += __shfl_xor_sync(0xffffffffu, v, 16);
+    }
+#pragma unroll
+    for (int s = 8; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    if (lane == 0) red[0][warp] = v;
+    if (CPLX && lane == 16) red[1][warp] = v;
   }
   __syncthreads();
-  if (threadIdx.x < mn) {
-    const int o = threadIdx.x;
-    double vr = MAXPLUS ? (double)zero : 0.0, vi = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      if (MAXPLUS) {
-        vr = fmax(vr, red[0][o][w]);
-      } else {
-        vr += red[0][o][w];
-        vi += red[1][o][w];
-      }
-    }
+  if (threadIdx.x < (CPLX ? 2 : 1)) {
+    double v = MAXPLUS ? (double)zero : 0.0;
+    for (int w = 0; w < 8; ++w) v = MAXPLUS ? fmax(v, red[0][w]) : v + red[threadIdx.x][w];
     double* dst = scratch + (((int64_t)b * chunks + chunk) * mn + o) * 2;
-    dst[0] = vr;
-    dst[1] = vi;
+    dst[threadIdx.x] = v;
+    if (!CPLX) dst[1] = 0.0;
   }
 }
 
 constexpr int kFinalThreads = 128;
 
+// CTA (b, output): thread t adds the partials of a contiguous run of chunks in order; thread 0
+// then adds the runs that hold any in order: a fixed association for a given chunk count.
 __global__ void __launch_bounds__(kFinalThreads) splitk_final_kernel(StepArgs a, const double* scratch,
                                                                     int32_t chunks, int32_t cplx) {
-  const int b = blockIdx.x;
-  const int m = (int)a.m, n = (int)a.n, mn = m * n;
+  const int b = blockIdx.x, o = blockIdx.y;
+  const int n = (int)a.n, mn = (int)a.m * n;
   float* C = a.C + b * a.c_bstride;
   __shared__ double part[2][kFinalThreads];
-  int lmax = -127;
-  // thread t adds the partials of a contiguous run of chunks in order; thread 0 then adds
-  // the runs in order: a fixed association for a given chunk count (deterministic)
-  const int per = (chunks + kFinalThreads - 1) / kFinalThreads;
+  const int per = (chunks + kFinalThreads - 1) / kFinalThreads, runs = (chunks + per - 1) / per;
   const double zero = a.maxplus ? __longlong_as_double(static_cast<long long>(0xfff0000000000000ull)) : 0.0;
-  for (int o = 0; o < mn; ++o) {
-    double sr = zero, si = 0.0;
-    const int c0 = threadIdx.x * per, c1 = min(chunks, c0 + per);
-    for (int c = c0; c < c1; ++c) {
-      const double* p = scratch + (((int64_t)b * chunks + c) * mn + o) * 2;
-      if (a.maxplus) {
-        sr = fmax(sr, p[0]);
-      } else {
-        sr += p[0];
-        si += p[1];
-      }
-    }
-    part[0][threadIdx.x] = sr;
-    part[1][threadIdx.x] = si;
-    __syncthreads();
-    double vr = zero, vi = 0.0;
-    if (threadIdx.x == 0)
-      for (int t = 0; t < kFinalThreads; ++t) {
-        if (a.maxplus) {
-          vr = fmax(vr, part[0][t]);
-        } else {
-          vr += part[0][t];
-          vi += part[1][t];
-        }
-      }
-    __syncthreads();  // every thread, every o: part is rewritten next iteration
-    if (threadIdx.x == 0) {
-      const int i = o / n, j = o % n;
-      const int64_t off = map_offset(a.rows, i) + map_offset(a.cols, j);
-      if (cplx) store_cplx(C, a.c_plane, off, (float)vr, (float)vi, a.c_split);
-      else C[off] = (float)vr;
-      if (a.recs) lmax = max(lmax, exp_of(cplx ? fmaxf(fabsf((float)vr), fabsf((float)vi)) : fabsf((float)vr)));
+  double sr = zero, si = 0.0;
+  const int c0 = threadIdx.x * per, c1 = min(chunks, c0 + per);
+  for (int c = c0; c < c1; ++c) {
+    const double2 p = *reinterpret_cast<const double2*>(scratch + (((int64_t)b * chunks + c) * mn + o) * 2);
+    if (a.maxplus) {
+      sr = fmax(sr, p.x);
+    } else {
+      sr += p.x;
+      si += p.y;
     }
   }
+  part[0][threadIdx.x] = sr;
+  part[1][threadIdx.x] = si;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double vr = zero, vi = 0.0;
+#pragma unroll 8
+  for (int t = 0; t < runs; ++t) {
+    if (a.maxplus) {
+      vr = fmax(vr, part[0][t]);
+    } else {
+      vr += part[0][t];
+      vi += part[1][t];
+    }
+  }
+  const int64_t off = map_offset(a.rows, o / n) + map_offset(a.cols, o % n);
+  if (cplx) store_cplx(C, a.c_plane, off, (float)vr, (float)vi, a.c_split);
+  else C[off] = (float)vr;
   if (a.recs) {
     ScaleRec* rc = a.recs + a.rec_c + (a.c_bstride ? b : 0);
-    atomicMax(&rc->emax, lmax);
-    if (threadIdx.x == 0) {
+    atomicMax(&rc->emax, exp_of(cplx ? fmaxf(fabsf((float)vr), fabsf((float)vi)) : fabsf((float)vr)));
+    if (o == 0) {
       const ScaleRec* ra = a.recs + a.rec_a + (a.a_bstride ? b : 0);
       const ScaleRec* rb = a.recs + a.rec_b + (a.b_bstride ? b : 0);
       rc->log2 = ra->log2 + rb->log2 + scale_exp(ra) + scale_exp(rb);
@@ -1008,11 +982,12 @@ int32_t splitk_chunks(int64_t k) { return (int32_t)((k + kSplitChunk - 1) / kSpl
 
 void launch_contract_splitk(const StepArgs& a, int32_t nb, bool cplx, double* scratch, cudaStream_t st) {
   const int32_t chunks = splitk_chunks(a.k);
-  dim3 grid((unsigned)chunks, (unsigned)nb);
+  const unsigned outs = (unsigned)(a.m * a.n);
+  dim3 grid((unsigned)chunks, (unsigned)nb, outs);
   if (cplx) splitk_partial_kernel<true><<<grid, 256, 0, st>>>(a, scratch, kSplitChunk, chunks);
   else if (a.maxplus) splitk_partial_kernel<false, true><<<grid, 256, 0, st>>>(a, scratch, kSplitChunk, chunks);
   else splitk_partial_kernel<false><<<grid, 256, 0, st>>>(a, scratch, kSplitChunk, chunks);
-  splitk_final_kernel<<<(unsigned)nb, kFinalThreads, 0, st>>>(a, scratch, chunks, cplx ? 1 : 0);
+  splitk_final_kernel<<<dim3((unsigned)nb, outs), kFinalThreads, 0, st>>>(a, scratch, chunks, cplx ? 1 : 0);
 }
 
 }  // namespace tn

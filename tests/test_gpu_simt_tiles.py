@@ -60,6 +60,36 @@ def test_tile_edges(tn, form, m, n, k):
         assert np.all(np.abs(out.imag - want.imag) <= g * (ar @ bi.T + ai @ br.T))
 
 
+@pytest.mark.parametrize("form", ["complex", "real", "maxplus"])
+@pytest.mark.parametrize("m,n,k", [(1, 1, 4096), (4, 4, 16384), (2, 3, 5003), (1, 16, 4097), (1, 1, 2 ** 20 + 2)])
+def test_split_k(tn, form, m, n, k):
+    """Few outputs, long k: a thread sums at most 16 terms in FP32 (32 products complex), the rest is
+    FP64, the result is rounded once: (2 * 16 + 3) 2^-24 of the absolute products for each of the
+    real and the imaginary part."""
+    rng = np.random.default_rng(k)
+    if form == "maxplus":
+        A, B = (rng.integers(-9000, 9000, size=s).astype(np.float64) for s in ((m, k), (n, k)))
+    else:
+        A, B = (rng.standard_normal(s) for s in ((m, k), (n, k)))
+        if form == "complex":
+            A, B = A + 1j * rng.standard_normal((m, k)), B + 1j * rng.standard_normal((n, k))
+    dt = np.complex64 if form == "complex" else np.float32
+    A, B = A.astype(dt), B.astype(dt)
+    net = Network([A, B], [(0, 2), (1, 2)], {0: m, 1: n, 2: k}, (0, 1))
+    plan = tn.Plan(net, Path([(0, 1)]), prec="fp32" if form == "complex" else "r32_fp32",
+                   semiring="maxplus" if form == "maxplus" else "standard")
+    assert plan.step(0)["cls"] == tn.TN_CLASS_SPLITK
+    out = np.zeros((m, n), dtype=np.complex128 if form == "complex" else np.float64)
+    plan.contract_host([A, B], out)
+    plan.destroy()
+    A, B = (x.astype(np.complex128 if form == "complex" else np.float64) for x in (A, B))
+    if form == "maxplus":
+        assert np.array_equal(out, np.max(A[:, None, :] + B[None, :, :], axis=2))
+        return
+    want, size = A @ B.T, np.abs(A) @ np.abs(B).T
+    assert np.all(np.abs(out - want) <= 2 * 35 * 2.0 ** -24 * size)
+
+
 @pytest.mark.parametrize("m,n,k", [(32, 64, 5), (256, 512, 40)])
 def test_interleaved_scaled(tn, m, n, k):
     """Extent-2 modes with rows and columns interleaved in the output, exponent scaling on: the
