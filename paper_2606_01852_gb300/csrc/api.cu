@@ -62,6 +62,7 @@ StepArgs step_args(const Plan& P, const StepRec& st) {
   a.c_bstride = C.batched ? fl(C) * C.size : 0;
   a.rows = st.rows;
   a.cols = st.cols;
+  a.blk = st.blk;
   a.recs = P.policy.exp_scaling ? reinterpret_cast<ScaleRec*>(P.dev + P.off_scale) : nullptr;
   a.rec_a = P.rec_index[st.a];
   a.rec_b = P.rec_index[st.b];

@@ -1741,7 +1741,7 @@ int64_t tc_launches(int64_t m, int64_t n, int64_t k, int32_t nb, int32_t prec, b
     }
   }
   if (prec != TN_C64_BF16X3 && prec != kPrecBF16x3M)
-    return tf32_launches(m, n, nb, prec == TN_R32_TF32 || prec == TN_R32_3XTF32);
+    return tf32_launches(m, n, k, nb, prec);
   const int64_t tiles = ((m + BM - 1) / BM) * ((n + BN - 1) / BN);
   const int64_t per = sm_band_tiles(tiles, nb);
   return (tiles + per - 1) / per;

@@ -5,11 +5,12 @@
 //                                      k-blocks, 3 stages, D_rr / D_ii / D_x accumulators
 //                                      (Re C = D_rr - D_ii, Im C = D_x); 192 threads (real
 //                                      tiles: 2 stages, 320 threads, two CTAs per SM);
-//   contract_tc3_kernel<REAL, SCALED>  3xTF32: eight warps split each staged tile into
-//                                      hi = RN_tf32(v) and lo = v - hi, hi.hi in 32-term
-//                                      chunks folded into round-to-nearest registers, cross
-//                                      terms in their own accumulator; 320 threads.
-// Real steps take 128 x 256 output tiles (two B tiles read as one 256-row operand).
+//   contract_tc3t_kernel<REAL, SCALED, BT>  3xTF32: sixteen warps split each staged tile into
+//                                      hi = RN_tf32(v) and lo = v - hi, A's into tensor memory;
+//                                      hi.hi in 32-term chunks folded into round-to-nearest
+//                                      registers, cross terms in their own accumulator; 576
+//                                      threads, tiles of 64-192 (real) or 32-64 (complex) columns.
+// Real TF32 steps take 128 x 256 output tiles (two B tiles read as one 256-row operand).
 // Every mbarrier wait is bounded by wall time; on expiry the CTA records an error code,
 // drains its copies, frees its tensor memory and returns.
 #include <cstdint>
@@ -241,104 +242,97 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
 // ---------------------------------------------------------------------------------
 // 3xTF32 with round-to-nearest accumulation across k.
 //
-// The tensor core's FP32 accumulator truncates each addition, so a long TMEM
-// accumulation drifts toward zero by ~k * 2^-25 relative (measured). Here the MMAs
-// accumulate only CK k-blocks (CK * 16 terms) into the TMEM chunk accumulator
-// (re @0, im @128; Re uses the instruction's negate-A bit for -A_im.B_im); eight
-// warps then add the chunk into running totals held in their registers with ordinary
-// round-to-nearest FP32 additions, and release the accumulator for the next chunk.
-// The same eight warps split every staged tile into hi/lo (so the MMA pipe waits only
-// for the short drain), and finally write the totals out. 128 x 128 tiles: the kernel is
-// bound by shared-memory operand reads (each 3xTF32 MMA re-reads its tiles), so the
-// wide tile keeps reads per flop low.
-// Warps: 0 TMA, 1 MMA + TMEM, 2-9 split / drain / epilogue (320 threads); warp w of
-// 2-9 drains TMEM lane quarter w % 4, columns 64 * ((w - 2) / 4) .. +63.
-
-// Stage layout (raw values and, in the lo buffers, their lo parts), 8 KiB tiles:
-//   A_re | A_im | -B_im | B_re | B_im
-// so that [B_re | B_im] and [-B_im | B_re] are each one 256-row operand: per k-atom
-// A_re.[B_re|B_im] and A_im.[-B_im|B_re] add into (Re, Im) with one 128 x 256 MMA each.
-// A real step (REAL) uses the A_re, B_re and B_im slots for A and the B tiles of columns
-// n0 .. n0 + 127 and n0 + 128 .. n0 + 255: a 128 x 256 tile, A.[B_0|B_1] per k-atom.
-struct C3 {
-  // CK = 2: 32-term chunks. Each truncating addition loses up to an ulp of the running chunk
-  // sum, so the error grows with the chunk; 64-term chunks were 5 % faster but left the
-  // FP32-accurate form at twice plain FP32's error on long paths of small steps.
-  static constexpr int BK = 16, ROWB = 64, CK = 2;
-  static constexpr int TILE_A = BM * ROWB;                  // 8 KiB
-  static constexpr int TILE_B = BN * ROWB;                  // 8 KiB
-  static constexpr int OFF_AI = TILE_A, OFF_BNEG = 2 * TILE_A;
-  static constexpr int OFF_BR = 2 * TILE_A + TILE_B, OFF_BI = 2 * TILE_A + 2 * TILE_B;
-  static constexpr int TMA_BYTES = 2 * TILE_A + 2 * TILE_B; // 32 KiB per stage by TMA
-  static constexpr int STAGE = 2 * TILE_A + 3 * TILE_B;     // 40 KiB
-  static constexpr int STAGES = 3, LO = 2;
-  static constexpr int THREADS = 320;
-  static constexpr int SMEM = (STAGES + LO) * STAGE + 1024 + 1024;
-  static constexpr uint32_t COLS = 512;  // re @0, im @128, re_lo @256, im_lo @384
+// The tensor core's FP32 accumulator truncates each addition, so a long TMEM accumulation
+// drifts toward zero by ~k * 2^-25 relative (measured). Here the hi.hi MMAs of 32 terms go into a
+// chunk accumulator, which warps add into running totals in their registers with ordinary
+// round-to-nearest FP32 additions (longer chunks lose more: 64 terms were 5 % faster but left the
+// FP32-accurate form at twice plain FP32's error on long paths); the cross terms (2^-11 of the
+// result) keep one accumulator over all of k. A complex tile's B planes are [-B_im | B_re | B_im],
+// so A_re.[B_re | B_im] and A_im.[-B_im | B_re] add into (Re | Im) with one MMA each.
+//
+// What bounds it: shared-memory bandwidth. Per k-block TMA writes the raw tiles, the split reads
+// them and writes hi and lo, and every MMA reads its operands (A and B three times). The split
+// therefore writes A's hi and lo into tensor memory (tcgen05.st, thread = row), where the MMAs
+// read them: no A stores to shared memory, no A reads from it. Per 32 terms of a real 128 x 192
+// tile that is 200 KB of shared-memory traffic for 1152 clocks of MMAs (a 128 x 256 tile with A in
+// shared memory: 336 KB for 1536). Tensor memory sets the tile: chunk and cross accumulators of N
+// columns and two buffers of A (hi and lo, 32 columns each, re and im) in 512 columns.
+//
+// Measured (GB300; before: 128 x 256 real, 128 x 128 complex tiles, A in shared memory, MMAs
+// issued from a divergent lane): real 16384 x 32768 x 1024 7.87 -> 5.21 ms (140 -> 211 TFLOP/s),
+// 2048 x 16384 x 8192 166 -> 234; complex 4096^3 231 -> 305, few tiles: 512 x 128 x 2048 179 -> 51 us,
+// 256 x 256 x 256 36 -> 14 us. cuBLAS's sustained TF32 rate over three products is 305.
+// BT rows of B per plane; the narrow tiles (64 real, 32 complex) put a small step's outputs on
+// more SMs.
+// Warps: 0 TMA, 1 MMA + TMEM, 2-17 split / fold / epilogue. Sixteen of them, because a block's
+// split and fold are a chain of latencies (shared memory, tensor memory, fences, barriers) that
+// eight warps could not finish within the block's MMAs (1920 against 1330 clocks): warp w owns
+// TMEM lanes 32 (w % 4) .. + 31, and of a row the part (w - 2) / 4 splits a quarter of A's terms
+// (real) or half of a plane's (complex) and folds every fourth 16-column unit.
+template <bool REAL, int BT>
+struct C3T {
+  static constexpr int BK = 32, ROWB = 128;
+  static constexpr int NP = REAL ? 1 : 2;
+  static constexpr int N = NP * BT;                         // MMA columns
+  static constexpr int TILE_A = BM * ROWB, TILE_B = BT * ROWB;
+  static constexpr int OFF_B = NP * TILE_A;                 // the B area: [B], or [-B_im | B_re | B_im]
+  static constexpr int AREA_B = (REAL ? 1 : 3) * TILE_B;
+  static constexpr int STAGE = OFF_B + AREA_B;
+  static constexpr int LOADED = NP * (TILE_A + TILE_B);     // TMA bytes per stage
+  static constexpr int LO = 2, FIT = (232448 - 1536 - 8 * (BM + BT) - LO * AREA_B) / STAGE;
+  static constexpr int STAGES = FIT < 5 ? FIT : 5;
+  static constexpr int THREADS = 576, WORKERS = 512;
+  static constexpr int OFFSETS = 8 * (BM + BT);             // output offsets of the rows and columns
+  static constexpr int SMEM = STAGES * STAGE + LO * AREA_B + 512 + OFFSETS + 1024;  // + barriers, alignment
+  static constexpr int ACOLS = NP * 2 * BK;                 // one buffer of A: plane p hi @32 p, lo @32 (NP + p)
+  static constexpr uint32_t COLS = 512;
+  // chunk accumulators: two where they fit, so that a chunk's hi.hi need not wait for the fold of
+  // the one before
+  static constexpr int HI = 3 * N + 2 * ACOLS <= 512 ? 2 : 1;
+  static constexpr int D_LO = HI * N, A_COL = D_LO + N;     // columns of the cross-term accumulator and of A
+  static constexpr int UNITS = BT / 16;                     // 16-column units of a plane
+  static constexpr int MINE = (UNITS + 3) / 4;              // units a warp folds at most
+  static constexpr int FOLDERS = UNITS >= 4 ? 16 : 4 * UNITS;
+  static constexpr int NB = BT / 32;                        // 32-column blocks of the tile
+  static_assert(A_COL + 2 * ACOLS <= 512 && N % 16 == 0 && TILE_B % 1024 == 0, "tensor memory and swizzle");
+  static_assert(SMEM <= 232448 && 4 * NB * NP * 32 * 33 * 4 <= STAGES * STAGE, "stages; epilogue transposes");
 };
 
-// 32 columns nb0 .. nb0 + 31 of this thread's row of a real result, v[OFF .. OFF + 31]: one
-// column of the warp's 32 rows per warp store when the rows are the unit-stride side, else
-// through shared memory (tr, this warp's 32 x 33 floats) one row per warp store. The lanes
-// compute the 32 column offsets once and pass them round by shuffles.
-template <int OFF>
-__device__ __forceinline__ void store_real_cols(float* C, const StepArgs& a, const float (&v)[64], int64_t nb0,
-                                                int64_t ro, bool row_ok, bool ok, bool rows_unit, float* tr,
-                                                int lane) {
-  const int64_t n = nb0 + lane;
-  const bool col_ok = ok && n < a.n;
-  const int64_t co = col_ok ? map_offset(a.cols, n) : 0;  // lane j: column nb0 + j
-  if (rows_unit) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int64_t co_j = __shfl_sync(0xffffffffu, co, j);
-      if (row_ok && nb0 + j < a.n) C[ro + co_j] = v[OFF + j];
-    }
-    return;
-  }
-#pragma unroll
-  for (int j = 0; j < 32; ++j) tr[lane * 33 + j] = v[OFF + j];
-  __syncwarp();
-  for (int r = 0; r < 32; ++r) {
-    const int64_t ro_r = __shfl_sync(0xffffffffu, ro, r);
-    const bool ok_r = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, r) != 0;
-    if (ok_r && col_ok) C[ro_r + co] = tr[r * 33 + lane];
-  }
-  __syncwarp();
-}
-
-template <bool REAL, bool SCALED>
-__global__ void __launch_bounds__(C3::THREADS, 1)
-    contract_tc3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                        StepArgs a, int64_t t_first, int* err) {
-  constexpr int STAGES = C3::STAGES, BK = C3::BK, ROWB = C3::ROWB, CK = C3::CK;
-  constexpr int TILE_A = C3::TILE_A, TILE_B = C3::TILE_B, STAGE = C3::STAGE;
-  constexpr int TN = REAL ? 2 * BN : BN;                                    // output columns per tile
-  constexpr int LOADED = REAL ? TILE_A + 2 * TILE_B : C3::TMA_BYTES;        // TMA bytes per stage
+template <bool REAL, bool SCALED, int BT>
+__global__ void __launch_bounds__(576, 1)
+    contract_tc3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                         StepArgs a, int64_t t_first, int* err) {
+  using G = C3T<REAL, BT>;
+  constexpr int STAGES = G::STAGES, BK = G::BK, ROWB = G::ROWB, NP = G::NP;
+  constexpr int TILE_A = G::TILE_A, TILE_B = G::TILE_B, STAGE = G::STAGE;
+  // B planes in the B area (hi in the stage, lo in the lo buffer)
+  constexpr int B_RE = REAL ? 0 : TILE_B, B_IM = 2 * TILE_B;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* lo_base = smem + STAGES * STAGE;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(lo_base + C3::LO * STAGE);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(lo_base + G::LO * G::AREA_B);
   uint64_t* full = bars;                     // [STAGES]
   uint64_t* empty = bars + STAGES;           // [STAGES]
-  uint64_t* conv_full = bars + 2 * STAGES;   // [2]
-  uint64_t* lo_empty = conv_full + 2;        // [2]
-  uint64_t* acc_full = lo_empty + 2;         // chunk accumulated
-  uint64_t* acc_empty = acc_full + 1;        // chunk drained
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
+  uint64_t* conv_full = bars + 2 * STAGES;   // [2] block split
+  uint64_t* lo_empty = conv_full + 2;        // [2] lo buffer and A buffer read
+  uint64_t* acc_full = lo_empty + 2;         // [HI] chunk accumulated
+  uint64_t* acc_empty = acc_full + G::HI;    // [HI] chunk folded
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + G::HI);
+  int64_t* row_off = reinterpret_cast<int64_t*>(bars + 64);  // [BM] output offsets of the tile's rows
+  int64_t* col_off = row_off + BM;                           // [BT] and columns
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + TN - 1) / TN;
+  // (the shuffle tells the compiler that the warp index is uniform)
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + BT - 1) / BT;
   const int64_t t = t_first + blockIdx.x;  // this launch's tiles start at t_first
   const int64_t per_group = GROUP_M * tiles_n;
   const int64_t first_m = (t / per_group) * GROUP_M;
   const int64_t gm = tiles_m - first_m < GROUP_M ? tiles_m - first_m : GROUP_M;
   const int64_t tm = first_m + (t % per_group) % gm, tn = (t % per_group) / gm;
-  const int m0 = static_cast<int>(tm * BM), n0 = static_cast<int>(tn * TN);
+  const int m0 = static_cast<int>(tm * BM), n0 = static_cast<int>(tn * BT);
   const int b = blockIdx.y;
   const int num_kb = static_cast<int>((a.k + BK - 1) / BK);
-  const int n_chunks = (num_kb + CK - 1) / CK;
-  const int pa = a.a_bstride ? (REAL ? b : 2 * b) : 0, pb = a.b_bstride ? (REAL ? b : 2 * b) : 0;
+  const int pa = a.a_bstride ? NP * b : 0, pb = a.b_bstride ? NP * b : 0;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -346,24 +340,26 @@ __global__ void __launch_bounds__(C3::THREADS, 1)
       mbar_init(&empty[s], 1);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&conv_full[i], 256);
+      mbar_init(&conv_full[i], G::WORKERS);
       mbar_init(&lo_empty[i], 1);
     }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, 8);
+    for (int i = 0; i < G::HI; ++i) {
+      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_empty[i], G::FOLDERS);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                 "r"(C3::COLS));
+                 "r"(G::COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -371,254 +367,241 @@ __global__ void __launch_bounds__(C3::THREADS, 1)
       for (int kb = 0; kb < num_kb; ++kb) {
         const int s = kb % STAGES;
         if (!mbar_wait(&empty[s], ((kb / STAGES) & 1) ^ 1)) {
-          atomicExch(err, 11);
+          atomicExch(err, 71);
           break;
         }
-        mbar_expect_tx(&full[s], LOADED);
+        mbar_expect_tx(&full[s], G::LOADED);
         uint8_t* st = smem + s * STAGE;
         const int k0 = kb * BK;
         tma_load_3d(st, &tmA, &full[s], k0, m0, pa);
-        if constexpr (REAL) {
-          // the second B tile may lie wholly past n: the box is then zero-filled
-          tma_load_3d(st + C3::OFF_BR, &tmB, &full[s], k0, n0, pb);
-          tma_load_3d(st + C3::OFF_BI, &tmB, &full[s], k0, n0 + BN, pb);
-        } else {
-          tma_load_3d(st + C3::OFF_AI, &tmA, &full[s], k0, m0, pa + 1);
-          tma_load_3d(st + C3::OFF_BR, &tmB, &full[s], k0, n0, pb);
-          tma_load_3d(st + C3::OFF_BI, &tmB, &full[s], k0, n0, pb + 1);
+        tma_load_3d(st + G::OFF_B + B_RE, &tmB, &full[s], k0, n0, pb);
+        if constexpr (!REAL) {
+          tma_load_3d(st + TILE_A, &tmA, &full[s], k0, m0, pa + 1);
+          tma_load_3d(st + G::OFF_B + B_IM, &tmB, &full[s], k0, n0, pb + 1);
         }
         issued = kb + 1;
       }
       for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-        if (!mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1)) atomicExch(err, 12);
+        if (!mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1)) atomicExch(err, 72);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_tf32(BM, 2 * BN);  // 128 x 256: (Re | Im) at once
-      const uint32_t d_hi = tmem, d_lo = tmem + 256;
-      bool ok = true;
-      for (int c = 0; c < n_chunks && ok; ++c) {
-        const int kb_end = min(num_kb, (c + 1) * CK);
-        for (int kb = c * CK; kb < kb_end; ++kb) {
-          const int s = kb % STAGES;
-          if (!mbar_wait(&full[s], (kb / STAGES) & 1) || !mbar_wait(&conv_full[kb & 1], (kb >> 1) & 1)) {
-            atomicExch(err, 14);
-            ok = false;
-            break;
-          }
-          fence_after();
-          const uint32_t st = su32(smem + s * STAGE);
-          const uint32_t lo = su32(lo_base + (kb & 1) * STAGE);
-          // the cross terms first: their accumulator runs over all of k (it is ~2^-11 of the
-          // result, so its own truncation is negligible) and is read once, after the last
-          // chunk, so a chunk's first k-block issues them before the wait for the previous
-          // chunk's fold, which then overlaps tensor-core work
-#pragma unroll
-          for (int j = 0; j < BK / 8; ++j) {
-            const uint64_t ar = smem_desc<ROWB>(st + j * 32), ai = smem_desc<ROWB>(st + C3::OFF_AI + j * 32);
-            const uint64_t b_ri = smem_desc<ROWB>(st + C3::OFF_BR + j * 32);    // [B_re | B_im]
-            const uint64_t b_nr = smem_desc<ROWB>(st + C3::OFF_BNEG + j * 32);  // [-B_im | B_re]
-            const uint64_t arl = smem_desc<ROWB>(lo + j * 32), ail = smem_desc<ROWB>(lo + C3::OFF_AI + j * 32);
-            const uint64_t bl_ri = smem_desc<ROWB>(lo + C3::OFF_BR + j * 32);
-            const uint64_t bl_nr = smem_desc<ROWB>(lo + C3::OFF_BNEG + j * 32);
-            mma_tf32(d_lo, arl, b_ri, idesc, (kb > 0 || j > 0) ? 1u : 0u);
-            if constexpr (!REAL) mma_tf32(d_lo, ail, b_nr, idesc, 1u);
-            mma_tf32(d_lo, ar, bl_ri, idesc, 1u);
-            if constexpr (!REAL) mma_tf32(d_lo, ai, bl_nr, idesc, 1u);
-          }
-          if (kb == c * CK) {
-            // the chunk accumulator must have been folded before the hi MMAs reuse it
-            if (!mbar_wait(acc_empty, (c & 1) ^ 1)) {
-              atomicExch(err, 13);
-              ok = false;
-              mma_commit(&empty[s]);
-              mma_commit(&lo_empty[kb & 1]);
-              break;
-            }
-            fence_after();
-          }
-          // hi.hi products into the main accumulators (Re | Im), so the main sums take only
-          // two truncating additions per 8 terms (one for a real step: its 256 columns are
-          // all hi.hi)
-#pragma unroll
-          for (int j = 0; j < BK / 8; ++j) {
-            const uint32_t acc = (kb > c * CK || j > 0) ? 1u : 0u;
-            const uint64_t ar = smem_desc<ROWB>(st + j * 32), ai = smem_desc<ROWB>(st + C3::OFF_AI + j * 32);
-            const uint64_t b_ri = smem_desc<ROWB>(st + C3::OFF_BR + j * 32);
-            const uint64_t b_nr = smem_desc<ROWB>(st + C3::OFF_BNEG + j * 32);
-            mma_tf32(d_hi, ar, b_ri, idesc, acc);
-            if constexpr (!REAL) mma_tf32(d_hi, ai, b_nr, idesc, 1u);
-          }
-          mma_commit(&empty[s]);
-          mma_commit(&lo_empty[kb & 1]);
-        }
-        mma_commit(acc_full);  // also on error, so the drain sees issued MMAs retire
+    // The whole warp runs the loop and one elected lane issues, so that the operands of the MMAs
+    // stay in uniform registers: issued by a lane on its own branch, an MMA of 64 columns cost 95
+    // clocks, three times its execution.
+    constexpr uint32_t idesc = idesc_tf32(BM, G::N);  // complex: (Re | Im) at once
+    const bool leader = elect_one();
+    const uint32_t d_lo = tmem + G::D_LO;
+    // descriptors of the first stage's and lo buffer's B areas; 16-byte units are added to them
+    const uint64_t hi0 = smem_desc<ROWB>(su32(smem + G::OFF_B)), lo0 = smem_desc<ROWB>(su32(lo_base));
+    bool mma_ok = true;
+    int s = 0;
+    for (int kb = 0; kb < num_kb; ++kb, s = s + 1 == STAGES ? 0 : s + 1) {
+      if (!mbar_wait(&conv_full[kb & 1], (kb >> 1) & 1)) {
+        if (leader) atomicExch(err, 74);
+        mma_ok = false;
+        break;
       }
-    }
-  } else {
-    const int et = threadIdx.x - 64;  // 0..255
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
-    float run_re[64], run_im[64];
+      fence_after();
+      const uint64_t hi = hi0 + static_cast<uint32_t>(s * (STAGE >> 4));
+      const uint64_t lo = lo0 + static_cast<uint32_t>((kb & 1) * (G::AREA_B >> 4));
+      const uint32_t at = tmem + G::A_COL + (kb & 1) * G::ACOLS;
+      const uint32_t ar = at, ai = at + BK, arl = at + NP * BK, ail = arl + BK;
+      // the cross terms first (their accumulator runs over all of k), so that they overlap the
+      // fold of the previous chunk; then, once that is folded, the chunk's hi.hi
+      if (leader) {
 #pragma unroll
-    for (int i = 0; i < 64; ++i) run_re[i] = run_im[i] = 0.f;
+        for (int j = 0; j < BK / 8; ++j) {
+          const uint64_t b_ri = hi + (B_RE >> 4) + 2 * j, bl_ri = lo + (B_RE >> 4) + 2 * j;
+          const uint64_t b_nr = hi + 2 * j, bl_nr = lo + 2 * j;
+          mma_tf32_ts(d_lo, arl + 8 * j, b_ri, idesc, (kb > 0 || j > 0) ? 1u : 0u);
+          if constexpr (!REAL) mma_tf32_ts(d_lo, ail + 8 * j, b_nr, idesc, 1u);
+          mma_tf32_ts(d_lo, ar + 8 * j, bl_ri, idesc, 1u);
+          if constexpr (!REAL) mma_tf32_ts(d_lo, ai + 8 * j, bl_nr, idesc, 1u);
+        }
+      }
+      const int h = kb % G::HI;
+      const uint32_t d_hi = tmem + h * G::N;
+      if (!mbar_wait(&acc_empty[h], ((kb / G::HI) & 1) ^ 1)) {
+        if (leader) atomicExch(err, 73);
+        mma_ok = false;
+        break;
+      }
+      fence_after();
+      if (leader) {
+#pragma unroll
+        for (int j = 0; j < BK / 8; ++j) {
+          mma_tf32_ts(d_hi, ar + 8 * j, hi + (B_RE >> 4) + 2 * j, idesc, j > 0 ? 1u : 0u);
+          if constexpr (!REAL) mma_tf32_ts(d_hi, ai + 8 * j, hi + 2 * j, idesc, 1u);
+        }
+        mma_commit(&empty[s]);
+        mma_commit(&lo_empty[kb & 1]);
+        mma_commit(&acc_full[h]);
+      }
+      __syncwarp();
+    }
+    if (!mma_ok && leader) mma_commit(&acc_full[0]);  // tracks the issued MMAs
+    __syncwarp();
+  } else {
+    const int et = threadIdx.x - 64;  // 0..511
+    const int q = warp & 3, part = (warp - 2) >> 2;
+    const int row = q * 32 + lane;
+    const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
+    const bool folds = part < G::UNITS;  // (warp-uniform)
+    float run[NP][G::MINE][16];
+#pragma unroll
+    for (int p = 0; p < NP; ++p)
+#pragma unroll
+      for (int i = 0; i < G::MINE; ++i)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) run[p][i][j] = 0.f;
     bool ok = true;
+    // output offsets, while the first loads are on their way
+    if (et < BM) row_off[et] = m0 + et < a.m ? map_offset(a.rows, m0 + et) : 0;
+    else if (et < BM + BT) col_off[et - BM] = n0 + et - BM < a.n ? map_offset(a.cols, n0 + et - BM) : 0;
     for (int kb = 0; kb <= num_kb; ++kb) {
-      // Fold chunk dc of the TMEM accumulators into the register totals and release
-      // them: once one k-block into the next chunk is split (so the MMA pipe restarts at
-      // once), and after the last k-block.
-      const int dc = kb == num_kb ? n_chunks - 1 : (kb % CK == 0 && kb > 0 ? kb / CK - 1 : -1);
       if (kb < num_kb) {
         const int s = kb % STAGES;
-        if (ok && (!mbar_wait(&full[s], (kb / STAGES) & 1) || !mbar_wait(&lo_empty[kb & 1], ((kb >> 1) & 1) ^ 1))) {
-          atomicExch(err, 15);
+        if (!mbar_wait(&full[s], (kb / STAGES) & 1) || !mbar_wait(&lo_empty[kb & 1], ((kb >> 1) & 1) ^ 1)) {
+          atomicExch(err, 75);
           ok = false;
+          break;
         }
-      }
-      if (kb < num_kb && ok) {
-        const int s = kb % STAGES;
-        float4* src = reinterpret_cast<float4*>(smem + s * STAGE);
-        float4* dst = reinterpret_cast<float4*>(lo_base + (kb & 1) * STAGE);
-        // hi = value rounded to the nearest TF32 (written back in place), lo = value - hi
-        // (exact); for B_im also -hi and -lo. kind::tf32 reads an FP32 operand by dropping
-        // its low 13 mantissa bits (tests/test_gpu_tc.py::test_tf32_operand_rounding), so hi
-        // is read exactly and only lo is truncated -- by at most 2^-10 of |lo|, with the
-        // sign of lo, i.e. without a bias. (Using the staged value itself as hi would have
-        // the hardware truncate it: a bias toward zero in every product.)
-        // float4s of A (A_re, A_im; a real step's A alone), then of the two B slots
-        constexpr int NA = (REAL ? TILE_A : 2 * TILE_A) / 16;
-        constexpr int SKIP = (C3::OFF_BR - (REAL ? TILE_A : 2 * TILE_A)) / 16;
-#pragma unroll 4
-        for (int i = et; i < LOADED / 16; i += 256) {
-          const int f = i < NA ? i : i + SKIP;  // skip the -B_im slot (and a real step's A_im)
-          const float4 v = src[f];
-          float4 h, l;
-          h.x = tf32_rn(v.x);
-          h.y = tf32_rn(v.y);
-          h.z = tf32_rn(v.z);
-          h.w = tf32_rn(v.w);
-          l.x = v.x - h.x;
-          l.y = v.y - h.y;
-          l.z = v.z - h.z;
-          l.w = v.w - h.w;
-          src[f] = h;
-          dst[f] = l;
-          if (!REAL && f >= C3::OFF_BI / 16) {
-            const int g = f - (C3::OFF_BI - C3::OFF_BNEG) / 16;
-            src[g] = make_float4(-h.x, -h.y, -h.z, -h.w);
-            dst[g] = make_float4(-l.x, -l.y, -l.z, -l.w);
+        fence_after();
+        // every shared-memory read of the block first: B's pieces, then A's
+        constexpr int PB = NP * TILE_B / 16 / G::WORKERS;
+        static_assert(PB * G::WORKERS * 16 == NP * TILE_B, "whole pieces per thread");
+        float4* src = reinterpret_cast<float4*>(smem + s * STAGE + G::OFF_B);
+        float4* dst = reinterpret_cast<float4*>(lo_base + (kb & 1) * G::AREA_B);
+        float4 bv[PB];
+#pragma unroll
+        for (int i = 0; i < PB; ++i) bv[i] = src[et + G::WORKERS * i + B_RE / 16];
+        // A: W terms of this thread's row (of plane part / 2 in a complex step), from the
+        // 128-byte swizzled tile (16-byte piece c at c ^ (row % 8)): hi rounded to the nearest
+        // TF32, lo the exact rest, into the buffer's columns
+        constexpr int W = REAL ? 8 : 16;
+        const int k_first = REAL ? 8 * part : 16 * (part & 1), plane = REAL ? 0 : part >> 1;
+        const uint8_t* arow = smem + s * STAGE + plane * TILE_A + row * ROWB;
+        const uint32_t at = tmem + lane_base + G::A_COL + (kb & 1) * G::ACOLS + plane * BK + k_first;
+        float h[W], l[W];
+#pragma unroll
+        for (int c = 0; c < W / 4; ++c) {
+          const float4 v = *reinterpret_cast<const float4*>(arow + (((k_first / 4 + c) ^ (row & 7)) << 4));
+          const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            h[4 * c + e] = tf32_rn(x[e]);
+            l[4 * c + e] = x[e] - h[4 * c + e];
           }
         }
+        tmem_st(at, h);
+        tmem_st(at + NP * BK, l);
+        // B: hi in place, lo into the lo buffer; of B_im also their negatives
+#pragma unroll
+        for (int i = 0; i < PB; ++i) {
+          const int f = et + G::WORKERS * i + B_RE / 16;
+          const float4 v = bv[i];
+          float4 x, y;
+          x.x = tf32_rn(v.x);
+          x.y = tf32_rn(v.y);
+          x.z = tf32_rn(v.z);
+          x.w = tf32_rn(v.w);
+          y.x = v.x - x.x;
+          y.y = v.y - x.y;
+          y.z = v.z - x.z;
+          y.w = v.w - x.w;
+          src[f] = x;
+          dst[f] = y;
+          if (!REAL && f >= B_IM / 16) {
+            const int g = f - B_IM / 16;
+            src[g] = make_float4(-x.x, -x.y, -x.z, -x.w);
+            dst[g] = make_float4(-y.x, -y.y, -y.z, -y.w);
+          }
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        fence_before();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(&conv_full[kb & 1]);
       }
-      if (dc >= 0 && ok) {
-        if (!mbar_wait(acc_full, dc & 1)) {
-          atomicExch(err, 16);
+      // fold chunk kb - 1 (its MMAs ran while this block was split) into the register totals with
+      // round-to-nearest additions and release the accumulator
+      if (kb > 0 && folds) {
+        const int d = (kb - 1) % G::HI;
+        if (!mbar_wait(&acc_full[d], ((kb - 1) / G::HI) & 1)) {
+          atomicExch(err, 76);
           ok = false;
-        } else {
-          fence_after();
-          float v[32];
-#pragma unroll
-          for (int p = 0; p < 2; ++p) {
-            const uint32_t col = lane_base + half * 64 + p * 32;
-            tmem_ld32(tmem + col, v);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) run_re[p * 32 + i] += v[i];
-            tmem_ld32(tmem + 128 + col, v);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) run_im[p * 32 + i] += v[i];
-            if (dc == n_chunks - 1) {  // last chunk: the cross terms too
-              tmem_ld32(tmem + 256 + col, v);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) run_re[p * 32 + i] += v[i];
-              tmem_ld32(tmem + 384 + col, v);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) run_im[p * 32 + i] += v[i];
-            }
-          }
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty);
+          break;
         }
+        fence_after();
+        auto add = [&](uint32_t first) {  // the accumulator at column `first`
+#pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            float v[G::MINE][16];
+#pragma unroll
+            for (int i = 0; i < G::MINE; ++i)
+              tmem_ld16_async(tmem + lane_base + first + p * BT + 16 * (part + 4 * i), v[i]);
+            tmem_ld_wait(v);
+#pragma unroll
+            for (int i = 0; i < G::MINE; ++i)
+#pragma unroll
+              for (int j = 0; j < 16; ++j) run[p][i][j] += v[i][j];
+          }
+        };
+        add(d * G::N);
+        if (kb == num_kb) add(G::D_LO);  // last chunk: the cross terms too
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[d]);
       }
     }
-    // epilogue: thread = TMEM lane (row); this warp's 64 columns
-    const int row = q * 32 + lane;
-    const int64_t m = static_cast<int64_t>(m0) + row;
-    const bool row_ok = ok && m < a.m;
-    const int64_t ro = row_ok ? map_offset(a.rows, m) : 0;
+    // Epilogue: the four warps of a lane quarter put their columns into 32 x 32 blocks in shared
+    // memory and store them in address order. The stage buffers are free: the last fold waited
+    // for the final MMA, which waited for every warp's last split; no TMA load is outstanding.
+    // (A warp that gave up a wait stores nothing; its barrier below still completes.)
     float* C = a.C + static_cast<int64_t>(b) * a.c_bstride;
-    // The stage buffers are free here: this warp's last drain waited for the final MMA,
-    // which waited for every warp's last split; no TMA load is outstanding.
-    // Row-by-row stores (one row per warp store, through shared memory when the columns
-    // are the unit-stride side): the address-ordered block store costs this kernel
-    // registers its split loop needs.
-    const bool rows_unit = a.rows.n > 0 && a.rows.stride[a.rows.n - 1] == 1;
-    float* tr = reinterpret_cast<float*>(smem) + (warp - 2) * 2 * 32 * 33;  // [2][32][33]
-    if constexpr (SCALED) {
+    constexpr int BLK = NP * 32 * 33;
+    float* tr = reinterpret_cast<float*>(smem) + q * G::NB * BLK;
+    if (folds) {
       const TcScale sc = tc_scale(a, b);
       int lmax = -127;
-      // (rows past m and columns past n hold zeros: their operands were zero-filled by TMA,
-      // as the k tail is)
 #pragma unroll
-      for (int i = 0; i < 64; ++i) {
-        run_re[i] = run_re[i] * sc.sa * sc.sb;
-        run_im[i] = run_im[i] * sc.sa * sc.sb;
-        lmax = max(lmax, REAL ? max(exp_of(fabsf(run_re[i])), exp_of(fabsf(run_im[i])))
-                              : exp_of(fmaxf(fabsf(run_re[i]), fabsf(run_im[i]))));
-      }
-      tc_scale_finish(a, b, lmax, t == 0 && threadIdx.x == 64);
-    }
-    if constexpr (REAL) {
-      // run_re: columns n0 + half * 64 + (0 .. 63), run_im: the same + 128; one row per
-      // warp store (through shared memory when the columns are the unit-stride side)
-      const int64_t c0 = static_cast<int64_t>(n0) + half * 64;
-      store_real_cols<0>(C, a, run_re, c0, ro, row_ok, ok, rows_unit, tr, lane);
-      store_real_cols<32>(C, a, run_re, c0 + 32, ro, row_ok, ok, rows_unit, tr, lane);
-      store_real_cols<0>(C, a, run_im, c0 + 128, ro, row_ok, ok, rows_unit, tr, lane);
-      store_real_cols<32>(C, a, run_im, c0 + 160, ro, row_ok, ok, rows_unit, tr, lane);
-    } else {
+      for (int i = 0; i < G::MINE; ++i) {
+        const int u = part + 4 * i;
+        float* t = tr + (u >> 1) * BLK + lane * 33 + 16 * (u & 1);
+        // (rows past m and columns past n hold zeros: their operands were zero-filled by TMA)
 #pragma unroll
-      for (int cb = 0; cb < 2; ++cb) {
-        const int64_t nb0 = static_cast<int64_t>(n0) + half * 64 + cb * 32;
-        const int64_t n = nb0 + lane;
-        const bool col_ok = ok && n < a.n;
-        const int64_t co = col_ok ? map_offset(a.cols, n) : 0;  // lane j: column nb0 + j
-        if (rows_unit) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int64_t co_j = __shfl_sync(0xffffffffu, co, j);
-            if (row_ok && nb0 + j < a.n) {
-              C[ro + co_j] = run_re[cb * 32 + j];
-              C[a.c_plane + ro + co_j] = run_im[cb * 32 + j];
-            }
+        for (int j = 0; j < 16; ++j) {
+          float re = run[0][i][j], im = REAL ? 0.f : run[NP - 1][i][j];
+          if constexpr (SCALED) {
+            re = re * sc.sa * sc.sb;
+            im = im * sc.sa * sc.sb;
+            lmax = max(lmax, exp_of(REAL ? fabsf(re) : fmaxf(fabsf(re), fabsf(im))));
           }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            tr[lane * 33 + j] = run_re[cb * 32 + j];
-            tr[32 * 33 + lane * 33 + j] = run_im[cb * 32 + j];
-          }
-          __syncwarp();
-          for (int r = 0; r < 32; ++r) {
-            const int64_t ro_r = __shfl_sync(0xffffffffu, ro, r);
-            const bool ok_r = __shfl_sync(0xffffffffu, row_ok ? 1 : 0, r) != 0;
-            if (ok_r && col_ok) {
-              C[ro_r + co] = tr[r * 33 + lane];
-              C[a.c_plane + ro_r + co] = tr[32 * 33 + r * 33 + lane];
-            }
-          }
-          __syncwarp();
+          t[j] = re;
+          if constexpr (!REAL) t[32 * 33 + j] = im;
         }
       }
+      if constexpr (SCALED) tc_scale_finish(a, b, lmax, t == 0 && threadIdx.x == 64);
+    }
+    // (the row offsets come from warps of other quarters: a barrier of all workers)
+    asm volatile("bar.sync 1, 512;" ::: "memory");
+    // blocks dealt out four at a time; a last round of fewer is shared by the warps
+    static_assert(G::NB % 4 != 3, "parts of the last round");
+    const int64_t rows_left = ok ? a.m - m0 - 32 * q : 0, cols_left = a.n - n0;
+#pragma unroll 1
+    for (int c0 = 0; c0 < G::NB; c0 += 4) {
+      const int left = G::NB - c0 < 4 ? G::NB - c0 : 4, parts = 4 / left;
+      const int c = c0 + part / parts;
+      store_block_planned<REAL>(C, a.c_plane, kFmtPlanar, tr + c * BLK, 33, 32 * 33, row_off + 32 * q, col_off + 32 * c,
+                                static_cast<int>(rows_left < 32 ? rows_left : 32),
+                                static_cast<int>(cols_left - 32 * c < 32 ? cols_left - 32 * c : 32), a.blk, lane,
+                                part % parts, parts);
     }
   }
   fence_before();
   __syncthreads();
   if (warp == 1) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C3::COLS));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(G::COLS));
   }
 }
 
@@ -628,10 +611,37 @@ __global__ void __launch_bounds__(C3::THREADS, 1)
 int64_t map_planes(bool batched, int32_t nb, bool real) {
   return (batched ? static_cast<int64_t>(nb) : 1) * (real ? 1 : 2);
 }
-// Output columns per tile of the TF32-family kernels: real steps take 128 x 256 tiles.
+// Tiles of a TF32 step: 128 x 256 real, 128 x 128 complex.
 int64_t tf32_tiles(int64_t m, int64_t n, bool real) {
   const int64_t tn = real ? 2 * BN : BN;
   return ((m + BM - 1) / BM) * ((n + tn - 1) / tn);
+}
+int64_t tc3t_tiles(int64_t m, int64_t n, int bt) { return ((m + BM - 1) / BM) * ((n + bt - 1) / bt); }
+
+// Columns of a 3xTF32 step's tile: the least waves x (k-blocks x time of one + time of a tile's
+// prologue and epilogue), in microseconds as measured with full waves (the bits do not depend on
+// it). Wide tiles have the cheaper k-blocks per output, narrow ones fill the SMs when there are
+// few outputs: real 1024 x 4096 x 256 33 / 25 / 35 us with 192 / 128 / 64 columns.
+int tc3t_bt(int64_t m, int64_t n, int64_t k, int32_t nb, bool real) {
+  struct Form {
+    int bt;
+    double block, tile;
+  };
+  static const Form kReal[] = {{192, 0.92, 6.7}, {128, 0.66, 4.9}, {64, 0.48, 3.8}};
+  static const Form kCplx[] = {{64, 1.0, 5.8}, {32, 0.70, 4.4}};
+  const int64_t sms = device_sms() > 0 ? device_sms() : 148;
+  const double kb = double((k + 31) / 32);
+  int best = 0;
+  double best_t = 0.0;
+  for (int i = 0; i < (real ? 3 : 2); ++i) {
+    const Form& f = real ? kReal[i] : kCplx[i];
+    const double waves = double((tc3t_tiles(m, n, f.bt) * nb + sms - 1) / sms), t = waves * (kb * f.block + f.tile);
+    if (best == 0 || t < best_t) {
+      best = f.bt;
+      best_t = t;
+    }
+  }
+  return best;
 }
 
 template <bool REAL, bool SCALED>
@@ -648,17 +658,28 @@ cudaError_t launch_tf32(const StepArgs& a, int32_t nb, int* err, cudaStream_t st
                       tb, a, err);
 }
 
-template <bool REAL, bool SCALED>
-cudaError_t launch_tc3(const StepArgs& a, int32_t nb, int* err, cudaStream_t st) {
+template <bool REAL, bool SCALED, int BT>
+cudaError_t launch_tc3t(const StepArgs& a, int32_t nb, int* err, cudaStream_t st) {
+  using G = C3T<REAL, BT>;
   static const cudaError_t configured = cudaFuncSetAttribute(
-      contract_tc3_kernel<REAL, SCALED>, cudaFuncAttributeMaxDynamicSharedMemorySize, C3::SMEM);
+      contract_tc3t_kernel<REAL, SCALED, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
   if (configured != cudaSuccess) return configured;
   CUtensorMap ta, tb;
-  if (!make_map(&ta, a.A, a.m, a.k, map_planes(a.a_bstride != 0, nb, REAL), a.a_plane, BM, C3::BK) ||
-      !make_map(&tb, a.B, a.n, a.k, map_planes(a.b_bstride != 0, nb, REAL), a.b_plane, BN, C3::BK))
+  if (!make_map(&ta, a.A, a.m, a.k, map_planes(a.a_bstride != 0, nb, REAL), a.a_plane, BM, G::BK) ||
+      !make_map(&tb, a.B, a.n, a.k, map_planes(a.b_bstride != 0, nb, REAL), a.b_plane, BT, G::BK))
     return cudaErrorInvalidValue;
-  return launch_bands(contract_tc3_kernel<REAL, SCALED>, tf32_tiles(a.m, a.n, REAL), nb, C3::THREADS, C3::SMEM, st,
+  return launch_bands(contract_tc3t_kernel<REAL, SCALED, BT>, tc3t_tiles(a.m, a.n, BT), nb, G::THREADS, G::SMEM, st,
                       ta, tb, a, err);
+}
+
+template <bool SCALED>
+cudaError_t launch_3xtf32(const StepArgs& a, int32_t nb, bool cplx, int* err, cudaStream_t st) {
+  const int bt = tc3t_bt(a.m, a.n, a.k, nb, !cplx);
+  if (cplx)
+    return bt == 32 ? launch_tc3t<false, SCALED, 32>(a, nb, err, st) : launch_tc3t<false, SCALED, 64>(a, nb, err, st);
+  if (bt == 64) return launch_tc3t<true, SCALED, 64>(a, nb, err, st);
+  if (bt == 128) return launch_tc3t<true, SCALED, 128>(a, nb, err, st);
+  return launch_tc3t<true, SCALED, 192>(a, nb, err, st);
 }
 
 }  // namespace
@@ -668,16 +689,19 @@ cudaError_t launch_contract_tf32(const StepArgs& a, int32_t nb, int32_t prec, bo
   const bool sc = a.recs != nullptr;
   if (!cplx) {
     if (prec == TN_R32_TF32) return sc ? launch_tf32<true, true>(a, nb, err, st) : launch_tf32<true, false>(a, nb, err, st);
-    if (prec == TN_R32_3XTF32) return sc ? launch_tc3<true, true>(a, nb, err, st) : launch_tc3<true, false>(a, nb, err, st);
+    if (prec == TN_R32_3XTF32) return sc ? launch_3xtf32<true>(a, nb, false, err, st) : launch_3xtf32<false>(a, nb, false, err, st);
     return cudaErrorNotSupported;
   }
   if (prec == TN_C64_TF32) return sc ? launch_tf32<false, true>(a, nb, err, st) : launch_tf32<false, false>(a, nb, err, st);
-  if (prec == TN_C64_3XTF32) return sc ? launch_tc3<false, true>(a, nb, err, st) : launch_tc3<false, false>(a, nb, err, st);
+  if (prec == TN_C64_3XTF32) return sc ? launch_3xtf32<true>(a, nb, true, err, st) : launch_3xtf32<false>(a, nb, true, err, st);
   return cudaErrorNotSupported;
 }
 
-int64_t tf32_launches(int64_t m, int64_t n, int32_t nb, bool real) {
-  const int64_t tiles = tf32_tiles(m, n, real);
+int64_t tf32_launches(int64_t m, int64_t n, int64_t k, int32_t nb, int32_t prec) {
+  const bool real = prec == TN_R32_TF32 || prec == TN_R32_3XTF32;
+  const int64_t tiles = prec == TN_C64_3XTF32 || prec == TN_R32_3XTF32
+                            ? tc3t_tiles(m, n, tc3t_bt(m, n, k, nb, real))
+                            : tf32_tiles(m, n, real);
   const int64_t per = sm_band_tiles(tiles, nb);
   return (tiles + per - 1) / per;
 }

@@ -69,6 +69,7 @@ struct StepArgs {
   int64_t a_bstride, b_bstride, c_bstride;  // floats
   int64_t a_plane, b_plane, c_plane;        // floats
   OffsetMap rows, cols;
+  BlockPlan blk;                            // address order of C's 32 x 32 blocks
   ScaleRec* recs;                           // null: no exponent scaling
   int32_t rec_a, rec_b, rec_c;
   int32_t c_split;                          // C's storage mode: 0 planar, 1 split, 2 split 3M
@@ -159,6 +160,6 @@ int64_t tc_launches(int64_t m, int64_t n, int64_t k, int32_t nb, int32_t prec, b
 // and the launches such a step makes.
 cudaError_t launch_contract_tf32(const StepArgs& a, int32_t nb, int32_t prec, bool cplx, int* err,
                                  cudaStream_t st);
-int64_t tf32_launches(int64_t m, int64_t n, int32_t nb, bool real);
+int64_t tf32_launches(int64_t m, int64_t n, int64_t k, int32_t nb, int32_t prec);
 
 }  // namespace tn

@@ -28,7 +28,36 @@ bool is_tc_prec(int32_t p) {
          p == TN_R32_3XTF32 || p == TN_R32_BF16X3;
 }
 
+// The weights of the low five bits of an index under `om`; false unless all are powers of two.
+bool bit_weights(const OffsetMap& om, int (&log2w)[5]) {
+  int n = 0;
+  for (int d = om.n - 1; d >= 0 && n < 5; --d) {
+    const uint32_t e = om.ext[d];
+    const int64_t w = om.stride[d];
+    if ((e & (e - 1u)) != 0u || w <= 0 || (w & (w - 1)) != 0) return false;
+    const int lw = __builtin_ctzll(static_cast<unsigned long long>(w));
+    for (int i = 0; (e >> i) > 1u && n < 5; ++i) log2w[n++] = lw + i;
+  }
+  return n == 5;
+}
+
 }  // namespace
+
+BlockPlan block_plan(const OffsetMap& rows, const OffsetMap& cols) {
+  BlockPlan p{};
+  int r[5], c[5];
+  if (!bit_weights(rows, r) || !bit_weights(cols, c)) return p;
+  int order[10];
+  std::iota(order, order + 10, 0);
+  auto weight = [&](int x) { return x < 5 ? r[x] : c[x - 5]; };
+  std::sort(order, order + 10, [&](int x, int y) { return weight(x) < weight(y); });
+  for (int k = 0; k < 10; ++k) {
+    p.e[k] = static_cast<int8_t>(weight(order[k]));
+    p.src[k] = static_cast<int8_t>(order[k]);
+  }
+  p.ok = 1;
+  return p;
+}
 
 // Rates of the kernel choice (t = max(bytes/B, flops/F), Sec. IV-C Eq. 6): B the HBM copy
 // rate, F per kernel family its peak in algorithmic flops (8 per complex MAC). Defaults:
@@ -364,6 +393,7 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
       err = "output interleaving too fine for the offset maps";
       return TN_ERR_UNSUPPORTED;
     }
+    st.blk = block_plan(st.rows, st.cols);
     const double flops = fm * double(st.m) * double(st.n) * double(st.k);
     const double bytes = eb * (double(st.m) * st.k + double(st.n) * st.k + double(st.m) * st.n);
     const double t_simt = std::max(bytes / g_cost.hbm_bytes_per_s, flops / g_cost.simt_flops);

@@ -55,6 +55,20 @@ __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uin
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
+// The same with A in tensor memory: 128 lanes (rows) x 8 columns (terms) at `a`.
+__device__ __forceinline__ void mma_tf32_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+// One lane of a fully active warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
                : "memory");
@@ -76,7 +90,47 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+// 16 consecutive fp32 columns of this thread's TMEM lane, not yet waited for: valid after
+// tmem_ld_wait on the same registers.
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];"
+      : TN_R8(0), TN_R8(8)
+      : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
 #undef TN_R8
+// Wait for every tcgen05.ld of this thread; the registers pass through the wait, so no use of
+// them can move above it.
+template <int U>
+__device__ __forceinline__ void tmem_ld_wait(float (&v)[U][16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int i = 0; i < 16; ++i) asm volatile("" : "+f"(v[u][i])::"memory");
+}
+
+// W (8 or 16) consecutive fp32 columns of this thread's TMEM lane, written (the caller waits:
+// tcgen05.wait::st).
+#define TN_V8(i) "r"(__float_as_uint(v[i + 0])), "r"(__float_as_uint(v[i + 1])), "r"(__float_as_uint(v[i + 2])), \
+                 "r"(__float_as_uint(v[i + 3])), "r"(__float_as_uint(v[i + 4])), "r"(__float_as_uint(v[i + 5])), \
+                 "r"(__float_as_uint(v[i + 6])), "r"(__float_as_uint(v[i + 7]))
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), TN_V8(0)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16};" ::"r"(taddr),
+      TN_V8(0), TN_V8(8)
+      : "memory");
+}
+#undef TN_V8
 
 // V consecutive 16-bit values (the low halves of x[]) as one store of 2V bytes.
 template <int V>
@@ -234,6 +288,7 @@ __device__ __forceinline__ void store_sorted(float* C, int64_t plane, int split,
       il += step(VB + k);
       al += int64_t(1) << e[VB + k];
     }
+#pragma unroll 1
   for (int s = part; s < (32 >> VB); s += parts) {
     int is = il;
     int64_t ah = 0;
@@ -370,6 +425,46 @@ __device__ __forceinline__ void store_block(float* C, int64_t plane, int split, 
   }
 }
 
+// Store one 32 x 32 block of a result tile from shared memory (t[r * pitch + c] = Re, t[cs + ...] =
+// Im) by the step's block plan: the address order is the plan's, worked out once on the host (a
+// sorting network per block, executed once per tile, costs an SM thousands of clocks of
+// instruction fetches). ro / co: offsets of the block's rows / columns in shared memory, of which
+// `rows` / `cols` are in range. A ragged block, or a map without power-of-two weights, is stored
+// one row per warp store. part of parts: this warp's share of the stores.
+template <bool REAL>
+__device__ __forceinline__ void store_block_planned(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
+                                                    const int64_t* ro, const int64_t* co, int rows, int cols,
+                                                    const BlockPlan& p, int lane, int part, int parts) {
+  if (p.ok && rows >= 32 && cols >= 32) {
+    const int64_t base = ro[0] + co[0];
+    int e[10], src[10], vb = 0;
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+      e[k] = p.e[k];
+      src[k] = p.src[k];
+    }
+    const int64_t align = REAL ? base : (base | plane);
+    bool run = true;  // the smallest weights are 1, 2, 4, ... and the block is aligned
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      run = run && e[k] == k && k < (!REAL && split ? 3 : 2) && (align & ((int64_t(2) << k) - 1)) == 0;
+      if (run) vb = k + 1;
+    }
+    if constexpr (!REAL) {
+      if (vb == 3) return store_sorted<3>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
+    }
+    if (vb == 2) return store_sorted<2, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
+    if (vb == 1) return store_sorted<1, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
+    return store_sorted<0, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
+  }
+  if (lane >= cols) return;
+  const int64_t c = co[lane];
+  for (int r = part; r < 32 && r < rows; r += parts) {
+    if constexpr (REAL) C[ro[r] + c] = t[r * pitch + lane];
+    else store_cplx(C, plane, ro[r] + c, t[r * pitch + lane], t[cs + r * pitch + lane], split);
+  }
+}
+
 // Exponent scaling on a tensor-core step. The operands are read as stored, so their
 // scales 2^-e_A and 2^-e_B multiply the accumulated result instead of each operand: the
 // same values as scaling on load, as a power of two commutes with every rounding in
@@ -432,10 +527,8 @@ bool make_map(CUtensorMap* map, const float* base, int64_t rows, int64_t k, int6
   return r == CUDA_SUCCESS;
 }
 
-// Tiles per batch entry in one launch of a one-tile-per-CTA kernel (one CTA per SM by its
-// shared memory): about kBandWaves waves of the SMs, for the reason given at
-// pair_band_tiles.
-int64_t sm_band_tiles(int64_t tiles, int32_t nb) {
+// SMs of the device (0: none).
+int device_sms() {
   static const int sms = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
@@ -443,6 +536,14 @@ int64_t sm_band_tiles(int64_t tiles, int32_t nb) {
       n = 0;
     return n;
   }();
+  return sms;
+}
+
+// Tiles per batch entry in one launch of a one-tile-per-CTA kernel (one CTA per SM by its
+// shared memory): about kBandWaves waves of the SMs, for the reason given at
+// pair_band_tiles.
+int64_t sm_band_tiles(int64_t tiles, int32_t nb) {
+  const int sms = device_sms();
   if (kBandWaves <= 0 || sms <= 0 || nb <= 0) return tiles;
   const int64_t want = (int64_t(sms) * kBandWaves + nb - 1) / nb;
   return want < tiles ? want : tiles;

@@ -23,6 +23,17 @@ struct OffsetMap {
   int64_t stride[kMaxDims];
 };
 
+// The address order of the 32 x 32 blocks of an output (blocks that start at multiples of 32 rows
+// and columns): when the low five bits of the row and of the column index each carry a
+// power-of-two weight in the output offset, bit k of an address-ordered element index weighs
+// 2^e[k] elements and comes from bit src[k] of the row (0-4) or column (5-9) index. ok 0: some
+// weight is not a power of two, or the map has fewer bits.
+struct BlockPlan {
+  int32_t ok;
+  int8_t e[10], src[10];
+};
+BlockPlan block_plan(const OffsetMap& rows, const OffsetMap& cols);
+
 // Per-leaf staging descriptor (a4): copy leaf t from its declared order into its
 // planned order, fixing sliced labels from the slice id, and split complex64 into
 // planar float32 (re plane, im plane).
@@ -83,6 +94,7 @@ struct StepRec {
   int32_t cls = TN_CLASS_SIMT;
   bool batched = false;
   OffsetMap rows{}, cols{};
+  BlockPlan blk{};
   int32_t ksplit = 1;  // SIMT steps too few tiles to fill the GPU: k cut in this many parts
   bool single_sm = false;  // tensor-core step kept on one SM per tile (tn_plan_autotune's choice)
   int32_t chain = -1;      // index of the step chain (a run of tiny CUDA-core steps) it is in
