@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
   uint64_t* acc_empty = acc_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + BN - 1) / BN;
   const int64_t t = t_first + blockIdx.x;  // this launch's tiles start at t_first
   const int64_t per_group = GROUP_M * tiles_n;
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -157,7 +157,9 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
         if (!mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1)) atomicExch(err, 22);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();  // (all lanes run the loop: see elect_one)
+      const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
       constexpr uint32_t id_w = idesc_bf16(BM, 2 * BN);   // A . [B_re | B_im] -> (Re | Im)
       constexpr uint32_t id_n = idesc_bf16(BM, BN);
       const uint32_t d_hi = tmem, d_lo = tmem + 256;
@@ -166,20 +168,21 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
         const int kb_end = min(num_kb, (c + 1) * CK);
         for (int kb = c * CK; kb < kb_end; ++kb) {
           const int s = kb % STAGES;
-          if (!mbar_wait(&full[s], (kb / STAGES) & 1)) {
-            atomicExch(err, 23);
+          if (!mbar_wait_warp(&full[s], (kb / STAGES) & 1)) {
+            if (leader) atomicExch(err, 23);
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t sa = su32(smem + s * STAGE), sb = sa + CB::OFF_B;
+          const uint64_t sa = desc0 + static_cast<uint32_t>(s * (STAGE >> 4)), sb = sa + (CB::OFF_B >> 4);
+          if (leader) {
 #pragma unroll
           for (int j = 0; j < BK / 16; ++j) {
             const uint32_t o = j * 32;
-            const uint64_t ar_l = smem_desc<ROWB>(sa + 2 * PLANE + o), ai_l = smem_desc<ROWB>(sa + 3 * PLANE + o);
-            const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PLANE + o);
-            const uint64_t b_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PLANE + o);
-            const uint64_t b_l = smem_desc<ROWB>(sb + 2 * PLANE + o), bi_l = smem_desc<ROWB>(sb + 3 * PLANE + o);
+            const uint64_t ar_l = sa + ((2 * PLANE + o) >> 4), ai_l = sa + ((3 * PLANE + o) >> 4);
+            const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PLANE + o) >> 4);
+            const uint64_t b_h = sb + ((o) >> 4), bi_h = sb + ((PLANE + o) >> 4);
+            const uint64_t b_l = sb + ((2 * PLANE + o) >> 4), bi_l = sb + ((3 * PLANE + o) >> 4);
             const uint32_t first = (kb > 0 || j > 0) ? 1u : 0u;
             mma_bf16(d_lo, ar_l, b_h, id_w, first);              // A_re_lo . [B_re_h | B_im_h]
             mma_bf16(d_lo, ai_l, bi_h, id_n | kNegateA, 1u);     // Re -= A_im_lo . B_im_h
@@ -188,29 +191,33 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
             mma_bf16(d_lo, ai_h, bi_l, id_n | kNegateA, 1u);
             mma_bf16(d_lo + 128, ai_h, b_l, id_n, 1u);
           }
+          }
           if (kb == c * CK) {
             // the chunk accumulator must have been folded before the hi MMAs reuse it
-            if (!mbar_wait(acc_empty, (c & 1) ^ 1)) {
-              atomicExch(err, 24);
+            if (!mbar_wait_warp(acc_empty, (c & 1) ^ 1)) {
+              if (leader) atomicExch(err, 24);
               ok = false;
-              mma_commit(&empty[s]);
+              if (leader) mma_commit(&empty[s]);
               break;
             }
             fence_after();
           }
+          if (leader) {
 #pragma unroll
           for (int j = 0; j < BK / 16; ++j) {
             const uint32_t o = j * 32;
-            const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PLANE + o);
-            const uint64_t b_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PLANE + o);
+            const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PLANE + o) >> 4);
+            const uint64_t b_h = sb + ((o) >> 4), bi_h = sb + ((PLANE + o) >> 4);
             const uint32_t acc = (kb > c * CK || j > 0) ? 1u : 0u;
             mma_bf16(d_hi, ar_h, b_h, id_w, acc);
             mma_bf16(d_hi, ai_h, bi_h, id_n | kNegateA, 1u);
             mma_bf16(d_hi + 128, ai_h, b_h, id_n, 1u);
           }
-          mma_commit(&empty[s]);
+          }
+          __syncwarp();
+          if (leader) mma_commit(&empty[s]);
         }
-        mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
+        if (leader) mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
       }
     }
   } else {
@@ -376,7 +383,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
 
   uint32_t rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + 2 * BM - 1) / (2 * BM), tiles_n = (a.n + BN - 1) / BN;
   const int64_t t = t_first + (blockIdx.x >> 1);  // this launch's tiles start at t_first
   const int64_t per_group = CB2::GROUP * tiles_n;
@@ -411,7 +418,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers initialised and the pair's TMEM allocated
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
   const bool skip = ld_leader_u32(skip_slot) != 0;  // one decision for the pair
 
   if (skip) {
@@ -439,7 +446,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 1) {
+    if (rank == 1) {
+      if (lane == 0) {
       // forward each landed stage to CTA 0, in order
       for (int kb = 0; kb < num_kb; ++kb) {
         if (!mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1)) {
@@ -448,18 +456,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
         }
         mbar_arrive_leader(&ready[kb % STAGES]);
       }
-    } else if (lane == 0) {
+      }
+    } else {
+      const bool leader = elect_one();
+      const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
       constexpr uint32_t id = idesc_bf16(2 * BM, BN);
       const uint32_t d_hi = tmem, d_lo = tmem + 256;
       // the cross terms (into D_lo) of one k-block: 8 MMAs per 16-deep atom
-      auto cross = [&](uint32_t sa, uint32_t sb, bool first_kb) {
+      auto cross = [&](uint64_t sa, uint64_t sb, bool first_kb) {
+        if (!leader) return;
 #pragma unroll
         for (int j = 0; j < BK / 16; ++j) {
           const uint32_t o = j * 32;
-          const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PA + o);
-          const uint64_t ar_l = smem_desc<ROWB>(sa + 2 * PA + o), ai_l = smem_desc<ROWB>(sa + 3 * PA + o);
-          const uint64_t br_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PB + o);
-          const uint64_t br_l = smem_desc<ROWB>(sb + 2 * PB + o), bi_l = smem_desc<ROWB>(sb + 3 * PB + o);
+          const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PA + o) >> 4);
+          const uint64_t ar_l = sa + ((2 * PA + o) >> 4), ai_l = sa + ((3 * PA + o) >> 4);
+          const uint64_t br_h = sb + ((o) >> 4), bi_h = sb + ((PB + o) >> 4);
+          const uint64_t br_l = sb + ((2 * PB + o) >> 4), bi_l = sb + ((3 * PB + o) >> 4);
           const uint32_t first = (!first_kb || j > 0) ? 1u : 0u;
           mma_bf16_pair(d_lo, ar_l, br_h, id, first);           // Re += A_re_lo . B_re_h
           mma_bf16_pair(d_lo, ai_l, bi_h, id | kNegateA, 1u);   // Re -= A_im_lo . B_im_h
@@ -472,12 +484,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
         }
       };
       // hi . hi of one k-block into the chunk accumulator D_hi: 4 MMAs per atom
-      auto hihi = [&](uint32_t sa, uint32_t sb, bool first_kb) {
+      auto hihi = [&](uint64_t sa, uint64_t sb, bool first_kb) {
+        if (!leader) return;
 #pragma unroll
         for (int j = 0; j < BK / 16; ++j) {
           const uint32_t o = j * 32;
-          const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PA + o);
-          const uint64_t br_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PB + o);
+          const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PA + o) >> 4);
+          const uint64_t br_h = sb + ((o) >> 4), bi_h = sb + ((PB + o) >> 4);
           const uint32_t acc = (!first_kb || j > 0) ? 1u : 0u;
           mma_bf16_pair(d_hi, ar_h, br_h, id, acc);
           mma_bf16_pair(d_hi, ai_h, bi_h, id | kNegateA, 1u);
@@ -485,9 +498,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
           mma_bf16_pair(d_hi + 128, ai_h, br_h, id, 1u);
         }
       };
-      auto stage_a = [&](int kb) { return su32(smem + (kb % STAGES) * STAGE); };
+      auto stage_a = [&](int kb) { return desc0 + static_cast<uint32_t>((kb % STAGES) * (STAGE >> 4)); };
       auto landed = [&](int kb) {
-        return mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1) && mbar_wait(&ready[kb % STAGES], (kb / STAGES) & 1);
+        return mbar_wait_warp(&full[kb % STAGES], (kb / STAGES) & 1) && mbar_wait_warp(&ready[kb % STAGES], (kb / STAGES) & 1);
       };
       // Per chunk: the cross terms of its first LEAD k-blocks are issued before the wait for
       // the previous chunk's fold (which both CTAs' warps must report, one of them across
@@ -501,38 +514,40 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
         const int lead_end = min(kb_end, kb0 + LEAD);
         for (int kb = kb0; kb < lead_end && ok; ++kb) {
           if (!landed(kb)) {
-            atomicExch(err, 55);
+            if (leader) atomicExch(err, 55);
             ok = false;
             break;
           }
           fence_after();
-          cross(stage_a(kb), stage_a(kb) + CB2::OFF_B, kb == 0);
+          cross(stage_a(kb), stage_a(kb) + (CB2::OFF_B >> 4), kb == 0);
         }
-        if (ok && !mbar_wait(acc_empty, (c & 1) ^ 1)) {  // the chunk accumulator is free
-          atomicExch(err, 56);
+        if (ok && !mbar_wait_warp(acc_empty, (c & 1) ^ 1)) {  // the chunk accumulator is free
+          if (leader) atomicExch(err, 56);
           ok = false;
         }
         if (!ok) {
-          mma_commit_pair(acc_full);  // let the fold see the issued MMAs retire
+          if (leader) mma_commit_pair(acc_full);  // let the fold see the issued MMAs retire
           break;
         }
         fence_after();
         for (int kb = kb0; kb < lead_end; ++kb) {
-          hihi(stage_a(kb), stage_a(kb) + CB2::OFF_B, kb == kb0);
-          mma_commit_pair(&empty[kb % STAGES]);
+          hihi(stage_a(kb), stage_a(kb) + (CB2::OFF_B >> 4), kb == kb0);
+          if (leader) mma_commit_pair(&empty[kb % STAGES]);
+          __syncwarp();
         }
         for (int kb = lead_end; kb < kb_end; ++kb) {
           if (!landed(kb)) {
-            atomicExch(err, 55);
+            if (leader) atomicExch(err, 55);
             ok = false;
             break;
           }
           fence_after();
-          cross(stage_a(kb), stage_a(kb) + CB2::OFF_B, false);
-          hihi(stage_a(kb), stage_a(kb) + CB2::OFF_B, false);
-          mma_commit_pair(&empty[kb % STAGES]);
+          cross(stage_a(kb), stage_a(kb) + (CB2::OFF_B >> 4), false);
+          hihi(stage_a(kb), stage_a(kb) + (CB2::OFF_B >> 4), false);
+          if (leader) mma_commit_pair(&empty[kb % STAGES]);
+          __syncwarp();
         }
-        mma_commit_pair(acc_full);  // also on error, so the fold sees issued MMAs retire
+        if (leader) mma_commit_pair(acc_full);  // also on error, so the fold sees issued MMAs retire
       }
     }
   } else {
@@ -659,7 +674,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
 
   uint32_t rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + 2 * BM - 1) / (2 * BM), tiles_n = (a.n + BN - 1) / BN;
   const int64_t tiles = tiles_m * tiles_n, total = tiles * nb;
   const int64_t cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
@@ -699,7 +714,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
   __syncthreads();
   cluster_sync_all();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
   const bool skip = ld_leader_u32(skip_slot) != 0;
 
   if (skip) {
@@ -732,7 +747,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 1) {
+    if (rank == 1) {
+      if (lane == 0) {
       // forward each landed stage to CTA 0, in order
       const int64_t mine = total > cluster ? (total - cluster + n_clusters - 1) / n_clusters : 0;
       const int64_t blocks = mine * num_kb;
@@ -743,17 +759,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
         }
         mbar_arrive_leader(&ready[g % STAGES]);
       }
-    } else if (lane == 0) {
+      }
+    } else {
+      const bool leader = elect_one();
+      const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
       constexpr uint32_t id = idesc_bf16(2 * BM, BN);
       const uint32_t d_hi = tmem, d_lo = tmem + 256;
-      auto cross = [&](uint32_t sa, uint32_t sb, bool first_kb) {
+      auto cross = [&](uint64_t sa, uint64_t sb, bool first_kb) {
+        if (!leader) return;
 #pragma unroll
         for (int j = 0; j < BK / 16; ++j) {
           const uint32_t o = j * 32;
-          const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PA + o);
-          const uint64_t ar_l = smem_desc<ROWB>(sa + 2 * PA + o), ai_l = smem_desc<ROWB>(sa + 3 * PA + o);
-          const uint64_t br_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PB + o);
-          const uint64_t br_l = smem_desc<ROWB>(sb + 2 * PB + o), bi_l = smem_desc<ROWB>(sb + 3 * PB + o);
+          const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PA + o) >> 4);
+          const uint64_t ar_l = sa + ((2 * PA + o) >> 4), ai_l = sa + ((3 * PA + o) >> 4);
+          const uint64_t br_h = sb + ((o) >> 4), bi_h = sb + ((PB + o) >> 4);
+          const uint64_t br_l = sb + ((2 * PB + o) >> 4), bi_l = sb + ((3 * PB + o) >> 4);
           const uint32_t first = (!first_kb || j > 0) ? 1u : 0u;
           mma_bf16_pair(d_lo, ar_l, br_h, id, first);
           mma_bf16_pair(d_lo, ai_l, bi_h, id | kNegateA, 1u);
@@ -765,12 +785,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
           mma_bf16_pair(d_lo + 128, ai_h, br_l, id, 1u);
         }
       };
-      auto hihi = [&](uint32_t sa, uint32_t sb, bool first_kb) {
+      auto hihi = [&](uint64_t sa, uint64_t sb, bool first_kb) {
+        if (!leader) return;
 #pragma unroll
         for (int j = 0; j < BK / 16; ++j) {
           const uint32_t o = j * 32;
-          const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PA + o);
-          const uint64_t br_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PB + o);
+          const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PA + o) >> 4);
+          const uint64_t br_h = sb + ((o) >> 4), bi_h = sb + ((PB + o) >> 4);
           const uint32_t acc = (!first_kb || j > 0) ? 1u : 0u;
           mma_bf16_pair(d_hi, ar_h, br_h, id, acc);
           mma_bf16_pair(d_hi, ai_h, bi_h, id | kNegateA, 1u);
@@ -780,10 +801,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
       };
       int64_t g = 0;   // k-blocks consumed over all items
       int64_t G = 0;   // chunks over all items
-      auto stage_of = [&](int64_t gg) { return su32(smem + (gg % STAGES) * STAGE); };
+      auto stage_of = [&](int64_t gg) { return desc0 + static_cast<uint32_t>((gg % STAGES) * (STAGE >> 4)); };
       auto landed = [&](int64_t gg) {
         const uint32_t ph = static_cast<uint32_t>((gg / STAGES) & 1);
-        return mbar_wait(&full[gg % STAGES], ph) && mbar_wait(&ready[gg % STAGES], ph);
+        return mbar_wait_warp(&full[gg % STAGES], ph) && mbar_wait_warp(&ready[gg % STAGES], ph);
       };
       constexpr int LEAD = 2;
       bool ok = true;
@@ -794,40 +815,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
           const int lead_end = c == 0 ? kb0 : min(kb_end, kb0 + LEAD);
           for (int kb = kb0; kb < lead_end && ok; ++kb) {
             if (!landed(g + (kb - kb0))) {
-              atomicExch(err, 55);
+              if (leader) atomicExch(err, 55);
               ok = false;
               break;
             }
             fence_after();
-            cross(stage_of(g + (kb - kb0)), stage_of(g + (kb - kb0)) + CB2::OFF_B, false);
+            cross(stage_of(g + (kb - kb0)), stage_of(g + (kb - kb0)) + (CB2::OFF_B >> 4), false);
           }
-          if (ok && !mbar_wait(acc_empty, static_cast<uint32_t>(G & 1) ^ 1)) {
-            atomicExch(err, 56);
+          if (ok && !mbar_wait_warp(acc_empty, static_cast<uint32_t>(G & 1) ^ 1)) {
+            if (leader) atomicExch(err, 56);
             ok = false;
           }
           if (!ok) {
-            mma_commit_pair(acc_full);
+            if (leader) mma_commit_pair(acc_full);
             break;
           }
           fence_after();
           for (int kb = kb0; kb < lead_end; ++kb) {
-            hihi(stage_of(g), stage_of(g) + CB2::OFF_B, kb == kb0);
-            mma_commit_pair(&empty[g % STAGES]);
+            hihi(stage_of(g), stage_of(g) + (CB2::OFF_B >> 4), kb == kb0);
+            if (leader) mma_commit_pair(&empty[g % STAGES]);
+            __syncwarp();
             ++g;
           }
           for (int kb = lead_end; kb < kb_end; ++kb) {
             if (!landed(g)) {
-              atomicExch(err, 55);
+              if (leader) atomicExch(err, 55);
               ok = false;
               break;
             }
             fence_after();
-            cross(stage_of(g), stage_of(g) + CB2::OFF_B, kb == 0);
-            hihi(stage_of(g), stage_of(g) + CB2::OFF_B, kb == kb0);
-            mma_commit_pair(&empty[g % STAGES]);
+            cross(stage_of(g), stage_of(g) + (CB2::OFF_B >> 4), kb == 0);
+            hihi(stage_of(g), stage_of(g) + (CB2::OFF_B >> 4), kb == kb0);
+            if (leader) mma_commit_pair(&empty[g % STAGES]);
+            __syncwarp();
             ++g;
           }
-          mma_commit_pair(acc_full);  // also on error, so the fold sees issued MMAs retire
+          if (leader) mma_commit_pair(acc_full);  // also on error, so the fold sees issued MMAs retire
         }
       }
     }
@@ -980,7 +1003,7 @@ __global__ void __launch_bounds__(CB3::THREADS, 1)
   uint64_t* acc_empty = acc_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + BN - 1) / BN;
   const int64_t t = t_first + blockIdx.x;  // this launch's tiles start at t_first
   const int64_t per_group = GROUP_M * tiles_n;
@@ -1012,7 +1035,7 @@ __global__ void __launch_bounds__(CB3::THREADS, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
   const int n_items = 3 * num_kb;  // (k-block, product) slots in order
 
   if (warp == 0) {
@@ -1035,7 +1058,9 @@ __global__ void __launch_bounds__(CB3::THREADS, 1)
         if (!mbar_wait(&full[it % SLOTS], (it / SLOTS) & 1)) atomicExch(err, 32);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
+      const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
       constexpr uint32_t id_n = idesc_bf16(BM, BN);
       bool ok = true;
       for (int c = 0; c < n_chunks && ok; ++c) {
@@ -1043,37 +1068,40 @@ __global__ void __launch_bounds__(CB3::THREADS, 1)
         for (int kb = c * CK; kb < kb_end && ok; ++kb) {
           for (int j = 0; j < 3; ++j) {
             const int it = 3 * kb + j, s = it % SLOTS;
-            if (!mbar_wait(&full[s], (it / SLOTS) & 1)) {
-              atomicExch(err, 33);
+            if (!mbar_wait_warp(&full[s], (it / SLOTS) & 1)) {
+              if (leader) atomicExch(err, 33);
               ok = false;
               break;
             }
             if (kb == c * CK && j == 0) {
               // the accumulators must have been folded before this chunk overwrites them
-              if (!mbar_wait(acc_empty, (c & 1) ^ 1)) {
-                atomicExch(err, 34);
+              if (!mbar_wait_warp(acc_empty, (c & 1) ^ 1)) {
+                if (leader) atomicExch(err, 34);
                 ok = false;
-                mma_commit(&empty[s]);
+                if (leader) mma_commit(&empty[s]);
                 break;
               }
             }
             fence_after();
-            const uint32_t sa = su32(smem + s * SLOT), sb = sa + CB3::OFF_B;
+            const uint64_t sa = desc0 + static_cast<uint32_t>(s * (SLOT >> 4)), sb = sa + (CB3::OFF_B >> 4);
             const uint32_t d = tmem + 128 * j;
+            if (leader) {
 #pragma unroll
             for (int q = 0; q < BK / 16; ++q) {
               const uint32_t o = q * 32;
-              const uint64_t ah = smem_desc<ROWB>(sa + o), al = smem_desc<ROWB>(sa + PLANE + o);
-              const uint64_t bh = smem_desc<ROWB>(sb + o), bl = smem_desc<ROWB>(sb + PLANE + o);
+              const uint64_t ah = sa + ((o) >> 4), al = sa + ((PLANE + o) >> 4);
+              const uint64_t bh = sb + ((o) >> 4), bl = sb + ((PLANE + o) >> 4);
               const uint32_t acc = (kb > c * CK || q > 0) ? 1u : 0u;
               mma_bf16(d, ah, bh, id_n, acc);   // hi.hi
               mma_bf16(d, ah, bl, id_n, 1u);    // hi.lo
               mma_bf16(d, al, bh, id_n, 1u);    // lo.hi
             }
-            mma_commit(&empty[s]);
+            }
+            __syncwarp();
+            if (leader) mma_commit(&empty[s]);
           }
         }
-        mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
+        if (leader) mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
       }
     }
   } else {
@@ -1192,7 +1220,7 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
   uint64_t* acc_empty = acc_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + BN - 1) / BN;
   const int64_t total = tiles_m * tiles_n * nb;
   const int num_kb = static_cast<int>((a.k + BK - 1) / BK);  // <= CK: one fold chunk per tile
@@ -1216,7 +1244,7 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1243,7 +1271,9 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
         if (!mbar_wait(&full[j % STAGES], static_cast<uint32_t>((j / STAGES) & 1))) atomicExch(err, 32);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
+      const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
       constexpr uint32_t id_w = idesc_bf16(BM, 2 * BN);
       constexpr uint32_t id_n = idesc_bf16(BM, BN);
       const uint32_t d_hi = tmem, d_lo = tmem + 256;
@@ -1251,27 +1281,28 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
       bool ok = true;
       for (int64_t w = blockIdx.x; w < total && ok; w += gridDim.x, ++q) {
         // the previous tile's accumulators must have been read
-        if (!mbar_wait(acc_empty, static_cast<uint32_t>(q & 1) ^ 1)) {
-          atomicExch(err, 33);
+        if (!mbar_wait_warp(acc_empty, static_cast<uint32_t>(q & 1) ^ 1)) {
+          if (leader) atomicExch(err, 33);
           break;
         }
         fence_after();
         for (int kb = 0; kb < num_kb; ++kb, ++g) {
           const int s = static_cast<int>(g % STAGES);
-          if (!mbar_wait(&full[s], static_cast<uint32_t>((g / STAGES) & 1))) {
-            atomicExch(err, 34);
+          if (!mbar_wait_warp(&full[s], static_cast<uint32_t>((g / STAGES) & 1))) {
+            if (leader) atomicExch(err, 34);
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t sa = su32(smem + s * STAGE), sb = sa + CB::OFF_B;
+          const uint64_t sa = desc0 + static_cast<uint32_t>(s * (STAGE >> 4)), sb = sa + (CB::OFF_B >> 4);
+          if (leader) {
 #pragma unroll
           for (int j = 0; j < BK / 16; ++j) {
             const uint32_t o = j * 32;
-            const uint64_t ar_l = smem_desc<ROWB>(sa + 2 * PLANE + o), ai_l = smem_desc<ROWB>(sa + 3 * PLANE + o);
-            const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PLANE + o);
-            const uint64_t b_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PLANE + o);
-            const uint64_t b_l = smem_desc<ROWB>(sb + 2 * PLANE + o), bi_l = smem_desc<ROWB>(sb + 3 * PLANE + o);
+            const uint64_t ar_l = sa + ((2 * PLANE + o) >> 4), ai_l = sa + ((3 * PLANE + o) >> 4);
+            const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PLANE + o) >> 4);
+            const uint64_t b_h = sb + ((o) >> 4), bi_h = sb + ((PLANE + o) >> 4);
+            const uint64_t b_l = sb + ((2 * PLANE + o) >> 4), bi_l = sb + ((3 * PLANE + o) >> 4);
             const uint32_t acc = (kb > 0 || j > 0) ? 1u : 0u;
             mma_bf16(d_lo, ar_l, b_h, id_w, acc);
             mma_bf16(d_lo, ai_l, bi_h, id_n | kNegateA, 1u);
@@ -1283,9 +1314,11 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
             mma_bf16(d_hi, ai_h, bi_h, id_n | kNegateA, 1u);
             mma_bf16(d_hi + 128, ai_h, b_h, id_n, 1u);
           }
-          mma_commit(&empty[s]);
+          }
+          __syncwarp();
+          if (leader) mma_commit(&empty[s]);
         }
-        mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
+        if (leader) mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
       }
     }
   } else {
@@ -1400,7 +1433,7 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
   uint64_t* acc_empty = bars + 3;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + BN - 1) / BN;
   const int64_t total = tiles_m * tiles_n * nb;
   const int num_kb = static_cast<int>((a.k + BK - 1) / BK);  // 1 or 2
@@ -1422,7 +1455,7 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1446,33 +1479,36 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
       if (g > 0 && !mbar_wait(full, static_cast<uint32_t>((g - 1) & 1))) atomicExch(err, 62);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
+      const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
       constexpr uint32_t id_w = idesc_bf16(BM, 2 * BN);
       constexpr uint32_t id_n = idesc_bf16(BM, BN);
       const uint32_t d_hi = tmem, d_lo = tmem + 256;
       int64_t g = 0, q = 0;
       bool ok = true;
       for (int64_t w = blockIdx.x; w < total && ok; w += gridDim.x, ++q) {
-        if (!mbar_wait(acc_empty, static_cast<uint32_t>(q & 1) ^ 1)) {  // the previous tile was read
-          atomicExch(err, 63);
+        if (!mbar_wait_warp(acc_empty, static_cast<uint32_t>(q & 1) ^ 1)) {  // the previous tile was read
+          if (leader) atomicExch(err, 63);
           break;
         }
         fence_after();
         for (int kb = 0; kb < num_kb; ++kb, ++g) {
-          if (!mbar_wait(full, static_cast<uint32_t>(g & 1))) {
-            atomicExch(err, 64);
+          if (!mbar_wait_warp(full, static_cast<uint32_t>(g & 1))) {
+            if (leader) atomicExch(err, 64);
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t sa = su32(smem), sb = sa + CB::OFF_B;
+          const uint64_t sa = desc0, sb = sa + (CB::OFF_B >> 4);
+          if (leader) {
 #pragma unroll
           for (int j = 0; j < BK / 16; ++j) {
             const uint32_t o = j * 32;
-            const uint64_t ar_l = smem_desc<ROWB>(sa + 2 * PLANE + o), ai_l = smem_desc<ROWB>(sa + 3 * PLANE + o);
-            const uint64_t ar_h = smem_desc<ROWB>(sa + o), ai_h = smem_desc<ROWB>(sa + PLANE + o);
-            const uint64_t b_h = smem_desc<ROWB>(sb + o), bi_h = smem_desc<ROWB>(sb + PLANE + o);
-            const uint64_t b_l = smem_desc<ROWB>(sb + 2 * PLANE + o), bi_l = smem_desc<ROWB>(sb + 3 * PLANE + o);
+            const uint64_t ar_l = sa + ((2 * PLANE + o) >> 4), ai_l = sa + ((3 * PLANE + o) >> 4);
+            const uint64_t ar_h = sa + ((o) >> 4), ai_h = sa + ((PLANE + o) >> 4);
+            const uint64_t b_h = sb + ((o) >> 4), bi_h = sb + ((PLANE + o) >> 4);
+            const uint64_t b_l = sb + ((2 * PLANE + o) >> 4), bi_l = sb + ((3 * PLANE + o) >> 4);
             const uint32_t acc = (kb > 0 || j > 0) ? 1u : 0u;
             mma_bf16(d_lo, ar_l, b_h, id_w, acc);
             mma_bf16(d_lo, ai_l, bi_h, id_n | kNegateA, 1u);
@@ -1484,9 +1520,11 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
             mma_bf16(d_hi, ai_h, bi_h, id_n | kNegateA, 1u);
             mma_bf16(d_hi + 128, ai_h, b_h, id_n, 1u);
           }
-          mma_commit(empty);
+          }
+          __syncwarp();
+          if (leader) mma_commit(empty);
         }
-        mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
+        if (leader) mma_commit(acc_full);  // also on error, so the fold sees issued MMAs retire
       }
     }
   } else {

@@ -28,11 +28,11 @@ namespace tn {
 namespace {
 
 // TF32 form (contract_tc_kernel). A complex stage holds A_re A_im B_re B_im (3 stages, one
-// CTA per SM; tensor memory D_rr @0, D_ii @128, D_x @256; warps 0 TMA, 1 MMA, 2-5 epilogue).
+// CTA per SM; tensor memory D_rr @0, D_ii @128, D_x @256; warps 0 TMA, 1 MMA, 2-9 epilogue).
 // A real one holds A B_0 B_1, the two B tiles of a 256-column tile, in 2 stages, and its
 // accumulator takes 256 columns: two CTAs fit on an SM, so one's epilogue overlaps the
-// other's MMAs; eight epilogue warps (2-9: warp w drains TMEM lane quarter w % 4, columns
-// 128 ((w - 2) / 4) .. + 127) store its 32K results.
+// other's MMAs. Eight epilogue warps store a tile's results: warp w drains TMEM lane quarter
+// w % 4, the first or second half of the columns.
 template <bool REAL>
 struct Cfg {
   static constexpr int BK = 32;                             // fp32 elements per k-block
@@ -42,11 +42,12 @@ struct Cfg {
   static constexpr int OFF_B = REAL ? TILE_A : 2 * TILE_A;  // first B tile
   static constexpr int STAGE = REAL ? TILE_A + 2 * TILE_B : 2 * TILE_A + 2 * TILE_B;
   static constexpr int STAGES = REAL ? 2 : 3;
-  static constexpr int THREADS = REAL ? 320 : 192;
+  static constexpr int THREADS = 320;
   static constexpr uint32_t TMEM_COLS = REAL ? 256 : 512;
-  static constexpr int SMEM = STAGES * STAGE + 1024 /*barriers*/ + 1024 /*align*/;
+  static constexpr int OFFSETS = 8 * (BM + (REAL ? 2 : 1) * BN);  // output offsets of the rows and columns
+  static constexpr int SMEM = STAGES * STAGE + 512 /*barriers*/ + OFFSETS + 1024 /*align*/;
   static_assert(SMEM <= 232448 && STAGE % 1024 == 0 && OFF_B % 1024 == 0, "stages fit, swizzle-aligned tiles");
-  static_assert((THREADS / 32 - 2) * 2 * 32 * 33 * 4 <= STAGES * STAGE, "epilogue transposes fit the stages");
+  static_assert(8 * 2 * 32 * 33 * 4 <= STAGES * STAGE, "epilogue transposes fit the stages");
 };
 
 // v rounded to the nearest value with 10 fraction bits (ties away from zero): half a unit in
@@ -60,8 +61,12 @@ __device__ __forceinline__ float tf32_rn(float v) {
 // n0 .. n0 + 127 and n0 + 128 .. n0 + 255 side by side, one 128 x 256 MMA per k-atom reads
 // the two as one operand, and the accumulator's 256 columns are the tile's output columns
 // in order. SCALED: exponent scaling (a.recs).
+// Measured (GB300; before: MMAs issued from a divergent lane, the block order sorted per block, four
+// epilogue warps for a complex tile): complex 4096^3 822 -> 952 TFLOP/s, 8192 x 8192 x 512
+// 439 -> 593, 1024 x 65536 x 256 304 -> 432; real 16384 x 32768 x 1024 539 -> 667, 8192 x 16384 x 256
+// 229 -> 343 (bound by its stores, 2.7 TB/s). cuBLAS sustains 914-930.
 template <bool REAL, bool SCALED>
-__global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
+__global__ void __launch_bounds__(Cfg<REAL>::THREADS, REAL ? 2 : 1)
     contract_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        StepArgs a, int64_t t_first, int* err) {
   using G = Cfg<REAL>;
@@ -75,8 +80,10 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
   uint64_t* empty = bars + STAGES;           // [STAGES]
   uint64_t* acc_full = bars + 2 * STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  int64_t* row_off = reinterpret_cast<int64_t*>(bars + 64);  // [BM] output offsets of the tile's rows
+  int64_t* col_off = row_off + BM;                           // [TN] and columns
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   // grouped raster over output tiles for L2 reuse of A and B tiles
   const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + TN - 1) / TN;
   const int64_t t = t_first + blockIdx.x;  // this launch's tiles start at t_first
@@ -108,7 +115,7 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform_u32(*tmem_slot);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -140,24 +147,25 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
         if (!mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1)) atomicExch(err, 2);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_tf32(BM, TN);
-      const uint32_t d_rr = tmem, d_ii = tmem + 128, d_x = tmem + 256;
-      for (int kb = 0; kb < num_kb; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = (kb / STAGES) & 1;
-        if (!mbar_wait(&full[s], ph)) {
-          atomicExch(err, 3);
-          break;
-        }
-        fence_after();
-        const uint32_t st = su32(smem + s * STAGE);
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = idesc_tf32(BM, TN);
+    const uint32_t d_rr = tmem, d_ii = tmem + 128, d_x = tmem + 256;
+    const uint64_t desc0 = smem_desc<ROWB>(su32(smem));
+    for (int kb = 0; kb < num_kb; ++kb) {
+      const int s = kb % STAGES;
+      const uint32_t ph = (kb / STAGES) & 1;
+      if (!mbar_wait_warp(&full[s], ph)) {
+        if (leader) atomicExch(err, 3);
+        break;
+      }
+      fence_after();
+      const uint64_t st = desc0 + static_cast<uint32_t>(s * (STAGE >> 4));
+      if (leader) {
 #pragma unroll
         for (int j = 0; j < BK / 8; ++j) {
           const uint32_t acc = (kb > 0 || j > 0) ? 1u : 0u;
-          const uint64_t ar = smem_desc<ROWB>(st + j * 32), ai = smem_desc<ROWB>(st + TILE_A + j * 32);
-          const uint64_t br = smem_desc<ROWB>(st + OFF_B + j * 32);
-          const uint64_t bi = smem_desc<ROWB>(st + OFF_B + TILE_B + j * 32);
+          const uint64_t ar = st + 2 * j, ai = st + (TILE_A >> 4) + 2 * j;
+          const uint64_t br = st + (OFF_B >> 4) + 2 * j, bi = st + ((OFF_B + TILE_B) >> 4) + 2 * j;
           if constexpr (REAL) {
             mma_tf32(tmem, ar, br, idesc, acc);  // br: the 256 B rows of both tiles
           } else {
@@ -169,31 +177,35 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
         }
         mma_commit(&empty[s]);
       }
-      mma_commit(acc_full);  // also on error: lets the epilogue see in-flight MMAs retire
+      __syncwarp();
     }
+    if (leader) mma_commit(acc_full);  // also on error: lets the epilogue see in-flight MMAs retire
+    __syncwarp();
   } else {
     // epilogue: TMEM lane quarter of this warp = warp % 4
-    const bool ok = mbar_wait(acc_full, 0);
-    if (!ok) atomicExch(err, 6);
+    // output offsets, while the first loads and MMAs run
+    for (int x = threadIdx.x - 64; x < BM + TN; x += 256) {
+      if (x < BM) row_off[x] = m0 + x < a.m ? map_offset(a.rows, m0 + x) : 0;
+      else col_off[x - BM] = n0 + x - BM < a.n ? map_offset(a.cols, n0 + x - BM) : 0;
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    const bool ok = mbar_wait_warp(acc_full, 0);
+    if (!ok && lane == 0) atomicExch(err, 6);
     fence_after();
-    const int q = warp & 3;
-    const int row = q * 32 + lane;
-    const int64_t m = static_cast<int64_t>(m0) + row;
-    const bool row_ok = ok && m < a.m;
-    const int64_t ro = row_ok ? map_offset(a.rows, m) : 0;
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const bool row_ok = ok && m0 + q * 32 + lane < a.m;
+    const int64_t rows_left = ok ? a.m - m0 - 32 * q : 0;
     float* C = a.C + static_cast<int64_t>(b) * a.c_bstride;
     const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
     // Each 32 x 32 block goes through shared memory (the drained stage buffers) and is
-    // stored in address order (store_block): 32 consecutive elements per warp store for
-    // the usual layouts.
+    // stored in address order: 32 consecutive elements per warp store for the usual layouts.
     float* tr = reinterpret_cast<float*>(smem) + (warp - 2) * 2 * 32 * 33;  // [2][32][33]
     const TcScale sc = tc_scale(a, b);
     int lmax = -127;
-    // this warp's 32-column blocks: all of a complex tile's, half of a real tile's
-    constexpr int NCB = REAL ? TN / 64 : TN / 32;
-    const int c_first = REAL ? ((warp - 2) >> 2) * NCB : 0;
-    for (int c = c_first; c < c_first + NCB; ++c) {
-      const int64_t nb0 = static_cast<int64_t>(n0) + c * 32;
+    constexpr int NCB = TN / 64;  // this warp's 32-column blocks
+#pragma unroll 1
+    for (int c = half * NCB; c < (half + 1) * NCB; ++c) {
+      const int64_t cols_left = a.n - n0 - 32 * c;
       if constexpr (REAL) {
         float v[32];
         tmem_ld32(tmem + lane_base + c * 32, v);
@@ -201,7 +213,7 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
         for (int j = 0; j < 32; ++j) {
           if constexpr (SCALED) {
             v[j] = v[j] * sc.sa * sc.sb;
-            if (row_ok && nb0 + j < a.n) lmax = max(lmax, exp_of(fabsf(v[j])));
+            if (row_ok && j < cols_left) lmax = max(lmax, exp_of(fabsf(v[j])));
           }
           tr[lane * 33 + j] = v[j];
         }
@@ -216,17 +228,16 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, 1)
           if constexpr (SCALED) {
             re = re * sc.sa * sc.sb;
             im = im * sc.sa * sc.sb;
-            if (row_ok && nb0 + j < a.n) lmax = max(lmax, exp_of(fmaxf(fabsf(re), fabsf(im))));
+            if (row_ok && j < cols_left) lmax = max(lmax, exp_of(fmaxf(fabsf(re), fabsf(im))));
           }
           tr[lane * 33 + j] = re;
           tr[32 * 33 + lane * 33 + j] = im;
         }
       }
       __syncwarp();
-      const int64_t n = nb0 + lane;
-      const bool col_ok = ok && n < a.n;
-      store_block<REAL>(C, a.c_plane, kFmtPlanar, tr, 33, 32 * 33, ro, col_ok ? map_offset(a.cols, n) : 0, row_ok,
-                        col_ok, lane);
+      store_block_planned<REAL>(C, a.c_plane, kFmtPlanar, tr, 33, 32 * 33, row_off + 32 * q, col_off + 32 * c,
+                                static_cast<int>(rows_left < 32 ? rows_left : 32),
+                                static_cast<int>(cols_left < 32 ? cols_left : 32), a.blk, lane, 0, 1);
       __syncwarp();
     }
     if constexpr (SCALED) tc_scale_finish(a, b, lmax, t == 0 && threadIdx.x == 64);
@@ -321,8 +332,7 @@ __global__ void __launch_bounds__(576, 1)
   int64_t* row_off = reinterpret_cast<int64_t*>(bars + 64);  // [BM] output offsets of the tile's rows
   int64_t* col_off = row_off + BM;                           // [BT] and columns
 
-  // (the shuffle tells the compiler that the warp index is uniform)
-  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int64_t tiles_m = (a.m + BM - 1) / BM, tiles_n = (a.n + BT - 1) / BT;
   const int64_t t = t_first + blockIdx.x;  // this launch's tiles start at t_first
   const int64_t per_group = GROUP_M * tiles_n;
@@ -359,7 +369,7 @@ __global__ void __launch_bounds__(576, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  const uint32_t tmem = uniform_u32(*tmem_slot);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -385,9 +395,6 @@ __global__ void __launch_bounds__(576, 1)
         if (!mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1)) atomicExch(err, 72);
     }
   } else if (warp == 1) {
-    // The whole warp runs the loop and one elected lane issues, so that the operands of the MMAs
-    // stay in uniform registers: issued by a lane on its own branch, an MMA of 64 columns cost 95
-    // clocks, three times its execution.
     constexpr uint32_t idesc = idesc_tf32(BM, G::N);  // complex: (Re | Im) at once
     const bool leader = elect_one();
     const uint32_t d_lo = tmem + G::D_LO;
@@ -396,7 +403,7 @@ __global__ void __launch_bounds__(576, 1)
     bool mma_ok = true;
     int s = 0;
     for (int kb = 0; kb < num_kb; ++kb, s = s + 1 == STAGES ? 0 : s + 1) {
-      if (!mbar_wait(&conv_full[kb & 1], (kb >> 1) & 1)) {
+      if (!mbar_wait_warp(&conv_full[kb & 1], (kb >> 1) & 1)) {
         if (leader) atomicExch(err, 74);
         mma_ok = false;
         break;
@@ -421,7 +428,7 @@ __global__ void __launch_bounds__(576, 1)
       }
       const int h = kb % G::HI;
       const uint32_t d_hi = tmem + h * G::N;
-      if (!mbar_wait(&acc_empty[h], ((kb / G::HI) & 1) ^ 1)) {
+      if (!mbar_wait_warp(&acc_empty[h], ((kb / G::HI) & 1) ^ 1)) {
         if (leader) atomicExch(err, 73);
         mma_ok = false;
         break;
@@ -461,8 +468,8 @@ __global__ void __launch_bounds__(576, 1)
     for (int kb = 0; kb <= num_kb; ++kb) {
       if (kb < num_kb) {
         const int s = kb % STAGES;
-        if (!mbar_wait(&full[s], (kb / STAGES) & 1) || !mbar_wait(&lo_empty[kb & 1], ((kb >> 1) & 1) ^ 1)) {
-          atomicExch(err, 75);
+        if (!mbar_wait_warp(&full[s], (kb / STAGES) & 1) || !mbar_wait_warp(&lo_empty[kb & 1], ((kb >> 1) & 1) ^ 1)) {
+          if (lane == 0) atomicExch(err, 75);
           ok = false;
           break;
         }
@@ -526,8 +533,8 @@ __global__ void __launch_bounds__(576, 1)
       // round-to-nearest additions and release the accumulator
       if (kb > 0 && folds) {
         const int d = (kb - 1) % G::HI;
-        if (!mbar_wait(&acc_full[d], ((kb - 1) / G::HI) & 1)) {
-          atomicExch(err, 76);
+        if (!mbar_wait_warp(&acc_full[d], ((kb - 1) / G::HI) & 1)) {
+          if (lane == 0) atomicExch(err, 76);
           ok = false;
           break;
         }

@@ -49,6 +49,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, uint64_t
   }
 }
 
+// The same for a whole warp (all lanes active): every lane gets the same answer, so the warp stays
+// together whatever happens to the wait.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(b, parity)) != 0;
+}
+
 // One contiguous global -> shared copy by the bulk-copy engine (cp.async.bulk): both
 // addresses 16-byte aligned, bytes a multiple of 16; completion counts `bytes` against the
 // barrier's transaction count.

@@ -63,7 +63,13 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t d, uint32_t a, uint64_t b, 
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d),
       "r"(a), "l"(b), "r"(idesc), "r"(acc));
 }
-// One lane of a fully active warp, always the same one.
+// The warp index and a value the same in every lane, as the compiler can see it.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
+__device__ __forceinline__ uint32_t uniform_u32(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+// One lane of a fully active warp, always the same one. The MMA warps run their loops with all
+// lanes and issue from the elected one, with the descriptors formed by adding to a warp-uniform
+// base, so that the operands of the MMAs stay in uniform registers: issued by a lane on a branch of
+// its own, an MMA cost 75-95 clocks whatever its size (measured).
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
@@ -288,7 +294,7 @@ __device__ __forceinline__ void store_sorted(float* C, int64_t plane, int split,
       il += step(VB + k);
       al += int64_t(1) << e[VB + k];
     }
-#pragma unroll 1
+#pragma unroll 2
   for (int s = part; s < (32 >> VB); s += parts) {
     int is = il;
     int64_t ah = 0;
