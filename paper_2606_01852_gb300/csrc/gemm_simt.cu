@@ -4,7 +4,7 @@
 // What bounds it: the FP32 pipe (128 FMAs per clock and SM) once k is a few tens, the output's
 // stores below that. One kernel template, three tile shapes: every output is one thread's
 // accumulator with k in order, so all shapes give the same bits and the choice is free
-// (simt_tile). A warp owns an (8 TM) x (4 TN) block of the tile, thread (lane / 4, lane % 4) the
+// (launch_form). A warp owns an (8 TM) x (4 TN) block of the tile, thread (lane / 4, lane % 4) the
 // TM x TN outputs of it; both operands sit in shared memory k-major, so a complex 4 x 8 thread
 // tile issues 128 FMAs per six 16-byte shared-memory loads. Global loads are 16 bytes along k
 // (scalar when k or the planes are not 4-aligned), one k-block ahead of the arithmetic in
@@ -24,7 +24,7 @@
 // waited for in place before): complex 2048 x 8192 x 1024 3.88 -> 2.30 ms (35.4 -> 59.7 TFLOP/s),
 // 1024 x 4096 x 16384 16.1 -> 9.5 ms; real 2048 x 8192 x 1024 1.30 -> 0.68 ms (26.5 -> 50.2);
 // max-plus the same 1.60 -> 1.16 ms (21.5 -> 29.6); few outputs, complex 32 x 2048 x 2048
-// 180 -> 54 us; shallow, complex 2048 x 16384 x 4 311 -> 132 us (0.87 -> 2.0 TB/s). What is left
+// 180 -> 54 us; shallow, complex 2048 x 16384 x 4 311 -> 108 us (0.87 -> 2.5 TB/s). What is left
 // is the shared-memory read bandwidth: a 16-byte load returns 512 bytes to a warp in 4 clocks,
 // 75 % (complex) or all (real, max-plus) of the packed instructions' time. Larger thread tiles
 // (8 x 16) cut that but leave 8 warps on an SM: slower (42.8 TFLOP/s real).
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(G::THREADS, G::MIN_CTAS) contract_simt_kernel(
     const int64_t r = br0 + lane, c = bc0 + lane;
     const bool rok = r < a.m, cok = c < a.n;
     store_block<!CPLX>(C, a.c_plane, a.c_split, t, 33, CS, rok ? map_offset(a.rows, r) : 0,
-                       cok ? map_offset(a.cols, c) : 0, rok, cok, lane, part, parts);
+                       cok ? map_offset(a.cols, c) : 0, rok, cok, a.blk, lane, part, parts);
   };
   if constexpr (8 * TM >= 32) {
     // the warp's block is (8 TM) x (4 TN): its 32 x 32 blocks one after the other
@@ -472,30 +472,49 @@ void launch(const StepArgs& a, int32_t nb, cudaStream_t st) {
   contract_simt_kernel<G><<<grid, G::THREADS, G::SMEM, st>>>(a);
 }
 
-// The tile of a step: the wide one (real) from two tiles per SM on -- with 160 tiles on 152 SMs
-// eight of them set the time --, the 64 x 64 one from one per SM, else the smallest (a step of few
-// outputs is bound by its serial k loop, and small tiles spread it over more SMs).
+// A tile shape's time per k term, in units of a full-rate 128 x 128 real (64 x 64 complex) tile:
+// `share` of an SM whose `resident` CTAs run together, `alone` for a CTA without company (latency
+// instead of throughput). From the shapes' rates: max-plus 29.6 / 26.9 / 19.3 TFLOP/s (128 x 128,
+// 64 x 128, 64 x 64), real 50.2 / 41.5 (64 x 128, 64 x 64), complex 60 (64 x 64); and steps of few
+// tiles: max-plus 256 128-square tiles 5.1 ms, the same as 512 64 x 128 ones 7.2 ms.
+struct TileCost {
+  double share, alone;
+  int resident;
+  double time(int64_t ctas, int num_sms) const {
+    const int64_t n = (ctas + num_sms - 1) / num_sms, rest = n % resident;
+    return double(n - rest) * share + (rest ? std::max(double(rest) * share, alone) : 0.0);
+  }
+};
+
+// The tile of a step: the least time by TileCost (the bits do not depend on it). Large tiles have
+// the better rate; with few outputs a step is bound by its serial k loop, and small tiles spread
+// it over more SMs.
 template <Arith AR>
 void launch_form(const StepArgs& a, int32_t nb, int num_sms, cudaStream_t st) {
-  auto fills = [&](int64_t tm, int64_t tn, int per_sm) {
-    const int64_t ctas = ((a.m + tm - 1) / tm) * ((a.n + tn - 1) / tn) * nb * (a.ksplit > 1 ? a.ksplit : 1);
-    return ctas >= int64_t(per_sm) * num_sms;
+  auto ctas = [&](int64_t tm, int64_t tn) {
+    return ((a.m + tm - 1) / tm) * ((a.n + tn - 1) / tn) * nb * (a.ksplit > 1 ? a.ksplit : 1);
   };
-  // real outputs take half the registers: an 8 x 8 thread tile. Max-plus reads a pair of terms per
-  // load: with 16 warps on an SM (128 x 128) 29.6 TFLOP/s, with 12 (64 x 128) 26.9, with the square
-  // tile's 4 x 8 per thread 19.3, so it keeps the 8 x 8 one down to one tile per SM; real 47.9,
-  // 50.2 and 41.5.
-  if constexpr (AR != Arith::Complex) {
-    using Wide = SimtCfg<AR, 8, 8, 1, 4>;
-    if constexpr (AR == Arith::MaxPlus) {
-      using Widest = SimtCfg<AR, 8, 8, 2, 4>;
-      if (fills(Widest::M, Widest::N, 2)) return launch<Widest>(a, nb, st);
-    }
-    if (fills(Wide::M, Wide::N, AR == Arith::MaxPlus ? 1 : 2)) return launch<Wide>(a, nb, st);
-  }
+  using Widest = SimtCfg<AR, 8, 8, 2, 4>;
+  using Wide = SimtCfg<AR, 8, 8, 1, 4>;
   using Square = SimtCfg<AR, 4, 8, 2, 2>;
   using Small = SimtCfg<AR, 2, 4, 2, 2>;
-  if (fills(Square::M, Square::N, 1)) launch<Square>(a, nb, st);
+  constexpr bool kCplx = AR == Arith::Complex, kMax = AR == Arith::MaxPlus;
+  constexpr TileCost square = kCplx ? TileCost{1.0, 1.8, 3} : (kMax ? TileCost{0.39, 0.6, 3} : TileCost{0.30, 0.5, 3});
+  constexpr TileCost small = kCplx ? TileCost{0.43, 0.75, 4} : (kMax ? TileCost{0.14, 0.25, 4} : TileCost{0.11, 0.22, 4});
+  const double t_square = square.time(ctas(Square::M, Square::N), num_sms);
+  const double t_small = small.time(ctas(Small::M, Small::N), num_sms);
+  const double t_rest = std::min(t_square, t_small);
+  if constexpr (!kCplx) {  // real outputs take half the registers: an 8 x 8 thread tile
+    constexpr TileCost wide = kMax ? TileCost{0.55, 1.0, 3} : TileCost{0.5, 0.9, 3};
+    const double t_wide = wide.time(ctas(Wide::M, Wide::N), num_sms);
+    if constexpr (kMax) {
+      constexpr TileCost widest{1.0, 1.2, 2};
+      const double t_widest = widest.time(ctas(Widest::M, Widest::N), num_sms);
+      if (t_widest <= t_wide && t_widest <= t_rest) return launch<Widest>(a, nb, st);
+    }
+    if (t_wide <= t_rest) return launch<Wide>(a, nb, st);
+  }
+  if (t_square <= t_small) launch<Square>(a, nb, st);
   else launch<Small>(a, nb, st);
 }
 

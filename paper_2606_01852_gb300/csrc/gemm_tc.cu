@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
       const int64_t n = static_cast<int64_t>(n0) + half * 64 + cb * 32 + lane;
       const bool col_ok = ok && n < a.n;
       store_block(C, a.c_plane, split, tr + cb * 32, 65, 32 * 65, ro, col_ok ? map_offset(a.cols, n) : 0, row_ok,
-                  col_ok, lane);
+                  col_ok, a.blk, lane);
     }
   }
   fence_before();
@@ -613,7 +613,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
         const int64_t n = static_cast<int64_t>(n0) + half * 64 + cb * 32 + lane;
         const bool col_ok = n < a.n;
         store_block(C, a.c_plane, split, tr + cb * 32, 65, 32 * 65, ro, col_ok ? map_offset(a.cols, n) : 0, row_ok,
-                    col_ok, lane);
+                    col_ok, a.blk, lane);
       }
     }
   }
@@ -859,17 +859,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
     const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
     float* tr = epi + (warp - 2) * 2 * 32 * 33;  // this warp's Re and Im transpose blocks
     const int split = a.c_split;
-    bool pow2 = a.m >= 32 && a.n >= 32;
-    for (int d = 0; d < a.rows.n; ++d) pow2 = pow2 && (a.rows.ext[d] & (a.rows.ext[d] - 1u)) == 0u;
-    for (int d = 0; d < a.cols.n; ++d) pow2 = pow2 && (a.cols.ext[d] & (a.cols.ext[d] - 1u)) == 0u;
-    // kept in shared memory (the same for every lane), not in registers
-    BlockOrder& ord = reinterpret_cast<BlockOrder*>(epi + 8 * 2 * 32 * 33)[warp - 2];
-    {
-      const BlockOrder o = block_order(pow2 ? map_offset(a.rows, lane) : 0, pow2 ? map_offset(a.cols, lane) : 0,
-                                       pow2, lane);
-      if (lane == 0) ord = o;
-      __syncwarp();
-    }
     int64_t G = 0;  // chunks folded over all items
     bool ok = true;
     for (int64_t w = cluster; w < total && ok; w += n_clusters) {
@@ -929,12 +918,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
         const int64_t n = static_cast<int64_t>(n0) + half * 64 + cb * 32 + lane;
         const bool col_ok = n < a.n;
         const int64_t co = col_ok ? map_offset(a.cols, n) : 0;
-        if (ord.ok && __all_sync(0xffffffffu, row_ok && col_ok)) {
-          const int64_t base = __shfl_sync(0xffffffffu, ro, 0) + __shfl_sync(0xffffffffu, co, 0);
-          store_ordered(C, a.c_plane, split, tr, 33, 32 * 33, base, ord, lane);
-        } else {
-          store_block(C, a.c_plane, split, tr, 33, 32 * 33, ro, co, row_ok, col_ok, lane);
-        }
+        store_block(C, a.c_plane, split, tr, 33, 32 * 33, ro, co, row_ok, col_ok, a.blk, lane);
         __syncwarp();
       }
     }
@@ -1157,7 +1141,7 @@ __global__ void __launch_bounds__(CB3::THREADS, 1)
       const int64_t n = static_cast<int64_t>(n0) + half * 64 + cb * 32 + lane;
       const bool col_ok = ok && n < a.n;
       store_block(C, a.c_plane, split, tr + cb * 32, 65, 32 * 65, ro, col_ok ? map_offset(a.cols, n) : 0, row_ok,
-                  col_ok, lane);
+                  col_ok, a.blk, lane);
     }
   }
   fence_before();
@@ -1326,20 +1310,6 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
     float* tr = epi + (warp - 2) * 2 * 32 * 33;  // this warp's Re and Im transpose blocks
     const int split = a.c_split;
-    // When every extent of the offset maps is a power of two, every full 32 x 32 block of
-    // the step has the address order of the first one: it is computed once here, and a
-    // full block only adds its base offset (the other blocks take store_block's checks).
-    bool pow2 = a.m >= 32 && a.n >= 32;
-    for (int d = 0; d < a.rows.n; ++d) pow2 = pow2 && (a.rows.ext[d] & (a.rows.ext[d] - 1u)) == 0u;
-    for (int d = 0; d < a.cols.n; ++d) pow2 = pow2 && (a.cols.ext[d] & (a.cols.ext[d] - 1u)) == 0u;
-    // kept in shared memory (the same for every lane), not in registers
-    BlockOrder& ord = reinterpret_cast<BlockOrder*>(epi + 8 * 2 * 32 * 33)[warp - 2];
-    {
-      const BlockOrder o = block_order(pow2 ? map_offset(a.rows, lane) : 0, pow2 ? map_offset(a.cols, lane) : 0,
-                                       pow2, lane);
-      if (lane == 0) ord = o;
-      __syncwarp();
-    }
     int64_t q = 0;  // tiles folded
     for (int64_t w = blockIdx.x; w < total; w += gridDim.x, ++q) {
       const TileCoord tc = tile_of(w, tiles_m, tiles_n);
@@ -1384,12 +1354,7 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
         const int64_t n = static_cast<int64_t>(tc.n0) + half * 64 + cb * 32 + lane;
         const bool col_ok = n < a.n;
         const int64_t co = col_ok ? map_offset(a.cols, n) : 0;
-        if (ord.ok && __all_sync(0xffffffffu, row_ok && col_ok)) {
-          const int64_t base = __shfl_sync(0xffffffffu, ro, 0) + __shfl_sync(0xffffffffu, co, 0);
-          store_ordered(C, a.c_plane, split, tr, 33, 32 * 33, base, ord, lane);
-        } else {
-          store_block(C, a.c_plane, split, tr, 33, 32 * 33, ro, co, row_ok, col_ok, lane);
-        }
+        store_block(C, a.c_plane, split, tr, 33, 32 * 33, ro, co, row_ok, col_ok, a.blk, lane);
         __syncwarp();
       }
     }
@@ -1533,16 +1498,6 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
     float* tr = epi + e * 2 * 32 * 33;             // this warp's Re and Im transpose block
     const int split = a.c_split;
-    bool pow2 = a.m >= 32 && a.n >= 32;
-    for (int d = 0; d < a.rows.n; ++d) pow2 = pow2 && (a.rows.ext[d] & (a.rows.ext[d] - 1u)) == 0u;
-    for (int d = 0; d < a.cols.n; ++d) pow2 = pow2 && (a.cols.ext[d] & (a.cols.ext[d] - 1u)) == 0u;
-    BlockOrder& ord = reinterpret_cast<BlockOrder*>(epi + CBS::EPI_WARPS * 2 * 32 * 33)[e];
-    {
-      const BlockOrder o = block_order(pow2 ? map_offset(a.rows, lane) : 0, pow2 ? map_offset(a.cols, lane) : 0,
-                                       pow2, lane);
-      if (lane == 0) ord = o;
-      __syncwarp();
-    }
     int64_t q = 0;
     for (int64_t w = blockIdx.x; w < total; w += gridDim.x, ++q) {
       const TileCoord tc = tile_of(w, tiles_m, tiles_n);
@@ -1572,12 +1527,7 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
       const int64_t n = static_cast<int64_t>(tc.n0) + cq * 32 + lane;
       const bool col_ok = n < a.n;
       const int64_t co = col_ok ? map_offset(a.cols, n) : 0;
-      if (ord.ok && __all_sync(0xffffffffu, row_ok && col_ok)) {
-        const int64_t base = __shfl_sync(0xffffffffu, ro, 0) + __shfl_sync(0xffffffffu, co, 0);
-        store_ordered(C, a.c_plane, split, tr, 33, 32 * 33, base, ord, lane);
-      } else {
-        store_block(C, a.c_plane, split, tr, 33, 32 * 33, ro, co, row_ok, col_ok, lane);
-      }
+      store_block(C, a.c_plane, split, tr, 33, 32 * 33, ro, co, row_ok, col_ok, a.blk, lane);
       __syncwarp();
     }
   }

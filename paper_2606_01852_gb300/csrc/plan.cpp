@@ -28,15 +28,21 @@ bool is_tc_prec(int32_t p) {
          p == TN_R32_3XTF32 || p == TN_R32_BF16X3;
 }
 
-// The weights of the low five bits of an index under `om`; false unless all are powers of two.
+// The weights of the low five bits of an index under `om` (blocks of 32 that start at multiples
+// of 32); false unless all are powers of two. The dims below the one that holds the fifth bit
+// are powers of two; that one is a multiple of the bits' range, or the outermost (a block then
+// ends inside it, or is ragged).
 bool bit_weights(const OffsetMap& om, int (&log2w)[5]) {
   int n = 0;
   for (int d = om.n - 1; d >= 0 && n < 5; --d) {
     const uint32_t e = om.ext[d];
     const int64_t w = om.stride[d];
-    if ((e & (e - 1u)) != 0u || w <= 0 || (w & (w - 1)) != 0) return false;
+    if (w <= 0 || (w & (w - 1)) != 0) return false;
+    const bool pow2 = (e & (e - 1u)) == 0u;
+    if (!pow2 && d > 0 && e % (32u >> n) != 0u) return false;
+    if (!pow2 && e < (32u >> n)) return false;
     const int lw = __builtin_ctzll(static_cast<unsigned long long>(w));
-    for (int i = 0; (e >> i) > 1u && n < 5; ++i) log2w[n++] = lw + i;
+    for (int i = 0; (pow2 ? (e >> i) > 1u : true) && n < 5; ++i) log2w[n++] = lw + i;
   }
   return n == 5;
 }

@@ -322,103 +322,66 @@ __device__ __forceinline__ void store_sorted(float* C, int64_t plane, int split,
 }
 
 // Store one 32 x 32 block of a result tile from shared memory (t[r * pitch + c] = Re,
-// t[cs + r * pitch + c] = Im; row r is lane r's row, column c lane c's column) in the
-// order of its addresses. When the block's offsets are linear in the bits of (r, c) with
-// power-of-two weights -- every row and column extent of the offset maps a power of two,
-// as in every network with extent-2 modes -- off(r, c) = off(0, 0) + sum of per-bit
-// weights, and the ten weights sorted ascending give the block's elements in address
-// order. Each lane then writes V consecutive addresses with one vector store per plane
-// (V up to 4 FP32 or 8 BF16 values, 16 bytes, as far as the smallest weights are 1, 2, 4,
-// ... and the block is aligned), and a warp store covers 32 V consecutive elements when
-// the following weights continue the sequence (interleaved row/column layouts included).
-// Otherwise (ragged block, other extents) it falls back to one row per store. ro / co:
-// this lane's row / column offset; row_ok / col_ok: in range.
-// The address order of a 32 x 32 block: the ten bit weights (log2; bits 0-4 of the row,
-// 5-9 of the column index) sorted ascending, with the bit each comes from; ok when the
-// block's offsets are linear in those bits with power-of-two weights. ro_rel / co_rel: this
-// lane's row / column offset relative to the block's first row / column.
-struct BlockOrder {
-  int e[10], src[10];
-  bool ok;
-};
-static_assert(sizeof(BlockOrder) <= 128, "a fold warp's block order slot");
-__device__ __forceinline__ BlockOrder block_order(int64_t ro_rel, int64_t co_rel, bool in_range, int lane) {
-  BlockOrder o;
-  bool lin = in_range;
-  int64_t pr = 0, pc = 0;
+// t[cs + r * pitch + c] = Im) in the order of its addresses, the step's block plan: each lane
+// writes V consecutive addresses with one vector store per plane (V as far as the smallest
+// weights are 1, 2, 4, ... and the block's base and the plane size are V-aligned; 16 bytes at
+// most), and a warp store covers 32 V consecutive elements when the following weights continue
+// the sequence (interleaved row/column layouts included). The plan is worked out once on the host:
+// a sorting network per block, executed once per tile, cost an SM thousands of clocks of
+// instruction fetches. base: offset of the block's first element. part of parts: the share of the
+// stores this warp makes when several share the block.
+template <bool REAL>
+__device__ __forceinline__ void store_planned(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
+                                              int64_t base, const BlockPlan& p, int lane, int part, int parts) {
+  int e[10], src[10], vb = 0;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int64_t wr = __shfl_sync(0xffffffffu, ro_rel, 1 << i);
-    const int64_t wc = __shfl_sync(0xffffffffu, co_rel, 1 << i);
-    o.e[i] = (wr > 0 && (wr & (wr - 1)) == 0) ? 63 - __clzll(wr) : -1;
-    o.e[5 + i] = (wc > 0 && (wc & (wc - 1)) == 0) ? 63 - __clzll(wc) : -1;
-    lin = lin && o.e[i] >= 0 && o.e[5 + i] >= 0;
-    pr += ((lane >> i) & 1) * wr;
-    pc += ((lane >> i) & 1) * wc;
+  for (int k = 0; k < 10; ++k) {
+    e[k] = p.e[k];
+    src[k] = p.src[k];
   }
-  lin = lin && pr == ro_rel && pc == co_rel;
-  o.ok = __all_sync(0xffffffffu, lin);
+  const int64_t align = REAL ? base : (base | plane);
+  bool run = true;
 #pragma unroll
-  for (int i = 0; i < 10; ++i) o.src[i] = i;
-  if (o.ok) {
-#pragma unroll
-    for (int i = 1; i < 10; ++i)
-#pragma unroll
-      for (int j = i; j > 0; --j)
-        if (o.e[j] < o.e[j - 1]) {
-          const int te = o.e[j];
-          o.e[j] = o.e[j - 1];
-          o.e[j - 1] = te;
-          const int ts = o.src[j];
-          o.src[j] = o.src[j - 1];
-          o.src[j - 1] = ts;
-        }
+  for (int k = 0; k < 3; ++k) {
+    run = run && e[k] == k && k < (!REAL && split ? 3 : 2) && (align & ((int64_t(2) << k) - 1)) == 0;
+    if (run) vb = k + 1;
   }
-  return o;
-}
-
-// The address-ordered stores of a block whose order is `o` (o.ok) and whose first element
-// is at `base`: each lane writes V consecutive addresses with one vector store per plane
-// (V as far as the smallest weights are 1, 2, 4, ... and base and the plane size are
-// V-aligned; 16 bytes at most).
-template <bool REAL = false>
-__device__ __forceinline__ void store_ordered(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
-                                              int64_t base, const BlockOrder& o, int lane, int part = 0,
-                                              int parts = 1) {
-  int vb = 0;
-  while (vb < (!REAL && split ? 3 : 2) && o.e[vb] == vb) ++vb;
-  while (vb > 0 && ((base | plane) & ((int64_t(1) << vb) - 1)) != 0) --vb;
   if constexpr (!REAL) {
-    if (vb == 3) {
-      store_sorted<3>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
-      return;
-    }
+    if (vb == 3) return store_sorted<3>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
   }
-  if (vb == 2) store_sorted<2, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
-  else if (vb == 1) store_sorted<1, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
-  else store_sorted<0, REAL>(C, plane, split, t, pitch, cs, base, o.e, o.src, lane, part, parts);
+  if (vb == 2) return store_sorted<2, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
+  if (vb == 1) return store_sorted<1, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
+  return store_sorted<0, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
 }
 
-// Store one 32 x 32 block of a result tile from shared memory (t[r * pitch + c] = Re,
-// t[cs + r * pitch + c] = Im; row r is lane r's row, column c lane c's column) in the
-// order of its addresses. When the block's offsets are linear in the bits of (r, c) with
-// power-of-two weights -- every row and column extent of the offset maps a power of two,
-// as in every network with extent-2 modes -- off(r, c) = off(0, 0) + sum of per-bit
-// weights, and the ten weights sorted ascending give the block's elements in address
-// order (block_order); a warp store then covers 32 V consecutive elements when the
-// following weights continue the sequence (interleaved row/column layouts included).
-// Otherwise (ragged block, other extents) it falls back to one row per store. ro / co:
-// this lane's row / column offset; row_ok / col_ok: in range. REAL: a real FP32 result
-// (one plane in t; plane, split and cs unused). part of parts: the share of the stores this
-// warp makes when several warps store one block.
+// The block at rows ro[0..31] and columns co[0..31] (output offsets in shared memory), of which
+// `rows` / `cols` are in range. A ragged block, or a map without a plan, is stored one row per
+// warp store. REAL: a real FP32 result (one plane in t; plane, split and cs unused).
+template <bool REAL>
+__device__ __forceinline__ void store_block_planned(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
+                                                    const int64_t* ro, const int64_t* co, int rows, int cols,
+                                                    const BlockPlan& p, int lane, int part, int parts) {
+  if (p.ok && rows >= 32 && cols >= 32) {
+    store_planned<REAL>(C, plane, split, t, pitch, cs, ro[0] + co[0], p, lane, part, parts);
+    return;
+  }
+  if (lane >= cols) return;
+  const int64_t c = co[lane];
+  for (int r = part; r < 32 && r < rows; r += parts) {
+    if constexpr (REAL) C[ro[r] + c] = t[r * pitch + lane];
+    else store_cplx(C, plane, ro[r] + c, t[r * pitch + lane], t[cs + r * pitch + lane], split);
+  }
+}
+
+// The same with the offsets in registers: ro / co are this lane's row / column offset, row_ok /
+// col_ok whether they are in range.
 template <bool REAL = false>
 __device__ __forceinline__ void store_block(float* C, int64_t plane, int split, const float* t, int pitch,
-                                            int cs, int64_t ro, int64_t co, bool row_ok, bool col_ok, int lane,
-                                            int part = 0, int parts = 1) {
-  const int64_t ro0 = __shfl_sync(0xffffffffu, ro, 0), co0 = __shfl_sync(0xffffffffu, co, 0);
-  const BlockOrder o = block_order(ro - ro0, co - co0, row_ok && col_ok, lane);
-  if (o.ok) {
-    store_ordered<REAL>(C, plane, split, t, pitch, cs, ro0 + co0, o, lane, part, parts);
+                                            int cs, int64_t ro, int64_t co, bool row_ok, bool col_ok,
+                                            const BlockPlan& p, int lane, int part = 0, int parts = 1) {
+  if (p.ok && __all_sync(0xffffffffu, row_ok && col_ok)) {
+    const int64_t base = __shfl_sync(0xffffffffu, ro, 0) + __shfl_sync(0xffffffffu, co, 0);
+    store_planned<REAL>(C, plane, split, t, pitch, cs, base, p, lane, part, parts);
     return;
   }
   for (int r = part; r < 32; r += parts) {
@@ -428,46 +391,6 @@ __device__ __forceinline__ void store_block(float* C, int64_t plane, int split, 
       if constexpr (REAL) C[ro_r + co] = t[r * pitch + lane];
       else store_cplx(C, plane, ro_r + co, t[r * pitch + lane], t[cs + r * pitch + lane], split);
     }
-  }
-}
-
-// Store one 32 x 32 block of a result tile from shared memory (t[r * pitch + c] = Re, t[cs + ...] =
-// Im) by the step's block plan: the address order is the plan's, worked out once on the host (a
-// sorting network per block, executed once per tile, costs an SM thousands of clocks of
-// instruction fetches). ro / co: offsets of the block's rows / columns in shared memory, of which
-// `rows` / `cols` are in range. A ragged block, or a map without power-of-two weights, is stored
-// one row per warp store. part of parts: this warp's share of the stores.
-template <bool REAL>
-__device__ __forceinline__ void store_block_planned(float* C, int64_t plane, int split, const float* t, int pitch, int cs,
-                                                    const int64_t* ro, const int64_t* co, int rows, int cols,
-                                                    const BlockPlan& p, int lane, int part, int parts) {
-  if (p.ok && rows >= 32 && cols >= 32) {
-    const int64_t base = ro[0] + co[0];
-    int e[10], src[10], vb = 0;
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-      e[k] = p.e[k];
-      src[k] = p.src[k];
-    }
-    const int64_t align = REAL ? base : (base | plane);
-    bool run = true;  // the smallest weights are 1, 2, 4, ... and the block is aligned
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      run = run && e[k] == k && k < (!REAL && split ? 3 : 2) && (align & ((int64_t(2) << k) - 1)) == 0;
-      if (run) vb = k + 1;
-    }
-    if constexpr (!REAL) {
-      if (vb == 3) return store_sorted<3>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
-    }
-    if (vb == 2) return store_sorted<2, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
-    if (vb == 1) return store_sorted<1, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
-    return store_sorted<0, REAL>(C, plane, split, t, pitch, cs, base, e, src, lane, part, parts);
-  }
-  if (lane >= cols) return;
-  const int64_t c = co[lane];
-  for (int r = part; r < 32 && r < rows; r += parts) {
-    if constexpr (REAL) C[ro[r] + c] = t[r * pitch + lane];
-    else store_cplx(C, plane, ro[r] + c, t[r * pitch + lane], t[cs + r * pitch + lane], split);
   }
 }
 
