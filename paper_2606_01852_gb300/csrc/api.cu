@@ -234,7 +234,7 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
       sp.bytes = 2.0 * (cplx ? 8.0 : 4.0) * staged;
       TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(sp.e0), st));
     }
-    launch_stage_leaves(descs, P.leafdesc.data(), T, P.dev, sb, nb, p > 0, cplx, recs, recidx, st);
+    launch_stage_leaves(descs, P.leafdesc.data(), T, P.dev, sb, nb, p > 0, cplx, recs, recidx, P.num_sms, st);
     if (P.prof_on) {
       TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(sp.e1), st));
       P.prof_pending.push_back(sp);

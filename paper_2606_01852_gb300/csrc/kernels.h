@@ -117,7 +117,7 @@ cudaError_t launch_contract_chain(const ChainStep* steps, const ChainTask* tasks
 // kernel, one launch per leaf; host_descs is the host copy of the table (grid sizes).
 void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, int32_t n_leaves, char* ws,
                          int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
-                         const int32_t* rec_index, cudaStream_t st);
+                         const int32_t* rec_index, int num_sms, cudaStream_t st);
 // With a.ksplit > 1 each part of k goes to its own CTAs and a second kernel combines the
 // partial tiles (in part order) and writes C.
 void launch_contract_simt(const StepArgs& a, int32_t nb, bool cplx, int num_sms, cudaStream_t st);

@@ -527,6 +527,9 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
       d.load_o = (inner >= 0 && in_o[inner]) ? 1 : 0;
       d.vec_load = (!d.load_o && d.ni > 0 && d.sstride[d.ipos[d.ni - 1]] == 1 && d.ext[d.ipos[d.ni - 1]] % 2 == 0)
                        ? 1 : 0;
+      d.linear = d.tiled;
+      for (int i = 0; i < d.rank; ++i)
+        if (d.sstride[i] != d.dstride[i]) d.linear = 0;
       // pipelined form: each group one 32-wide chunk, 16-byte loads, and the rest index's
       // fastest positions multiplying to exactly the tiles one CTA walks
       d.fast = 0;

@@ -66,6 +66,8 @@ struct LeafDesc {
   int32_t fast;                    // the pipelined form applies: Po = Pi = 32, 16-byte loads, and
                                    // the last `nlo` rest positions span exactly the tiles of a CTA
   int32_t nlo;
+  int32_t linear;                  // the planned order is the declared one: a copy's source is one
+                                   // contiguous run
   int8_t ipos[kMaxLeafRank], rpos[kMaxLeafRank];
   int64_t dstride[kMaxLeafRank];   // stride of each planned position in the staged copy
 };
