@@ -2,24 +2,33 @@
 //
 // Each network has its own path and its own plan (the same planner as tn_plan: step
 // analysis, GEMM-oriented reordering of Sec. IV-A, liveness offsets), flattened into
-// compact device tables. One CTA takes the next network from an atomic queue and runs
-// its whole path: stage the leaves into the network's arena (planned orders), then for
-// each step C = A (m x k) . B (n x k)^T written through the output offset maps, with
-// every thread of the CTA working on the step. With exponent scaling each tensor is
-// renormalised in place after it is made (an exact power of two chosen from its largest
-// entry) and the exponents are summed per network in an int64; the network's result is
-// (value, log2 scale) and ln|Z| = ln|value| + log2 * ln 2 in FP64 on the host side. In the
-// max-plus semiring (real, unscaled) a step is C = max_k (A + B) instead. (Taking the
-// costliest networks first was measured: 1.4-1.5x slower on both ensembles -- the big
-// arenas then run at the same time and contend for L2 -- so the queue stays in order.)
+// compact device tables (one copy for all networks of one shape and path). One CTA, or one
+// warp, takes the next network from an atomic queue and runs its whole path: stage the leaves
+// into the network's arena (planned orders), then for each step C = A (m x k) . B (n x k)^T
+// written through the output offset maps. With exponent scaling each tensor counts as
+// renormalised by an exact power of two chosen from its largest entry: the step's stores also
+// take the maximum, and whoever reads the tensor multiplies by the power of two, so that a step
+// has one pass and one barrier. The exponents are summed per network in an int64; the network's
+// result is (value, log2 scale) and ln|Z| = ln|value| + log2 * ln 2 in FP64 on the host side. In
+// the max-plus semiring (real, unscaled) a step is C = max_k (A + B) instead.
+//
+// What bounds it: latency, of the steps one after another (tens per network, most of them under
+// 100 terms) and, in the few large steps, of the loads whose lanes are k floats apart. So
+// small steps run one output per thread with no table and no division, steps of at least 8
+// outputs per thread run 4 x 4 (complex: 4 x 2) outputs per thread with 16-byte loads, and the
+// networks are queued by falling cost so that the large ones do not end last. 4096 Ising
+// networks of 20-60 vertices: 3.98 -> 0.60 ms (0.89 ms in the caller's order and with 64
+// registers a thread, 0.64 ms with 80, 0.60 with 128: the tiles want registers more than the
+// small steps want warps); 1024 king's graphs of 4-7 a side, max-plus: 14.0 -> 1.8 ms.
 // The CTA width (threads per network) and CTAs per SM are chosen by an autotuner that
 // times the real batch; the launch (queue reset + kernel) can be replayed as a CUDA graph.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
 #include <memory>
+#include <numeric>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -31,289 +40,395 @@
 namespace tn {
 namespace {
 
-__device__ __forceinline__ int bexp_of(float v) { return ((__float_as_int(v) >> 23) & 0xff) - 127; }
 __device__ __forceinline__ float bpow2_neg(int e) {
   e = max(-126, min(127, e));
   return __int_as_float((127 - e) << 23);
 }
 
-template <bool CPLX>
-__device__ void renormalise(float* t, int size, int* smax, long long* slog) {
-  int lmax = -127;
-  for (int i = threadIdx.x; i < size; i += blockDim.x) {
-    float v = fabsf(t[i]);
-    if (CPLX) v = fmaxf(v, fabsf(t[size + i]));
-    lmax = max(lmax, bexp_of(v));
+// The threads that run one network: a whole CTA, or one warp.
+template <bool WARP>
+struct Team {
+  static __device__ __forceinline__ int rank() { return WARP ? threadIdx.x & 31 : threadIdx.x; }
+  static __device__ __forceinline__ int size() { return WARP ? 32 : blockDim.x; }
+  static __device__ __forceinline__ void sync() {
+    if (WARP) __syncwarp();
+    else __syncthreads();
   }
-  for (int o = 16; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(smax, lmax);
-  __syncthreads();
-  const int e = *smax < -126 ? 0 : *smax;  // an all-zero tensor is left as is
-  if (e != 0) {
-    const float s = bpow2_neg(e);
-    for (int i = threadIdx.x; i < size; i += blockDim.x) {
-      t[i] *= s;
-      if (CPLX) t[size + i] *= s;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    *slog += e;
-    *smax = -127;
-  }
-  __syncthreads();
-}
+};
 
-// leaves whose exponents one pass takes together (networks with more renormalise leaf by leaf)
-constexpr int kLeafExpCap = 256;
-
-// Output offset of row x (x < m) or of column x - m (x >= m) of step S: the mixed-radix
-// digits over the merged dims, each times its stride.
-__device__ __forceinline__ int step_offset(const BStep& S, int x) {
+__device__ __forceinline__ int map_offset(const int32_t* __restrict__ ext, const int32_t* __restrict__ str, int nd,
+                                          bool pow2, int x) {
   int off = 0;
-  if (x < S.m) {
-    for (int d = S.nr - 1; d >= 0; --d) {
-      off += (x % S.rext[d]) * S.rstr[d];
-      x /= S.rext[d];
+  if (pow2) {
+#pragma unroll 4
+    for (int d = 0; d < nd; ++d) {
+      const int w = __ldg(ext + d);
+      off += ((x >> (w & 31)) & (w >> 8)) * __ldg(str + d);
     }
   } else {
-    x -= S.m;
-    for (int d = S.nc - 1; d >= 0; --d) {
-      off += (x % S.cext[d]) * S.cstr[d];
-      x /= S.cext[d];
+    for (int d = nd - 1; d >= 0; --d) {
+      const int w = __ldg(ext + d);
+      off += (x % w) * __ldg(str + d);
+      x /= w;
     }
   }
   return off;
 }
 
-template <bool CPLX, bool MAXPLUS = false>
-__global__ void batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves,
-                             const BStep* __restrict__ steps, int32_t n_nets, const float* __restrict__ in,
-                             float* arena, int32_t* queue, int32_t scaling, double* values, double* logs,
-                             int32_t smem_arena, int32_t tab_ints) {
-  // dynamic shared memory: [arena: smem_arena floats | offset table: tab_ints ints]
-  extern __shared__ float s_arena[];
-  int* s_tab = reinterpret_cast<int*>(s_arena + smem_arena);
-  __shared__ int s_lexp[kLeafExpCap];  // per-leaf maximum exponents
-  __shared__ int s_net;
-  __shared__ int s_max;
-  __shared__ long long s_log;
-  constexpr int NP = CPLX ? 2 : 1;
-  if (threadIdx.x == 0) s_max = -127;
-  while (true) {
-    if (threadIdx.x == 0) {
-      s_net = atomicAdd(queue, 1);
-      s_log = 0;
+// Output offset of row x (x < m) or of column x - m (x >= m) of step S.
+__device__ __forceinline__ int step_offset(const BStep* __restrict__ S, int nr, int nc, bool pow2, int m, int x) {
+  return x < m ? map_offset(S->rext, S->rstr, nr, pow2, x) : map_offset(S->cext, S->cstr, nc, pow2, x - m);
+}
+
+template <int KV>
+__device__ __forceinline__ void load_k(const float* p, float s, float (&v)[KV]) {
+  if constexpr (KV == 4) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x * s, v[1] = x.y * s, v[2] = x.z * s, v[3] = x.w * s;
+  } else if constexpr (KV == 2) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x * s, v[1] = x.y * s;
+  } else {
+    v[0] = *p * s;
+  }
+}
+
+// RM x RN outputs of one thread, each its own chain over k in order (so an output's bits do not
+// depend on the tile it is computed in): rows a + ra[r], columns b + rb[c], KV terms per load.
+template <bool CPLX, bool MAXPLUS, int RM, int RN, int KV>
+__device__ __forceinline__ void dot_tile(const float* a, int ai, const int (&ra)[RM], const float* b, int bi,
+                                         const int (&rb)[RN], int k, float sa, float sb, float (&cr)[RM][RN],
+                                         float (&ci)[RM][RN]) {
+#pragma unroll
+  for (int r = 0; r < RM; ++r)
+#pragma unroll
+    for (int c = 0; c < RN; ++c) {
+      cr[r][c] = MAXPLUS ? __int_as_float(0xff800000) : 0.f;  // max-plus: its zero is -inf, its product +
+      ci[r][c] = 0.f;
     }
-    __syncthreads();
-    const int w = s_net;
+#pragma unroll(RM * RN == 1 ? 4 : 1)
+  for (int t = 0; t < k; t += KV) {
+    float xr[RM][KV], xi[RM][KV];
+#pragma unroll
+    for (int r = 0; r < RM; ++r) {
+      load_k<KV>(a + ra[r] + t, sa, xr[r]);
+      if (CPLX) load_k<KV>(a + ai + ra[r] + t, sa, xi[r]);
+    }
+#pragma unroll
+    for (int c = 0; c < RN; ++c) {
+      float yr[KV], yi[KV];
+      load_k<KV>(b + rb[c] + t, sb, yr);
+      if (CPLX) load_k<KV>(b + bi + rb[c] + t, sb, yi);
+#pragma unroll
+      for (int q = 0; q < KV; ++q)
+#pragma unroll
+        for (int r = 0; r < RM; ++r) {
+          if (CPLX) {
+            cr[r][c] = fmaf(xr[r][q], yr[q], fmaf(-xi[r][q], yi[q], cr[r][c]));
+            ci[r][c] = fmaf(xr[r][q], yi[q], fmaf(xi[r][q], yr[q], ci[r][c]));
+          } else if (MAXPLUS) {
+            cr[r][c] = fmaxf(cr[r][c], xr[r][q] + yr[q]);
+          } else {
+            cr[r][c] = fmaf(xr[r][q], yr[q], cr[r][c]);
+          }
+        }
+    }
+  }
+}
+
+// One step in the arena `ar` by the team; returns the largest output's bits (sign cleared), this
+// thread's outputs only. RM x RN tiles are dealt to warps in patches of 32 >> bj by 1 << bj
+// threads, a thread's rows tm apart and its columns tn apart, so that neighbouring threads read
+// neighbouring rows. 1 x 1: output o to thread o, in order.
+template <bool CPLX, bool MAXPLUS, bool WARP, int RM, int RN, int KV>
+__device__ __forceinline__ int run_step(float* ar, const BStep* __restrict__ S, int m, int n, int k, int nr, int nc,
+                                        bool pow2, int a, int b, int c, float sa, float sb, const int* tab) {
+  int mx = 0;
+  float cr[RM][RN], ci[RM][RN];
+  auto store = [&](int off, float vr, float vi) {
+    ar[c + off] = vr;
+    float v = fabsf(vr);
+    if (CPLX) {
+      ar[c + m * n + off] = vi;
+      v = fmaxf(v, fabsf(vi));
+    }
+    mx = max(mx, __float_as_int(v));
+  };
+  if constexpr (RM == 1) {
+    const int nsh = (n & (n - 1)) == 0 ? 31 - __clz(n) : -1;
+    for (int o = Team<WARP>::rank(); o < m * n; o += Team<WARP>::size()) {
+      const int i = nsh >= 0 ? o >> nsh : o / n, j = o - i * n;
+      const int ra[1] = {i * k}, rb[1] = {j * k};
+      dot_tile<CPLX, MAXPLUS, 1, 1, KV>(ar + a, m * k, ra, ar + b, n * k, rb, k, sa, sb, cr, ci);
+      store(map_offset(S->rext, S->rstr, nr, pow2, i) + map_offset(S->cext, S->cstr, nc, pow2, j), cr[0][0], ci[0][0]);
+    }
+  } else {
+    const int tm = (m + RM - 1) / RM, tn = (n + RN - 1) / RN;
+    const int bj = tn >= 8 ? 3 : tn >= 4 ? 2 : tn >= 2 ? 1 : 0;
+    const int lane = threadIdx.x & 31;
+    const int li = lane >> bj, lj = lane & ((1 << bj) - 1);
+    const int pn = (tn + (1 << bj) - 1) >> bj, pm = (tm + (32 >> bj) - 1) >> (5 - bj);
+    for (int p = Team<WARP>::rank() >> 5; p < pm * pn; p += Team<WARP>::size() >> 5) {
+      const int pi = p / pn, pj = p - pi * pn;
+      const int ti = (pi << (5 - bj)) + li, tj = (pj << bj) + lj;
+      if (ti >= tm || tj >= tn) continue;
+      int ra[RM], rb[RN];
+#pragma unroll
+      for (int r = 0; r < RM; ++r) ra[r] = min(ti + r * tm, m - 1) * k;
+#pragma unroll
+      for (int q = 0; q < RN; ++q) rb[q] = min(tj + q * tn, n - 1) * k;
+      dot_tile<CPLX, MAXPLUS, RM, RN, KV>(ar + a, m * k, ra, ar + b, n * k, rb, k, sa, sb, cr, ci);
+#pragma unroll
+      for (int q = 0; q < RN; ++q) {
+        const int j = tj + q * tn;
+        if (j >= n) continue;
+        const int oc = tab ? tab[m + j] : map_offset(S->cext, S->cstr, nc, pow2, j);
+#pragma unroll
+        for (int r = 0; r < RM; ++r) {
+          const int i = ti + r * tm;
+          if (i < m) store((tab ? tab[i] : map_offset(S->rext, S->rstr, nr, pow2, i)) + oc, cr[r][q], ci[r][q]);
+        }
+      }
+    }
+  }
+  return mx;
+}
+
+// Step outputs whose exponents a team keeps (bytes of shared memory per CTA / per warp's share):
+// networks with more steps renormalise each output in place.
+constexpr int kExpBytes = 2048;
+
+// CTAs of at most this many threads take the form with register tiles (128 registers a thread);
+// wider ones, which the autotuner does not try, run one output per thread
+constexpr int kTileThreads = 256;
+
+// leaves above this many elements are staged by the whole team, the others by groups of 8 threads
+constexpr int kGroupLeaf = 64;
+
+template <bool CPLX, bool MAXPLUS, bool WARP, bool TILES>
+__global__ void __launch_bounds__(TILES ? kTileThreads : 1024, TILES ? 2 : 1)
+batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves, const BStep* __restrict__ steps,
+             int32_t n_nets, const float* __restrict__ packed, float* arena, int32_t* queue, int32_t scaling,
+             double* values, double* logs, int32_t smem_arena, int32_t tab_ints) {
+  // dynamic shared memory: [arenas: smem_arena floats per team | offset tables: tab_ints per team]
+  extern __shared__ __align__(16) float s_arena[];
+  __shared__ int s_exp[kExpBytes / 4];  // the step outputs' largest exponents: ints, or bytes (+127) per warp
+  __shared__ int s_net;
+  __shared__ long long s_log;
+  using T = Team<WARP>;
+  constexpr int RM = 4, RN = CPLX ? 2 : 4;
+  const int teams = WARP ? blockDim.x >> 5 : 1, team = WARP ? threadIdx.x >> 5 : 0;
+  const int rank = T::rank(), size = T::size(), lane = threadIdx.x & 31;
+  int* s_tab = reinterpret_cast<int*>(s_arena + smem_arena * teams) + team * tab_ints;
+  const int exp_cap = WARP ? kExpBytes / teams : kExpBytes / 4;
+  uint8_t* w_exp = reinterpret_cast<uint8_t*>(s_exp) + (WARP ? team * exp_cap : 0);
+  while (true) {
+    int w = 0;
+    if (WARP) {
+      if (lane == 0) w = atomicAdd(queue, 1);
+      w = __shfl_sync(0xffffffffu, w, 0);
+    } else {
+      if (rank == 0) {
+        s_net = atomicAdd(queue, 1);
+        s_log = 0;
+      }
+      __syncthreads();
+      w = s_net;
+    }
     if (w >= n_nets) break;
     const BNet net = nets[w];
     // the network's arena: in shared memory when it fits the launch's shared-memory arena
-    // (smem_arena floats per CTA), else its own slice of the global batch arena
-    float* ar = net.arena_floats <= smem_arena ? s_arena : arena + net.arena;
-    // stage the leaves (declared order -> planned order; complex64 -> planar)
-    for (int l = 0; l < net.n_leaves; ++l) {
-      const BLeaf& L = leaves[net.leaf0 + l];
-      for (int e = threadIdx.x; e < L.size; e += blockDim.x) {
-        int r = e, src = 0;
-        for (int d = L.rank - 1; d >= 0; --d) {
-          src += (r % L.ext[d]) * L.sstride[d];
-          r /= L.ext[d];
+    // (smem_arena floats per team), else its own slice of the global batch arena
+    float* ar = net.arena_floats <= smem_arena ? s_arena + team * smem_arena : arena + net.arena;
+    const float* in = packed + net.in * (CPLX ? 2 : 1);
+    const BLeaf* L0 = leaves + net.leaf0;
+    const BStep* S0 = steps + net.step0;
+    const bool defer = net.n_steps <= exp_cap;
+    long long lsum = 0;  // this thread's share of the exponents' sum
+    if (!WARP && scaling)
+      for (int i = rank; i < min(max(net.n_steps, 2), exp_cap); i += size) s_exp[i] = -127;
+    // Leaves (declared order -> planned order; complex64 -> planar), each scaled by its own exact
+    // power of two: small ones by groups of 8 threads, whose own elements they scale
+    bool big = false;
+    for (int l0 = 0; l0 < net.n_leaves; l0 += size >> 3) {
+      const int l = l0 + (rank >> 3), sub = lane & 7;
+      int4 h = make_int4(0, 0, 0, 0);
+      if (l < net.n_leaves) h = __ldg(reinterpret_cast<const int4*>(L0 + l));
+      big = big || h.z > kGroupLeaf;
+      const bool mine = h.z <= kGroupLeaf;
+      int mx = 0;
+      if (mine)
+        for (int e = sub; e < h.z; e += 8) {
+          const int src = h.x + map_offset(L0[l].ext, L0[l].sstride, h.w & 0xff, h.w < 0, e);
+          if (CPLX) {
+            const float2 v = reinterpret_cast<const float2*>(in)[src];
+            ar[h.y + e] = v.x;
+            ar[h.y + h.z + e] = v.y;
+            mx = max(mx, __float_as_int(fmaxf(fabsf(v.x), fabsf(v.y))));
+          } else {
+            const float v = in[src];
+            ar[h.y + e] = v;
+            mx = max(mx, __float_as_int(fabsf(v)));
+          }
         }
-        if (CPLX) {
-          const float2 v = reinterpret_cast<const float2*>(in)[L.src + src];
-          ar[L.dst + e] = v.x;
-          ar[L.dst + L.size + e] = v.y;
-        } else {
-          ar[L.dst + e] = in[L.src + src];
+      if (!MAXPLUS && scaling) {
+        for (int o = 4; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        int e = (mx >> 23) - 127;
+        if (e < -126) e = 0;  // an all-zero leaf is left as is
+        if (mine && e != 0) {
+          const float sc = bpow2_neg(e);
+          for (int i = sub; i < h.z; i += 8) {
+            ar[h.y + i] *= sc;
+            if (CPLX) ar[h.y + h.z + i] *= sc;
+          }
+          if (sub == 0) lsum += e;
         }
       }
     }
-    __syncthreads();
-    if (scaling && net.n_leaves <= kLeafExpCap) {
-      // every leaf renormalised in one pass: per-leaf maxima by shared-memory atomics, then
-      // each leaf scaled by its own exact power of two (the same exponents as one leaf at a
-      // time, with three barriers instead of three per leaf)
-      for (int l = threadIdx.x; l < net.n_leaves; l += blockDim.x) s_lexp[l] = -127;
-      __syncthreads();
-      for (int l = 0; l < net.n_leaves; ++l) {
-        const BLeaf& L = leaves[net.leaf0 + l];
-        int lmax = -127;
-        for (int i = threadIdx.x; i < L.size; i += blockDim.x) {
-          float v = fabsf(ar[L.dst + i]);
-          if (CPLX) v = fmaxf(v, fabsf(ar[L.dst + L.size + i]));
-          lmax = max(lmax, bexp_of(v));
-        }
-        if (lmax > -127) atomicMax(&s_lexp[l], lmax);
-      }
-      __syncthreads();
-      long long sum = 0;
-      for (int l = 0; l < net.n_leaves; ++l) {
-        const BLeaf& L = leaves[net.leaf0 + l];
-        const int e = s_lexp[l] < -126 ? 0 : s_lexp[l];  // an all-zero leaf is left as is
-        sum += e;
-        if (e == 0) continue;
-        const float sc = bpow2_neg(e);
-        for (int i = threadIdx.x; i < L.size; i += blockDim.x) {
-          ar[L.dst + i] *= sc;
-          if (CPLX) ar[L.dst + L.size + i] *= sc;
-        }
-      }
-      if (threadIdx.x == 0) s_log += sum;
-      __syncthreads();
-    } else if (scaling) {
-      for (int l = 0; l < net.n_leaves; ++l) {
-        const BLeaf& L = leaves[net.leaf0 + l];
-        renormalise<CPLX>(ar + L.dst, L.size, &s_max, &s_log);
-      }
-    }
-    for (int s = 0; s < net.n_steps; ++s) {
-      const BStep& S = steps[net.step0 + s];
-      const int mn = S.m * S.n;
-      // the output offset of every row and column, once per step (not once per element)
-      const bool tab = S.m + S.n <= tab_ints;
-      if (tab) {
-        for (int x = threadIdx.x; x < S.m + S.n; x += blockDim.x) s_tab[x] = step_offset(S, x);
+    // the largest exponent over the team, every thread's answer; slot: two taken in turn
+    auto team_exp = [&](int mx, int slot) {
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      if (!WARP) {
+        if (lane == 0) atomicMax(&s_exp[slot], (mx >> 23) - 127);
         __syncthreads();
+        const int e = s_exp[slot];
+        if (rank == 0) s_exp[slot ^ 1] = -127;  // read by nobody until the barrier after the scaling
+        return e;
       }
-      for (int o = threadIdx.x; o < mn; o += blockDim.x) {
-        const int i = o / S.n, j = o - i * S.n;
-        const float* A = ar + S.a + i * S.k;
-        const float* B = ar + S.b + j * S.k;
-        // max-plus (real, unscaled): the semiring's zero is -inf, its product +
-        float cr = MAXPLUS ? __int_as_float(0xff800000) : 0.f, ci = 0.f;
-        for (int t = 0; t < S.k; ++t) {
-          if (CPLX) {
-            const float xr = A[t], xi = A[S.a_size + t], yr = B[t], yi = B[S.b_size + t];
-            cr = fmaf(xr, yr, fmaf(-xi, yi, cr));
-            ci = fmaf(xr, yi, fmaf(xi, yr, ci));
-          } else if (MAXPLUS) {
-            cr = fmaxf(cr, A[t] + B[t]);
-          } else {
-            cr = fmaf(A[t], B[t], cr);
-          }
-        }
-        const int off = tab ? s_tab[i] + s_tab[S.m + j] : step_offset(S, i) + step_offset(S, S.m + j);
-        ar[S.c + off] = cr;
-        if (CPLX) ar[S.c + S.c_size + off] = ci;
+      return (mx >> 23) - 127;
+    };
+    auto scale_in_place = [&](int off, int elems, int e) {
+      if (e < -126) e = 0;
+      if (e != 0) {
+        const float sc = bpow2_neg(e);
+        for (int i = rank; i < elems * (CPLX ? 2 : 1); i += size) ar[off + i] *= sc;
       }
-      __syncthreads();
-      if (scaling) renormalise<CPLX>(ar + S.c, S.c_size, &s_max, &s_log);
-    }
-    if (threadIdx.x == 0) {
-      // scalar results (closed networks): value and log2 scale
-      values[2 * (int64_t)w] = ar[net.root];
-      values[2 * (int64_t)w + 1] = CPLX ? ar[net.root + net.root_size] : 0.0;
-      logs[w] = double(s_log) * 0.69314718055994530942;
-    }
-    __syncthreads();
-  }
-}
-
-// The warp-per-network form of batch_kernel (K-FUSE): each warp takes networks from the
-// queue and runs a whole path with warp-synchronous steps -- no block barriers between
-// steps, and as many networks in flight per SM as resident warps. The same tables, the
-// same arithmetic per output element (one lane, k in order) and the same exact power-of-two
-// renormalisation, so a network's value does not depend on the form that computed it.
-template <bool CPLX>
-__device__ int warp_renormalise(float* t, int size, int lane) {
-  int lmax = -127;
-  for (int i = lane; i < size; i += 32) {
-    float v = fabsf(t[i]);
-    if (CPLX) v = fmaxf(v, fabsf(t[size + i]));
-    lmax = max(lmax, bexp_of(v));
-  }
-  for (int o = 16; o > 0; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  const int e = lmax < -126 ? 0 : lmax;  // an all-zero tensor is left as is
-  if (e != 0) {
-    const float sc = bpow2_neg(e);
-    for (int i = lane; i < size; i += 32) {
-      t[i] *= sc;
-      if (CPLX) t[size + i] *= sc;
-    }
-  }
-  __syncwarp();
-  return e;
-}
-
-template <bool CPLX, bool MAXPLUS = false>
-__global__ void batch_warp_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves,
-                                  const BStep* __restrict__ steps, int32_t n_nets, const float* __restrict__ in,
-                                  float* arena, int32_t* queue, int32_t scaling, double* values, double* logs,
-                                  int32_t smem_arena, int32_t tab_ints) {
-  // dynamic shared memory: [arenas: smem_arena floats per warp | tables: tab_ints ints per warp]
-  extern __shared__ float s_arena[];
-  const int lane = threadIdx.x & 31;
-  int* s_tab = reinterpret_cast<int*>(s_arena + smem_arena * (blockDim.x >> 5)) + (threadIdx.x >> 5) * tab_ints;
-  while (true) {
-    int w = 0;
-    if (lane == 0) w = atomicAdd(queue, 1);
-    w = __shfl_sync(0xffffffffu, w, 0);
-    if (w >= n_nets) break;
-    const BNet net = nets[w];
-    float* ar = net.arena_floats <= smem_arena ? s_arena + (threadIdx.x >> 5) * smem_arena : arena + net.arena;
-    long long slog = 0;
-    for (int l = 0; l < net.n_leaves; ++l) {
-      const BLeaf& L = leaves[net.leaf0 + l];
-      for (int e = lane; e < L.size; e += 32) {
-        int r = e, src = 0;
-        for (int d = L.rank - 1; d >= 0; --d) {
-          src += (r % L.ext[d]) * L.sstride[d];
-          r /= L.ext[d];
-        }
-        if (CPLX) {
-          const float2 v = reinterpret_cast<const float2*>(in)[L.src + src];
-          ar[L.dst + e] = v.x;
-          ar[L.dst + L.size + e] = v.y;
-        } else {
-          ar[L.dst + e] = in[L.src + src];
-        }
-      }
-    }
-    __syncwarp();
-    if (scaling)
+      if (rank == 0) lsum += e;
+      T::sync();
+    };
+    if (WARP) __syncwarp();
+    if (WARP ? __any_sync(0xffffffffu, big) : __syncthreads_or(big)) {
+      int turn = 0;
       for (int l = 0; l < net.n_leaves; ++l) {
-        const BLeaf& L = leaves[net.leaf0 + l];
-        slog += warp_renormalise<CPLX>(ar + L.dst, L.size, lane);
-      }
-    for (int s = 0; s < net.n_steps; ++s) {
-      const BStep& S = steps[net.step0 + s];
-      const int mn = S.m * S.n;
-      const bool tab = S.m + S.n <= tab_ints;
-      if (tab) {
-        for (int x = lane; x < S.m + S.n; x += 32) s_tab[x] = step_offset(S, x);
-        __syncwarp();
-      }
-      for (int o = lane; o < mn; o += 32) {
-        const int i = o / S.n, j = o - i * S.n;
-        const float* A = ar + S.a + i * S.k;
-        const float* B = ar + S.b + j * S.k;
-        float cr = MAXPLUS ? __int_as_float(0xff800000) : 0.f, ci = 0.f;
-        for (int t = 0; t < S.k; ++t) {
+        const int4 h = __ldg(reinterpret_cast<const int4*>(L0 + l));
+        if (h.z <= kGroupLeaf) continue;
+        int mx = 0;
+        for (int e = rank; e < h.z; e += size) {
+          const int src = h.x + map_offset(L0[l].ext, L0[l].sstride, h.w & 0xff, h.w < 0, e);
           if (CPLX) {
-            const float xr = A[t], xi = A[S.a_size + t], yr = B[t], yi = B[S.b_size + t];
-            cr = fmaf(xr, yr, fmaf(-xi, yi, cr));
-            ci = fmaf(xr, yi, fmaf(xi, yr, ci));
-          } else if (MAXPLUS) {
-            cr = fmaxf(cr, A[t] + B[t]);
+            const float2 v = reinterpret_cast<const float2*>(in)[src];
+            ar[h.y + e] = v.x;
+            ar[h.y + h.z + e] = v.y;
+            mx = max(mx, __float_as_int(fmaxf(fabsf(v.x), fabsf(v.y))));
           } else {
-            cr = fmaf(A[t], B[t], cr);
+            const float v = in[src];
+            ar[h.y + e] = v;
+            mx = max(mx, __float_as_int(fabsf(v)));
           }
         }
-        const int off = tab ? s_tab[i] + s_tab[S.m + j] : step_offset(S, i) + step_offset(S, S.m + j);
-        ar[S.c + off] = cr;
-        if (CPLX) ar[S.c + S.c_size + off] = ci;
+        if (!MAXPLUS && scaling) {
+          const int e = team_exp(mx, turn);
+          if (WARP) __syncwarp();
+          scale_in_place(h.y, h.z, e);
+          turn ^= 1;
+        }
       }
-      __syncwarp();
-      if (scaling) slog += warp_renormalise<CPLX>(ar + S.c, S.c_size, lane);
+      if (!WARP && scaling) {
+        // the two slots back as the steps expect them
+        T::sync();
+        if (rank < 2) s_exp[rank] = -127;
+      }
+      T::sync();
     }
-    if (lane == 0) {
-      values[2 * (int64_t)w] = ar[net.root];
-      values[2 * (int64_t)w + 1] = CPLX ? ar[net.root + net.root_size] : 0.0;
-      logs[w] = double(slog) * 0.69314718055994530942;
+    for (int s = 0; s < net.n_steps; ++s) {
+      const BStep* S = S0 + s;
+      const int4 h0 = __ldg(reinterpret_cast<const int4*>(S)), h1 = __ldg(reinterpret_cast<const int4*>(S) + 1);
+      if (rank < 2 && s + 1 < net.n_steps) {
+        // the next step's record into L1 while this one runs
+        int x;
+        asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(x) : "l"(reinterpret_cast<const char*>(S + 1) + rank * 128));
+      }
+      const int m = h0.w, n = h1.x, k = h1.y, mn = m * n;
+      const int nr = (h1.z >> 27) & 15, nc = h1.w >> 27;
+      const bool pow2 = h1.z < 0;
+      float sa = 1.f, sb = 1.f;
+      if (!MAXPLUS && scaling && defer) {
+        auto scale_of = [&](int id) {
+          if (id == kBLeafId) return 1.f;
+          const int e = WARP ? int(w_exp[id]) - 127 : s_exp[id];
+          return e < -126 ? 1.f : bpow2_neg(e);  // an all-zero tensor is left as is
+        };
+        sa = scale_of(h1.z & kBLeafId);
+        sb = scale_of(h1.w & kBLeafId);
+      }
+      int mx = 0;
+      if (rank - lane >= mn) {
+        // no output for this warp
+      } else if (TILES && m >= RM && n >= RN && mn >= 8 * size) {
+        const int* tab = nullptr;
+        if (m + n <= tab_ints) {
+          for (int x = rank; x < m + n; x += size) s_tab[x] = step_offset(S, nr, nc, pow2, m, x);
+          tab = s_tab;
+          T::sync();
+        }
+        if constexpr (!TILES) {
+        } else if ((k & 3) == 0 && !CPLX)
+          mx = run_step<CPLX, MAXPLUS, WARP, RM, RN, CPLX ? 2 : 4>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa,
+                                                                  sb, tab);
+        else if ((k & 1) == 0)
+          mx = run_step<CPLX, MAXPLUS, WARP, RM, RN, 2>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, tab);
+        else
+          mx = run_step<CPLX, MAXPLUS, WARP, RM, RN, 1>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, tab);
+      } else if ((k & 3) == 0) {
+        mx = run_step<CPLX, MAXPLUS, WARP, 1, 1, 4>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, nullptr);
+      } else if ((k & 1) == 0) {
+        mx = run_step<CPLX, MAXPLUS, WARP, 1, 1, 2>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, nullptr);
+      } else {
+        mx = run_step<CPLX, MAXPLUS, WARP, 1, 1, 1>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, nullptr);
+      }
+      if (!MAXPLUS && scaling) {
+        __syncwarp();
+        if (defer) {
+          mx = __reduce_max_sync(0xffffffffu, mx);
+          if (lane == 0) {
+            if (WARP) w_exp[s] = static_cast<uint8_t>(mx >> 23);
+            else if (mx) atomicMax(&s_exp[s], (mx >> 23) - 127);
+          }
+        } else {
+          const int e = team_exp(mx, s & 1);
+          if (WARP) __syncwarp();
+          scale_in_place(h0.z, mn, e);
+          continue;
+        }
+      }
+      T::sync();
     }
-    __syncwarp();
+    float sr = 1.f;
+    if (!MAXPLUS && scaling) {
+      if (defer) {
+        for (int i = rank; i < net.n_steps; i += size) {
+          const int e = WARP ? int(w_exp[i]) - 127 : s_exp[i];
+          lsum += e < -126 ? 0 : e;
+        }
+        if (net.n_steps > 0) {
+          const int e = WARP ? int(w_exp[net.n_steps - 1]) - 127 : s_exp[net.n_steps - 1];
+          if (e >= -126) sr = bpow2_neg(e);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+      if (!WARP) {
+        if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&s_log), static_cast<unsigned long long>(lsum));
+        __syncthreads();
+        lsum = s_log;
+      }
+    }
+    if (rank == 0) {
+      // scalar results (closed networks): value and log2 scale
+      values[2 * (int64_t)net.index] = ar[net.root] * sr;
+      values[2 * (int64_t)net.index + 1] = CPLX ? ar[net.root + net.root_size] * sr : 0.0;
+      logs[net.index] = double(lsum) * 0.69314718055994530942;
+    }
+    T::sync();
   }
 }
 
@@ -352,9 +467,9 @@ struct tn_batch_s {
 
 namespace tn {
 
-template <typename K>
-cudaError_t set_smem(K kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+template <bool CPLX, bool MAXPLUS, bool WARP>
+auto batch_form(bool tiles) {
+  return tiles ? batch_kernel<CPLX, MAXPLUS, WARP, true> : batch_kernel<CPLX, MAXPLUS, WARP, false>;
 }
 
 cudaError_t launch_batch_kernel(const BNet* nets, const BLeaf* leaves, const BStep* steps, int32_t n_nets,
@@ -366,37 +481,31 @@ cudaError_t launch_batch_kernel(const BNet* nets, const BLeaf* leaves, const BSt
   const float* in = static_cast<const float*>(packed);
   const int sc = scaling ? 1 : 0;
   // dynamic shared memory: an arena and an offset table per CTA, or per warp in the warp form
+  smem_arena &= ~63;  // arenas are multiples of 64 floats
   const int smem = (smem_arena + tab_ints) * 4 * (warp ? threads / 32 : 1);
-  if (warp) {
-    if (cplx) {
-      if (smem && (e = set_smem(batch_warp_kernel<true>, smem)) != cudaSuccess) return e;
-      batch_warp_kernel<true><<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, sc, values,
-                                                           logs, smem_arena, tab_ints);
-    } else if (maxplus) {
-      if (smem && (e = set_smem(batch_warp_kernel<false, true>, smem)) != cudaSuccess) return e;
-      batch_warp_kernel<false, true><<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, 0,
-                                                                  values, logs, smem_arena, tab_ints);
-    } else {
-      if (smem && (e = set_smem(batch_warp_kernel<false>, smem)) != cudaSuccess) return e;
-      batch_warp_kernel<false><<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, sc,
-                                                            values, logs, smem_arena, tab_ints);
-    }
-    return cudaGetLastError();
-  }
-  if (cplx) {
-    if (smem && (e = set_smem(batch_kernel<true>, smem)) != cudaSuccess) return e;
-    batch_kernel<true><<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, sc, values, logs,
-                                                    smem_arena, tab_ints);
-  } else if (maxplus) {
-    if (smem && (e = set_smem(batch_kernel<false, true>, smem)) != cudaSuccess) return e;
-    batch_kernel<false, true><<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, 0, values,
-                                                           logs, smem_arena, tab_ints);
-  } else {
-    if (smem && (e = set_smem(batch_kernel<false>, smem)) != cudaSuccess) return e;
-    batch_kernel<false><<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, sc, values,
-                                                     logs, smem_arena, tab_ints);
-  }
+  const bool tiles = threads <= kTileThreads;
+  auto kernel = warp ? (cplx ? batch_form<true, false, true>(tiles)
+                             : maxplus ? batch_form<false, true, true>(tiles) : batch_form<false, false, true>(tiles))
+                     : (cplx ? batch_form<true, false, false>(tiles)
+                             : maxplus ? batch_form<false, true, false>(tiles) : batch_form<false, false, false>(tiles));
+  if (smem && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    return e;
+  kernel<<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, maxplus ? 0 : sc, values, logs,
+                                      smem_arena, tab_ints);
   return cudaGetLastError();
+}
+
+// Replace the extents of a digit map by the digits' places where all are powers of two.
+static bool digit_places(int32_t* ext, int n) {
+  int sh = 0;
+  for (int d = 0; d < n; ++d)
+    if (ext[d] < 1 || (ext[d] & (ext[d] - 1)) != 0 || ext[d] >= 1 << 23) return false;
+  for (int d = n - 1; d >= 0; --d) {
+    const int32_t mask = ext[d] - 1;
+    ext[d] = sh | mask << 8;
+    sh += __builtin_popcount(static_cast<unsigned>(mask));
+  }
+  return true;
 }
 
 bool batch_template(const Plan& P, BatchTemplate& T, std::string& err) {
@@ -425,14 +534,14 @@ bool batch_template(const Plan& P, BatchTemplate& T, std::string& err) {
       return false;
     }
     BLeaf L{};
-    L.src = T.input_elems;
+    L.src = static_cast<int32_t>(T.input_elems);
     L.dst = foff(t);
     L.size = (int32_t)R.size;
-    L.rank = d.rank;
     for (int r = 0; r < d.rank; ++r) {
       L.ext[r] = (int32_t)d.ext[r];
       L.sstride[r] = (int32_t)d.sstride[r];
     }
+    L.rank = d.rank | (digit_places(L.ext, d.rank) ? kBPow2 : 0);
     int64_t full = 1;
     for (int32_t x : R.decl) full *= P.extent[x];
     T.input_elems += full;
@@ -447,14 +556,9 @@ bool batch_template(const Plan& P, BatchTemplate& T, std::string& err) {
     S.a = foff(st.a);
     S.b = foff(st.b);
     S.c = foff(st.out);
-    S.a_size = (int32_t)P.tensors[st.a].size;
-    S.b_size = (int32_t)P.tensors[st.b].size;
-    S.c_size = (int32_t)P.tensors[st.out].size;
     S.m = (int32_t)st.m;
     S.n = (int32_t)st.n;
     S.k = (int32_t)st.k;
-    S.nr = (int8_t)st.rows.n;
-    S.nc = (int8_t)st.cols.n;
     for (int d = 0; d < st.rows.n; ++d) {
       S.rext[d] = (int32_t)st.rows.ext[d];
       S.rstr[d] = (int32_t)st.rows.stride[d];
@@ -463,6 +567,16 @@ bool batch_template(const Plan& P, BatchTemplate& T, std::string& err) {
       S.cext[d] = (int32_t)st.cols.ext[d];
       S.cstr[d] = (int32_t)st.cols.stride[d];
     }
+    int32_t rext[kBMaxDims], cext[kBMaxDims];
+    std::copy(S.rext, S.rext + kBMaxDims, rext);
+    std::copy(S.cext, S.cext + kBMaxDims, cext);
+    const bool pow2 = digit_places(rext, st.rows.n) && digit_places(cext, st.cols.n);
+    if (pow2) {
+      std::copy(rext, rext + kBMaxDims, S.rext);
+      std::copy(cext, cext + kBMaxDims, S.cext);
+    }
+    S.pa = (st.a < P.n_leaves ? kBLeafId : st.a - P.n_leaves) | st.rows.n << 27 | (pow2 ? kBPow2 : 0);
+    S.pb = (st.b < P.n_leaves ? kBLeafId : st.b - P.n_leaves) | st.cols.n << 27;
     T.steps.push_back(S);
     T.max_tab = std::max<int32_t>(T.max_tab, static_cast<int32_t>(st.m + st.n));
     T.flops += (P.is_complex ? 8.0 : 2.0) * double(st.m) * double(st.n) * double(st.k);
@@ -515,6 +629,8 @@ tn_status tn_batch_plan(int32_t n_nets, const tn_network* nets, const tn_path* p
     return TN_ERR_UNSUPPORTED;
   }
   int64_t in_off = 0;
+  std::unordered_map<std::string, std::pair<size_t, size_t>> tables;
+  std::vector<double> cost;
   tn_dtype_policy hp = policy;
   hp.flags |= TN_PLAN_HOST_ONLY;
   hp.max_slice_batch = 1;
@@ -543,20 +659,26 @@ tn_status tn_batch_plan(int32_t n_nets, const tn_network* nets, const tn_path* p
     }
     BNet bn{};
     bn.arena = B->arena_floats;
-    bn.leaf0 = (int32_t)B->leaves.size();
+    bn.index = w;
+    // networks of one shape and path share their tables (which then stay in L2)
+    std::string key(reinterpret_cast<const char*>(T.leaves.data()), T.leaves.size() * sizeof(BLeaf));
+    key.append(reinterpret_cast<const char*>(T.steps.data()), T.steps.size() * sizeof(BStep));
+    const auto [at, fresh] = tables.emplace(std::move(key), std::make_pair(B->leaves.size(), B->steps.size()));
+    bn.leaf0 = (int32_t)at->second.first;
     bn.n_leaves = (int32_t)T.leaves.size();
-    bn.step0 = (int32_t)B->steps.size();
+    bn.step0 = (int32_t)at->second.second;
     bn.n_steps = (int32_t)T.steps.size();
     bn.root = T.root;
     bn.root_size = T.root_size;
     bn.arena_floats = static_cast<int32_t>(T.arena_floats);
-    for (BLeaf L : T.leaves) {
-      B->leaf_offset.push_back(in_off + L.src);
-      L.src += in_off;
-      B->leaves.push_back(L);
+    bn.in = in_off;
+    for (const BLeaf& L : T.leaves) B->leaf_offset.push_back(in_off + L.src);
+    if (fresh) {
+      B->leaves.insert(B->leaves.end(), T.leaves.begin(), T.leaves.end());
+      B->steps.insert(B->steps.end(), T.steps.begin(), T.steps.end());
     }
     in_off += T.input_elems;
-    B->steps.insert(B->steps.end(), T.steps.begin(), T.steps.end());
+    cost.push_back(T.flops);
     B->flops += T.flops;
     B->arena_floats += T.arena_floats;
     B->max_arena_floats = std::max(B->max_arena_floats, T.arena_floats);
@@ -564,6 +686,13 @@ tn_status tn_batch_plan(int32_t n_nets, const tn_network* nets, const tn_path* p
     B->nets.push_back(bn);
   }
   B->leaf_offset.push_back(in_off);
+  // the costliest networks first
+  std::vector<int32_t> order(n_nets);
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return cost[x] > cost[y]; });
+  std::vector<BNet> queued;
+  for (int32_t w : order) queued.push_back(B->nets[w]);
+  B->nets.swap(queued);
   if ((policy.flags & TN_PLAN_HOST_ONLY) == 0) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||

@@ -15,33 +15,37 @@ namespace tn {
 constexpr int kBMaxDims = 8;    // merged offset dims per side in the batch tables
 constexpr int kBMaxRank = 8;    // planned leaf rank in the batch tables
 
-struct BLeaf {
-  int64_t src;                  // element offset in the packed input buffer
+// Mixed-radix digit maps (planned positions of a leaf, merged dims of a step's rows and
+// columns): digit d of an index times its stride, summed. When every extent is a power of two
+// (and below 2^23) ext[d] holds the digit's place instead, shift | (extent - 1) << 8, so that a
+// digit costs a shift and a mask and does not wait for the one before it.
+struct alignas(16) BLeaf {
+  int32_t src;                  // element offset in the network's own inputs
   int32_t dst;                  // float offset in the network's arena (real plane)
   int32_t size;
-  int32_t rank;
-  int32_t pad;
+  int32_t rank;                 // planned positions | kBPow2
   int32_t ext[kBMaxRank];
   int32_t sstride[kBMaxRank];   // declared stride of each planned position
 };
 
-struct BStep {
-  int32_t a, b, c;              // float offsets in the arena (real planes)
-  int32_t a_size, b_size, c_size;
+struct alignas(16) BStep {
+  int32_t a, b, c;              // float offsets in the arena (real planes; imaginary ones follow them)
   int32_t m, n, k;
-  int8_t nr, nc;
-  int16_t pad;
+  int32_t pa, pb;               // producing step (kBLeafId: a leaf) | row / column dims << 27 (pa: | kBPow2)
   int32_t rext[kBMaxDims], rstr[kBMaxDims];
   int32_t cext[kBMaxDims], cstr[kBMaxDims];
 };
+constexpr int32_t kBPow2 = INT32_MIN;           // the map's extents are all powers of two
+constexpr int32_t kBLeafId = (1 << 27) - 1;
 
 struct BNet {
   int64_t arena;                // float offset of the network's arena in the batch arena
+  int64_t in;                   // element offset of its inputs in the packed input buffer
   int32_t leaf0, n_leaves;      // index range in the leaf table
   int32_t step0, n_steps;       // index range in the step table
   int32_t root, root_size;      // float offset and size of the result tensor
   int32_t arena_floats;         // size of the network's arena
-  int32_t pad;
+  int32_t index;                // row of its results
 };
 
 // One network's tables, offsets relative to the network itself (arena floats from 0,

@@ -256,6 +256,7 @@ struct tn_server_s {
       tab_ints = std::max(tab_ints, std::min(pt.T.max_tab, kMaxTabInts));
       BNet bn{};
       bn.arena = arena;
+      bn.index = static_cast<int32_t>(nets.size());
       bn.leaf0 = (int32_t)leaves.size();
       bn.n_leaves = (int32_t)pt.T.leaves.size();
       bn.step0 = (int32_t)steps.size();
@@ -263,10 +264,8 @@ struct tn_server_s {
       bn.root = pt.T.root;
       bn.root_size = pt.T.root_size;
       bn.arena_floats = static_cast<int32_t>(pt.T.arena_floats);
-      for (BLeaf L : pt.T.leaves) {
-        L.src += in_elems;
-        leaves.push_back(L);
-      }
+      bn.in = in_elems;
+      leaves.insert(leaves.end(), pt.T.leaves.begin(), pt.T.leaves.end());
       steps.insert(steps.end(), pt.T.steps.begin(), pt.T.steps.end());
       in_elems += pt.T.input_elems;
       arena += pt.T.arena_floats;
