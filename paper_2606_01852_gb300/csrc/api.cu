@@ -103,8 +103,13 @@ tn_status check_device_error(Plan& P) {
   return TN_OK;
 }
 
-tn_status upload_chain_table(Plan& P) {
-  if (P.chains.empty() || !P.dev) return TN_OK;
+tn_status upload_tables(Plan& P) {
+  if (!P.dev) return TN_OK;
+  for (int32_t t = 0; t < P.n_leaves; ++t) P.leafdesc[t].dst = P.tensors[t].offset;
+  cudaError_t e = cudaMemcpy(P.dev + P.off_leafdesc, P.leafdesc.data(), sizeof(LeafDesc) * P.leafdesc.size(),
+                             cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(P.dev + P.off_recidx, P.rec_index.data(), sizeof(int32_t) * P.n_leaves, cudaMemcpyHostToDevice);
   auto packed = [](uint32_t e) {
     const uint32_t sh = (e & (e - 1u)) == 0u ? static_cast<uint32_t>(__builtin_ctz(e)) : 0xffu;
     return e | (sh << 24);
@@ -144,22 +149,22 @@ tn_status upload_chain_table(Plan& P) {
       }
       table.push_back(cs);
     }
-  cudaError_t e = cudaMemcpy(P.dev + P.off_chain, table.data(), sizeof(ChainStep) * table.size(),
-                             cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !table.empty())
+    e = cudaMemcpy(P.dev + P.off_chain, table.data(), sizeof(ChainStep) * table.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !table.empty())
     e = cudaMemcpy(P.dev + P.off_chain_tasks, P.chain_tasks.data(), 4 * P.chain_tasks.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !table.empty())
     e = cudaMemcpy(P.dev + P.off_chain_levels, P.chain_levels.data(), 4 * P.chain_levels.size(),
                    cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
-    set_error(std::string("writing the step-chain table: ") + cudaGetErrorString(e));
+    set_error(std::string("writing the plan's tables: ") + cudaGetErrorString(e));
     return TN_ERR_CUDA;
   }
   return TN_OK;
 }
 
 tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t count, void* output,
-                     double* log_scale, void* stream, std::string& err, void* pinned) {
+                     double* log_scale, void* stream, std::string& err) {
   if (!P.dev) {
     err = "plan was built with TN_PLAN_HOST_ONLY (no device workspace)";
     return TN_ERR_INVALID;
@@ -182,31 +187,12 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
   const bool scaling = P.policy.exp_scaling != 0;
   const int32_t T = P.n_leaves, S = (int32_t)P.steps.size();
   const int32_t root = T + S - 1;
-  for (int32_t t = 0; t < T; ++t) {
-    P.leafdesc[t].src = inputs[t];
-    P.leafdesc[t].dst = P.tensors[t].offset;
-  }
-  // descriptors from pageable memory (the copy is staged before the call returns), or from
-  // the caller's pinned buffer
-  const void* desc_src = P.leafdesc.data();
-  const void* rec_src = P.rec_index.data();
-  if (pinned) {
-    char* pb = static_cast<char*>(pinned);
-    std::memcpy(pb, P.leafdesc.data(), sizeof(LeafDesc) * P.leafdesc.size());
-    std::memcpy(pb + sizeof(LeafDesc) * T, P.rec_index.data(), sizeof(int32_t) * T);
-    desc_src = pb;
-    rec_src = pb + sizeof(LeafDesc) * T;
-  }
-  TN_CUDA_TRY(cudaMemcpyAsync(P.dev + P.off_leafdesc, desc_src, sizeof(LeafDesc) * P.leafdesc.size(),
-                              cudaMemcpyHostToDevice, st));
   ScaleRec* recs = scaling ? reinterpret_cast<ScaleRec*>(P.dev + P.off_scale) : nullptr;
   int32_t* recidx = reinterpret_cast<int32_t*>(P.dev + P.off_recidx);
-  if (scaling) TN_CUDA_TRY(cudaMemcpyAsync(recidx, rec_src, sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
   const LeafDesc* descs = reinterpret_cast<const LeafDesc*>(P.dev + P.off_leafdesc);
   double* acc = reinterpret_cast<double*>(P.dev + P.off_acc);
   int64_t* ref = reinterpret_cast<int64_t*>(P.dev + P.off_ref);
   int* errw = reinterpret_cast<int*>(P.dev + P.off_err);
-  TN_CUDA_TRY(cudaMemsetAsync(errw, 0, sizeof(int), st));
   const int64_t npass = (count + P.batch - 1) / P.batch;
   for (int64_t p = 0; p < npass; ++p) {
     const int32_t nb = (int32_t)std::min<int64_t>(P.batch, count - p * P.batch);
@@ -234,7 +220,8 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
       sp.bytes = 2.0 * (cplx ? 8.0 : 4.0) * staged;
       TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(sp.e0), st));
     }
-    launch_stage_leaves(descs, P.leafdesc.data(), T, P.dev, sb, nb, p > 0, cplx, recs, recidx, P.num_sms, st);
+    launch_stage_leaves(descs, P.leafdesc.data(), inputs, T, P.dev, p == 0 ? errw : nullptr, sb, nb, p > 0, cplx, recs,
+                        recidx, P.num_sms, st);
     if (P.prof_on) {
       TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(sp.e1), st));
       P.prof_pending.push_back(sp);
@@ -430,7 +417,7 @@ tn_status tn_plan(const tn_network* net, const tn_path* path, const int32_t* sli
     return TN_ERR_OOM;
   }
   P.dev = static_cast<char*>(mem);
-  const tn_status cs = upload_chain_table(P);
+  const tn_status cs = upload_tables(P);
   if (cs != TN_OK) {
     cudaFree(mem);
     delete h;
@@ -474,7 +461,7 @@ tn_status tn_plan_launches(tn_plan_t plan, int64_t slice_count, int64_t* out) {
   int64_t n = 0;
   for (int64_t p = 0; p < npass; ++p) {
     const int32_t nb = (int32_t)std::min<int64_t>(P.batch, slice_count - p * P.batch);
-    if (T > 0) n += 1;  // stage_leaves_kernel
+    n += (T + kMaxLeafSrcs - 1) / kMaxLeafSrcs;  // stage_leaves_kernel
     for (int32_t t = 0; t < T; ++t)
       if (P.leafdesc[t].tiled && !(p > 0 && !P.tensors[t].batched)) n += 1;
     for (int32_t q = 0; q < (int32_t)P.steps.size(); ++q) {
@@ -654,7 +641,7 @@ tn_status tn_contract_graph(tn_plan_t plan, const void* const* inputs, void* out
   tn_status s = tn_contract(plan, inputs, output, out_log_scale, stream);
   if (s != TN_OK) return s;
   if (P.g_done) {
-    // the previous graph's copy nodes read the pinned buffer: let its last launch finish
+    // let the previous graph's last launch finish
     cudaEventSynchronize(static_cast<cudaEvent_t>(P.g_done));
   } else if (cudaEventCreateWithFlags(reinterpret_cast<cudaEvent_t*>(&P.g_done), cudaEventDisableTiming) !=
              cudaSuccess) {
@@ -663,11 +650,6 @@ tn_status tn_contract_graph(tn_plan_t plan, const void* const* inputs, void* out
   }
   if (P.g_exec) cudaGraphExecDestroy(static_cast<cudaGraphExec_t>(P.g_exec));
   P.g_exec = nullptr;
-  if (!P.g_pinned && cudaMallocHost(&P.g_pinned, (sizeof(LeafDesc) + sizeof(int32_t)) * T + 16) != cudaSuccess) {
-    P.g_pinned = nullptr;
-    set_error("pinned descriptor buffer");
-    return TN_ERR_OOM;
-  }
   cudaStream_t cap = nullptr;
   if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) {
     set_error("graph capture stream");
@@ -677,7 +659,7 @@ tn_status tn_contract_graph(tn_plan_t plan, const void* const* inputs, void* out
   std::string err;
   s = TN_OK;
   if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) s = TN_ERR_CUDA;
-  if (s == TN_OK) s = run_slices(P, inputs, 0, P.n_slices, output, out_log_scale, cap, err, P.g_pinned);
+  if (s == TN_OK) s = run_slices(P, inputs, 0, P.n_slices, output, out_log_scale, cap, err);
   cudaError_t e = cudaStreamEndCapture(cap, &g);
   cudaGraphExec_t ge = nullptr;
   if (s == TN_OK && e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
@@ -762,7 +744,6 @@ tn_status tn_plan_destroy(tn_plan_t plan) {
     cudaEventDestroy(static_cast<cudaEvent_t>(plan->P.g_done));
   }
   if (plan->P.g_exec) cudaGraphExecDestroy(static_cast<cudaGraphExec_t>(plan->P.g_exec));
-  if (plan->P.g_pinned) cudaFreeHost(plan->P.g_pinned);
   if (plan->P.dev) cudaFree(plan->P.dev);
   for (auto& r : plan->P.prof_pending) {
     cudaEventDestroy(static_cast<cudaEvent_t>(r.e0));

@@ -114,8 +114,11 @@ cudaError_t launch_contract_chain(const ChainStep* steps, const ChainTask* tasks
                                   bool maxplus, cudaStream_t st);
 
 // Small leaves: one CTA per leaf. Large leaves (LeafDesc::tiled): the tiled permutation
-// kernel, one launch per leaf; host_descs is the host copy of the table (grid sizes).
-void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, int32_t n_leaves, char* ws,
+// kernel, one launch per leaf; host_descs is the host copy of the table (grid sizes). inputs: the
+// caller's leaves, which the launches carry as parameters. errw != nullptr: set to 0.
+constexpr int32_t kMaxLeafSrcs = 3584;  // leaves of one launch (28 KB of parameters); more take several
+void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, const void* const* inputs,
+                         int32_t n_leaves, char* ws, int* errw,
                          int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
                          const int32_t* rec_index, int num_sms, cudaStream_t st);
 // With a.ksplit > 1 each part of k goes to its own CTAs and a second kernel combines the

@@ -21,12 +21,23 @@ namespace tn {
 // ---------------------------------------------------------------------------------
 // leaf staging (a4)
 
-__global__ void stage_leaves_kernel(const LeafDesc* __restrict__ descs, char* __restrict__ ws,
-                                    int64_t slice_begin, int32_t nb, int32_t only_batched,
-                                    int32_t is_complex, ScaleRec* recs, const int32_t* rec_index,
-                                    int32_t rec_batched_base) {
+template <int N>
+struct LeafSrcs {
+  const void* p[N];
+};
+
+// The leaves' addresses come as a parameter: nothing is copied to the device for a call. (The
+// descriptors, 1.2 KB a leaf, used to be copied with the addresses in them on every call, from
+// pageable memory: 15 us of the 48 us that an amplitude of a 12-qubit circuit took.)
+template <int N>
+__global__ void stage_leaves_kernel(const LeafDesc* __restrict__ descs, const __grid_constant__ LeafSrcs<N> srcs,
+                                    char* __restrict__ ws, int* errw, int64_t slice_begin, int32_t nb,
+                                    int32_t only_batched, int32_t is_complex, ScaleRec* recs,
+                                    const int32_t* rec_index) {
+  if (errw && blockIdx.x == 0 && threadIdx.x == 0) *errw = 0;
   const LeafDesc& d = descs[blockIdx.x];
   if (d.tiled || (only_batched && !d.batched)) return;
+  const void* leaf = srcs.p[blockIdx.x];
   const int32_t copies = d.batched ? nb : 1;
   const int64_t total = d.size * copies;
   int lmax = -127;
@@ -34,21 +45,30 @@ __global__ void stage_leaves_kernel(const LeafDesc* __restrict__ descs, char* __
     const int64_t b = i / d.size;
     int64_t e = i - b * d.size;
     int64_t src = 0;
-    for (int r = d.rank - 1; r >= 0; --r) {
-      const uint32_t x = d.ext[r];
-      src += (e % x) * d.sstride[r];
-      e /= x;
+    if (d.size <= INT32_MAX) {
+      uint32_t e32 = static_cast<uint32_t>(e);
+      for (int r = d.rank - 1; r >= 0; --r) {
+        const uint32_t x = d.ext[r];
+        src += (e32 % x) * d.sstride[r];
+        e32 /= x;
+      }
+    } else {
+      for (int r = d.rank - 1; r >= 0; --r) {
+        const uint32_t x = d.ext[r];
+        src += (e % x) * d.sstride[r];
+        e /= x;
+      }
     }
     const int64_t sid = slice_begin + b;
     for (int q = 0; q < d.n_sl; ++q) src += ((sid / d.sl_div[q]) % d.sl_ext[q]) * d.sl_stride[q];
     const int64_t el = i - b * d.size;
     if (is_complex) {
-      const float2 v = reinterpret_cast<const float2*>(d.src)[src];
+      const float2 v = static_cast<const float2*>(leaf)[src];
       float* dst = reinterpret_cast<float*>(ws + d.dst) + b * cplx_floats(d.split) * d.size;
       store_cplx(dst, d.size, el, v.x, v.y, d.split);
       if (recs) lmax = max(lmax, exp_of(fmaxf(fabsf(v.x), fabsf(v.y))));
     } else {
-      const float v = reinterpret_cast<const float*>(d.src)[src];
+      const float v = static_cast<const float*>(leaf)[src];
       float* dst = reinterpret_cast<float*>(ws + d.dst) + b * d.size;
       dst[el] = v;
       if (recs) lmax = max(lmax, exp_of(fabsf(v)));
@@ -79,7 +99,7 @@ __global__ void stage_leaves_kernel(const LeafDesc* __restrict__ descs, char* __
 // plane, or eight BF16 values per plane in the split form). When the declared innermost
 // position is itself in the output group, loads run along the output group instead.
 template <bool CPLX>
-__global__ void __launch_bounds__(256, 5) stage_leaf_tiled_kernel(const LeafDesc* __restrict__ descs, int32_t leaf,
+__global__ void __launch_bounds__(256, 5) stage_leaf_tiled_kernel(const LeafDesc* __restrict__ descs, int32_t leaf, const void* leaf_src,
                                                                char* __restrict__ ws, int64_t slice_begin,
                                                                ScaleRec* recs, const int32_t* rec_index) {
   constexpr int TT = kTilesInFlight;  // tiles per CTA iteration (loads of all before any store)
@@ -99,7 +119,7 @@ __global__ void __launch_bounds__(256, 5) stage_leaf_tiled_kernel(const LeafDesc
   const int64_t blk0 = int64_t(blockIdx.x) * kTilesPerCta;
   const int64_t blk1 = blk0 + kTilesPerCta < tiles ? blk0 + kTilesPerCta : tiles;
   const int64_t Pi = d.Pi, Po = d.Po;
-  const bool vec = CPLX && d.vec_load && (reinterpret_cast<uintptr_t>(d.src) & 15) == 0;
+  const bool vec = CPLX && d.vec_load && (reinterpret_cast<uintptr_t>(leaf_src) & 15) == 0;
   const int64_t np = CPLX ? cplx_floats(d.split) : 1;
   float* base = reinterpret_cast<float*>(ws + d.dst) + int64_t(b) * np * d.size;
   if (tid < TT) s_built[tid][0] = s_built[tid][1] = -1;
@@ -119,7 +139,7 @@ __global__ void __launch_bounds__(256, 5) stage_leaf_tiled_kernel(const LeafDesc
     }
     // ---- load the tiles: tre[u][ti][to] = element (output-group go0 + to, input-group gi0 + ti)
     if (vec) {
-      const float4* src4 = reinterpret_cast<const float4*>(d.src);
+      const float4* src4 = reinterpret_cast<const float4*>(leaf_src);
       const int ti = 2 * (tid & 15);
       float4 v[TT][2];
 #pragma unroll
@@ -156,12 +176,12 @@ __global__ void __launch_bounds__(256, 5) stage_leaf_tiled_kernel(const LeafDesc
           if (gi < Pi && go < Po) {
             const int64_t so = s_cur[u].src0 + s_isrc[u][ti] + s_osrc[u][to];
             if (CPLX) {
-              const float2 w = __ldg(reinterpret_cast<const float2*>(d.src) + so);
+              const float2 w = __ldg(reinterpret_cast<const float2*>(leaf_src) + so);
               tre[u][ti][to] = w.x;
               tim[u][ti][to] = w.y;
               lmax = max(lmax, exp_of(fmaxf(fabsf(w.x), fabsf(w.y))));
             } else {
-              const float w = __ldg(reinterpret_cast<const float*>(d.src) + so);
+              const float w = __ldg(reinterpret_cast<const float*>(leaf_src) + so);
               tre[u][ti][to] = w;
               lmax = max(lmax, exp_of(fabsf(w)));
             }
@@ -285,7 +305,7 @@ __device__ __forceinline__ void store_tile_row(float* base, int64_t size, int64_
 }
 
 template <int SPLIT>
-__global__ void __launch_bounds__(256, 4) stage_leaf_fast_kernel(const LeafDesc* __restrict__ descs, int32_t leaf,
+__global__ void __launch_bounds__(256, 4) stage_leaf_fast_kernel(const LeafDesc* __restrict__ descs, int32_t leaf, const void* leaf_src,
                                                                  char* __restrict__ ws, int64_t slice_begin,
                                                                  ScaleRec* recs, const int32_t* rec_index) {
   const LeafDesc& d = descs[leaf];
@@ -305,7 +325,7 @@ __global__ void __launch_bounds__(256, 4) stage_leaf_fast_kernel(const LeafDesc*
   }
   __syncthreads();
   const int64_t hsrc = s_hi[0], hdst = s_hi[1];
-  const float4* src4 = reinterpret_cast<const float4*>(d.src);
+  const float4* src4 = reinterpret_cast<const float4*>(leaf_src);
   float* base = reinterpret_cast<float*>(ws + d.dst) + int64_t(b) * cplx_floats(d.split) * d.size;
   const int ti = 2 * (tid & 15), to0 = tid >> 4;
   const int64_t sa = s_isrc[ti] + s_osrc[to0], sb = s_isrc[ti] + s_osrc[to0 + 16];
@@ -346,7 +366,7 @@ __global__ void __launch_bounds__(256, 4) stage_leaf_fast_kernel(const LeafDesc*
 // are 4-aligned. A 3001 x 1500 and a 1999 x 1500 complex leaf 142 -> 34 us (the tiled kernel moved
 // 0.84 TB/s of the ragged tiles, this one 3.5).
 template <bool CPLX, int SPLIT>
-__global__ void __launch_bounds__(256) stage_leaf_linear_kernel(const LeafDesc* __restrict__ descs, int32_t leaf,
+__global__ void __launch_bounds__(256) stage_leaf_linear_kernel(const LeafDesc* __restrict__ descs, int32_t leaf, const void* leaf_src,
                                                                 char* __restrict__ ws, int64_t slice_begin,
                                                                 ScaleRec* recs, const int32_t* rec_index) {
   const LeafDesc& d = descs[leaf];
@@ -354,7 +374,7 @@ __global__ void __launch_bounds__(256) stage_leaf_linear_kernel(const LeafDesc* 
   const int64_t sid = slice_begin + b, size = d.size;
   int64_t off = 0;
   for (int q = 0; q < d.n_sl; ++q) off += ((sid / d.sl_div[q]) % d.sl_ext[q]) * d.sl_stride[q];
-  const float* src = static_cast<const float*>(d.src) + (CPLX ? 2 : 1) * off;
+  const float* src = static_cast<const float*>(leaf_src) + (CPLX ? 2 : 1) * off;
   float* dst = reinterpret_cast<float*>(ws + d.dst) + int64_t(b) * (CPLX ? cplx_floats(SPLIT) : 1) * size;
   const bool vec = (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (size & 3) == 0;
   const int64_t G = 4 * int64_t(gridDim.x) * blockDim.x;
@@ -434,12 +454,27 @@ __global__ void __launch_bounds__(256) stage_leaf_linear_kernel(const LeafDesc* 
   }
 }
 
-void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, int32_t n_leaves, char* ws,
+template <int N>
+static void launch_small_leaves(const LeafDesc* descs, const void* const* inputs, int32_t n, char* ws, int* errw,
+                                int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
+                                const int32_t* rec_index, cudaStream_t st) {
+  LeafSrcs<N> srcs;
+  std::copy(inputs, inputs + n, srcs.p);
+  stage_leaves_kernel<N><<<n, 128, 0, st>>>(descs, srcs, ws, errw, slice_begin, nb, only_batched ? 1 : 0,
+                                            is_complex ? 1 : 0, recs, rec_index);
+}
+
+void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, const void* const* inputs,
+                         int32_t n_leaves, char* ws, int* errw,
                          int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
                          const int32_t* rec_index, int num_sms, cudaStream_t st) {
   if (n_leaves <= 0) return;
-  stage_leaves_kernel<<<n_leaves, 128, 0, st>>>(descs, ws, slice_begin, nb, only_batched ? 1 : 0,
-                                                is_complex ? 1 : 0, recs, rec_index, 0);
+  for (int32_t t = 0; t < n_leaves; t += kMaxLeafSrcs) {
+    const int32_t n = std::min(n_leaves - t, kMaxLeafSrcs);
+    const auto launch = n <= 128 ? launch_small_leaves<128> : n <= 512 ? launch_small_leaves<512> : launch_small_leaves<kMaxLeafSrcs>;
+    launch(descs + t, inputs + t, n, ws, t == 0 ? errw : nullptr, slice_begin, nb, only_batched, is_complex, recs,
+           rec_index + t, st);
+  }
   for (int32_t t = 0; t < n_leaves; ++t) {
     const LeafDesc& h = host_descs[t];
     if (!h.tiled || (only_batched && !h.batched)) continue;
@@ -448,31 +483,31 @@ void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, int3
       dim3 grid(static_cast<unsigned>(std::min<int64_t>(want, int64_t(num_sms) * 8)),
                 static_cast<unsigned>(h.batched ? nb : 1));
       if (!is_complex)
-        stage_leaf_linear_kernel<false, kFmtPlanar><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_linear_kernel<false, kFmtPlanar><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       else if (h.split == kFmtSplit3M)
-        stage_leaf_linear_kernel<true, kFmtSplit3M><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_linear_kernel<true, kFmtSplit3M><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       else if (h.split == kFmtSplit)
-        stage_leaf_linear_kernel<true, kFmtSplit><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_linear_kernel<true, kFmtSplit><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       else
-        stage_leaf_linear_kernel<true, kFmtPlanar><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_linear_kernel<true, kFmtPlanar><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       continue;
     }
     const int64_t tiles = h.Pr * ((h.Po + 31) / 32) * ((h.Pi + 31) / 32);
     const int64_t ctas = (tiles + kTilesPerCta - 1) / kTilesPerCta;
     dim3 grid(static_cast<unsigned>(ctas), static_cast<unsigned>(h.batched ? nb : 1));
-    if (h.fast && (reinterpret_cast<uintptr_t>(h.src) & 15) == 0) {  // 16-byte loads need an aligned source
+    if (h.fast && (reinterpret_cast<uintptr_t>(inputs[t]) & 15) == 0) {  // 16-byte loads need an aligned source
       if (h.split == kFmtSplit3M)
-        stage_leaf_fast_kernel<kFmtSplit3M><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_fast_kernel<kFmtSplit3M><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       else if (h.split == kFmtSplit)
-        stage_leaf_fast_kernel<kFmtSplit><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_fast_kernel<kFmtSplit><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       else
-        stage_leaf_fast_kernel<kFmtPlanar><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+        stage_leaf_fast_kernel<kFmtPlanar><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
       continue;
     }
     if (is_complex)
-      stage_leaf_tiled_kernel<true><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+      stage_leaf_tiled_kernel<true><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
     else
-      stage_leaf_tiled_kernel<false><<<grid, 256, 0, st>>>(descs, t, ws, slice_begin, recs, rec_index);
+      stage_leaf_tiled_kernel<false><<<grid, 256, 0, st>>>(descs, t, inputs[t], ws, slice_begin, recs, rec_index);
   }
 }
 

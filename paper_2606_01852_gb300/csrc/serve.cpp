@@ -383,9 +383,9 @@ struct tn_server_s {
       return nullptr;
     }
     in->P.dev = static_cast<char*>(mem);
-    if (upload_chain_table(in->P) != TN_OK) {
+    if (upload_tables(in->P) != TN_OK) {
       cudaFree(mem);
-      err = "writing a request workspace's step-chain table failed";
+      err = "writing a request workspace's tables failed";
       fatal = true;
       return nullptr;
     }

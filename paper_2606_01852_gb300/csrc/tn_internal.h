@@ -38,7 +38,6 @@ BlockPlan block_plan(const OffsetMap& rows, const OffsetMap& cols);
 // planned order, fixing sliced labels from the slice id, and split complex64 into
 // planar float32 (re plane, im plane).
 struct LeafDesc {
-  const void* src;          // caller's leaf, declared order
   int64_t dst;              // byte offset of the staged tensor in the workspace
   int64_t size;             // elements of one staged copy (sliced labels removed)
   int32_t rank;             // planned rank
@@ -166,15 +165,12 @@ struct Plan {
   std::vector<double> prof_step_ms, prof_last_step_ms;
   uint64_t uid = 0;                 // unique per plan (serve pools key on it)
   // tn_contract_graph: the captured call (graph exec), the pointers and stream it was
-  // captured for, a pinned copy of the leaf descriptors and scale-record indices its copy
-  // nodes read, and an event after its last launch (the pinned copy is rewritten only
-  // after that event)
+  // captured for, and an event after its last launch (the graph is replaced only after it)
   void* g_exec = nullptr;
   std::vector<const void*> g_inputs;
   void* g_out = nullptr;
   double* g_ls = nullptr;
   void* g_stream = nullptr;
-  void* g_pinned = nullptr;
   void* g_done = nullptr;
   // stats
   tn_plan_stats stats{};
@@ -191,18 +187,15 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
 // (no chain is launched, or memory is short) tensors live in path order, and chains run in it.
 void assign_workspace(Plan& P, int64_t batch, bool level_order = true);
 
-// executor
-// pinned: null (descriptors copied from pageable host memory, staged before the call
-// returns), or a pinned buffer of sizeof(LeafDesc) x n_leaves + 4 x n_leaves bytes that the
-// descriptor and record-index copies read from (capturable in a CUDA graph)
+// executor (launches only, capturable in a CUDA graph)
 tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t count,
-                     void* output, double* log_scale, void* stream, std::string& err,
-                     void* pinned = nullptr);
+                     void* output, double* log_scale, void* stream, std::string& err);
 
 void set_error(const std::string& msg);
 tn_status check_device_error(Plan& P);
-// writes the step chains' ChainStep table into the workspace (once P.dev is set)
-tn_status upload_chain_table(Plan& P);
+// writes the tables that calls do not change into the workspace (once P.dev is set): the leaves'
+// descriptors and scale-record indices, the step chains
+tn_status upload_tables(Plan& P);
 
 // true when the tcgen05 kernels are compiled in
 bool tc_supported();
