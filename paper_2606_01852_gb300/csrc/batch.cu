@@ -588,9 +588,6 @@ bool batch_template(const Plan& P, BatchTemplate& T, std::string& err) {
 }  // namespace tn
 
 namespace {
-constexpr int64_t kMaxSmemPerCta = 227 * 1024;  // dynamic shared memory one CTA may take
-constexpr int64_t kSmemPerSm = 224 * 1024;      // what the SM's resident CTAs share (with headroom)
-
 tn_status launch_batch(tn_batch_s* B, const void* packed, double* values, double* logs, cudaStream_t st) {
   const bool warp = B->nets_per_cta > 1;
   const int64_t ctas_needed = warp ? (B->n_nets + B->nets_per_cta - 1) / B->nets_per_cta : B->n_nets;

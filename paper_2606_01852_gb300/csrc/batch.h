@@ -64,6 +64,9 @@ struct BatchTemplate {
 // element by element)
 constexpr int32_t kMaxTabInts = 4096;
 
+constexpr int64_t kMaxSmemPerCta = 227 * 1024;  // dynamic shared memory one CTA may take
+constexpr int64_t kSmemPerSm = 224 * 1024;      // what the SM's resident CTAs share (with headroom)
+
 // Tables of a closed, unsliced network from its plan (workspace assigned for one copy, no
 // tensor-core steps); false with a reason when the batched kernel cannot run it.
 bool batch_template(const Plan& P, BatchTemplate& T, std::string& err);
