@@ -151,7 +151,7 @@ def _load():
         "tn_selftest_bounded_wait": [vp, i32, i64, vp],
         "tn_serve_create": [C.POINTER(tn_serve_config), C.POINTER(vp)],
         "tn_serve_submit": [vp, vp, C.POINTER(vp), C.POINTER(u64)],
-        "tn_serve_submit_batch": [vp, i32, C.POINTER(vp), C.POINTER(C.POINTER(vp)), C.POINTER(u64)],
+        "tn_serve_submit_batch": [vp, i32, C.POINTER(vp), C.POINTER(vp), C.POINTER(u64)],
         "tn_serve_poll": [vp, u64, vp, vp, i32],
         "tn_serve_destroy": [vp],
         "tn_serve_stats_get": [vp, C.POINTER(tn_serve_stats)],
@@ -203,6 +203,20 @@ def _ptr(x):
     if isinstance(x, np.ndarray):
         return x.ctypes.data
     raise TypeError(f"cannot take the address of {type(x)}")
+
+
+_no_bytes = C.c_char * 0
+
+
+def _addresses(xs):
+    """_ptr of each. Writable C-contiguous arrays (a list of them, as a request's leaves are) give
+    their address by the buffer protocol, in half the time of ndarray.ctypes."""
+    if all(type(x) is np.ndarray for x in xs):
+        try:
+            return [C.addressof(_no_bytes.from_buffer(x)) for x in xs]
+        except (TypeError, ValueError, BufferError):
+            pass
+    return [_ptr(x) for x in xs]
 
 
 SEMIRINGS = {"standard": 0, "maxplus": 1}
@@ -305,8 +319,7 @@ class Plan:
     def _inputs(self, inputs):
         if len(inputs) != self.n_leaves:
             raise ValueError(f"expected {self.n_leaves} inputs, got {len(inputs)}")
-        arr = (C.c_void_p * self.n_leaves)(*[_ptr(t) for t in inputs])
-        return arr
+        return (C.c_void_p * self.n_leaves)(*_addresses(inputs))
 
     def contract(self, inputs, output, log_scale=None, stream=None):
         check(lib.tn_contract(self.handle, self._inputs(inputs), _ptr(output), _ptr(log_scale),
@@ -541,7 +554,7 @@ class Server:
         plans = (C.c_void_p * max(1, n))(*[p.handle.value if hasattr(p.handle, "value") else p.handle
                                           for p, _ in requests])
         arrs = [p._inputs(x) for p, x in requests]
-        ins = (C.POINTER(C.c_void_p) * max(1, n))(*[C.cast(a, C.POINTER(C.c_void_p)) for a in arrs])
+        ins = (C.c_void_p * max(1, n))(*[C.addressof(a) for a in arrs])
         tickets = (C.c_uint64 * max(1, n))()
         check(lib.tn_serve_submit_batch(self.handle, n, plans, ins, tickets))
         return list(tickets)[:n]
