@@ -110,9 +110,15 @@ tn_status upload_tables(Plan& P) {
                              cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(P.dev + P.off_recidx, P.rec_index.data(), sizeof(int32_t) * P.n_leaves, cudaMemcpyHostToDevice);
-  auto packed = [](uint32_t e) {
-    const uint32_t sh = (e & (e - 1u)) == 0u ? static_cast<uint32_t>(__builtin_ctz(e)) : 0xffu;
-    return e | (sh << 24);
+  auto places = [](uint32_t* ext, const auto& dims) {
+    bool pow2 = true;
+    for (int d = 0; d < dims.n; ++d) pow2 = pow2 && (dims.ext[d] & (dims.ext[d] - 1u)) == 0u;
+    uint32_t sh = 0;
+    for (int d = dims.n - 1; d >= 0; --d) {
+      const uint32_t e = static_cast<uint32_t>(dims.ext[d]);
+      ext[d] = pow2 ? sh << 24 | (e - 1u) : 0xffu << 24 | e;
+      sh += static_cast<uint32_t>(__builtin_ctz(e));
+    }
   };
   std::vector<ChainStep> table;
   for (const ChainRec& c : P.chains)
@@ -139,14 +145,10 @@ tn_status upload_tables(Plan& P) {
       cs.batched = P.steps[q].batched ? 1 : 0;
       cs.nr = a.rows.n;
       cs.nc = a.cols.n;
-      for (int d = 0; d < a.rows.n; ++d) {
-        cs.ext[d] = packed(a.rows.ext[d]);
-        cs.stride[d] = (int32_t)a.rows.stride[d];
-      }
-      for (int d = 0; d < a.cols.n; ++d) {
-        cs.ext[kMaxDims + d] = packed(a.cols.ext[d]);
-        cs.stride[kMaxDims + d] = (int32_t)a.cols.stride[d];
-      }
+      places(cs.ext, a.rows);
+      places(cs.ext + kMaxDims, a.cols);
+      for (int d = 0; d < a.rows.n; ++d) cs.stride[d] = (int32_t)a.rows.stride[d];
+      for (int d = 0; d < a.cols.n; ++d) cs.stride[kMaxDims + d] = (int32_t)a.cols.stride[d];
       table.push_back(cs);
     }
   if (e == cudaSuccess && !table.empty())

@@ -12,7 +12,11 @@
 // A run of one level needs no barrier and takes as many CTAs as give each lane one output.
 // Measured (GB300): the 702 steps 1036 us in one CTA step after step (1.5 us each) -> 40 us; 27
 // steps of one level (110592 outputs) 284 -> 33 us on one cluster -> ~8 us on 216 CTAs; the
-// 12-qubit amplitude's 57 steps (12 levels) 84 -> 29 us.
+// 12-qubit amplitude's 57 steps (12 levels) 84 -> 26 -> 19.5 us, the last by taking branches out
+// of a lane's chain: a level was ~2000 clocks for 2 terms and 300 more for every 4, nearly all of
+// it branches and dependent loads of the dims, and is ~1500 and 60 now. (Software-pipelined or
+// 16-term groups were slower: spills, and instructions that one CTA runs once cost their fetch.)
+#include <cstddef>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -28,6 +32,8 @@ constexpr int kChainThreads = 512;
 constexpr int kChainWarps = kChainThreads / 32;
 constexpr int kStepWords = sizeof(ChainStep) / 4;
 constexpr int kLaneWords = (kStepWords + 31) / 32;
+static_assert(offsetof(ChainStep, ext) % 16 == 0 && offsetof(ChainStep, stride) % 16 == 0 && kMaxDims % 4 == 0,
+              "four places per 16-byte load");
 static_assert(sizeof(ChainStep) % 16 == 0, "ChainStep copied as 32-bit words, table entries 16-byte aligned");
 
 // every CTA of the cluster (the grid): the stores and atomics before it are visible to the loads after it
@@ -41,24 +47,52 @@ __device__ __forceinline__ void level_barrier() {
   }
 }
 
-// Offset of index i under the merged dims d0 .. d1 - 1 of a step (last fastest): extents packed
-// with their log2 (0xff: not a power of two), strides in elements.
-__device__ __forceinline__ int dims_offset(const ChainStep& S, int d0, int d1, uint32_t i) {
+// Offset of index i under the nd merged dims of one side of a step (last fastest). Extents that are
+// all powers of two come as places (shift << 24 | mask), whose digits do not wait for one
+// another; a place beyond nd is 0, so four are taken without a branch. Else as 0xff << 24 | extent.
+__device__ __forceinline__ int dims_offset(const uint32_t* ext, const int32_t* stride, int nd, uint32_t i) {
+  const uint4 e = *reinterpret_cast<const uint4*>(ext);
   int off = 0;
-  for (int d = d1 - 1; d >= d0; --d) {
-    const uint32_t e = S.ext[d] & 0xffffffu, sh = S.ext[d] >> 24;
-    uint32_t q, r;
-    if (sh != 0xffu) {
-      q = i >> sh;
-      r = i & (e - 1u);
-    } else {
-      q = i / e;
-      r = i - q * e;
+  if (e.x >> 24 != 0xffu) {
+    const int4 st = *reinterpret_cast<const int4*>(stride);
+    off = static_cast<int>((i >> (e.x >> 24)) & e.x & 0xffffffu) * st.x +
+          static_cast<int>((i >> (e.y >> 24)) & e.y & 0xffffffu) * st.y +
+          static_cast<int>((i >> (e.z >> 24)) & e.z & 0xffffffu) * st.z +
+          static_cast<int>((i >> (e.w >> 24)) & e.w & 0xffffffu) * st.w;
+#pragma unroll 1
+    for (int d = 4; d < nd; ++d) off += static_cast<int>((i >> (ext[d] >> 24)) & ext[d] & 0xffffffu) * stride[d];
+  } else {
+#pragma unroll 1
+    for (int d = nd - 1; d >= 0; --d) {
+      const uint32_t x = ext[d] & 0xffffffu, q = i / x;
+      off += static_cast<int>(i - q * x) * stride[d];
+      i = q;
     }
-    off += static_cast<int>(r) * S.stride[d];
-    i = q;
   }
   return off;
+}
+
+// Bring p's sector into L1 (no value is waited for).
+__device__ __forceinline__ void touch(const float* p) {
+  float x;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p) : "memory");
+}
+
+template <bool CPLX, bool MAXPLUS>
+__device__ __forceinline__ void add_term(float xr, float xi, float yr, float yi, float sa, float sb, float& accr,
+                                         float& acci) {
+  const float vr = xr * sa, wr = yr * sb;
+  if (CPLX) {
+    const float vi = xi * sa, wi = yi * sb;
+    accr = fmaf(vr, wr, accr);
+    accr = fmaf(-vi, wi, accr);
+    acci = fmaf(vr, wi, acci);
+    acci = fmaf(vi, wr, acci);
+  } else if (MAXPLUS) {
+    accr = fmaxf(accr, vr + wr);
+  } else {
+    accr = fmaf(vr, wr, accr);
+  }
 }
 
 // One task: outputs first .. first + count - 1 of batch entry b of step S, a lane per output.
@@ -80,42 +114,71 @@ __device__ __forceinline__ void run_task(const ChainStep& S, const ChainTask& t,
   const float* B = S.B + b * S.b_bstride;
   float* C = S.C + b * S.c_bstride;
   const int k = S.k;
+  // rows of a multiple of four terms start 16-byte aligned (tensors do at 256), of two at 8
+  const int bits = k | S.a_plane | S.b_plane | S.a_bstride | S.b_bstride;
+  const int vec = (bits & 3) == 0 ? 4 : k == 2 && (bits & 1) == 0 ? 2 : 1;
   int lmax = -127;
   for (int idx = t.first + lane; idx < t.first + t.count; idx += 32) {
     const int r = S.n_shift >= 0 ? idx >> S.n_shift : idx / S.n, c = idx - r * S.n;
     const float* ar = A + r * k;
     const float* br = B + c * k;
     float accr = kZero, acci = kZero;
-    for (int k0 = 0; k0 < k; k0 += U) {
-      float xr[U], yr[U], xi[CPLX ? U : 1], yi[CPLX ? U : 1];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (k0 + u >= k) break;
-        xr[u] = ar[k0 + u];
-        yr[u] = br[k0 + u];
+    if (vec == 4) {
+      // whole groups of four terms: no branches but the loop's (a lone warp waits for each). Deep
+      // rows: every 32-byte sector is asked for before the first is waited for
+#pragma unroll 1
+      for (int k0 = 8; k0 < k; k0 += 8) {
+        touch(ar + k0);
+        touch(br + k0);
         if (CPLX) {
-          xi[u] = ar[S.a_plane + k0 + u];
-          yi[u] = br[S.b_plane + k0 + u];
+          touch(ar + S.a_plane + k0);
+          touch(br + S.b_plane + k0);
         }
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (k0 + u >= k) break;
-        const float vr = xr[u] * sa, wr = yr[u] * sb;
+#pragma unroll 1
+      for (int k0 = 0; k0 < k; k0 += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(ar + k0), y = *reinterpret_cast<const float4*>(br + k0);
+        float4 u{}, w{};
         if (CPLX) {
-          const float vi = xi[u] * sa, wi = yi[u] * sb;
-          accr = fmaf(vr, wr, accr);
-          accr = fmaf(-vi, wi, accr);
-          acci = fmaf(vr, wi, acci);
-          acci = fmaf(vi, wr, acci);
-        } else if (MAXPLUS) {
-          accr = fmaxf(accr, vr + wr);
-        } else {
-          accr = fmaf(vr, wr, accr);
+          u = *reinterpret_cast<const float4*>(ar + S.a_plane + k0);
+          w = *reinterpret_cast<const float4*>(br + S.b_plane + k0);
+        }
+        add_term<CPLX, MAXPLUS>(x.x, u.x, y.x, w.x, sa, sb, accr, acci);
+        add_term<CPLX, MAXPLUS>(x.y, u.y, y.y, w.y, sa, sb, accr, acci);
+        add_term<CPLX, MAXPLUS>(x.z, u.z, y.z, w.z, sa, sb, accr, acci);
+        add_term<CPLX, MAXPLUS>(x.w, u.w, y.w, w.w, sa, sb, accr, acci);
+      }
+    } else if (vec == 2) {
+      const float2 x = *reinterpret_cast<const float2*>(ar), y = *reinterpret_cast<const float2*>(br);
+      float2 u{}, w{};
+      if (CPLX) {
+        u = *reinterpret_cast<const float2*>(ar + S.a_plane);
+        w = *reinterpret_cast<const float2*>(br + S.b_plane);
+      }
+      add_term<CPLX, MAXPLUS>(x.x, u.x, y.x, w.x, sa, sb, accr, acci);
+      add_term<CPLX, MAXPLUS>(x.y, u.y, y.y, w.y, sa, sb, accr, acci);
+    } else {
+#pragma unroll 1
+      for (int k0 = 0; k0 < k; k0 += U) {
+        float xr[U], yr[U], xi[U], yi[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (k0 + u >= k) break;
+          xr[u] = ar[k0 + u];
+          yr[u] = br[k0 + u];
+          if (CPLX) {
+            xi[u] = ar[S.a_plane + k0 + u];
+            yi[u] = br[S.b_plane + k0 + u];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (k0 + u >= k) break;
+          add_term<CPLX, MAXPLUS>(xr[u], xi[u], yr[u], yi[u], sa, sb, accr, acci);
         }
       }
     }
-    const int off = dims_offset(S, 0, S.nr, r) + dims_offset(S, kMaxDims, kMaxDims + S.nc, c);
+    const int off = dims_offset(S.ext, S.stride, S.nr, r) + dims_offset(S.ext + kMaxDims, S.stride + kMaxDims, S.nc, c);
     if (CPLX) store_cplx(C, S.c_plane, off, accr, acci, S.c_split);
     else C[off] = accr;
     if (S.recs) lmax = max(lmax, exp_of(CPLX ? fmaxf(fabsf(accr), fabsf(acci)) : fabsf(accr)));

@@ -90,8 +90,9 @@ struct ChainStep {
   int32_t a_bstride, b_bstride, c_bstride;
   int32_t rec_a, rec_b, rec_c;
   int32_t c_split, batched, nr, nc;
-  // merged dims: rows at 0 .. nr - 1, columns at kMaxDims .. kMaxDims + nc - 1; the extent in the
-  // low 24 bits, its log2 (0xff: not a power of two) above
+  // merged dims: rows at 0 .. nr - 1, columns at kMaxDims .. kMaxDims + nc - 1; a side's extents
+  // all powers of two: extent - 1 in the low 24 bits, the log2 of the later dims' extents above;
+  // else the extents, with 0xff above
   uint32_t ext[2 * kMaxDims];
   int32_t stride[2 * kMaxDims];
 };
