@@ -196,6 +196,14 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
   int64_t* ref = reinterpret_cast<int64_t*>(P.dev + P.off_ref);
   int* errw = reinterpret_cast<int*>(P.dev + P.off_err);
   const int64_t npass = (count + P.batch - 1) / P.batch;
+  // gate runs read leaves where they are and write the output as they go: not where these overlap
+  bool runs = !P.gate_runs.empty();
+  for (const GateRun& g : P.gate_runs) {
+    if (g.leaf < 0) continue;
+    const uintptr_t x = reinterpret_cast<uintptr_t>(inputs[g.leaf]), y = reinterpret_cast<uintptr_t>(output);
+    const uintptr_t nx = static_cast<uintptr_t>(P.tensors[g.leaf].size * elem_bytes(P)), ny = static_cast<uintptr_t>(P.out_elems * (cplx ? 16 : 8));
+    runs = runs && (x + nx <= y || y + ny <= x);
+  }
   for (int64_t p = 0; p < npass; ++p) {
     const int32_t nb = (int32_t)std::min<int64_t>(P.batch, count - p * P.batch);
     const int64_t sb = begin + p * P.batch;
@@ -216,14 +224,14 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
       double staged = 0.0;
       for (int32_t t = 0; t < T; ++t) {
         const TensorRec& R = P.tensors[t];
-        if (p > 0 && !R.batched) continue;
+        if ((p > 0 && !R.batched) || (runs && P.leafdesc[t].direct)) continue;
         staged += double(R.size) * (R.batched ? nb : 1);
       }
       sp.bytes = 2.0 * (cplx ? 8.0 : 4.0) * staged;
       TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(sp.e0), st));
     }
-    launch_stage_leaves(descs, P.leafdesc.data(), inputs, T, P.dev, p == 0 ? errw : nullptr, sb, nb, p > 0, cplx, recs,
-                        recidx, P.num_sms, st);
+    launch_stage_leaves(descs, P.leafdesc.data(), inputs, T, P.dev, p == 0 ? errw : nullptr, sb, nb, p > 0, runs,
+                        cplx, recs, recidx, P.num_sms, st);
     if (P.prof_on) {
       TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(sp.e1), st));
       P.prof_pending.push_back(sp);
@@ -262,6 +270,37 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
         continue;
       }
       if (!sr.batched && p > 0) continue;  // slice-invariant: computed once, kept
+      if (runs && sr.gates >= 0) {
+        const GateRun& g = P.gate_runs[sr.gates];
+        if (s != g.first) continue;
+        Plan::ProfRec pr{};
+        if (P.prof_on) {
+          pr.e0 = take_event(P);
+          pr.e1 = take_event(P);
+          pr.cls = TN_CLASS_STREAM;
+          pr.step = s;
+          for (int32_t q = s; q < s + g.n; ++q)
+            pr.flops += (cplx ? 8.0 : 2.0) * double(P.steps[q].m) * double(P.steps[q].n) * double(P.steps[q].k);
+          pr.bytes = double(elem_bytes(P)) * double(sr.m * sr.k) * (g.root ? 3.0 : 2.0);
+          TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(pr.e0), st));
+        }
+        GateArgs ga = g.args;
+        ga.in = g.leaf >= 0 ? static_cast<const float*>(inputs[g.leaf])
+                            : reinterpret_cast<const float*>(P.dev + P.tensors[sr.a].offset);
+        ga.out = g.root ? output : P.dev + P.tensors[P.steps[s + g.n - 1].out].offset;
+        ga.log_scale = g.root ? log_scale : nullptr;
+        for (int32_t q = 0; q < g.n; ++q) {
+          const StepArgs a = step_args(P, P.steps[s + q]);
+          ga.gate[q].b = a.B;
+          ga.gate[q].b_plane = static_cast<int32_t>(a.b_plane);
+        }
+        TN_CUDA_TRY(launch_gate_run(ga, cplx, st));
+        if (P.prof_on) {
+          TN_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(pr.e1), st));
+          P.prof_pending.push_back(pr);
+        }
+        continue;
+      }
       StepArgs a = step_args(P, sr);
       const int32_t nbs = sr.batched ? nb : 1;
       Plan::ProfRec pr{};
@@ -293,6 +332,7 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
         P.prof_pending.push_back(pr);
       }
     }
+    if (runs && P.gate_runs.back().root) continue;
     const TensorRec& R = P.tensors[root];
     const int64_t np = cplx ? 2 : 1;
     launch_accumulate_root(reinterpret_cast<const float*>(P.dev + R.offset), R.size,
@@ -465,7 +505,7 @@ tn_status tn_plan_launches(tn_plan_t plan, int64_t slice_count, int64_t* out) {
     const int32_t nb = (int32_t)std::min<int64_t>(P.batch, slice_count - p * P.batch);
     n += (T + kMaxLeafSrcs - 1) / kMaxLeafSrcs;  // stage_leaves_kernel
     for (int32_t t = 0; t < T; ++t)
-      if (P.leafdesc[t].tiled && !(p > 0 && !P.tensors[t].batched)) n += 1;
+      if (P.leafdesc[t].tiled && !P.leafdesc[t].direct && !(p > 0 && !P.tensors[t].batched)) n += 1;
     for (int32_t q = 0; q < (int32_t)P.steps.size(); ++q) {
       const StepRec& st = P.steps[q];
       if (st.chain >= 0) {  // one launch per step chain, at its first step
@@ -474,6 +514,10 @@ tn_status tn_plan_launches(tn_plan_t plan, int64_t slice_count, int64_t* out) {
         continue;
       }
       if (!st.batched && p > 0) continue;
+      if (st.gates >= 0) {  // one launch per gate run, at its first step
+        n += q == P.gate_runs[st.gates].first;
+        continue;
+      }
       const int32_t nbs = st.batched ? nb : 1;
       if (st.cls == TN_CLASS_TC)
         n += tc_launches(st.m, st.n, st.k, nbs, form, pairs && !st.single_sm, P.policy.exp_scaling != 0);
@@ -481,7 +525,7 @@ tn_status tn_plan_launches(tn_plan_t plan, int64_t slice_count, int64_t* out) {
       else if (st.cls == TN_CLASS_SIMT) n += st.ksplit > 1 ? 2 : 1;
       else n += 1;
     }
-    n += 1;  // the slice sum (or the output widening)
+    if (P.gate_runs.empty() || !P.gate_runs.back().root) n += 1;  // the slice sum (or the output widening)
   }
   *out = n;
   return TN_OK;

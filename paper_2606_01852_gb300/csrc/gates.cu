@@ -1,0 +1,189 @@
+// Gate runs (sm_103a): consecutive big x small steps on one tensor, in one pass over it.
+//
+// A step whose small operand is square (k = n = 2, 4, 8, 16: gates on a state) only replaces bits
+// of the big tensor's index: the k bits give way to as many n bits, every other bit moves to its
+// place in the output. So a run of them is one fixed permutation of index bits ("wires") with a
+// small matrix applied to some wires on the way. A tile holds all values of the wires that the
+// run's gates act on and of the lowest few bits of the run's input and of its output, so that
+// both are moved in whole sectors; a CTA loads it into shared memory, applies the gates in place
+// and stores it. A leaf is read where the caller has it, instead of being staged in the planned
+// order first; a run that ends the path writes the caller's FP64 output itself.
+//
+// Every output is summed over k in order with the FMAs of contract_stream_kernel: the same bits as
+// a pass per step.
+//
+// What bounds it: HBM, as a pass per step does, but with one read and one write for the run. Four
+// two-qubit gates on 26 qubits with a leaf's staging and the output's widening moved 6.5 GB in 1.21 ms;
+// the run moves 1.6 GB in @@ ms. A tile of 2^13 complex elements takes 64 KB, three CTAs an SM,
+// so that some load or store while others compute. Shared-memory addresses are linear over the wires
+// (XOR): a tile wire at local bit p >= 5 also flips one of the five bank bits, chosen so that the lanes of
+// the load, of every gate and of the store meet different banks.
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+#include "kernels.h"
+#include "widen.cuh"
+
+namespace tn {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kThreadBits = 8;
+constexpr int kIters = 1 << (kGateTileBits - kThreadBits);
+
+template <bool CPLX, int KB>
+__device__ __forceinline__ void gate_pass(float* re, float* im, const GateStep& g, const float2* mat, int t) {
+  constexpr int K = 1 << KB;
+  const int groups = 1 << (t - KB), tid = threadIdx.x;
+  int base0 = 0;
+#pragma unroll
+  for (int b = 0; b < kThreadBits; ++b) base0 ^= (tid >> b) & 1 ? g.rest[b] : 0;
+  int ko[K];
+#pragma unroll
+  for (int q = 0; q < K; ++q) {
+    ko[q] = 0;
+#pragma unroll
+    for (int b = 0; b < KB; ++b) ko[q] ^= (q >> b) & 1 ? g.wire[b] : 0;
+  }
+  float2 m[KB <= 2 ? K * K : 1];
+  if constexpr (KB <= 2) {
+#pragma unroll
+    for (int i = 0; i < K * K; ++i) m[i] = mat[i];
+  }
+  for (int i = tid; i < groups; i += kThreads) {
+    int base = base0;
+#pragma unroll
+    for (int b = kThreadBits; b < kGateTileBits; ++b) base ^= (i >> b) & 1 ? g.rest[b] : 0;
+    float xr[K], xi[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      xr[q] = re[base ^ ko[q]];
+      if (CPLX) xi[q] = im[base ^ ko[q]];
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      float cr = 0.f, ci = 0.f;
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        const float2 y = KB <= 2 ? m[KB <= 2 ? j * K + q : 0] : mat[j * K + q];
+        if (CPLX) {
+          cr = fmaf(xr[q], y.x, cr);
+          cr = fmaf(-xi[q], y.y, cr);
+          ci = fmaf(xr[q], y.y, ci);
+          ci = fmaf(xi[q], y.x, ci);
+        } else {
+          cr = fmaf(xr[q], y.x, cr);
+        }
+      }
+      re[base ^ ko[j]] = cr;
+      if (CPLX) im[base ^ ko[j]] = ci;
+    }
+  }
+}
+
+template <bool CPLX>
+__global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_constant__ GateArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int64_t s_in[kIters], s_out[kIters];
+  __shared__ int s_ia[kIters], s_oa[kIters];
+  const int t = a.t, tid = threadIdx.x;
+  float *re = sm, *im = sm + (1 << t);
+  float2* mats = reinterpret_cast<float2*>(sm + (CPLX ? 2 : 1) * (1 << t));
+  for (int g = 0, o = 0; g < a.n_gates; ++g) {
+    const int kk = 1 << (2 * a.gate[g].bits);
+    for (int i = tid; i < kk; i += kThreads)
+      mats[o + i] = make_float2(__ldg(a.gate[g].b + i), CPLX ? __ldg(a.gate[g].b + a.gate[g].b_plane + i) : 0.f);
+    o += kk;
+  }
+  if (tid < kIters) {
+    int64_t si = 0, so = 0;
+    int ai = 0, ao = 0;
+#pragma unroll
+    for (int b = kThreadBits; b < kGateTileBits; ++b)
+      if ((tid >> (b - kThreadBits)) & 1) {
+        si += a.in_off[b];
+        so += a.out_off[b];
+        ai ^= a.in_addr[b];
+        ao ^= a.out_addr[b];
+      }
+    s_in[tid] = si;
+    s_out[tid] = so;
+    s_ia[tid] = ai;
+    s_oa[tid] = ao;
+  }
+  int64_t in = 0, out = 0;
+  int ia = 0, oa = 0;
+  for (int b = 0; b < a.outer; ++b)
+    if ((blockIdx.x >> b) & 1) {
+      in += a.in_outer[b];
+      out += a.out_outer[b];
+    }
+#pragma unroll
+  for (int b = 0; b < kThreadBits; ++b)
+    if ((tid >> b) & 1) {
+      in += a.in_off[b];
+      out += a.out_off[b];
+      ia ^= a.in_addr[b];
+      oa ^= a.out_addr[b];
+    }
+  __syncthreads();
+  const int iters = 1 << (t - kThreadBits);
+  constexpr int U = 8;  // elements in flight per thread
+  for (int i0 = 0; i0 < iters; i0 += U) {
+    float2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u >= iters) break;
+      const int64_t e = in + s_in[i0 + u];
+      if (!CPLX) v[u].x = __ldg(a.in + e);
+      else if (a.interleaved) v[u] = __ldg(reinterpret_cast<const float2*>(a.in) + e);
+      else v[u] = make_float2(__ldg(a.in + e), __ldg(a.in + a.in_plane + e));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u >= iters) break;
+      re[ia ^ s_ia[i0 + u]] = v[u].x;
+      if (CPLX) im[ia ^ s_ia[i0 + u]] = v[u].y;
+    }
+  }
+  __syncthreads();
+  for (int g = 0, o = 0; g < a.n_gates; ++g) {
+    const GateStep& s = a.gate[g];
+    if (s.bits == 1) gate_pass<CPLX, 1>(re, im, s, mats + o, t);
+    else if (s.bits == 2) gate_pass<CPLX, 2>(re, im, s, mats + o, t);
+    else if (s.bits == 3) gate_pass<CPLX, 3>(re, im, s, mats + o, t);
+    else gate_pass<CPLX, 4>(re, im, s, mats + o, t);
+    o += 1 << (2 * s.bits);
+    __syncthreads();
+  }
+#pragma unroll 4
+  for (int i = 0; i < iters; ++i) {
+    const int64_t e = out + s_out[i];
+    const float x = re[oa ^ s_oa[i]], y = CPLX ? im[oa ^ s_oa[i]] : 0.f;
+    if (!a.widen) {
+      float* o = static_cast<float*>(a.out);
+      o[e] = x;
+      if (CPLX) o[a.out_plane + e] = y;
+    } else if (CPLX) {
+      static_cast<double2*>(a.out)[e] = make_double2(f64_of_f32(x), f64_of_f32(y));
+    } else {
+      static_cast<double*>(a.out)[e] = f64_of_f32(x);
+    }
+  }
+  if (a.log_scale && blockIdx.x == 0 && tid == 0) *a.log_scale = 0.0;
+}
+
+}  // namespace
+
+cudaError_t launch_gate_run(const GateArgs& a, bool cplx, cudaStream_t st) {
+  auto kernel = cplx ? gate_run_kernel<true> : gate_run_kernel<false>;
+  int bytes = (cplx ? 8 : 4) << a.t;
+  for (int g = 0; g < a.n_gates; ++g) bytes += 8 << (2 * a.gate[g].bits);
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  kernel<<<1u << a.outer, kThreads, bytes, st>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace tn

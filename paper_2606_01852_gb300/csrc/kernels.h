@@ -116,12 +116,15 @@ cudaError_t launch_contract_chain(const ChainStep* steps, const ChainTask* tasks
 
 // Small leaves: one CTA per leaf. Large leaves (LeafDesc::tiled): the tiled permutation
 // kernel, one launch per leaf; host_descs is the host copy of the table (grid sizes). inputs: the
-// caller's leaves, which the launches carry as parameters. errw != nullptr: set to 0.
+// caller's leaves, which the launches carry as parameters. errw != nullptr: set to 0. skip_direct: leaves
+// that a gate run reads where they are (LeafDesc::direct) are left out.
 constexpr int32_t kMaxLeafSrcs = 3584;  // leaves of one launch (28 KB of parameters); more take several
 void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, const void* const* inputs,
                          int32_t n_leaves, char* ws, int* errw,
-                         int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
-                         const int32_t* rec_index, int num_sms, cudaStream_t st);
+                         int64_t slice_begin, int32_t nb, bool only_batched, bool skip_direct, bool is_complex,
+                         ScaleRec* recs, const int32_t* rec_index, int num_sms, cudaStream_t st);
+// A run of gates (GateRun::args with the call's pointers filled in).
+cudaError_t launch_gate_run(const GateArgs& a, bool cplx, cudaStream_t st);
 // With a.ksplit > 1 each part of k goes to its own CTAs and a second kernel combines the
 // partial tiles (in part order) and writes C.
 void launch_contract_simt(const StepArgs& a, int32_t nb, bool cplx, int num_sms, cudaStream_t st);

@@ -14,6 +14,7 @@
 #include "mbarrier.cuh"
 #include "scale.cuh"
 #include "split_bf16.cuh"
+#include "widen.cuh"
 #include "staging.cuh"
 
 namespace tn {
@@ -32,11 +33,11 @@ struct LeafSrcs {
 template <int N>
 __global__ void stage_leaves_kernel(const LeafDesc* __restrict__ descs, const __grid_constant__ LeafSrcs<N> srcs,
                                     char* __restrict__ ws, int* errw, int64_t slice_begin, int32_t nb,
-                                    int32_t only_batched, int32_t is_complex, ScaleRec* recs,
+                                    int32_t only_batched, int32_t skip_direct, int32_t is_complex, ScaleRec* recs,
                                     const int32_t* rec_index) {
   if (errw && blockIdx.x == 0 && threadIdx.x == 0) *errw = 0;
   const LeafDesc& d = descs[blockIdx.x];
-  if (d.tiled || (only_batched && !d.batched)) return;
+  if (d.tiled || (only_batched && !d.batched) || (skip_direct && d.direct)) return;
   const void* leaf = srcs.p[blockIdx.x];
   const int32_t copies = d.batched ? nb : 1;
   const int64_t total = d.size * copies;
@@ -456,28 +457,28 @@ __global__ void __launch_bounds__(256) stage_leaf_linear_kernel(const LeafDesc* 
 
 template <int N>
 static void launch_small_leaves(const LeafDesc* descs, const void* const* inputs, int32_t n, char* ws, int* errw,
-                                int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
-                                const int32_t* rec_index, cudaStream_t st) {
+                                int64_t slice_begin, int32_t nb, bool only_batched, bool skip_direct, bool is_complex,
+                                ScaleRec* recs, const int32_t* rec_index, cudaStream_t st) {
   LeafSrcs<N> srcs;
   std::copy(inputs, inputs + n, srcs.p);
   stage_leaves_kernel<N><<<n, 128, 0, st>>>(descs, srcs, ws, errw, slice_begin, nb, only_batched ? 1 : 0,
-                                            is_complex ? 1 : 0, recs, rec_index);
+                                            skip_direct ? 1 : 0, is_complex ? 1 : 0, recs, rec_index);
 }
 
 void launch_stage_leaves(const LeafDesc* descs, const LeafDesc* host_descs, const void* const* inputs,
                          int32_t n_leaves, char* ws, int* errw,
-                         int64_t slice_begin, int32_t nb, bool only_batched, bool is_complex, ScaleRec* recs,
-                         const int32_t* rec_index, int num_sms, cudaStream_t st) {
+                         int64_t slice_begin, int32_t nb, bool only_batched, bool skip_direct, bool is_complex,
+                         ScaleRec* recs, const int32_t* rec_index, int num_sms, cudaStream_t st) {
   if (n_leaves <= 0) return;
   for (int32_t t = 0; t < n_leaves; t += kMaxLeafSrcs) {
     const int32_t n = std::min(n_leaves - t, kMaxLeafSrcs);
     const auto launch = n <= 128 ? launch_small_leaves<128> : n <= 512 ? launch_small_leaves<512> : launch_small_leaves<kMaxLeafSrcs>;
-    launch(descs + t, inputs + t, n, ws, t == 0 ? errw : nullptr, slice_begin, nb, only_batched, is_complex, recs,
-           rec_index + t, st);
+    launch(descs + t, inputs + t, n, ws, t == 0 ? errw : nullptr, slice_begin, nb, only_batched, skip_direct, is_complex,
+           recs, rec_index + t, st);
   }
   for (int32_t t = 0; t < n_leaves; ++t) {
     const LeafDesc& h = host_descs[t];
-    if (!h.tiled || (only_batched && !h.batched)) continue;
+    if (!h.tiled || (only_batched && !h.batched) || (skip_direct && h.direct)) continue;
     if (h.linear) {
       const int64_t want = (h.size + 2047) / 2048;  // two rounds a thread, up to eight CTAs per SM
       dim3 grid(static_cast<unsigned>(std::min<int64_t>(want, int64_t(num_sms) * 8)),
@@ -832,30 +833,6 @@ void launch_contract_stream(const StepArgs& a, int32_t nb, bool cplx, int num_sm
 // last pass writes sum + comp straight to the caller's output (and the log scale), so a
 // one-pass call never touches the accumulator, and a one-slice call (widen_root_kernel)
 // does no FP64 arithmetic at all.
-
-// The binary64 value of a binary32 value, exactly, from the two formats' fields with integer
-// operations only (this GPU's FP64 pipe is narrow; a conversion per output element would
-// bound a one-slice open output): the exponent is rebiased from 127 to 1023 and the 23
-// fraction bits move to the top of the 52; subnormal inputs are normalised; zeros and
-// infinities keep their sign, and a NaN its sign and payload with the quiet bit set (as an
-// IEEE 754 conversion returns a signaling NaN quieted).
-__device__ __forceinline__ double f64_of_f32(float f) {
-  const uint32_t u = __float_as_uint(f);
-  const uint64_t sign = static_cast<uint64_t>(u >> 31) << 63;
-  const uint32_t e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-  uint64_t bits;
-  if (e == 0xffu) {
-    bits = sign | (uint64_t(0x7ff) << 52) | (uint64_t(m) << 29) | (m ? uint64_t(1) << 51 : 0);
-  } else if (e != 0u) {
-    bits = sign | (uint64_t(e + (1023 - 127)) << 52) | (uint64_t(m) << 29);
-  } else if (m == 0u) {
-    bits = sign;
-  } else {  // m * 2^-149 with the leading one at bit p: exponent p - 149, fraction below it
-    const int p = 31 - __clz(static_cast<int>(m));
-    bits = sign | (uint64_t(p - 149 + 1023) << 52) | ((uint64_t(m) << (52 - p)) & ((uint64_t(1) << 52) - 1));
-  }
-  return __longlong_as_double(static_cast<long long>(bits));
-}
 
 __global__ void accumulate_root_kernel(const float* __restrict__ root, int64_t size, int32_t nb,
                                        int64_t bstride, int64_t plane, int32_t cplx, double* acc,

@@ -119,6 +119,7 @@ bool build_offset_map(const std::vector<int32_t>& side, const std::vector<int32_
 
 }  // namespace
 
+static void find_gate_runs(Plan& P);
 tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* sliced,
                      int32_t n_sliced, const tn_dtype_policy& pol, Plan& P, std::string& err) {
   std::ostringstream es;
@@ -579,7 +580,244 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
   S0.flops = fl_fixed + fl_batched * double(P.n_slices);
   S0.bytes = by_fixed + by_batched * double(P.n_slices);
   P.out_elems = P.tensors[root].size;
+  find_gate_runs(P);
   return TN_OK;
+}
+
+// ---- gate runs (gates.cu) ----------------------------------------------------------------------
+
+static int log2_of(int64_t x) {
+  return x > 0 && (x & (x - 1)) == 0 ? __builtin_ctzll(static_cast<unsigned long long>(x)) : -1;
+}
+
+// The offset of each bit of a mixed-radix index (last dim fastest), low bit first; false unless the
+// extents are powers of two with `bits` bits in all.
+template <typename E, typename St>
+static bool index_bits(const E* ext, const St* stride, int n, int bits, std::vector<int64_t>& w) {
+  w.clear();
+  for (int d = n - 1; d >= 0; --d) {
+    const int l = log2_of(ext[d]);
+    if (l < 0) return false;
+    for (int i = 0; i < l; ++i) w.push_back(int64_t(stride[d]) << i);
+  }
+  return (int)w.size() == bits;
+}
+
+namespace {
+
+// The wires of a run under construction: a wire is a bit of the first step's big operand.
+struct Wires {
+  int bits = 0;                         // of the big tensor's index
+  std::vector<int64_t> in;              // offset of each wire in the run's input
+  std::vector<int> at;                  // its bit in the current tensor's index
+  std::vector<std::vector<int>> gates;  // wires of each gate, lowest index bit first
+};
+
+// Apply step st to the wires; false if it is not a gate on them.
+bool add_gate(const StepRec& st, Wires& W) {
+  const int kb = log2_of(st.k), mb = log2_of(st.m);
+  if (st.cls != TN_CLASS_STREAM || st.n != st.k || kb < 1 || kb > 4 || mb < 0 || kb + mb != W.bits) return false;
+  std::vector<int64_t> row, col;
+  if (!index_bits(st.rows.ext, st.rows.stride, st.rows.n, mb, row) ||
+      !index_bits(st.cols.ext, st.cols.stride, st.cols.n, kb, col))
+    return false;
+  std::vector<int> at(W.bits), gate(kb);
+  std::vector<bool> seen(W.bits, false);
+  for (int w = 0; w < W.bits; ++w) {
+    const int b = W.at[w], to = log2_of(b < kb ? col[b] : row[b - kb]);
+    if (to < 0 || to >= W.bits || seen[to]) return false;
+    seen[to] = true;
+    at[w] = to;
+    if (b < kb) gate[b] = w;
+  }
+  W.at = at;
+  W.gates.push_back(gate);
+  return true;
+}
+
+// The n wires with the smallest offsets.
+std::vector<int> lowest(const std::vector<int64_t>& off, int n) {
+  std::vector<int> o(off.size());
+  std::iota(o.begin(), o.end(), 0);
+  std::sort(o.begin(), o.end(), [&](int x, int y) { return off[x] < off[y]; });
+  o.resize(std::min<size_t>(o.size(), n));
+  return o;
+}
+
+// The tile of a run: the gates' wires, and the lowest of the input and of the output so that whole
+// 64-byte (FP32 planes: 32-byte) pieces move; then up to 128-byte pieces while the tile stays at 2^12
+// elements and there are 512 tiles. Empty if it does not fit.
+std::vector<int> tile_wires(const Wires& W, const std::vector<int64_t>& out, bool pairs, bool widen, bool cplx) {
+  std::vector<bool> has(W.bits, false);
+  int n = 0;
+  auto add = [&](int w) {
+    n += !has[w];
+    has[w] = true;
+  };
+  for (const auto& g : W.gates)
+    for (int w : g) add(w);
+  const int lo_in = 3, lo_out = widen && cplx ? 2 : 3, hi_in = pairs ? 4 : 5, hi_out = widen ? (cplx ? 3 : 4) : 5;
+  for (int w : lowest(W.in, lo_in)) add(w);
+  for (int w : lowest(out, lo_out)) add(w);
+  if (n > kGateTileBits) return {};
+  auto grow = [&](const std::vector<int>& ws) {
+    for (int w : ws)
+      if (n < 12 && W.bits - n > 9) add(w);
+  };
+  grow(lowest(out, hi_out));
+  grow(lowest(W.in, hi_in));
+  for (int w : lowest(W.in, W.bits))
+    if (n < 8) add(w);
+  std::vector<int> tile;
+  for (int w = 0; w < W.bits; ++w)
+    if (has[w]) tile.push_back(w);
+  return tile;
+}
+
+// Fill the run's tables for the tile; out: offset of each wire in the run's output.
+bool gate_args(const Wires& W, const std::vector<int64_t>& out, const std::vector<int>& tile, GateArgs& a) {
+  const int t = (int)tile.size();
+  if (t < 8 || t > kGateTileBits || W.bits - t > kGateMaxOuter) return false;
+  std::vector<bool> in_tile(W.bits, false);
+  for (int w : tile) in_tile[w] = true;
+  auto by = [&](const std::vector<int64_t>& off) {
+    std::vector<int> o = tile;
+    std::sort(o.begin(), o.end(), [&](int x, int y) { return off[x] < off[y]; });
+    return o;
+  };
+  const std::vector<int> by_in = by(W.in), by_out = by(out);
+  // bank bit of every tile wire: the input's lowest wires differ, the output's lowest do, and the
+  // five are spread evenly
+  std::vector<int> bank(W.bits, -1);
+  int count[5] = {0, 0, 0, 0, 0};
+  auto give = [&](int w, const std::vector<int>& apart_from) {
+    if (bank[w] >= 0) return;
+    int best = -1;
+    bool best_used = true;
+    for (int r = 0; r < 5; ++r) {
+      bool used = false;
+      for (int x : apart_from) used = used || bank[x] == r;
+      if (best < 0 || std::make_pair(used, count[r]) < std::make_pair(best_used, count[best])) best = r, best_used = used;
+    }
+    bank[w] = best;
+    ++count[best];
+  };
+  const std::vector<int> low_in(by_in.begin(), by_in.begin() + 4), low_out(by_out.begin(), by_out.begin() + 3);
+  for (int w : low_in) give(w, low_in);
+  for (int w : low_out) give(w, low_out);
+  for (const auto& g : W.gates)
+    for (int w : g) give(w, g);
+  for (int w : by_in) give(w, {});
+  // local bits: the first wire of each bank takes that bit, the others the bits from 5 on
+  std::vector<int> addr(W.bits, 0);
+  bool taken[5] = {false, false, false, false, false};
+  int next = 5;
+  for (int w : by_in) {
+    if (!taken[bank[w]]) {
+      taken[bank[w]] = true;
+      addr[w] = 1 << bank[w];
+    } else {
+      addr[w] = 1 << next++ | 1 << bank[w];
+    }
+  }
+  if (next != t) return false;  // a bank without a wire (t >= 8 wires spread over five: does not happen)
+  // an order of tile wires that starts with `first`, whose five lane wires differ in bank as far as can be
+  auto lanes_first = [&](std::vector<int> order, int first) {
+    bool used[5] = {false, false, false, false, false};
+    for (int i = 0; i < first; ++i) used[bank[order[i]]] = true;
+    for (int i = first; i < 5 && i < (int)order.size(); ++i) {
+      int pick = i;
+      for (int j = i; j < (int)order.size(); ++j)
+        if (!used[bank[order[j]]]) {
+          pick = j;
+          break;
+        }
+      std::rotate(order.begin() + i, order.begin() + pick, order.begin() + pick + 1);
+      used[bank[order[i]]] = true;
+    }
+    return order;
+  };
+  const std::vector<int> lo = lanes_first(by_in, 4), so = lanes_first(by_out, 3);
+  a.t = t;
+  a.outer = W.bits - t;
+  a.n_gates = (int)W.gates.size();
+  for (int i = 0; i < t; ++i) {
+    a.in_off[i] = W.in[lo[i]];
+    a.in_addr[i] = addr[lo[i]];
+    a.out_off[i] = out[so[i]];
+    a.out_addr[i] = addr[so[i]];
+  }
+  int o = 0;
+  for (int w : lowest(out, W.bits))  // neighbouring tiles write neighbouring pieces
+    if (!in_tile[w]) {
+      a.in_outer[o] = W.in[w];
+      a.out_outer[o++] = out[w];
+    }
+  for (int g = 0; g < a.n_gates; ++g) {
+    GateStep& s = a.gate[g];
+    s.bits = (int)W.gates[g].size();
+    std::vector<int> rest;
+    for (int w : by_in)
+      if (std::find(W.gates[g].begin(), W.gates[g].end(), w) == W.gates[g].end()) rest.push_back(w);
+    rest = lanes_first(rest, 0);
+    for (int i = 0; i < s.bits; ++i) s.wire[i] = addr[W.gates[g][i]];
+    for (size_t i = 0; i < rest.size(); ++i) s.rest[i] = addr[rest[i]];
+  }
+  return true;
+}
+
+}  // namespace
+
+// Gate runs of a plan of one slice without scaling: from each step that can start one, as many
+// steps as a tile holds. A run of one step pays only if it also saves the leaf's staging or the
+// output's widening.
+static void find_gate_runs(Plan& P) {
+  const int32_t T = P.n_leaves, S = (int32_t)P.steps.size();
+  if (P.n_slices != 1 || P.policy.exp_scaling || P.policy.semiring == TN_SEMIRING_MAXPLUS) return;
+  for (int32_t s = 0; s < S;) {
+    const StepRec& st = P.steps[s];
+    Wires W;
+    W.bits = log2_of(st.m * st.k);
+    GateRun best, run;
+    if (st.cls == TN_CLASS_STREAM && W.bits >= 8) {
+      run.first = s;
+      if (st.a < T) {
+        const LeafDesc& d = P.leafdesc[st.a];
+        if (!d.split && d.n_sl == 0 && index_bits(d.ext, d.sstride, d.rank, W.bits, W.in)) run.leaf = st.a;
+      }
+      if (run.leaf < 0) {
+        W.in.clear();
+        for (int i = 0; i < W.bits; ++i) W.in.push_back(int64_t(1) << i);
+      }
+      W.at.resize(W.bits);
+      std::iota(W.at.begin(), W.at.end(), 0);
+      for (int32_t q = s; q < S && q - s < kGateMaxRun; ++q) {
+        const StepRec& sq = P.steps[q];
+        if ((q > s && sq.a != T + q - 1) || sq.b - T >= s || P.tensors[sq.b].split || !add_gate(sq, W)) break;
+        if (P.tensors[sq.out].split) break;
+        const bool widen = q == S - 1;
+        std::vector<int64_t> out(W.bits);
+        for (int w = 0; w < W.bits; ++w) out[w] = int64_t(1) << W.at[w];
+        const std::vector<int> tile = tile_wires(W, out, run.leaf >= 0 && P.is_complex, widen, P.is_complex);
+        run.args = GateArgs{};
+        if (tile.empty() || !gate_args(W, out, tile, run.args)) continue;
+        run.n = q - s + 1;
+        run.root = widen;
+        best = run;
+      }
+    }
+    if (best.n >= 2 || (best.n == 1 && (best.leaf >= 0 || best.root))) {
+      best.args.interleaved = best.leaf >= 0 && P.is_complex;
+      best.args.widen = best.root;
+      best.args.in_plane = best.args.out_plane = int64_t(1) << W.bits;
+      if (best.leaf >= 0) P.leafdesc[best.leaf].direct = 1;
+      for (int32_t q = s; q < s + best.n; ++q) P.steps[q].gates = (int32_t)P.gate_runs.size();
+      P.gate_runs.push_back(best);
+      s += best.n;
+    } else {
+      ++s;
+    }
+  }
 }
 
 // Step chains: maximal runs (two or more) of consecutive tiny CUDA-core steps, each run one

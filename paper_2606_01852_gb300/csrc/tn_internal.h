@@ -55,6 +55,7 @@ struct LeafDesc {
   // order outside the output group, slowest first) and the rest (rpos[0..nr-1]). A CTA
   // moves one 32 x 32 tile (output-group index x input-group index) through shared
   // memory, reading along the input group and writing along the output group.
+  int32_t direct;                  // read by a gate run where the caller has it
   int32_t tiled;                   // staged by the tiled kernel (else by the per-leaf kernel)
   int32_t no, ni, nr;
   int32_t load_o;                  // the declared order's innermost position is in the
@@ -99,6 +100,38 @@ struct StepRec {
   int32_t ksplit = 1;  // SIMT steps too few tiles to fill the GPU: k cut in this many parts
   bool single_sm = false;  // tensor-core step kept on one SM per tile (tn_plan_autotune's choice)
   int32_t chain = -1;      // index of the step chain (a run of tiny CUDA-core steps) it is in
+  int32_t gates = -1;      // index of the gate run it is in
+};
+
+// A gate run: steps first .. first + n - 1, each on the output of the one before, in one pass over
+// the tensor (gates.cu). Offsets are in elements, addresses in floats of a tile's plane; the
+// tile's bits are listed in the order in which threads take them (thread bits first).
+constexpr int kGateTileBits = 13;   // complex elements of a tile, log2: 64 KB of shared memory
+constexpr int kGateMaxRun = 8;
+constexpr int kGateMaxOuter = 30;
+struct GateStep {
+  const float* b;                   // n x k
+  int32_t b_plane, bits;            // bits: log2 k = log2 n
+  int32_t wire[4];                  // addresses of the k (and n) index bits, lowest first
+  int32_t rest[kGateTileBits];      // addresses of the tile's other bits
+};
+struct GateArgs {
+  const float* in;
+  void* out;
+  double* log_scale;                // set to 0 (may be null)
+  int64_t in_plane, out_plane;
+  int32_t t, outer, n_gates;        // log2 of a tile's elements and of the tiles
+  int32_t interleaved, widen;       // in: (re, im) pairs; out: the FP64 output
+  int64_t in_outer[kGateMaxOuter], out_outer[kGateMaxOuter];
+  int64_t in_off[kGateTileBits], out_off[kGateTileBits];
+  int32_t in_addr[kGateTileBits], out_addr[kGateTileBits];
+  GateStep gate[kGateMaxRun];
+};
+struct GateRun {
+  int32_t first = 0, n = 0;
+  int32_t leaf = -1;                // the leaf it reads where the caller has it
+  bool root = false;                // it writes the output
+  GateArgs args{};
 };
 
 // A step chain: steps first .. first + n - 1 run in one launch (entries table .. table + n - 1
@@ -138,6 +171,7 @@ struct Plan {
   int64_t n_rec_unbatched = 0, n_rec_total = 0;
   int64_t off_leafdesc = 0;         // LeafDesc table
   int64_t off_chain = 0;            // ChainStep table of the step chains
+  std::vector<GateRun> gate_runs;
   std::vector<ChainRec> chains;
   std::vector<int32_t> chain_tasks;   // ChainTask, four ints each
   std::vector<int32_t> chain_levels;
