@@ -16,8 +16,8 @@
 // two-qubit gates on 26 qubits with a leaf's staging and the output's widening moved 6.5 GB in 1.21 ms;
 // the run moves 1.6 GB in @@ ms. A tile of 2^13 complex elements takes 64 KB, three CTAs an SM,
 // so that some load or store while others compute. Shared-memory addresses are linear over the wires
-// (XOR): a tile wire at local bit p >= 5 also flips one of the five bank bits, chosen so that the lanes of
-// the load, of every gate and of the store meet different banks.
+// (XOR): a tile wire above the bank bits also flips one of them, chosen so that the lanes of the
+// load, of every gate and of the store meet different banks.
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -32,10 +32,23 @@ constexpr int kThreads = 256;
 constexpr int kThreadBits = 8;
 constexpr int kIters = 1 << (kGateTileBits - kThreadBits);
 
+// An element of the tile at a byte address (real: y is not stored).
+template <bool CPLX>
+__device__ __forceinline__ float2 get(const char* tile, int at) {
+  if constexpr (CPLX) return *reinterpret_cast<const float2*>(tile + at);
+  else return make_float2(*reinterpret_cast<const float*>(tile + at), 0.f);
+}
+template <bool CPLX>
+__device__ __forceinline__ void put(char* tile, int at, float2 v) {
+  if constexpr (CPLX) *reinterpret_cast<float2*>(tile + at) = v;
+  else *reinterpret_cast<float*>(tile + at) = v.x;
+}
+
 template <bool CPLX, int KB>
-__device__ __forceinline__ void gate_pass(float* re, float* im, const GateStep& g, const float2* mat, int t) {
+__device__ __forceinline__ void gate_pass(char* tile, const GateStep& g, const float2* mat, int t) {
   constexpr int K = 1 << KB;
   const int groups = 1 << (t - KB), tid = threadIdx.x;
+  if (tid >= groups) return;
   int base0 = 0;
 #pragma unroll
   for (int b = 0; b < kThreadBits; ++b) base0 ^= (tid >> b) & 1 ? g.rest[b] : 0;
@@ -51,45 +64,45 @@ __device__ __forceinline__ void gate_pass(float* re, float* im, const GateStep& 
 #pragma unroll
     for (int i = 0; i < K * K; ++i) m[i] = mat[i];
   }
-  for (int i = tid; i < groups; i += kThreads) {
-    int base = base0;
+  const int rounds = groups > kThreads ? groups / kThreads : 1;
+  for (int i = 0; i < rounds; ++i) {
+    int base = base0;  // i is every thread's
 #pragma unroll
-    for (int b = kThreadBits; b < kGateTileBits; ++b) base ^= (i >> b) & 1 ? g.rest[b] : 0;
-    float xr[K], xi[K];
+    for (int b = kThreadBits; b < kGateTileBits; ++b) base ^= (i >> (b - kThreadBits)) & 1 ? g.rest[b] : 0;
+    float2 x[K];
 #pragma unroll
-    for (int q = 0; q < K; ++q) {
-      xr[q] = re[base ^ ko[q]];
-      if (CPLX) xi[q] = im[base ^ ko[q]];
-    }
+    for (int q = 0; q < K; ++q) x[q] = get<CPLX>(tile, base ^ ko[q]);
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-      float cr = 0.f, ci = 0.f;
+      float2 c = make_float2(0.f, 0.f);
 #pragma unroll
       for (int q = 0; q < K; ++q) {
         const float2 y = KB <= 2 ? m[KB <= 2 ? j * K + q : 0] : mat[j * K + q];
+        c.x = fmaf(x[q].x, y.x, c.x);
         if (CPLX) {
-          cr = fmaf(xr[q], y.x, cr);
-          cr = fmaf(-xi[q], y.y, cr);
-          ci = fmaf(xr[q], y.y, ci);
-          ci = fmaf(xi[q], y.x, ci);
-        } else {
-          cr = fmaf(xr[q], y.x, cr);
+          c.x = fmaf(-x[q].y, y.y, c.x);
+          c.y = fmaf(x[q].x, y.y, c.y);
+          c.y = fmaf(x[q].y, y.x, c.y);
         }
       }
-      re[base ^ ko[j]] = cr;
-      if (CPLX) im[base ^ ko[j]] = ci;
+      put<CPLX>(tile, base ^ ko[j], c);
     }
   }
 }
 
+// What a round of the load or of the store adds to a thread's offset (bytes) and address.
+struct __align__(16) Round {
+  int64_t off;
+  int at;
+};
+
 template <bool CPLX>
 __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_constant__ GateArgs a) {
-  extern __shared__ __align__(16) float sm[];
-  __shared__ int64_t s_in[kIters], s_out[kIters];
-  __shared__ int s_ia[kIters], s_oa[kIters];
+  extern __shared__ __align__(16) char tile[];
+  __shared__ Round s_in[kIters], s_out[kIters];
   const int t = a.t, tid = threadIdx.x;
-  float *re = sm, *im = sm + (1 << t);
-  float2* mats = reinterpret_cast<float2*>(sm + (CPLX ? 2 : 1) * (1 << t));
+  const int in_bytes = CPLX && a.interleaved ? 8 : 4, out_bytes = (a.widen ? 8 : 4) * (CPLX && a.widen ? 2 : 1);
+  float2* mats = reinterpret_cast<float2*>(tile + ((CPLX ? 8 : 4) << t));
   for (int g = 0, o = 0; g < a.n_gates; ++g) {
     const int kk = 1 << (2 * a.gate[g].bits);
     for (int i = tid; i < kk; i += kThreads)
@@ -97,20 +110,17 @@ __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_cons
     o += kk;
   }
   if (tid < kIters) {
-    int64_t si = 0, so = 0;
-    int ai = 0, ao = 0;
+    Round ri{0, 0}, ro{0, 0};
 #pragma unroll
     for (int b = kThreadBits; b < kGateTileBits; ++b)
       if ((tid >> (b - kThreadBits)) & 1) {
-        si += a.in_off[b];
-        so += a.out_off[b];
-        ai ^= a.in_addr[b];
-        ao ^= a.out_addr[b];
+        ri.off += a.in_off[b] * in_bytes;
+        ro.off += a.out_off[b] * out_bytes;
+        ri.at ^= a.in_addr[b];
+        ro.at ^= a.out_addr[b];
       }
-    s_in[tid] = si;
-    s_out[tid] = so;
-    s_ia[tid] = ai;
-    s_oa[tid] = ao;
+    s_in[tid] = ri;
+    s_out[tid] = ro;
   }
   int64_t in = 0, out = 0;
   int ia = 0, oa = 0;
@@ -127,6 +137,8 @@ __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_cons
       ia ^= a.in_addr[b];
       oa ^= a.out_addr[b];
     }
+  const char* src = reinterpret_cast<const char*>(a.in) + in * in_bytes;
+  char* dst = static_cast<char*>(a.out) + out * out_bytes;
   __syncthreads();
   const int iters = 1 << (t - kThreadBits);
   constexpr int U = 8;  // elements in flight per thread
@@ -135,40 +147,39 @@ __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_cons
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (i0 + u >= iters) break;
-      const int64_t e = in + s_in[i0 + u];
-      if (!CPLX) v[u].x = __ldg(a.in + e);
-      else if (a.interleaved) v[u] = __ldg(reinterpret_cast<const float2*>(a.in) + e);
-      else v[u] = make_float2(__ldg(a.in + e), __ldg(a.in + a.in_plane + e));
+      const char* p = src + s_in[i0 + u].off;
+      if (!CPLX) v[u].x = __ldg(reinterpret_cast<const float*>(p));
+      else if (a.interleaved) v[u] = __ldg(reinterpret_cast<const float2*>(p));
+      else v[u] = make_float2(__ldg(reinterpret_cast<const float*>(p)), __ldg(reinterpret_cast<const float*>(p) + a.in_plane));
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (i0 + u >= iters) break;
-      re[ia ^ s_ia[i0 + u]] = v[u].x;
-      if (CPLX) im[ia ^ s_ia[i0 + u]] = v[u].y;
+      put<CPLX>(tile, ia ^ s_in[i0 + u].at, v[u]);
     }
   }
   __syncthreads();
   for (int g = 0, o = 0; g < a.n_gates; ++g) {
     const GateStep& s = a.gate[g];
-    if (s.bits == 1) gate_pass<CPLX, 1>(re, im, s, mats + o, t);
-    else if (s.bits == 2) gate_pass<CPLX, 2>(re, im, s, mats + o, t);
-    else if (s.bits == 3) gate_pass<CPLX, 3>(re, im, s, mats + o, t);
-    else gate_pass<CPLX, 4>(re, im, s, mats + o, t);
+    if (s.bits == 1) gate_pass<CPLX, 1>(tile, s, mats + o, t);
+    else if (s.bits == 2) gate_pass<CPLX, 2>(tile, s, mats + o, t);
+    else if (s.bits == 3) gate_pass<CPLX, 3>(tile, s, mats + o, t);
+    else gate_pass<CPLX, 4>(tile, s, mats + o, t);
     o += 1 << (2 * s.bits);
     __syncthreads();
   }
 #pragma unroll 4
   for (int i = 0; i < iters; ++i) {
-    const int64_t e = out + s_out[i];
-    const float x = re[oa ^ s_oa[i]], y = CPLX ? im[oa ^ s_oa[i]] : 0.f;
+    const Round r = s_out[i];
+    const float2 v = get<CPLX>(tile, oa ^ r.at);
+    char* p = dst + r.off;
     if (!a.widen) {
-      float* o = static_cast<float*>(a.out);
-      o[e] = x;
-      if (CPLX) o[a.out_plane + e] = y;
+      *reinterpret_cast<float*>(p) = v.x;
+      if (CPLX) reinterpret_cast<float*>(p)[a.out_plane] = v.y;
     } else if (CPLX) {
-      static_cast<double2*>(a.out)[e] = make_double2(f64_of_f32(x), f64_of_f32(y));
+      *reinterpret_cast<double2*>(p) = make_double2(f64_of_f32(v.x), f64_of_f32(v.y));
     } else {
-      static_cast<double*>(a.out)[e] = f64_of_f32(x);
+      *reinterpret_cast<double*>(p) = f64_of_f32(v.x);
     }
   }
   if (a.log_scale && blockIdx.x == 0 && tid == 0) *a.log_scale = 0.0;

@@ -674,8 +674,10 @@ std::vector<int> tile_wires(const Wires& W, const std::vector<int64_t>& out, boo
   return tile;
 }
 
-// Fill the run's tables for the tile; out: offset of each wire in the run's output.
-bool gate_args(const Wires& W, const std::vector<int64_t>& out, const std::vector<int>& tile, GateArgs& a) {
+// Fill the run's tables for the tile; out: offset of each wire in the run's output. Addresses are
+// in bytes, an element (re, im) or a real one: 16 or 32 to a pass of the banks.
+bool gate_args(const Wires& W, const std::vector<int64_t>& out, const std::vector<int>& tile, bool cplx, GateArgs& a) {
+  const int nbank = cplx ? 4 : 5, esh = cplx ? 3 : 2;
   const int t = (int)tile.size();
   if (t < 8 || t > kGateTileBits || W.bits - t > kGateMaxOuter) return false;
   std::vector<bool> in_tile(W.bits, false);
@@ -686,15 +688,15 @@ bool gate_args(const Wires& W, const std::vector<int64_t>& out, const std::vecto
     return o;
   };
   const std::vector<int> by_in = by(W.in), by_out = by(out);
-  // bank bit of every tile wire: the input's lowest wires differ, the output's lowest do, and the
-  // five are spread evenly
+  // bank bit of every tile wire: the input's lowest wires differ, the output's lowest do, and all
+  // are spread evenly
   std::vector<int> bank(W.bits, -1);
   int count[5] = {0, 0, 0, 0, 0};
   auto give = [&](int w, const std::vector<int>& apart_from) {
     if (bank[w] >= 0) return;
     int best = -1;
     bool best_used = true;
-    for (int r = 0; r < 5; ++r) {
+    for (int r = 0; r < nbank; ++r) {
       bool used = false;
       for (int x : apart_from) used = used || bank[x] == r;
       if (best < 0 || std::make_pair(used, count[r]) < std::make_pair(best_used, count[best])) best = r, best_used = used;
@@ -708,24 +710,24 @@ bool gate_args(const Wires& W, const std::vector<int64_t>& out, const std::vecto
   for (const auto& g : W.gates)
     for (int w : g) give(w, g);
   for (int w : by_in) give(w, {});
-  // local bits: the first wire of each bank takes that bit, the others the bits from 5 on
+  // local bits: the first wire of each bank takes that bit, the others the bits above the banks'
   std::vector<int> addr(W.bits, 0);
   bool taken[5] = {false, false, false, false, false};
-  int next = 5;
+  int next = nbank;
   for (int w : by_in) {
     if (!taken[bank[w]]) {
       taken[bank[w]] = true;
-      addr[w] = 1 << bank[w];
+      addr[w] = 1 << bank[w] << esh;
     } else {
-      addr[w] = 1 << next++ | 1 << bank[w];
+      addr[w] = (1 << next++ | 1 << bank[w]) << esh;
     }
   }
   if (next != t) return false;  // a bank without a wire (t >= 8 wires spread over five: does not happen)
-  // an order of tile wires that starts with `first`, whose five lane wires differ in bank as far as can be
+  // an order of tile wires that starts with `first`, whose lane wires differ in bank as far as can be
   auto lanes_first = [&](std::vector<int> order, int first) {
     bool used[5] = {false, false, false, false, false};
     for (int i = 0; i < first; ++i) used[bank[order[i]]] = true;
-    for (int i = first; i < 5 && i < (int)order.size(); ++i) {
+    for (int i = first; i < nbank && i < (int)order.size(); ++i) {
       int pick = i;
       for (int j = i; j < (int)order.size(); ++j)
         if (!used[bank[order[j]]]) {
@@ -800,7 +802,7 @@ static void find_gate_runs(Plan& P) {
         for (int w = 0; w < W.bits; ++w) out[w] = int64_t(1) << W.at[w];
         const std::vector<int> tile = tile_wires(W, out, run.leaf >= 0 && P.is_complex, widen, P.is_complex);
         run.args = GateArgs{};
-        if (tile.empty() || !gate_args(W, out, tile, run.args)) continue;
+        if (tile.empty() || !gate_args(W, out, tile, P.is_complex, run.args)) continue;
         run.n = q - s + 1;
         run.root = widen;
         best = run;

@@ -104,7 +104,7 @@ struct StepRec {
 };
 
 // A gate run: steps first .. first + n - 1, each on the output of the one before, in one pass over
-// the tensor (gates.cu). Offsets are in elements, addresses in floats of a tile's plane; the
+// the tensor (gates.cu). Offsets are in elements, addresses in bytes of the tile; the
 // tile's bits are listed in the order in which threads take them (thread bits first).
 constexpr int kGateTileBits = 13;   // complex elements of a tile, log2: 64 KB of shared memory
 constexpr int kGateMaxRun = 8;

@@ -15,6 +15,9 @@ namespace tn {
 // IEEE 754 conversion returns a signaling NaN quieted).
 __device__ __forceinline__ double f64_of_f32(float f) {
   const uint32_t u = __float_as_uint(f);
+  if ((u & 0x7f800000u) - 0x00800000u < 0x7f000000u)  // a normal number, by its two halves
+    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                            static_cast<int>(u << 29));
   const uint64_t sign = static_cast<uint64_t>(u >> 31) << 63;
   const uint32_t e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
   uint64_t bits;
