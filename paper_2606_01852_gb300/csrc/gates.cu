@@ -12,12 +12,17 @@
 // Every output is summed over k in order with the FMAs of contract_stream_kernel: the same bits as
 // a pass per step.
 //
-// What bounds it: HBM, as a pass per step does, but with one read and one write for the run. Four
-// two-qubit gates on 26 qubits with a leaf's staging and the output's widening moved 6.5 GB in 1.21 ms;
-// the run moves 1.6 GB in @@ ms. A tile of 2^13 complex elements takes 64 KB, three CTAs an SM,
-// so that some load or store while others compute. Shared-memory addresses are linear over the wires
-// (XOR): a tile wire above the bank bits also flips one of them, chosen so that the lanes of the
-// load, of every gate and of the store meet different banks.
+// What bounds it: the instructions of a tile's way through shared memory, no longer HBM. Four
+// two-qubit gates on 26 qubits with the leaf's staging and the output's widening moved 6.5 GB in 1.21
+// ms; the run moves 1.6 GB in 0.43 ms, with 5 instructions of 8 issue slots used: per element 64
+// FMAs, 20 others for the gates, 35 for load, FP64 and store. A tile of 2^12 complex elements
+// takes 32 KB, six CTAs of 128 threads an SM: some load or store while others compute, and a thread's
+// share of 32 elements pays for its setup (256 threads: 0.54 -> 0.48 ms). Sixteen loads in flight
+// and rounds in Gray code order: 0.48 -> 0.43. Measured and slower: tiles dealt to resident CTAs
+// (their phases align: 0.84), two elements to a packed FMA (0.52-0.98: registers).
+// Shared-memory addresses are linear over the wires (XOR): a tile wire above the bank bits also
+// flips one of them, chosen so that the lanes of the load, of every gate and of the store meet
+// different banks.
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -28,8 +33,8 @@
 namespace tn {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kThreadBits = 8;
+constexpr int kThreads = 128;
+constexpr int kThreadBits = 7;
 constexpr int kIters = 1 << (kGateTileBits - kThreadBits);
 
 // An element of the tile at a byte address (real: y is not stored).
@@ -65,10 +70,10 @@ __device__ __forceinline__ void gate_pass(char* tile, const GateStep& g, const f
     for (int i = 0; i < K * K; ++i) m[i] = mat[i];
   }
   const int rounds = groups > kThreads ? groups / kThreads : 1;
+  int base = base0;
+  // the rounds in Gray code order: one bit of the group's index changes from each to the next
   for (int i = 0; i < rounds; ++i) {
-    int base = base0;  // i is every thread's
-#pragma unroll
-    for (int b = kThreadBits; b < kGateTileBits; ++b) base ^= (i >> (b - kThreadBits)) & 1 ? g.rest[b] : 0;
+    if (i > 0) base ^= g.rest[kThreadBits + __ffs(i) - 1];
     float2 x[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) x[q] = get<CPLX>(tile, base ^ ko[q]);
@@ -97,9 +102,10 @@ struct __align__(16) Round {
 };
 
 template <bool CPLX>
-__global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_constant__ GateArgs a) {
+__global__ void __launch_bounds__(kThreads, 6) gate_run_kernel(const __grid_constant__ GateArgs a) {
   extern __shared__ __align__(16) char tile[];
   __shared__ Round s_in[kIters], s_out[kIters];
+  __shared__ int64_t s_tile[2];
   const int t = a.t, tid = threadIdx.x;
   const int in_bytes = CPLX && a.interleaved ? 8 : 4, out_bytes = (a.widen ? 8 : 4) * (CPLX && a.widen ? 2 : 1);
   float2* mats = reinterpret_cast<float2*>(tile + ((CPLX ? 8 : 4) << t));
@@ -122,13 +128,24 @@ __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_cons
     s_in[tid] = ri;
     s_out[tid] = ro;
   }
+  if (tid < 32) {  // the tile's offsets
+    int64_t x = 0, y = 0;
+    if (tid < a.outer && (blockIdx.x >> tid) & 1) {
+      x = a.in_outer[tid];
+      y = a.out_outer[tid];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+    if (tid == 0) {
+      s_tile[0] = x;
+      s_tile[1] = y;
+    }
+  }
   int64_t in = 0, out = 0;
   int ia = 0, oa = 0;
-  for (int b = 0; b < a.outer; ++b)
-    if ((blockIdx.x >> b) & 1) {
-      in += a.in_outer[b];
-      out += a.out_outer[b];
-    }
 #pragma unroll
   for (int b = 0; b < kThreadBits; ++b)
     if ((tid >> b) & 1) {
@@ -137,26 +154,28 @@ __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_cons
       ia ^= a.in_addr[b];
       oa ^= a.out_addr[b];
     }
-  const char* src = reinterpret_cast<const char*>(a.in) + in * in_bytes;
-  char* dst = static_cast<char*>(a.out) + out * out_bytes;
   __syncthreads();
+  const char* src = reinterpret_cast<const char*>(a.in) + (in + s_tile[0]) * in_bytes;
+  char* dst = static_cast<char*>(a.out) + (out + s_tile[1]) * out_bytes;
   const int iters = 1 << (t - kThreadBits);
-  constexpr int U = 8;  // elements in flight per thread
-  for (int i0 = 0; i0 < iters; i0 += U) {
-    float2 v[U];
+  auto fetch = [&](int i) {
+    const char* p = src + s_in[i].off;
+    if (!CPLX) return make_float2(__ldg(reinterpret_cast<const float*>(p)), 0.f);
+    if (a.interleaved) return __ldg(reinterpret_cast<const float2*>(p));
+    return make_float2(__ldg(reinterpret_cast<const float*>(p)), __ldg(reinterpret_cast<const float*>(p) + a.in_plane));
+  };
+  constexpr int U = 16;  // elements in flight per thread
+  if (iters >= U) {
+    for (int i0 = 0; i0 < iters; i0 += U) {
+      float2 v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (i0 + u >= iters) break;
-      const char* p = src + s_in[i0 + u].off;
-      if (!CPLX) v[u].x = __ldg(reinterpret_cast<const float*>(p));
-      else if (a.interleaved) v[u] = __ldg(reinterpret_cast<const float2*>(p));
-      else v[u] = make_float2(__ldg(reinterpret_cast<const float*>(p)), __ldg(reinterpret_cast<const float*>(p) + a.in_plane));
-    }
+      for (int u = 0; u < U; ++u) v[u] = fetch(i0 + u);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (i0 + u >= iters) break;
-      put<CPLX>(tile, ia ^ s_in[i0 + u].at, v[u]);
+      for (int u = 0; u < U; ++u) put<CPLX>(tile, ia ^ s_in[i0 + u].at, v[u]);
     }
+  } else {
+#pragma unroll 2
+    for (int i = 0; i < iters; ++i) put<CPLX>(tile, ia ^ s_in[i].at, fetch(i));
   }
   __syncthreads();
   for (int g = 0, o = 0; g < a.n_gates; ++g) {
@@ -177,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 3) gate_run_kernel(const __grid_cons
       *reinterpret_cast<float*>(p) = v.x;
       if (CPLX) reinterpret_cast<float*>(p)[a.out_plane] = v.y;
     } else if (CPLX) {
-      *reinterpret_cast<double2*>(p) = make_double2(f64_of_f32(v.x), f64_of_f32(v.y));
+      *reinterpret_cast<double2*>(p) = f64_of_f32(v);
     } else {
       *reinterpret_cast<double*>(p) = f64_of_f32(v.x);
     }

@@ -908,7 +908,7 @@ __global__ void __launch_bounds__(256) widen_root_kernel(const float* __restrict
     for (int i = 0; i < 2; ++i) {
       const int64_t e = e0 + i * G;
       if (e >= size) continue;
-      if (cplx) reinterpret_cast<double2*>(out)[e] = make_double2(f64_of_f32(re[i]), f64_of_f32(im[i]));
+      if (cplx) reinterpret_cast<double2*>(out)[e] = f64_of_f32(make_float2(re[i], im[i]));
       else reinterpret_cast<double*>(out)[e] = f64_of_f32(re[i]);
     }
   }

@@ -15,9 +15,6 @@ namespace tn {
 // IEEE 754 conversion returns a signaling NaN quieted).
 __device__ __forceinline__ double f64_of_f32(float f) {
   const uint32_t u = __float_as_uint(f);
-  if ((u & 0x7f800000u) - 0x00800000u < 0x7f000000u)  // a normal number, by its two halves
-    return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
-                            static_cast<int>(u << 29));
   const uint64_t sign = static_cast<uint64_t>(u >> 31) << 63;
   const uint32_t e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
   uint64_t bits;
@@ -32,6 +29,20 @@ __device__ __forceinline__ double f64_of_f32(float f) {
     bits = sign | (uint64_t(p - 149 + 1023) << 52) | ((uint64_t(m) << (52 - p)) & ((uint64_t(1) << 52) - 1));
   }
   return __longlong_as_double(static_cast<long long>(bits));
+}
+
+// The same for a normal number, by its two halves.
+__device__ __forceinline__ bool is_normal(float f) {
+  return (__float_as_uint(f) & 0x7f800000u) - 0x00800000u < 0x7f000000u;
+}
+__device__ __forceinline__ double f64_of_normal(float f) {
+  const uint32_t u = __float_as_uint(f);
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                          static_cast<int>(u << 29));
+}
+__device__ __forceinline__ double2 f64_of_f32(float2 v) {
+  if (is_normal(v.x) && is_normal(v.y)) return make_double2(f64_of_normal(v.x), f64_of_normal(v.y));
+  return make_double2(f64_of_f32(v.x), f64_of_f32(v.y));
 }
 
 }  // namespace tn
