@@ -24,6 +24,7 @@
 #include "kernels.h"
 #include "scale.cuh"
 #include "split_bf16.cuh"
+#include "pdl.cuh"
 
 namespace tn {
 namespace {
@@ -201,6 +202,8 @@ __global__ void __launch_bounds__(kChainThreads) contract_chain_kernel(const Cha
                                                                        int32_t skip_unbatched) {
   static_assert(!(CPLX && MAXPLUS), "the max-plus semiring is real");
   __shared__ ChainStep s_step[kChainWarps];
+  pdl_wait();
+  pdl_next();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w = blockIdx.x * kChainWarps + warp, W = gridDim.x * kChainWarps;
   ChainStep& S = s_step[warp];
@@ -287,15 +290,17 @@ cudaError_t launch(const ChainStep* steps, const ChainTask* tasks, const int32_t
   // one level: no barrier, so no cluster and no limit on the CTAs
   const int c = n_levels == 1 || ctas < most ? ctas : most;
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = static_cast<unsigned>(c);
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = static_cast<unsigned>(c);
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3(static_cast<unsigned>(c));
   cfg.blockDim = dim3(kChainThreads);
   cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = n_levels == 1 ? 0 : 1;
+  cfg.attrs = at;
+  cfg.numAttrs = n_levels == 1 ? 1 : 2;
   return cudaLaunchKernelEx(&cfg, kern, steps, tasks, levels, n_levels, nb, static_cast<int32_t>(skip_unbatched));
 }
 

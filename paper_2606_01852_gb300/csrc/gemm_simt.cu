@@ -42,6 +42,7 @@
 #include "scale.cuh"
 #include "split_bf16.cuh"
 #include "tc_common.cuh"
+#include "pdl.cuh"
 
 namespace tn {
 namespace {
@@ -262,6 +263,8 @@ __global__ void __launch_bounds__(G::THREADS, G::MIN_CTAS) contract_simt_kernel(
   extern __shared__ __align__(16) float sm[];
   const float fill = MP ? __int_as_float(0xff800000) : 0.f;  // the semiring's zero
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  pdl_next();
   const int64_t tiles_n = (a.n + G::N - 1) / G::N;
   const int64_t tile = blockIdx.x;
   const int64_t m0 = (tile / tiles_n) * G::M, n0 = (tile % tiles_n) * G::N;
@@ -438,6 +441,8 @@ __global__ void __launch_bounds__(G::THREADS, G::MIN_CTAS) contract_simt_kernel(
 // Combine the k parts of a split SIMT step in part order (sum, or max for max-plus) and
 // write C through the offset maps. One thread per output element of every batch entry.
 __global__ void simt_combine_kernel(StepArgs a, int32_t nb, int32_t cplx) {
+  pdl_wait();
+  pdl_next();
   const int64_t mn = a.m * a.n, np = cplx ? 2 : 1;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nb * mn;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -469,7 +474,7 @@ void launch(const StepArgs& a, int32_t nb, cudaStream_t st) {
   (void)set;
   const int64_t tiles = ((a.m + G::M - 1) / G::M) * ((a.n + G::N - 1) / G::N);
   dim3 grid((unsigned)tiles, (unsigned)nb, (unsigned)(a.ksplit > 1 ? a.ksplit : 1));
-  contract_simt_kernel<G><<<grid, G::THREADS, G::SMEM, st>>>(a);
+  launch_pdl(contract_simt_kernel<G>, grid, G::THREADS, G::SMEM, st, a);
 }
 
 // A tile shape's time per k term, in units of a full-rate 128 x 128 real (64 x 64 complex) tile:
@@ -538,7 +543,7 @@ void launch_contract_simt(const StepArgs& a, int32_t nb, bool cplx, int num_sms,
   if (a.ksplit > 1) {
     const int64_t total = int64_t(nb) * a.m * a.n;
     const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 4096);
-    simt_combine_kernel<<<blocks, 256, 0, st>>>(a, nb, cplx ? 1 : 0);
+    launch_pdl(simt_combine_kernel, blocks, 256, 0, st, a, nb, cplx ? 1 : 0);
   }
 }
 

@@ -29,6 +29,7 @@
 #include "mbarrier.cuh"
 #include "split_bf16.cuh"
 #include "tc_common.cuh"
+#include "pdl.cuh"
 
 namespace tn {
 namespace {
@@ -136,6 +137,8 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -404,6 +407,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
     }
     mbar_init(acc_full, 1);
     mbar_init(acc_empty, 16);
+    pdl_wait();  // the call's first launch clears the error word
     *skip_slot = *reinterpret_cast<volatile int*>(err) != 0 ? 1u : 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
@@ -419,6 +423,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
   cluster_sync_all();  // both CTAs' barriers initialised and the pair's TMEM allocated
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
   const bool skip = ld_leader_u32(skip_slot) != 0;  // one decision for the pair
 
   if (skip) {
@@ -700,6 +706,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
     }
     mbar_init(acc_full, 1);
     mbar_init(acc_empty, 16);
+    pdl_wait();  // the call's first launch clears the error word
     *skip_slot = *reinterpret_cast<volatile int*>(err) != 0 ? 1u : 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
@@ -715,6 +722,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CB2::THREADS, 1)
   cluster_sync_all();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
   const bool skip = ld_leader_u32(skip_slot) != 0;
 
   if (skip) {
@@ -1020,6 +1029,8 @@ __global__ void __launch_bounds__(CB3::THREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
   const int n_items = 3 * num_kb;  // (k-block, product) slots in order
 
   if (warp == 0) {
@@ -1229,6 +1240,8 @@ __global__ void __launch_bounds__(CB::THREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1421,6 +1434,8 @@ __global__ void __launch_bounds__(CBS::THREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1657,7 +1672,7 @@ cudaError_t launch_tcb(const StepArgs& a, int32_t nb, int* err, cudaStream_t st,
       if (clusters > 0) {
         const int64_t items = pair_tiles * static_cast<int64_t>(nb);
         const int64_t g = items < clusters ? items : clusters;
-        contract_tcb2p_kernel<<<static_cast<unsigned>(2 * g), CB2::THREADS, CB2P::SMEM, st>>>(ta, tb, a, nb, err);
+        launch_pdl(contract_tcb2p_kernel, static_cast<unsigned>(2 * g), CB2::THREADS, CB2P::SMEM, st, ta, tb, a, nb, err);
         return cudaGetLastError();
       }
     }
@@ -1665,7 +1680,7 @@ cudaError_t launch_tcb(const StepArgs& a, int32_t nb, int* err, cudaStream_t st,
     for (int64_t t0 = 0; t0 < pair_tiles; t0 += per_launch) {
       const int64_t cnt = pair_tiles - t0 < per_launch ? pair_tiles - t0 : per_launch;
       dim3 grid(static_cast<unsigned>(2 * cnt), static_cast<unsigned>(nb));
-      contract_tcb2_kernel<<<grid, CB2::THREADS, CB2::SMEM, st>>>(ta, tb, a, t0, err);
+      launch_pdl(contract_tcb2_kernel, grid, CB2::THREADS, CB2::SMEM, st, ta, tb, a, t0, err);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
@@ -1682,7 +1697,7 @@ cudaError_t launch_tcb(const StepArgs& a, int32_t nb, int* err, cudaStream_t st,
     if (e != cudaSuccess) return e;
     const int64_t items = tiles * static_cast<int64_t>(nb);
     const unsigned grid = static_cast<unsigned>(items < sms ? items : sms);
-    contract_tcb_shallow_kernel<<<grid, CBS::THREADS, CBS::SMEM, st>>>(ta, tb, a, nb, err);
+    launch_pdl(contract_tcb_shallow_kernel, grid, CBS::THREADS, CBS::SMEM, st, ta, tb, a, nb, err);
     return cudaGetLastError();
   }
   if (a.k <= CBP::MAX_K) {
@@ -1693,7 +1708,7 @@ cudaError_t launch_tcb(const StepArgs& a, int32_t nb, int* err, cudaStream_t st,
     if (e != cudaSuccess) return e;
     const int64_t items = tiles * static_cast<int64_t>(nb);
     const unsigned grid = static_cast<unsigned>(items < sms ? items : sms);
-    contract_tcb_persistent_kernel<<<grid, CB::THREADS, CBP::SMEM, st>>>(ta, tb, a, nb, err);
+    launch_pdl(contract_tcb_persistent_kernel, grid, CB::THREADS, CBP::SMEM, st, ta, tb, a, nb, err);
     return cudaGetLastError();
   }
   return launch_bands(contract_tcb_kernel<false>, tiles, nb, CB::THREADS, CB::SMEM, st, ta, tb, a, err);

@@ -23,6 +23,7 @@
 #include "scale.cuh"
 #include "split_bf16.cuh"
 #include "tc_common.cuh"
+#include "pdl.cuh"
 
 namespace tn {
 namespace {
@@ -116,6 +117,8 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, REAL ? 2 : 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -370,6 +373,8 @@ __global__ void __launch_bounds__(576, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = uniform_u32(*tmem_slot);
+  pdl_wait();
+  pdl_next();
 
   if (warp == 0) {
     if (lane == 0) {

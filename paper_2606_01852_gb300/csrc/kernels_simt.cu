@@ -15,6 +15,7 @@
 #include "scale.cuh"
 #include "split_bf16.cuh"
 #include "widen.cuh"
+#include "pdl.cuh"
 #include "staging.cuh"
 
 namespace tn {
@@ -892,17 +893,19 @@ __global__ void accumulate_root_kernel(const float* __restrict__ root, int64_t s
 
 // One slice in one pass: the output is that slice's value, widened exactly; no FP64
 // arithmetic. Grid-stride, two elements (e, e + G) per thread per iteration.
-__global__ void __launch_bounds__(256) widen_root_kernel(const float* __restrict__ root, int64_t size,
+__global__ void __launch_bounds__(256) widen_root_kernel(const float* root, int64_t size,
                                                          int64_t plane, int32_t cplx, void* out,
                                                          const ScaleRec* rec, double* log_scale) {
+  pdl_wait();
+  pdl_next();
   const int64_t G = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < size; e0 += 2 * G) {
     float re[2], im[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int64_t e = e0 + i * G;
-      re[i] = e < size ? __ldg(root + e) : 0.f;
-      im[i] = cplx && e < size ? __ldg(root + plane + e) : 0.f;
+      re[i] = e < size ? __ldcg(root + e) : 0.f;
+      im[i] = cplx && e < size ? __ldcg(root + plane + e) : 0.f;
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -923,7 +926,7 @@ void launch_accumulate_root(const float* root, int64_t size, int32_t nb, int64_t
   if (first && last && nb == 1) {
     const int64_t want = (size + 511) / 512;
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, int64_t(num_sms) * 8));
-    widen_root_kernel<<<blocks, 256, 0, st>>>(root, size, plane, cplx ? 1 : 0, out,
+    launch_pdl(widen_root_kernel, blocks, 256, 0, st, root, size, plane, cplx ? 1 : 0, out,
                                               recs && !maxplus ? recs + rec_root : nullptr, log_scale);
     return;
   }
@@ -952,6 +955,8 @@ void launch_accumulate_root(const float* root, int64_t size, int32_t nb, int64_t
 template <bool CPLX, bool MAXPLUS = false>
 __global__ void __launch_bounds__(256) splitk_partial_kernel(StepArgs a, double* scratch, int64_t kc,
                                                              int32_t chunks) {
+  pdl_wait();
+  pdl_next();
   static_assert(!(CPLX && MAXPLUS), "the max-plus semiring is real");
   const int chunk = blockIdx.x, b = blockIdx.y, o = blockIdx.z;
   const int n = (int)a.n, mn = (int)a.m * n;
@@ -1053,6 +1058,8 @@ constexpr int kFinalThreads = 128;
 // then adds the runs that hold any in order: a fixed association for a given chunk count.
 __global__ void __launch_bounds__(kFinalThreads) splitk_final_kernel(StepArgs a, const double* scratch,
                                                                     int32_t chunks, int32_t cplx) {
+  pdl_wait();
+  pdl_next();
   const int b = blockIdx.x, o = blockIdx.y;
   const int n = (int)a.n, mn = (int)a.m * n;
   float* C = a.C + b * a.c_bstride;
@@ -1104,10 +1111,10 @@ void launch_contract_splitk(const StepArgs& a, int32_t nb, bool cplx, double* sc
   const int32_t chunks = splitk_chunks(a.k);
   const unsigned outs = (unsigned)(a.m * a.n);
   dim3 grid((unsigned)chunks, (unsigned)nb, outs);
-  if (cplx) splitk_partial_kernel<true><<<grid, 256, 0, st>>>(a, scratch, kSplitChunk, chunks);
-  else if (a.maxplus) splitk_partial_kernel<false, true><<<grid, 256, 0, st>>>(a, scratch, kSplitChunk, chunks);
-  else splitk_partial_kernel<false><<<grid, 256, 0, st>>>(a, scratch, kSplitChunk, chunks);
-  splitk_final_kernel<<<dim3((unsigned)nb, outs), kFinalThreads, 0, st>>>(a, scratch, chunks, cplx ? 1 : 0);
+  if (cplx) launch_pdl(splitk_partial_kernel<true>, grid, 256, 0, st, a, scratch, kSplitChunk, chunks);
+  else if (a.maxplus) launch_pdl(splitk_partial_kernel<false, true>, grid, 256, 0, st, a, scratch, kSplitChunk, chunks);
+  else launch_pdl(splitk_partial_kernel<false>, grid, 256, 0, st, a, scratch, kSplitChunk, chunks);
+  launch_pdl(splitk_final_kernel, dim3((unsigned)nb, outs), kFinalThreads, 0, st, a, scratch, chunks, cplx ? 1 : 0);
 }
 
 }  // namespace tn

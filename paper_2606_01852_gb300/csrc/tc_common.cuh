@@ -13,6 +13,7 @@
 #include "mbarrier.cuh"
 #include "scale.cuh"
 #include "split_bf16.cuh"
+#include "pdl.cuh"
 
 namespace tn {
 namespace {
@@ -485,7 +486,7 @@ cudaError_t launch_bands(Kern kern, int64_t tiles, int32_t nb, int threads, int 
   const int64_t per = sm_band_tiles(tiles, nb);
   for (int64_t t0 = 0; t0 < tiles; t0 += per) {
     const int64_t cnt = tiles - t0 < per ? tiles - t0 : per;
-    kern<<<dim3(static_cast<unsigned>(cnt), static_cast<unsigned>(nb)), threads, smem, st>>>(ta, tb, a, t0, err);
+    launch_pdl(kern, dim3(static_cast<unsigned>(cnt), static_cast<unsigned>(nb)), threads, smem, st, ta, tb, a, t0, err);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
