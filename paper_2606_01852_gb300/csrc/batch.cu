@@ -56,19 +56,20 @@ struct Team {
   }
 };
 
-__device__ __forceinline__ int map_offset(const int32_t* __restrict__ ext, const int32_t* __restrict__ str, int nd,
-                                          bool pow2, int x) {
+// The offset of index x under a digit map of nd digits (arrays 16-byte aligned; places beyond nd
+// are 0, so four are taken without a branch).
+__device__ __forceinline__ int map_offset(const int32_t* ext, const int32_t* str, int nd, bool pow2, int x) {
   int off = 0;
   if (pow2) {
-#pragma unroll 4
-    for (int d = 0; d < nd; ++d) {
-      const int w = __ldg(ext + d);
-      off += ((x >> (w & 31)) & (w >> 8)) * __ldg(str + d);
-    }
+    const int4 e = *reinterpret_cast<const int4*>(ext), st = *reinterpret_cast<const int4*>(str);
+    off = ((x >> (e.x & 31)) & (e.x >> 8)) * st.x + ((x >> (e.y & 31)) & (e.y >> 8)) * st.y +
+          ((x >> (e.z & 31)) & (e.z >> 8)) * st.z + ((x >> (e.w & 31)) & (e.w >> 8)) * st.w;
+#pragma unroll 1
+    for (int d = 4; d < nd; ++d) off += ((x >> (ext[d] & 31)) & (ext[d] >> 8)) * str[d];
   } else {
     for (int d = nd - 1; d >= 0; --d) {
-      const int w = __ldg(ext + d);
-      off += (x % w) * __ldg(str + d);
+      const int w = ext[d];
+      off += (x % w) * str[d];
       x /= w;
     }
   }
@@ -76,7 +77,7 @@ __device__ __forceinline__ int map_offset(const int32_t* __restrict__ ext, const
 }
 
 // Output offset of row x (x < m) or of column x - m (x >= m) of step S.
-__device__ __forceinline__ int step_offset(const BStep* __restrict__ S, int nr, int nc, bool pow2, int m, int x) {
+__device__ __forceinline__ int step_offset(const BStep* S, int nr, int nc, bool pow2, int m, int x) {
   return x < m ? map_offset(S->rext, S->rstr, nr, pow2, x) : map_offset(S->cext, S->cstr, nc, pow2, x - m);
 }
 
@@ -141,7 +142,7 @@ __device__ __forceinline__ void dot_tile(const float* a, int ai, const int (&ra)
 // threads, a thread's rows tm apart and its columns tn apart, so that neighbouring threads read
 // neighbouring rows. 1 x 1: output o to thread o, in order.
 template <bool CPLX, bool MAXPLUS, bool WARP, int RM, int RN, int KV>
-__device__ __forceinline__ int run_step(float* ar, const BStep* __restrict__ S, int m, int n, int k, int nr, int nc,
+__device__ __forceinline__ int run_step(float* ar, const BStep* S, int m, int n, int k, int nr, int nc,
                                         bool pow2, int a, int b, int c, float sa, float sb, const int* tab) {
   int mx = 0;
   float cr[RM][RN], ci[RM][RN];
@@ -215,6 +216,8 @@ batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves, co
   __shared__ int s_exp[kExpBytes / 4];  // the step outputs' largest exponents: ints, or bytes (+127) per warp
   __shared__ int s_net;
   __shared__ long long s_log;
+  constexpr int kRec = sizeof(BStep) / 16;
+  __shared__ int4 s_step[2][WARP ? 1 : kRec];  // this step's record and the next one's
   using T = Team<WARP>;
   constexpr int RM = 4, RN = CPLX ? 2 : 4;
   const int teams = WARP ? blockDim.x >> 5 : 1, team = WARP ? threadIdx.x >> 5 : 0;
@@ -247,6 +250,7 @@ batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves, co
     long long lsum = 0;  // this thread's share of the exponents' sum
     if (!WARP && scaling)
       for (int i = rank; i < min(max(net.n_steps, 2), exp_cap); i += size) s_exp[i] = -127;
+    if (!WARP && rank < kRec && net.n_steps > 0) s_step[0][rank] = __ldg(reinterpret_cast<const int4*>(S0) + rank);
     // Leaves (declared order -> planned order; complex64 -> planar), each scaled by its own exact
     // power of two: small ones by groups of 8 threads, whose own elements they scale
     bool big = false;
@@ -341,13 +345,12 @@ batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves, co
       T::sync();
     }
     for (int s = 0; s < net.n_steps; ++s) {
-      const BStep* S = S0 + s;
-      const int4 h0 = __ldg(reinterpret_cast<const int4*>(S)), h1 = __ldg(reinterpret_cast<const int4*>(S) + 1);
-      if (rank < 2 && s + 1 < net.n_steps) {
-        // the next step's record into L1 while this one runs
-        int x;
-        asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(x) : "l"(reinterpret_cast<const char*>(S + 1) + rank * 128));
-      }
+      // (a record read from L2 by every step cost it more than its arithmetic)
+      const BStep* S = WARP ? S0 + s : reinterpret_cast<const BStep*>(s_step[s & 1]);
+      const int4 h0 = reinterpret_cast<const int4*>(S)[0], h1 = reinterpret_cast<const int4*>(S)[1];
+      int4 next;
+      const bool fetch = !WARP && rank < kRec && s + 1 < net.n_steps;
+      if (fetch) next = __ldg(reinterpret_cast<const int4*>(S0 + s + 1) + rank);
       const int m = h0.w, n = h1.x, k = h1.y, mn = m * n;
       const int nr = (h1.z >> 27) & 15, nc = h1.w >> 27;
       const bool pow2 = h1.z < 0;
@@ -386,6 +389,7 @@ batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves, co
       } else {
         mx = run_step<CPLX, MAXPLUS, WARP, 1, 1, 1>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, nullptr);
       }
+      if (fetch) s_step[(s + 1) & 1][rank] = next;
       if (!MAXPLUS && scaling) {
         __syncwarp();
         if (defer) {
