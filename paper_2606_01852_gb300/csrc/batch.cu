@@ -19,7 +19,9 @@
 // networks are queued by falling cost so that the large ones do not end last. 4096 Ising
 // networks of 20-60 vertices: 3.98 -> 0.60 ms (0.89 ms in the caller's order and with 64
 // registers a thread, 0.64 ms with 80, 0.60 with 128: the tiles want registers more than the
-// small steps want warps); 1024 king's graphs of 4-7 a side, max-plus: 14.0 -> 1.8 ms.
+// small steps want warps), 0.58 with the step records in shared memory, 0.38 with run_panels;
+// 1024 king's graphs of 4-7 a side, max-plus: 14.0 -> 1.8 -> 0.89 ms. A small step is now ~1300
+// clocks: 200-300 for its record, 850 for an output, 250 for the maximum and the barrier.
 // The CTA width (threads per network) and CTAs per SM are chosen by an autotuner that
 // times the real batch; the launch (queue reset + kernel) can be replayed as a CUDA graph.
 #include <algorithm>
@@ -96,10 +98,8 @@ __device__ __forceinline__ void load_k(const float* p, float s, float (&v)[KV]) 
 
 // RM x RN outputs of one thread, each its own chain over k in order (so an output's bits do not
 // depend on the tile it is computed in): rows a + ra[r], columns b + rb[c], KV terms per load.
-template <bool CPLX, bool MAXPLUS, int RM, int RN, int KV>
-__device__ __forceinline__ void dot_tile(const float* a, int ai, const int (&ra)[RM], const float* b, int bi,
-                                         const int (&rb)[RN], int k, float sa, float sb, float (&cr)[RM][RN],
-                                         float (&ci)[RM][RN]) {
+template <bool MAXPLUS, int RM, int RN>
+__device__ __forceinline__ void dot_init(float (&cr)[RM][RN], float (&ci)[RM][RN]) {
 #pragma unroll
   for (int r = 0; r < RM; ++r)
 #pragma unroll
@@ -107,6 +107,11 @@ __device__ __forceinline__ void dot_tile(const float* a, int ai, const int (&ra)
       cr[r][c] = MAXPLUS ? __int_as_float(0xff800000) : 0.f;  // max-plus: its zero is -inf, its product +
       ci[r][c] = 0.f;
     }
+}
+template <bool CPLX, bool MAXPLUS, int RM, int RN, int KV>
+__device__ __forceinline__ void dot_tile(const float* a, int ai, const int (&ra)[RM], const float* b, int bi,
+                                         const int (&rb)[RN], int k, float sa, float sb, float (&cr)[RM][RN],
+                                         float (&ci)[RM][RN]) {
 #pragma unroll(RM * RN == 1 ? 4 : 1)
   for (int t = 0; t < k; t += KV) {
     float xr[RM][KV], xi[RM][KV];
@@ -160,6 +165,7 @@ __device__ __forceinline__ int run_step(float* ar, const BStep* S, int m, int n,
     for (int o = Team<WARP>::rank(); o < m * n; o += Team<WARP>::size()) {
       const int i = nsh >= 0 ? o >> nsh : o / n, j = o - i * n;
       const int ra[1] = {i * k}, rb[1] = {j * k};
+      dot_init<MAXPLUS>(cr, ci);
       dot_tile<CPLX, MAXPLUS, 1, 1, KV>(ar + a, m * k, ra, ar + b, n * k, rb, k, sa, sb, cr, ci);
       store(map_offset(S->rext, S->rstr, nr, pow2, i) + map_offset(S->cext, S->cstr, nc, pow2, j), cr[0][0], ci[0][0]);
     }
@@ -178,6 +184,7 @@ __device__ __forceinline__ int run_step(float* ar, const BStep* S, int m, int n,
       for (int r = 0; r < RM; ++r) ra[r] = min(ti + r * tm, m - 1) * k;
 #pragma unroll
       for (int q = 0; q < RN; ++q) rb[q] = min(tj + q * tn, n - 1) * k;
+      dot_init<MAXPLUS>(cr, ci);
       dot_tile<CPLX, MAXPLUS, RM, RN, KV>(ar + a, m * k, ra, ar + b, n * k, rb, k, sa, sb, cr, ci);
 #pragma unroll
       for (int q = 0; q < RN; ++q) {
@@ -192,6 +199,71 @@ __device__ __forceinline__ int run_step(float* ar, const BStep* S, int m, int n,
       }
     }
   }
+  return mx;
+}
+
+// A step of a network whose arena is in global memory: its operands' rows are k floats apart, and
+// lanes that read their own rows touch a line each, eight times over. Here 32 terms of the rows of a
+// (4 G) x 32 tile of outputs (G = threads / 8) are brought into shared memory by whole lines, and each
+// thread's 4 x 4 outputs run over them, k in order as everywhere: the same bits. The rows are
+// the larger operand's, 36 floats apart (a quarter warp's 16-byte reads then meet different
+// banks). A 32 x 16 x 512 step was 88 us of its CTA and a 64 x 256 x 16 one 47: 4096 Ising networks
+// 0.58 -> 0.38 ms, 1024 king's graphs 1.80 -> 0.89 ms.
+constexpr int kPanelRow = 36;
+__host__ __device__ constexpr int panel_floats(int threads) { return (threads / 2 + 32) * kPanelRow; }
+
+template <bool MAXPLUS>
+__device__ __forceinline__ int run_panels(float* ar, const BStep* S, int m, int n, int k, int nr, int nc, bool pow2,
+                                          int a, int b, int c, float sa, float sb, const int* tab, float* panel) {
+  const int tid = threadIdx.x, T = blockDim.x, G = T >> 3;
+  const bool by_a = m >= n;
+  const float* P = ar + (by_a ? a : b);
+  const float* Q = ar + (by_a ? b : a);
+  const float sp = by_a ? sa : sb, sq = by_a ? sb : sa;
+  const int np = by_a ? m : n, nq = by_a ? n : m;
+  const int ti = tid >> 3, tj = tid & 7;
+  float* pq = panel + 4 * G * kPanelRow;
+  int ra[4], rb[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    ra[r] = (ti + G * r) * kPanelRow;
+    rb[r] = (tj + 8 * r) * kPanelRow;
+  }
+  int mx = 0;
+  for (int p0 = 0; p0 < np; p0 += 4 * G)
+    for (int q0 = 0; q0 < nq; q0 += 32) {
+      float cr[4][4], ci[4][4];
+      dot_init<MAXPLUS>(cr, ci);
+      for (int t0 = 0; t0 < k; t0 += 32) {
+        const int kc = min(32, k - t0), t = t0 + 4 * tj;
+        __syncthreads();  // the panels' last reads
+        if (4 * tj < kc) {
+          for (int r = ti; r < 4 * G && p0 + r < np; r += G) {
+            float v[4];
+            load_k<4>(P + (p0 + r) * k + t, sp, v);
+            *reinterpret_cast<float4*>(panel + r * kPanelRow + 4 * tj) = make_float4(v[0], v[1], v[2], v[3]);
+          }
+          for (int r = ti; r < 32 && q0 + r < nq; r += G) {
+            float v[4];
+            load_k<4>(Q + (q0 + r) * k + t, sq, v);
+            *reinterpret_cast<float4*>(pq + r * kPanelRow + 4 * tj) = make_float4(v[0], v[1], v[2], v[3]);
+          }
+        }
+        __syncthreads();
+        dot_tile<false, MAXPLUS, 4, 4, 4>(panel, 0, ra, pq, 0, rb, kc, 1.f, 1.f, cr, ci);
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          const int p = p0 + ti + G * x, q = q0 + tj + 8 * y;
+          if (p >= np || q >= nq) continue;
+          const int i = by_a ? p : q, j = by_a ? q : p;
+          ar[c + (tab ? tab[i] + tab[m + j]
+                      : map_offset(S->rext, S->rstr, nr, pow2, i) + map_offset(S->cext, S->cstr, nc, pow2, j))] = cr[x][y];
+          mx = max(mx, __float_as_int(fabsf(cr[x][y])));
+        }
+    }
   return mx;
 }
 
@@ -365,7 +437,19 @@ batch_kernel(const BNet* __restrict__ nets, const BLeaf* __restrict__ leaves, co
         sb = scale_of(h1.w & kBLeafId);
       }
       int mx = 0;
-      if (rank - lane >= mn) {
+      // (k deep enough for the panels to pay, and no more than half of a tile's rows empty)
+      const bool panels = TILES && !WARP && !CPLX && ar != s_arena && smem_arena >= panel_floats(blockDim.x) &&
+                          (k & 3) == 0 && k >= 16 && max(m, n) >= 16 && min(m, n) >= 8 && mn * (k >> 4) >= 16 * size;
+      if (panels) {
+        if constexpr (TILES && !WARP && !CPLX) {
+          const int* tab = nullptr;
+          if (m + n <= tab_ints) {
+            for (int x = rank; x < m + n; x += size) s_tab[x] = step_offset(S, nr, nc, pow2, m, x);
+            tab = s_tab;  // (complete at the panels' first barrier)
+          }
+          mx = run_panels<MAXPLUS>(ar, S, m, n, k, nr, nc, pow2, h0.x, h0.y, h0.z, sa, sb, tab, s_arena);
+        }
+      } else if (rank - lane >= mn) {
         // no output for this warp
       } else if (TILES && m >= RM && n >= RN && mn >= 8 * size) {
         const int* tab = nullptr;

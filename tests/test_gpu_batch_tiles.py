@@ -1,5 +1,6 @@
 """The batched kernel's step forms at their edges: register tiles with ragged rows and columns,
-loads of 4, 2 and 1 terms, extents that are not powers of two, leaves staged by groups and by the
+loads of 4, 2 and 1 terms, panels
+of large steps in shared memory, extents that are not powers of two, leaves staged by groups and by the
 whole team, and more steps than the exponents a team keeps. Every launch shape gives the same bits
 (one thread runs an output's terms in order), and the value is the direct sum's within FP32's error
 bound for the sum: every term is positive (or bounded by its absolute sum), so each of the
@@ -15,9 +16,9 @@ from tn_inputs.network import Network, Path
 pytestmark = pytest.mark.gpu
 
 SIZES = [(1, 1, 1), (4, 4, 2), (5, 7, 3), (16, 16, 8), (17, 33, 4), (64, 33, 6), (37, 130, 4), (100, 101, 1), (130, 3, 16),
-         (2, 300, 2), (64, 128, 32), (129, 64, 12)]
+         (2, 300, 2), (64, 128, 32), (129, 64, 12), (70, 33, 36), (33, 70, 20), (16, 8, 512), (300, 40, 52), (97, 97, 16)]
 # (threads, CTAs per SM, networks per CTA, shared arena): tiles from 256 outputs on in the first, never in the last
-SHAPES = [(32, 4, 1), (128, 2, 1, 4096), (256, 2, 1), (512, 1, 1), (32, 2, 4), (32, 1, 16)]
+SHAPES = [(32, 4, 1), (128, 2, 1, 4096), (256, 1, 1, 8192), (64, 2, 1, 2304), (256, 2, 1), (512, 1, 1), (32, 2, 4), (32, 1, 16)]
 
 
 @pytest.fixture(scope="module")
