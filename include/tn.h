@@ -49,7 +49,7 @@ typedef enum {
  *               FP32 accumulation.
  * Steps too small or too thin for a tensor-core tile run on the FP32 SIMT kernels
  * whatever the form (tn_plan_step reports each step's kernel). Real networks take the
- * TF32 and 3XTF32 forms on 128 x 256 tiles; R32_BF16X3 is not built. Exponent scaling
+ * TF32 (128 x 256 tiles) and 3XTF32 (128 x 192 and narrower) forms; R32_BF16X3 is not built. Exponent scaling
  * runs in every form but the 3M product (the tensor-core kernels apply the operands' exact
  * power-of-two scales to the accumulated result, the same values as scaling the operands
  * on load; scaled BF16X3 steps keep one SM per tile). tn_plan returns TN_ERR_UNSUPPORTED
@@ -158,7 +158,7 @@ typedef struct {
   int32_t ksplit;          /* SIMT steps: k cut in this many parts (then two launches) */
   int32_t single_sm;       /* tensor-core steps: 1 if kept on one SM per tile (tn_plan_autotune) */
   int32_t chain;           /* -1, or the step chain the step runs in: a run of consecutive tiny
-                              CUDA-core steps executed by one CTA in one launch (the profile
+                              CUDA-core steps executed by one cluster in one launch (the profile
                               attributes the chain's time to its first step) */
   int32_t reserved;
 } tn_step_info;
@@ -242,7 +242,8 @@ tn_status tn_plan_layout(tn_plan_t plan, int32_t id, int32_t* modes_out, int32_t
 
 /* The number of kernel launches one tn_contract_slices call over slice_count slices makes
  * (the same for any first slice): staging, every step (two for split-k steps, several for a
- * deep step on paired SMs, launched in bands of tiles), and the slice sum, per pass. */
+ * deep step on paired SMs, launched in bands of tiles; one for a run of gates), and the slice sum
+ * (none where a run of gates writes the output), per pass. */
 tn_status tn_plan_launches(tn_plan_t plan, int64_t slice_count, int64_t* out);
 
 /* Description of step s (host only). */
@@ -276,8 +277,8 @@ tn_status tn_plan_autotune(tn_plan_t plan, const void* const* inputs, void* outp
  * private stream; later calls with the same pointers and stream launch the captured graph
  * (one launch instead of one per step and pass), with the same results bit for bit. A call
  * with other pointers or another stream re-captures (after the previous graph's last launch
- * has finished). The first call allocates the graph and a pinned copy of the leaf
- * descriptors; tn_plan_destroy frees them. The inputs are read at launch time, so new values
+ * has finished). The first call allocates the graph; tn_plan_destroy
+ * frees it. The inputs are read at launch time, so new values
  * in the same buffers are contracted by a replay. TN_ERR_INVALID while per-step profiling is
  * on (tn_plan_profile) or for a host-only plan; TN_ERR_CUDA if capture fails. */
 tn_status tn_contract_graph(tn_plan_t plan, const void* const* inputs, void* output, double* out_log_scale,
@@ -415,8 +416,8 @@ typedef struct tn_batch_s* tn_batch_t;
 
 /* Plan n_nets independent CLOSED networks (each with its own path; no slicing) for one
  * persistent launch: every network gets the same analysis and mode reordering as
- * tn_plan (Sec. II-B, Sec. IV-A) and its own arena; one CTA contracts one network at a
- * time, taking networks from an atomic queue. policy.prec must be TN_C64_FP32_SIMT or
+ * tn_plan (Sec. II-B, Sec. IV-A) and its own arena; one CTA (or warp) contracts one network
+ * at a time, the costliest first, from an atomic queue. policy.prec must be TN_C64_FP32_SIMT or
  * TN_R32_FP32_SIMT; policy.exp_scaling renormalises every tensor by an exact power of two
  * as it is made and sums the exponents per network in an int64; policy.semiring may be
  * TN_SEMIRING_MAXPLUS with R32 and no scaling (each value is then the network's max-plus

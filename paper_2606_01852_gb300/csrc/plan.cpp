@@ -441,7 +441,7 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
       P.tensors[st.b].split = mode;
     }
   }
-  // ---- leaf descriptors (sources filled per call)
+  // ---- leaf descriptors (a call's launches carry the sources)
   P.leafdesc.assign(T, LeafDesc{});
   int64_t leaf_permutes = 0;
   for (int32_t t = 0; t < T; ++t) {
