@@ -555,9 +555,27 @@ struct tn_batch_s {
 
 namespace tn {
 
+// The kernel of a form, allowed all the shared memory that a CTA may take beside its static part
+// (once: launches of several threads do not meet in it).
+using BatchKernel = void (*)(const BNet*, const BLeaf*, const BStep*, int32_t, const float*, float*, int32_t*, int32_t,
+                             double*, double*, int32_t, int32_t);
+static cudaError_t allow_smem(BatchKernel kernel) {
+  cudaFuncAttributes fa{};
+  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kMaxSmemPerCta - static_cast<int64_t>(fa.sharedSizeBytes)));
+}
 template <bool CPLX, bool MAXPLUS, bool WARP>
-auto batch_form(bool tiles) {
-  return tiles ? batch_kernel<CPLX, MAXPLUS, WARP, true> : batch_kernel<CPLX, MAXPLUS, WARP, false>;
+BatchKernel batch_form(bool tiles, cudaError_t& e) {
+  if (tiles) {
+    static const cudaError_t set = allow_smem(batch_kernel<CPLX, MAXPLUS, WARP, true>);
+    e = set;
+    return batch_kernel<CPLX, MAXPLUS, WARP, true>;
+  }
+  static const cudaError_t set = allow_smem(batch_kernel<CPLX, MAXPLUS, WARP, false>);
+  e = set;
+  return batch_kernel<CPLX, MAXPLUS, WARP, false>;
 }
 
 cudaError_t launch_batch_kernel(const BNet* nets, const BLeaf* leaves, const BStep* steps, int32_t n_nets,
@@ -572,12 +590,11 @@ cudaError_t launch_batch_kernel(const BNet* nets, const BLeaf* leaves, const BSt
   smem_arena &= ~63;  // arenas are multiples of 64 floats
   const int smem = (smem_arena + tab_ints) * 4 * (warp ? threads / 32 : 1);
   const bool tiles = threads <= kTileThreads;
-  auto kernel = warp ? (cplx ? batch_form<true, false, true>(tiles)
-                             : maxplus ? batch_form<false, true, true>(tiles) : batch_form<false, false, true>(tiles))
-                     : (cplx ? batch_form<true, false, false>(tiles)
-                             : maxplus ? batch_form<false, true, false>(tiles) : batch_form<false, false, false>(tiles));
-  if (smem && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-    return e;
+  auto kernel = warp ? (cplx ? batch_form<true, false, true>(tiles, e)
+                             : maxplus ? batch_form<false, true, true>(tiles, e) : batch_form<false, false, true>(tiles, e))
+                     : (cplx ? batch_form<true, false, false>(tiles, e)
+                             : maxplus ? batch_form<false, true, false>(tiles, e) : batch_form<false, false, false>(tiles, e));
+  if (e != cudaSuccess) return e;
   kernel<<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, maxplus ? 0 : sc, values, logs,
                                       smem_arena, tab_ints);
   return cudaGetLastError();

@@ -206,14 +206,22 @@ __global__ void __launch_bounds__(kThreads, 6) gate_run_kernel(const __grid_cons
 
 }  // namespace
 
-cudaError_t launch_gate_run(const GateArgs& a, bool cplx, cudaStream_t st) {
-  auto kernel = cplx ? gate_run_kernel<true> : gate_run_kernel<false>;
-  int bytes = (cplx ? 8 : 4) << a.t;
-  for (int g = 0; g < a.n_gates; ++g) bytes += 8 << (2 * a.gate[g].bits);
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e != cudaSuccess) return e;
-  kernel<<<1u << a.outer, kThreads, bytes, st>>>(a);
+template <bool CPLX>
+static cudaError_t launch(const GateArgs& a, cudaStream_t st) {
+  // (once, for the largest tile and matrices: launches of several threads do not meet in it)
+  constexpr int elem = CPLX ? 8 : 4;
+  static const cudaError_t configured =
+      cudaFuncSetAttribute(gate_run_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (elem << kGateTileBits) + kGateMaxRun * 256 * int(sizeof(float2)));
+  if (configured != cudaSuccess) return configured;
+  int bytes = elem << a.t;
+  for (int g = 0; g < a.n_gates; ++g) bytes += int(sizeof(float2)) << (2 * a.gate[g].bits);
+  gate_run_kernel<CPLX><<<1u << a.outer, kThreads, bytes, st>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t launch_gate_run(const GateArgs& a, bool cplx, cudaStream_t st) {
+  return cplx ? launch<true>(a, st) : launch<false>(a, st);
 }
 
 }  // namespace tn

@@ -8,6 +8,9 @@
 // it, so the last one's completion is everybody's. The first launch of a call is an ordinary one.
 // Such a kernel reads what other kernels write by ordinary loads, L2 loads or TMA, never by the
 // read-only path (__ldg, __restrict__): its lines and the compiler may be older than the wait.
+// Measured (GB300): one amplitude of a 12-qubit circuit (3 launches) 28.7 -> 24.1 us, 16 amplitudes
+// of a 20-qubit one (20 launches) 255 -> 212 us, a 20 x 20 spin glass 12.02 -> 11.81 ms; a 4 x 4
+// kicked Ising model replayed from a graph (109 launches) 0.93 ms with and without.
 #pragma once
 
 #include <utility>
