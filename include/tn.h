@@ -160,7 +160,9 @@ typedef struct {
   int32_t chain;           /* -1, or the step chain the step runs in: a run of consecutive tiny
                               CUDA-core steps executed by one cluster in one launch (the profile
                               attributes the chain's time to its first step) */
-  int32_t reserved;
+  int32_t gate_run;        /* -1, or the gate run the step is in: consecutive steps that each apply a
+                              small square matrix to the output of the one before, executed in one
+                              launch (the profile attributes the run's time to its first step) */
 } tn_step_info;
 
 /* How a tensor's copies are stored in the workspace. PLANAR: FP32 (complex: the real

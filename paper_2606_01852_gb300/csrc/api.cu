@@ -30,13 +30,17 @@ thread_local std::string g_last_error;
 constexpr int64_t kLevelOrderBytes = int64_t(64) << 20;
 
 // Assign the workspace for b slices a pass, chains in level order if that fits `budget` and
-// costs little; its size.
+// costs little, gate runs (which hold one tensor more at most) if that fits; its size.
 int64_t batch_footprint(Plan& P, int64_t b, int64_t budget) {
   assign_workspace(P, b, true);
   int64_t held = 0;
   for (const StepRec& st : P.steps)
     if (st.chain >= 0) held += P.tensors[st.out].bytes;
   if (held > kLevelOrderBytes || P.total_bytes > budget || !P.workspace_ok) assign_workspace(P, b, false);
+  if (P.total_bytes > budget && !P.gate_runs.empty()) {
+    drop_gate_runs(P);
+    return batch_footprint(P, b, budget);
+  }
   return P.total_bytes;
 }
 
@@ -555,7 +559,7 @@ tn_status tn_plan_step(tn_plan_t plan, int32_t s, tn_step_info* out) {
   out->ksplit = st.ksplit;
   out->single_sm = st.single_sm ? 1 : 0;
   out->chain = st.chain;
-  out->reserved = 0;
+  out->gate_run = st.gates;
   return TN_OK;
 }
 

@@ -748,6 +748,7 @@ tn_status tn_batch_plan(int32_t n_nets, const tn_network* nets, const tn_path* p
       set_error("tn_batch_plan: network " + std::to_string(w) + " has open labels (closed networks only)");
       return TN_ERR_UNSUPPORTED;
     }
+    drop_gate_runs(P);  // the batched kernel runs the steps one after another
     assign_workspace(P, 1, false);
     if (!P.workspace_ok) {
       set_error("tn_batch_plan: workspace self-check failed");

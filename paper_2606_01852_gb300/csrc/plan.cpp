@@ -898,8 +898,37 @@ static void find_chains(Plan& P, int64_t batch, bool level_order) {
   }
 }
 
+void drop_gate_runs(Plan& P) {
+  for (StepRec& st : P.steps) st.gates = -1;
+  for (LeafDesc& d : P.leafdesc) d.direct = 0;
+  P.gate_runs.clear();
+}
+
+// Every gate run's output apart from all that exists when the run starts and is read in it or after
+// it: the run is one launch, whose blocks store while others have not loaded yet. Worked out
+// from what the kernel reads and writes, not from the lifetimes that the offsets come from.
+static bool gate_runs_ok(const Plan& P) {
+  const int32_t T = P.n_leaves, N = T + (int32_t)P.steps.size();
+  for (const GateRun& g : P.gate_runs) {
+    if (g.root) continue;  // writes the caller's output
+    const int32_t last = g.first + g.n - 1;
+    const TensorRec& C = P.tensors[P.steps[last].out];
+    for (int32_t t = 0; t < N; ++t) {
+      const TensorRec& R = P.tensors[t];
+      const bool before = t < T || t - T < g.first;
+      const bool used = R.consumer < 0 || R.consumer >= g.first;
+      if (!before || !used || t == g.leaf) continue;
+      if (R.offset < C.offset + C.bytes && C.offset < R.offset + R.bytes) return false;
+    }
+  }
+  return true;
+}
+
 // Liveness: a leaf is born when the pass stages it (event -1) and a step output at its
-// step; each dies at its consuming step (the root after the final accumulation). Two
+// step; each dies at its consuming step (the root after the final accumulation). A gate run's
+// input and gates die at its last step: it reads them while it writes that step's output. (Its inner
+// results, and a leaf that it reads where the caller has it, are in the workspace only for calls
+// that run its steps one by one, in path order.) Two
 // tensors share memory only if their lifetimes are disjoint. Offsets are static, so
 // every pass replays the same layout -- which is why a pinned tensor (made once in the
 // first pass, read by every pass) is reserved over the whole timeline [-1, inf]: a
@@ -922,11 +951,18 @@ void assign_workspace(Plan& P, int64_t batch, bool level_order) {
     const ChainRec& c = P.chains[P.steps[s].chain];
     return c.first + c.n - 1;
   };
+  // the last step of tensor t's gate run, if it is the run's input or one of its gates
+  auto run_reads = [&](int32_t t, int32_t s) {
+    if (P.steps[s].gates < 0) return s;
+    const GateRun& g = P.gate_runs[P.steps[s].gates];
+    const bool inner = P.steps[s].a == t && s > g.first;
+    return inner || t == g.leaf ? s : g.first + g.n - 1;
+  };
   std::vector<int32_t> birth(N), death(N);
   for (int32_t t = 0; t < N; ++t) {
     TensorRec& R = P.tensors[t];
     birth[t] = t < T ? -1 : writes(R.producer);
-    death[t] = R.consumer < 0 ? S : reads(R.consumer);
+    death[t] = R.consumer < 0 ? S : std::max(reads(R.consumer), run_reads(t, R.consumer));
     if (R.pinned) {
       birth[t] = -1;
       death[t] = kInf;
@@ -1003,6 +1039,7 @@ void assign_workspace(Plan& P, int64_t batch, bool level_order) {
       if (time && mem) P.workspace_ok = false;
     }
   }
+  P.workspace_ok = P.workspace_ok && gate_runs_ok(P);
   int64_t cur = P.arena_bytes;
   // cross-slice accumulator [sum re, sum im, comp re, comp im] per output element: only
   // calls of more than one pass keep it between passes (the last pass writes the output)

@@ -191,6 +191,7 @@ struct tn_server_s {
     Plan path_order;  // the batched kernel runs the steps one after another: the smaller arena
     if (simt_only && P.batch == 1) {
       path_order = P;
+      drop_gate_runs(path_order);
       assign_workspace(path_order, 1, false);
     }
     if (simt_only && P.batch == 1 && path_order.workspace_ok && batch_template(path_order, pt.T, why)) {

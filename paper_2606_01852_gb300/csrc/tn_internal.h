@@ -220,6 +220,8 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
 // runs its steps by tree level, so every tensor it touches is alive for the whole chain; else
 // (no chain is launched, or memory is short) tensors live in path order, and chains run in it.
 void assign_workspace(Plan& P, int64_t batch, bool level_order = true);
+// Every step of the plan as a launch of its own (before assign_workspace: lifetimes without runs).
+void drop_gate_runs(Plan& P);
 
 // executor (launches only, capturable in a CUDA graph)
 tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t count,
