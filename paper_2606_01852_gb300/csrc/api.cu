@@ -41,6 +41,7 @@ int64_t batch_footprint(Plan& P, int64_t b, int64_t budget) {
     drop_gate_runs(P);
     return batch_footprint(P, b, budget);
   }
+  if (P.total_bytes > budget && b == 1 && !P.chains.empty()) smallest_workspace(P);
   return P.total_bytes;
 }
 

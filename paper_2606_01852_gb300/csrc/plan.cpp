@@ -837,6 +837,7 @@ static void find_chains(Plan& P, int64_t batch, bool level_order) {
   P.chains.clear();
   P.chain_tasks.clear();
   P.chain_levels.clear();
+  if (P.step_by_step) return;
   const int64_t cw = P.is_complex ? 4 : 1;
   auto tiny = [&](const StepRec& st) {
     return st.cls == TN_CLASS_SIMT && st.ksplit == 1 &&
@@ -902,6 +903,12 @@ void drop_gate_runs(Plan& P) {
   for (StepRec& st : P.steps) st.gates = -1;
   for (LeafDesc& d : P.leafdesc) d.direct = 0;
   P.gate_runs.clear();
+}
+
+void smallest_workspace(Plan& P) {
+  drop_gate_runs(P);
+  P.step_by_step = true;
+  assign_workspace(P, P.batch, false);
 }
 
 // Every gate run's output apart from all that exists when the run starts and is read in it or after

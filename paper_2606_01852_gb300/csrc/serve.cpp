@@ -49,6 +49,7 @@ struct Instance {
 };
 
 struct PlanPool {
+  std::unique_ptr<Plan> smallest;  // the plan in the least memory (made when it exceeds the budget)
   std::vector<std::unique_ptr<Instance>> inst;
 };
 
@@ -380,7 +381,17 @@ struct tn_server_s {
     PlanPool& pool = pools[plan->P.uid];
     for (auto& in : pool.inst)
       if (!in->busy) return in.get();
-    const int64_t need = plan->P.total_bytes;
+    // chains in level order, their tables and gate runs may take the workspace past a budget that the
+    // plan's steps one by one fit
+    const Plan* layout = &plan->P;
+    if (cfg.hbm_budget_bytes > 0 && layout->total_bytes > cfg.hbm_budget_bytes) {
+      if (!pool.smallest) {
+        pool.smallest = std::make_unique<Plan>(*layout);
+        smallest_workspace(*pool.smallest);
+      }
+      if (pool.smallest->workspace_ok) layout = pool.smallest.get();
+    }
+    const int64_t need = layout->total_bytes;
     if (cfg.hbm_budget_bytes > 0 && hbm_in_use + need > cfg.hbm_budget_bytes) evict_idle(need);
     if (cfg.hbm_budget_bytes > 0 && hbm_in_use + need > cfg.hbm_budget_bytes) {
       if (running.empty()) {
@@ -390,7 +401,7 @@ struct tn_server_s {
       return nullptr;
     }
     auto in = std::make_unique<Instance>();
-    in->P = plan->P;
+    in->P = *layout;
     in->P.dev = nullptr;
     void* mem = nullptr;
     if (cudaMalloc(&mem, (size_t)need) != cudaSuccess) {

@@ -171,6 +171,7 @@ struct Plan {
   int64_t n_rec_unbatched = 0, n_rec_total = 0;
   int64_t off_leafdesc = 0;         // LeafDesc table
   int64_t off_chain = 0;            // ChainStep table of the step chains
+  bool step_by_step = false;        // neither chains nor gate runs (smallest_workspace)
   std::vector<GateRun> gate_runs;
   std::vector<ChainRec> chains;
   std::vector<int32_t> chain_tasks;   // ChainTask, four ints each
@@ -222,6 +223,8 @@ tn_status build_plan(const tn_network* net, const tn_path* path, const int32_t* 
 void assign_workspace(Plan& P, int64_t batch, bool level_order = true);
 // Every step of the plan as a launch of its own (before assign_workspace: lifetimes without runs).
 void drop_gate_runs(Plan& P);
+// The least memory that the plan runs in: a launch per step, tensors in path order.
+void smallest_workspace(Plan& P);
 
 // executor (launches only, capturable in a CUDA graph)
 tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t count,
