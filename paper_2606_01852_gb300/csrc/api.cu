@@ -108,6 +108,8 @@ tn_status check_device_error(Plan& P) {
   return TN_OK;
 }
 
+cudaError_t uploads_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 tn_status upload_tables(Plan& P) {
   if (!P.dev) return TN_OK;
   for (int32_t t = 0; t < P.n_leaves; ++t) P.leafdesc[t].dst = P.tensors[t].offset;
@@ -163,6 +165,7 @@ tn_status upload_tables(Plan& P) {
   if (e == cudaSuccess && !table.empty())
     e = cudaMemcpy(P.dev + P.off_chain_levels, P.chain_levels.data(), 4 * P.chain_levels.size(),
                    cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = uploads_done();
   if (e != cudaSuccess) {
     set_error(std::string("writing the plan's tables: ") + cudaGetErrorString(e));
     return TN_ERR_CUDA;

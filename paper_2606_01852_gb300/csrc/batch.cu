@@ -824,7 +824,8 @@ tn_status tn_batch_plan(int32_t n_nets, const tn_network* nets, const tn_path* p
         cudaMemcpy(B->d_leaves, B->leaves.data(), sizeof(BLeaf) * B->leaves.size(), cudaMemcpyHostToDevice) !=
             cudaSuccess ||
         (!B->steps.empty() && cudaMemcpy(B->d_steps, B->steps.data(), sizeof(BStep) * B->steps.size(),
-                                         cudaMemcpyHostToDevice) != cudaSuccess)) {
+                                         cudaMemcpyHostToDevice) != cudaSuccess) ||
+        uploads_done() != cudaSuccess) {
       cudaFree(mem);
       set_error("tn_batch_plan: table upload failed");
       return TN_ERR_CUDA;

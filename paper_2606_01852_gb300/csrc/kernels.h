@@ -114,6 +114,10 @@ cudaError_t launch_contract_chain(const ChainStep* steps, const ChainTask* tasks
                                   int32_t n_levels, int32_t ctas, int32_t nb, bool skip_unbatched, bool cplx,
                                   bool maxplus, cudaStream_t st);
 
+// Wait for cudaMemcpy calls from pageable memory: such a call may return when its bytes are staged,
+// before they are on the device, and a non-blocking stream does not wait for the legacy stream.
+cudaError_t uploads_done();
+
 // Small leaves: one CTA per leaf. Large leaves (LeafDesc::tiled): the tiled permutation
 // kernel, one launch per leaf; host_descs is the host copy of the table (grid sizes). inputs: the
 // caller's leaves, which the launches carry as parameters. errw != nullptr: set to 0. skip_direct: leaves
