@@ -267,10 +267,6 @@ __device__ __forceinline__ int run_panels(float* ar, const BStep* S, int m, int 
   return mx;
 }
 
-// Step outputs whose exponents a team keeps (bytes of shared memory per CTA / per warp's share):
-// networks with more steps renormalise each output in place.
-constexpr int kExpBytes = 2048;
-
 // CTAs of at most this many threads take the form with register tiles (128 registers a thread);
 // wider ones, which the autotuner does not try, run one output per thread
 constexpr int kTileThreads = 256;
@@ -555,27 +551,11 @@ struct tn_batch_s {
 
 namespace tn {
 
-// The kernel of a form, allowed all the shared memory that a CTA may take beside its static part
-// (once: launches of several threads do not meet in it).
 using BatchKernel = void (*)(const BNet*, const BLeaf*, const BStep*, int32_t, const float*, float*, int32_t*, int32_t,
                              double*, double*, int32_t, int32_t);
-static cudaError_t allow_smem(BatchKernel kernel) {
-  cudaFuncAttributes fa{};
-  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(kMaxSmemPerCta - static_cast<int64_t>(fa.sharedSizeBytes)));
-}
 template <bool CPLX, bool MAXPLUS, bool WARP>
-BatchKernel batch_form(bool tiles, cudaError_t& e) {
-  if (tiles) {
-    static const cudaError_t set = allow_smem(batch_kernel<CPLX, MAXPLUS, WARP, true>);
-    e = set;
-    return batch_kernel<CPLX, MAXPLUS, WARP, true>;
-  }
-  static const cudaError_t set = allow_smem(batch_kernel<CPLX, MAXPLUS, WARP, false>);
-  e = set;
-  return batch_kernel<CPLX, MAXPLUS, WARP, false>;
+BatchKernel batch_form(bool tiles) {
+  return tiles ? batch_kernel<CPLX, MAXPLUS, WARP, true> : batch_kernel<CPLX, MAXPLUS, WARP, false>;
 }
 
 cudaError_t launch_batch_kernel(const BNet* nets, const BLeaf* leaves, const BStep* steps, int32_t n_nets,
@@ -590,10 +570,15 @@ cudaError_t launch_batch_kernel(const BNet* nets, const BLeaf* leaves, const BSt
   smem_arena &= ~63;  // arenas are multiples of 64 floats
   const int smem = (smem_arena + tab_ints) * 4 * (warp ? threads / 32 : 1);
   const bool tiles = threads <= kTileThreads;
-  auto kernel = warp ? (cplx ? batch_form<true, false, true>(tiles, e)
-                             : maxplus ? batch_form<false, true, true>(tiles, e) : batch_form<false, false, true>(tiles, e))
-                     : (cplx ? batch_form<true, false, false>(tiles, e)
-                             : maxplus ? batch_form<false, true, false>(tiles, e) : batch_form<false, false, false>(tiles, e));
+  auto kernel = warp ? (cplx ? batch_form<true, false, true>(tiles)
+                             : maxplus ? batch_form<false, true, true>(tiles) : batch_form<false, false, true>(tiles))
+                     : (cplx ? batch_form<true, false, false>(tiles)
+                             : maxplus ? batch_form<false, true, false>(tiles) : batch_form<false, false, false>(tiles));
+  // (an allowance belongs to the current device, so each launch that needs one sets it;
+  // always the largest, so launches of several threads do not meet in it)
+  if (smem + kBatchStaticSmem > kDefaultSmem)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kMaxSmemPerCta) - kBatchStaticSmem);
   if (e != cudaSuccess) return e;
   kernel<<<grid, threads, smem, st>>>(nets, leaves, steps, n_nets, in, arena, queue, maxplus ? 0 : sc, values, logs,
                                       smem_arena, tab_ints);

@@ -64,6 +64,12 @@ struct BatchTemplate {
 // element by element)
 constexpr int32_t kMaxTabInts = 4096;
 
+// Step outputs whose exponents a team keeps (bytes of shared memory per CTA / per warp's share):
+// networks with more steps renormalise each output in place.
+constexpr int kExpBytes = 2048;
+// the kernel's static shared memory at most: the exponents, two step records, scalars
+constexpr int kBatchStaticSmem = kExpBytes + 2 * int(sizeof(BStep)) + 64;
+
 constexpr int64_t kMaxSmemPerCta = 227 * 1024;  // dynamic shared memory one CTA may take
 constexpr int64_t kSmemPerSm = 224 * 1024;      // what the SM's resident CTAs share (with headroom)
 

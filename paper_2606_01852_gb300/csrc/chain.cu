@@ -16,6 +16,7 @@
 // of a lane's chain: a level was ~2000 clocks for 2 terms and 300 more for every 4, nearly all of
 // it branches and dependent loads of the dims, and is ~1500 and 60 now. (Software-pipelined or
 // 16-term groups were slower: spills, and instructions that one CTA runs once cost their fetch.)
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 
@@ -261,32 +262,45 @@ __global__ void __launch_bounds__(kChainThreads) contract_chain_kernel(const Cha
   }
 }
 
+// kChainMaxCtas if the kernel may take and the device has room for so large a cluster, else 8. The
+// allowance (clusters above 8 are not portable) belongs to the current device, so each
+// launch that needs it sets it; the room is the device's, asked for once.
+template <bool CPLX, bool MAXPLUS>
+int largest_cluster() {
+  auto kern = contract_chain_kernel<CPLX, MAXPLUS>;
+  int dev = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 8;
+  }
+  constexpr int kKnown = 64;
+  static std::atomic<int> known[kKnown];
+  const int slot = dev < kKnown ? dev : -1;
+  int most = slot >= 0 ? known[slot].load(std::memory_order_relaxed) : 0;
+  if (most > 0) return most;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kChainMaxCtas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(kChainMaxCtas);
+  cfg.blockDim = dim3(kChainThreads);
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  most = 8;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) cudaGetLastError();
+  else if (n >= 1) most = kChainMaxCtas;
+  if (slot >= 0) known[slot].store(most, std::memory_order_relaxed);
+  return most;
+}
+
 template <bool CPLX, bool MAXPLUS>
 cudaError_t launch(const ChainStep* steps, const ChainTask* tasks, const int32_t* levels, int32_t n_levels,
                    int32_t ctas, int32_t nb, bool skip_unbatched, cudaStream_t st) {
   auto kern = contract_chain_kernel<CPLX, MAXPLUS>;
-  // clusters of 16 need the non-portable size and room for one on the device
-  static const int most = [kern] {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      cudaGetLastError();
-      return 8;
-    }
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kChainMaxCtas;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3(kChainMaxCtas);
-    cfg.blockDim = dim3(kChainThreads);
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      return 8;
-    }
-    return static_cast<int>(kChainMaxCtas);
-  }();
+  const int most = n_levels > 1 && ctas > 8 ? largest_cluster<CPLX, MAXPLUS>() : 8;
   // one level: no barrier, so no cluster and no limit on the CTAs
   const int c = n_levels == 1 || ctas < most ? ctas : most;
   cudaLaunchConfig_t cfg{};

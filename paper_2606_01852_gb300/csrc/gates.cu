@@ -208,14 +208,17 @@ __global__ void __launch_bounds__(kThreads, 6) gate_run_kernel(const __grid_cons
 
 template <bool CPLX>
 static cudaError_t launch(const GateArgs& a, cudaStream_t st) {
-  // (once, for the largest tile and matrices: launches of several threads do not meet in it)
   constexpr int elem = CPLX ? 8 : 4;
-  static const cudaError_t configured =
-      cudaFuncSetAttribute(gate_run_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (elem << kGateTileBits) + kGateMaxRun * 256 * int(sizeof(float2)));
-  if (configured != cudaSuccess) return configured;
+  constexpr int fixed = 2 * kIters * int(sizeof(Round)) + 2 * int(sizeof(int64_t));  // the kernel's own arrays
   int bytes = elem << a.t;
   for (int g = 0; g < a.n_gates; ++g) bytes += int(sizeof(float2)) << (2 * a.gate[g].bits);
+  // (an allowance belongs to the current device, so each launch that needs one sets it;
+  // always the largest, so launches of several threads do not meet in it)
+  if (bytes + fixed > kDefaultSmem) {
+    const cudaError_t e = cudaFuncSetAttribute(gate_run_kernel<CPLX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (elem << kGateTileBits) + kGateMaxRun * 256 * int(sizeof(float2)));
+    if (e != cudaSuccess) return e;
+  }
   gate_run_kernel<CPLX><<<1u << a.outer, kThreads, bytes, st>>>(a);
   return cudaGetLastError();
 }

@@ -469,9 +469,7 @@ __global__ void simt_combine_kernel(StepArgs a, int32_t nb, int32_t cplx) {
 
 template <typename G>
 void launch(const StepArgs& a, int32_t nb, cudaStream_t st) {
-  static const bool set = cudaFuncSetAttribute(contract_simt_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               G::SMEM) == cudaSuccess;
-  (void)set;
+  static_assert(G::SMEM <= kDefaultSmem, "no allowance to set");
   const int64_t tiles = ((a.m + G::M - 1) / G::M) * ((a.n + G::N - 1) / G::N);
   dim3 grid((unsigned)tiles, (unsigned)nb, (unsigned)(a.ksplit > 1 ? a.ksplit : 1));
   launch_pdl(contract_simt_kernel<G>, grid, G::THREADS, G::SMEM, st, a);

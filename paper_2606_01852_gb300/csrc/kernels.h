@@ -114,6 +114,9 @@ cudaError_t launch_contract_chain(const ChainStep* steps, const ChainTask* tasks
                                   int32_t n_levels, int32_t ctas, int32_t nb, bool skip_unbatched, bool cplx,
                                   bool maxplus, cudaStream_t st);
 
+// Shared memory that any kernel may take without an allowance.
+constexpr int kDefaultSmem = 48 * 1024;
+
 // Wait for cudaMemcpy calls from pageable memory: such a call may return when its bytes are staged,
 // before they are on the device, and a non-blocking stream does not wait for the legacy stream.
 cudaError_t uploads_done();
