@@ -2,6 +2,7 @@
 // which packs compatible small requests into one launch of the same kernel.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -72,6 +73,13 @@ constexpr int kBatchStaticSmem = kExpBytes + 2 * int(sizeof(BStep)) + 64;
 
 constexpr int64_t kMaxSmemPerCta = 227 * 1024;  // dynamic shared memory one CTA may take
 constexpr int64_t kSmemPerSm = 224 * 1024;      // what the SM's resident CTAs share (with headroom)
+
+// Floats of the shared-memory arena of a packed launch's CTAs, per_sm of them on an SM together with
+// their offset tables: an SM's 228 KB hold, per CTA, 1 KB of the system's and the static part too.
+inline int32_t pack_arena_floats(int per_sm, int32_t tab_ints, int64_t max_arena) {
+  const int64_t share = std::min(int64_t(228 * 1024) / per_sm - 1024, kMaxSmemPerCta) - kBatchStaticSmem;
+  return static_cast<int32_t>(std::max<int64_t>(0, std::min(share / 256 * 64 - tab_ints, max_arena)));
+}
 
 // Tables of a closed, unsliced network from its plan (workspace assigned for one copy, no
 // tensor-core steps); false with a reason when the batched kernel cannot run it.

@@ -321,8 +321,7 @@ struct tn_server_s {
     const int threads = few ? 256 : 128;
     const int per_sm = few ? (int)((n + num_sms - 1) / num_sms) : 4;
     const int grid = (int)std::min<size_t>(n, (size_t)num_sms * per_sm);
-    const int32_t smem_arena = (int32_t)std::max<int64_t>(
-        0, std::min<int64_t>(std::min(kSmemPerSm / per_sm, kMaxSmemPerCta - 4096) / 4 - tab_ints, max_arena));
+    const int32_t smem_arena = pack_arena_floats(per_sm, tab_ints, max_arena);
     double* vals = reinterpret_cast<double*>(d + off_out);
     double* logs = vals + 2 * n;
     if (e == cudaSuccess)
