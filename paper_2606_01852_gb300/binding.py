@@ -151,7 +151,7 @@ def _load():
         "tn_selftest_bounded_wait": [vp, i32, i64, vp],
         "tn_serve_create": [C.POINTER(tn_serve_config), C.POINTER(vp)],
         "tn_serve_submit": [vp, vp, C.POINTER(vp), C.POINTER(u64)],
-        "tn_serve_submit_batch": [vp, i32, C.POINTER(vp), C.POINTER(vp), C.POINTER(u64)],
+        "tn_serve_submit_batch": [vp, i32, C.POINTER(vp), vp, C.POINTER(u64)],
         "tn_serve_poll": [vp, u64, vp, vp, i32],
         "tn_serve_destroy": [vp],
         "tn_serve_stats_get": [vp, C.POINTER(tn_serve_stats)],
