@@ -245,7 +245,9 @@ tn_status tn_plan_layout(tn_plan_t plan, int32_t id, int32_t* modes_out, int32_t
 /* The number of kernel launches one tn_contract_slices call over slice_count slices makes
  * (the same for any first slice): staging, every step (two for split-k steps, several for a
  * deep step on paired SMs, launched in bands of tiles; one for a run of gates), and the slice sum
- * (none where a run of gates writes the output), per pass. */
+ * (none where a run of gates writes the output), per pass. A call whose output or log scale
+ * overlaps a leaf that a run of gates reads directly makes a launch for each of its steps
+ * instead, with the leaf's staging and the output's widening; it is not counted here. */
 tn_status tn_plan_launches(tn_plan_t plan, int64_t slice_count, int64_t* out);
 
 /* Description of step s (host only). */

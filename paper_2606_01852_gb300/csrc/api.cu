@@ -204,13 +204,18 @@ tn_status run_slices(Plan& P, const void* const* inputs, int64_t begin, int64_t 
   int64_t* ref = reinterpret_cast<int64_t*>(P.dev + P.off_ref);
   int* errw = reinterpret_cast<int*>(P.dev + P.off_err);
   const int64_t npass = (count + P.batch - 1) / P.batch;
-  // gate runs read leaves where they are and write the output as they go: not where these overlap
+  // gate runs read leaves where they are and write the output and the log scale as they go: not
+  // where these overlap
   bool runs = !P.gate_runs.empty();
   for (const GateRun& g : P.gate_runs) {
     if (g.leaf < 0) continue;
-    const uintptr_t x = reinterpret_cast<uintptr_t>(inputs[g.leaf]), y = reinterpret_cast<uintptr_t>(output);
-    const uintptr_t nx = static_cast<uintptr_t>(P.tensors[g.leaf].size * elem_bytes(P)), ny = static_cast<uintptr_t>(P.out_elems * (cplx ? 16 : 8));
-    runs = runs && (x + nx <= y || y + ny <= x);
+    const uintptr_t x = reinterpret_cast<uintptr_t>(inputs[g.leaf]);
+    const uintptr_t nx = static_cast<uintptr_t>(P.tensors[g.leaf].size * elem_bytes(P));
+    auto apart = [&](const void* p, int64_t bytes) {
+      const uintptr_t y = reinterpret_cast<uintptr_t>(p);
+      return p == nullptr || x + nx <= y || y + static_cast<uintptr_t>(bytes) <= x;
+    };
+    runs = runs && apart(output, P.out_elems * (cplx ? 16 : 8)) && apart(log_scale, sizeof(double));
   }
   for (int64_t p = 0; p < npass; ++p) {
     const int32_t nb = (int32_t)std::min<int64_t>(P.batch, count - p * P.batch);

@@ -78,3 +78,23 @@ def test_kicked_ising():
     plan.destroy()
     assert len(set(got)) == 1
     assert abs(got[0] - oracle.contract(net, path)) < FP32_BAR
+
+
+def test_log_scale_in_the_leaf():
+    """The log scale (0 without scaling) in the memory of the leaf that the run reads: the general path, with
+    the bits of separate buffers."""
+    tn = ensure_built()
+    net, path = gate_network(18, 4, 2, seed=5)
+    plan = tn.Plan(net, path)
+    tensors = [torch.tensor(np.asarray(t)).to(torch.complex64).cuda() for t in net.tensors]
+    out = torch.zeros(1 << 18, dtype=torch.complex128, device="cuda")
+    plan.contract(tensors, out)
+    want = bits(out).clone()
+    plan.profile(True)
+    plan.contract(tensors, out)
+    assert plan.profile_read()["launches"][tn.TN_CLASS_STREAM] == 1
+    inside = tensors[0].reshape(-1)[1000:1001].view(torch.float64)
+    plan.contract(tensors, out, inside)
+    assert plan.profile_read()["launches"][tn.TN_CLASS_STREAM] == 4
+    assert torch.equal(bits(out), want) and inside.item() == 0.0
+    plan.destroy()
