@@ -541,13 +541,15 @@ def run_ours(args):
         prec, fpk["source"]["alu"]) if cls == 2 else (peaks["_source"] if cls in (1, 3, 4) else fpk["source"]["alu"])
     path_roof = path_roofline(plan, prec, semiring, peaks, ms_max, cplx, count=round(slices_per_step), form=form)
     perm = None
-    if prof["launches"][4] > 0 and prof["ms"][4] > 0:
+    # (a leaf that a run of gates reads where the caller has it is not staged)
+    tiled = [t for t in range(len(w.net.modes)) if plan.tensor(t)["tiled"]]
+    staged = [t for t in tiled if plan.tensor(t)["consumer"] < 0 or plan.step(plan.tensor(t)["consumer"])["gate_run"] < 0]
+    if prof["launches"][4] > 0 and prof["ms"][4] > 0 and (staged or not tiled):
         # leaf staging (the permutation kernels): staged bytes read + written over its event time
         gbs = prof["bytes"][4] / (prof["ms"][4] / 1e3) / 1e9
         perm = {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": gbs / peaks["hbm_gbs"], "bytes_per_step": prof["bytes"][4] / args.steps,
-                "ms_per_step": prof["ms"][4] / args.steps, "tiled_leaves": sum(
-                    1 for t in range(len(w.net.modes)) if plan.tensor(t)["tiled"])}
+                "ms_per_step": prof["ms"][4] / args.steps, "tiled_leaves": len(staged)}
 
     # end to end through the public C ABI with host buffers
     host_in = [np.ascontiguousarray(np.asarray(t, dtype=np.complex64 if cplx else np.float32))
