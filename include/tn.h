@@ -185,7 +185,8 @@ typedef struct {
   int32_t tiled;           /* leaves: staged by the tiled permutation kernel (one launch per
                               pass that stages it) rather than the per-leaf kernel: 1 its
                               general form, 2 its pipelined form (each index group one 32-wide
-                              chunk, 16-byte loads; used when the source is 16-byte aligned) */
+                              chunk, 16-byte loads; used when the source is 16-byte aligned);
+                              not staged where a run of gates reads it in place */
 } tn_tensor_info;
 
 /* Rates of the kernel choice, the roofline cost model of Sec. IV-C Eq. 6: a step's time

@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(Cfg<REAL>::THREADS, REAL ? 2 : 1)
 //
 // Measured (GB300; before: 128 x 256 real, 128 x 128 complex tiles, A in shared memory, MMAs
 // issued from a divergent lane): real 16384 x 32768 x 1024 7.87 -> 5.21 ms (140 -> 211 TFLOP/s),
-// 2048 x 16384 x 8192 166 -> 234; complex 4096^3 231 -> 305, few tiles: 512 x 128 x 2048 179 -> 51 us,
+// 2048 x 16384 x 8192 166 -> 234; complex 4096^3 231 -> 305, few tiles: 512 x 128 x 2048 178 -> 53 us,
 // 256 x 256 x 256 36 -> 14 us. cuBLAS's sustained TF32 rate over three products is 305.
 // BT rows of B per plane; the narrow tiles (64 real, 32 complex) put a small step's outputs on
 // more SMs.

@@ -55,8 +55,8 @@ struct LeafDesc {
   // order outside the output group, slowest first) and the rest (rpos[0..nr-1]). A CTA
   // moves one 32 x 32 tile (output-group index x input-group index) through shared
   // memory, reading along the input group and writing along the output group.
-  int32_t direct;                  // read by a gate run where the caller has it
   int32_t tiled;                   // staged by the tiled kernel (else by the per-leaf kernel)
+  int32_t direct;                  // (any leaf) read by a gate run where the caller has it
   int32_t no, ni, nr;
   int32_t load_o;                  // the declared order's innermost position is in the
                                    // output group: load along it instead
@@ -183,7 +183,7 @@ struct Plan {
   bool workspace_ok = false;        // liveness assignment passed its self-check
   // device state
   char* dev = nullptr;
-  std::vector<LeafDesc> leafdesc;   // host copy; src filled per call
+  std::vector<LeafDesc> leafdesc;   // host copy; dst filled when the tables are uploaded
   int num_sms = 148;
   // per-class timing (tn_plan_profile): event pairs around step launches
   struct ProfRec {

@@ -23,8 +23,8 @@
   ktri44    : kicked Ising on a 4x4 triangular lattice, 8 Trotter steps;
   tcgemm    : one dense step of the 14-cycle circuit's shape (2^14 x 2^14 outputs, k = 2^13), the
               small case the tensor-core kernel is profiled on;
-  sv26      : a 2^26-element state leaf in a shuffled declared order absorbing 4 gates (the
-              large-leaf permutation case);
+  sv26      : a 2^26-element state leaf in a shuffled declared order absorbing 4 gates (one
+              gate run; with scaling or slices the large-leaf permutation case);
   kings16   : maximum independent set of a 16x16 King's subgraph (site density 0.8, seed 1;
               209 vertices), contracted in the max-plus semiring (FP32, exact integers);
   kings_batch: maximum independent sets of many King's subgraphs (L in [4, 7], density 0.8),
@@ -146,7 +146,7 @@ def rc40open():
 def sv26():
     """A 26-qubit state (one 2^26-element leaf, 512 MiB in complex64) declared in a shuffled
     qubit order, absorbing four Haar-random two-qubit gates; the open output is the new
-    state in qubit order. Its leaf is the permutation the staging kernel exists for."""
+    state in qubit order. One gate run; a plan with scaling or slices stages the permuted leaf."""
     net = circuits.state_network(26, 4, 26)
     return Workload(net.name, net, circuits.state_path(net), (), {})
 
