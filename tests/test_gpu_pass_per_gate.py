@@ -93,3 +93,31 @@ def test_permuted_state(tn, qubits, seed):
     contract(tn, plan, leaves, out, 3, 8 << qubits)
     plan.destroy()
     assert torch.equal(torch.view_as_real(out).view(torch.int64), torch.view_as_real(want).view(torch.int64))
+
+
+@pytest.mark.parametrize("arity", [1, 4])
+def test_a_single_gate_is_not_slower_in_a_run(tn, arity):
+    """One gate on a real 26-qubit state: the run (which saves the staging and the widening) against the launch
+    per step of a call whose output overlaps the leaf, the best of several calls each."""
+    net, path = gate_chain_network(n_qubits=26, n_gates=1, seed=60 + arity, arity=arity, real=True)
+    plan = tn.Plan(net, path, prec="r32_fp32")
+    assert plan.step(0)["gate_run"] == 0
+    tensors = [torch.tensor(np.asarray(t)).to(torch.float32).cuda() for t in net.tensors]
+    out = torch.zeros(1 << 26, dtype=torch.float64, device="cuda")
+    leaves, over = overlapping(tensors, 1 << 26, True)
+
+    def best(ins, o):
+        times = []
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            leaves[0].copy_(tensors[0].reshape(-1))
+            e0.record()
+            plan.contract(ins, o)
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1))
+        return min(times)
+
+    run, steps = best(tensors, out), best(leaves, over)
+    plan.destroy()
+    assert run < steps
